@@ -194,3 +194,41 @@ def tolerance(case: dict):
     if case["op"] in ("encode", "dequant"):
         return "exact"
     return {"rel": 7e-3} if case.get("dtype") == "bf16" else {"rel": 8e-4}
+
+
+def _pot_values(n: int, k: int, bits: int, group: int, dtype: str, gen: torch.Generator) -> torch.Tensor:
+    """The weights that `_codes` stands for, [n, k] FP64, from the format's definition: sign * 2^E * scale with the top level on
+    the group's largest magnitude, the scale an FP16 number (rounded once to BF16 for BF16 products)."""
+    w, qmax = _weights(n, k, gen), (1 << (bits - 1)) - 1
+    out = torch.empty(n, k, dtype=torch.float64, device="cuda")
+    for r in range(0, n, 2048):
+        g = w[r:r + 2048].double().view(-1, k // group, group)
+        s = (g.abs().amax(2, keepdim=True) * 2.0 ** -qmax).clamp(2.0 ** -14, (2 - 2.0 ** -10) * 2.0 ** (15 - qmax)).to(torch.float16).double()
+        level = torch.ones_like(g)
+        for e in range(qmax):  # |w| / s above 2^(e + 1/2)
+            level = torch.where(g * g > s * s * 2.0 ** (2 * e + 1), 2.0 ** (e + 1), level)
+        if dtype == "bf16":
+            s = s.to(torch.bfloat16).double()
+        out[r:r + 2048] = torch.where(g < 0, -level, level).mul_(s).view(-1, k)
+    return out
+
+
+def exact(case: dict, seed: int):
+    """What `run` returns for these inputs, in FP64 from plain torch; the encoder's results are whole numbers."""
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    op, bits, group = case["op"], case["bits"], case["group"]
+    if op == "encode":
+        return None
+    if op == "decode":
+        h, f = case["hidden"], case["ffn"]
+        ys = []
+        for _ in range(case["layers"]):
+            for n, k in ((3 * h, h), (h, h), (f, h), (f, h), (h, f)):
+                w = _pot_values(n, k, bits, group, "f16", gen)
+                ys.append(w @ _activations(1, k, "f16", gen)[0].double())
+        return ys
+    w = _pot_values(case["n"], case["k"], bits, group, case["dtype"], gen)
+    if op == "dequant":
+        return w
+    x = _activations(case.get("m", 1), case["k"], case["dtype"], gen).double()
+    return w @ x[0] if op == "gemv" else x @ w.T
