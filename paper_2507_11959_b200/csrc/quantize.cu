@@ -1,8 +1,9 @@
-// Set-up kernels: reference quantizers (Eq. 2 and the uniform twin), scale validation and the
-// canonical <-> tiled repack.  None of these is on the timed path; they are written for
-// exactness (FP64 threshold tests, correctly rounded conversions), not speed.
+// Bringing in a matrix: the quantizers (Eq. 2 with its scale rules, and the uniform twin), scale validation and the
+// canonical <-> tiled repack.  Results are exact (exact threshold tests, correctly rounded conversions).
 #include "common.cuh"
 #include "layout.cuh"
+
+#include <type_traits>
 
 namespace pot {
 
@@ -14,12 +15,345 @@ __device__ __forceinline__ uint16_t clamp_scale_bits(uint16_t sb, int bits) {
     return sb < lo ? lo : (sb > hi ? hi : sb);
 }
 
-// One warp per group.  codes are staged in shared memory, then packed 32 bits at a time.
-// rule 0: top level on max|w|; 1: Algorithm 1's s0; 2: given; 3: Algorithm 1's grid search.
-template <int BITS, bool UNIFORM>
-__global__ void __launch_bounds__(256) quantize_kernel(const __half* __restrict__ W, int64_t N, int64_t K, int G,
-                                                       int rule, __half* __restrict__ S, __half* __restrict__ Z,
-                                                       uint32_t* __restrict__ packed) {
+// ------------------------------------------------------------------------------------------
+// PoT quantizer
+// ------------------------------------------------------------------------------------------
+// Eq. 2 by exact comparisons in FP32: E >= k + 1  <=>  |w| / S > 2^(k + 1/2)  <=>  w^2 > 4^k (2 S^2).  The squares of two
+// FP16 numbers have 22 significant bits and exponents from 2^-48 to 2^32, so both sides are exact; as 4^k adds k << 24 to an
+// FP32 pattern, the number of k that satisfy it is the difference of the patterns, rounded up to a multiple of 2^24.
+template <int BITS>
+__device__ __forceinline__ uint32_t pot_code(uint32_t h, float two_s2) {
+    const float w = __half2float(__ushort_as_half((uint16_t)h));
+    const float w2 = w * w;
+    const int steps = ((__float_as_int(w2) - __float_as_int(two_s2) - 1) >> 24) + 1;
+    const uint32_t E = w2 > two_s2 ? (uint32_t)min(steps, qmax_of(BITS)) : 0u;
+    return w < 0.f ? E | (1u << (BITS - 1)) : E;
+}
+__device__ __forceinline__ float pot_two_s2(uint16_t sb) {
+    const float S = __half2float(__ushort_as_half(sb));
+    return 2.f * (S * S);
+}
+
+// Rules TOP, PAPER_S0 and GIVEN.  Bound by HBM (2 bytes read and BITS / 8 written per weight): a thread takes 8 consecutive
+// weights with one 16-byte load, G / 8 neighbouring lanes share a group and find its largest magnitude with shuffles on the
+// FP16 patterns, and the 8 BITS bits of a thread leave as whole words (n = 3: four lanes give three words).  QZ_UNROLL loads
+// per thread are in flight.  11008 x 4096: 40 us at 3 bits (before, one warp per group in FP64 and codes packed bit by bit:
+// 299 us), 36 us at 2 and 4 bits (329, 483 us); the ALU pipe is what is left (156 instructions per 8 weights).
+constexpr int QZ_THREADS = 256;
+constexpr int QZ_UNROLL = 2;
+
+template <int BITS>
+__global__ void __launch_bounds__(QZ_THREADS) pot_quantize_kernel(const uint4* __restrict__ W, int64_t pieces, int ppg_shift,
+                                                                  int rule, uint16_t* __restrict__ S,
+                                                                  uint32_t* __restrict__ packed) {
+    constexpr int QMAX = qmax_of(BITS);
+    const int64_t base = (int64_t)blockIdx.x * (QZ_THREADS * QZ_UNROLL) + threadIdx.x;
+    uint4 v[QZ_UNROLL];
+#pragma unroll
+    for (int u = 0; u < QZ_UNROLL; ++u) {
+        const int64_t c = base + u * QZ_THREADS;
+        v[u] = c < pieces ? __ldg(W + c) : make_uint4(0, 0, 0, 0);
+    }
+#pragma unroll
+    for (int u = 0; u < QZ_UNROLL; ++u) {
+        const int64_t c = base + u * QZ_THREADS;   // pieces is a multiple of G / 8: the lanes of a group are all in range or all out
+        const bool live = c < pieces;
+        const uint32_t r[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+        uint16_t sb;
+        if (rule == POT_SCALE_GIVEN) {
+            sb = live ? S[c >> ppg_shift] : (uint16_t)0x0400;
+        } else {
+            __half2 m2 = __habs2(*reinterpret_cast<const __half2*>(&r[0]));  // (the maximum of a number and a NaN is the number)
+#pragma unroll
+            for (int j = 1; j < 4; ++j) m2 = __hmax2(m2, __habs2(*reinterpret_cast<const __half2*>(&r[j])));
+            uint32_t mag = (uint32_t)__half_as_ushort(__hmax(__low2half(m2), __high2half(m2)));
+            if (mag > 0x7C00u) mag = 0;
+            mag = max(mag, __shfl_xor_sync(0xffffffffu, mag, 1));
+            mag = max(mag, __shfl_xor_sync(0xffffffffu, mag, 2));
+            mag = max(mag, __shfl_xor_sync(0xffffffffu, mag, 4));
+            if (ppg_shift == 4) mag = max(mag, __shfl_xor_sync(0xffffffffu, mag, 8));
+            const float amax = __half2float(__ushort_as_half((uint16_t)mag));
+            // PAPER_S0: an 11-bit number over 2^QMAX - 1 <= 127 is either exact or at least 2^-19 of its value away from the
+            // midpoint of two FP16 numbers, so that rounding it to FP32 first changes nothing
+            const float s = rule == POT_SCALE_TOP ? amax * (1.f / (float)(1 << QMAX)) : __fdiv_rn(amax, (float)((1 << QMAX) - 1));
+            sb = clamp_scale_bits(__half_as_ushort(__float2half_rn(s)), BITS);
+            if (live && (c & ((1 << ppg_shift) - 1)) == 0) S[c >> ppg_shift] = sb;
+        }
+        const float two_s2 = pot_two_s2(sb);
+        uint32_t bits = 0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) bits |= pot_code<BITS>((r[j >> 1] >> (16 * (j & 1))) & 0xFFFFu, two_s2) << (j * BITS);
+        if constexpr (BITS == 2) {
+            if (live) reinterpret_cast<uint16_t*>(packed)[c] = (uint16_t)bits;
+        } else if constexpr (BITS == 4) {
+            if (live) packed[c] = bits;
+        } else {
+            const uint32_t next = __shfl_down_sync(0xffffffffu, bits, 1);
+            const int j = (int)(c & 3);
+            if (live && j < 3) packed[(c >> 2) * 3 + j] = (bits >> (8 * j)) | (next << (24 - 8 * j));
+        }
+    }
+}
+
+// Algorithm 1 (rule SEARCH): s0 = max|w| / (2^QMAX - 1); b = 0.01 i, i = 1 .. 200; keep the first minimiser of
+//   Q1(i) = sum_k (|w_k| - s_i 2^E_k(i))^2,  s_i = s0 b,
+// as a plain sequential loop in FP64 (terms in the order k = 0 .. G-1, multiply and add rounded separately) finds it.
+// One warp per group.  Evaluated term by term these are 200 G FP64 terms per group.  Instead
+//   Q1(i) = W2 + D(i),  D(i) = s_i^2 B(i) - 2 s_i A(i),   W2 = sum w^2,  A(i) = sum |w| 2^E(i),  B(i) = sum 4^E(i),
+// and 2^E = 1 + sum_k 2^k [i <= I_k(w)], 4^E = 1 + sum_k 3 4^k [i <= I_k(w)], where I_k(w) is the largest i whose
+// threshold sqrt(2) 2^k s_i lies below |w|: every (weight, k) adds one entry to a histogram over i, and A and B are suffix
+// sums of it.  I_k = I_0 >> k, because s_i scales exactly when i is doubled.  I_0 comes from one FP32 multiplication; where
+// that is too close to an integer the comparison of the sequential loop itself decides.  A and B are integers (A in units of
+// the last place of the group's smallest weight), hence exact.
+// D is evaluated in FP32, off by at most SEARCH_TOL32 T, T = s^2 B + 2 s A (7 roundings of 2^-24 T and the sequential loop's
+// own 131 2^-53 Q1).  A candidate whose lower bound is above the smallest upper bound cannot be the minimiser.  Mostly one
+// candidate is left; else the same bounds in FP64 (SEARCH_TOL64: 16 + 131 roundings of 2^-53), and if several are left even
+// then (equal or all but equal sums) the sequential loop decides between those: the result is that of the plain loop
+// bit for bit.
+// What bounds it: instruction issue (82 % of the issue slots, 750 instructions per group of 128 at 3 bits, two thirds of them the
+// histogram's entries and the 200 evaluations).  11008 x 4096, groups of 128 (64), 3 bits: 9184 us term by term, 280 us so;
+// 4 bits 12424 (12873), 476 (631) us; 2 bits, groups of 64: 5974, 376 us.
+constexpr float SEARCH_TOL32 = 6e-7f;
+constexpr double SEARCH_TOL64 = 2e-14;
+constexpr int SEARCH_BINS = 224;     // 7 candidates per lane; 201 .. 224 stay empty
+constexpr int SEARCH_NC = 7;         // candidates per lane: i = 7 lane + 1 .. 7 lane + 7
+constexpr int SEARCH_LOW_BITS = 22;  // WIDE: A's bins are two 32-bit sums, and no bin of 128 weights x QMAX entries overflows
+
+__device__ __forceinline__ double search_scale(double s0, int i) { return __dmul_rn(s0, __dmul_rn(0.01, (double)i)); }
+
+// The candidates that may be the minimiser: bit c of the result stands for i = 7 lane + 1 + c.  hist: zeroed.
+// WIDE = false: 128 weights times the largest one times 2^QMAX is below 2^32 in units of the last place, so that all sums of A
+// are 32-bit numbers.
+template <int BITS, int PER, bool WIDE>
+__device__ __forceinline__ uint32_t search_candidates(const uint32_t (&h)[PER], uint32_t emin, double s0, uint32_t (&hist)[3][SEARCH_BINS], int lane) {
+    constexpr int QMAX = qmax_of(BITS), NC = SEARCH_NC;
+    using Sum = typename std::conditional<WIDE, uint64_t, uint32_t>::type;
+    const float inv = __fdiv_rn(1.f, (float)(s0 * 0.014142135623730951));
+    Sum sum_a = 0;  // the parts of A and B that all candidates share: the leading terms and the entries with I_k >= 200
+    uint32_t sum_b = PER;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        const uint32_t m = h[j] & 0x7FFFu, e = m >> 10;
+        const float w = __half2float(__ushort_as_half((uint16_t)m));
+        const uint32_t v = m == 0 ? 0u : (e ? (m & 0x3FFu) | 0x400u : m);
+        const Sum vj = (Sum)v << (m == 0 ? 0u : max(e, 1u) - emin);
+        sum_a += vj;
+        const float x = w * inv, near = rintf(x);
+        int I0 = (int)x;  // (x is not an integer unless the test below is true: x is within 3 2^-24 of its value)
+        if (fabsf(x - near) < fmaf(x, 2.5e-7f, 1e-6f)) {
+            const double sc = search_scale(s0, (int)near);
+            I0 = (int)near - 1 + ((double)(w * w) > 2.0 * __dmul_rn(sc, sc) ? 1 : 0);
+        }
+#pragma unroll
+        for (int k = 0; k < QMAX; ++k) {
+            const int I = I0 >> k;
+            if (I >= 200) {
+                sum_a += vj << k;
+                sum_b += 3u << (2 * k);
+            } else if (I >= 1) {
+                const Sum vk = vj << k;
+                if constexpr (WIDE) {
+                    atomicAdd(&hist[0][I - 1], (uint32_t)vk & ((1u << SEARCH_LOW_BITS) - 1));
+                    const uint32_t hi = (uint32_t)(vk >> SEARCH_LOW_BITS);
+                    if (hi) atomicAdd(&hist[1][I - 1], hi);
+                } else {
+                    atomicAdd(&hist[0][I - 1], vk);
+                }
+                atomicAdd(&hist[2][I - 1], 3u << (2 * k));
+            }
+        }
+    }
+    Sum base_a;
+    if constexpr (WIDE) base_a = ((uint64_t)__reduce_add_sync(0xffffffffu, (uint32_t)(sum_a >> 24)) << 24) + __reduce_add_sync(0xffffffffu, (uint32_t)sum_a & 0xFFFFFFu);
+    else base_a = __reduce_add_sync(0xffffffffu, sum_a);
+    sum_b = __reduce_add_sync(0xffffffffu, sum_b);
+    __syncwarp();
+    Sum A[NC];
+    uint32_t Bc[NC];
+#pragma unroll
+    for (int c = NC - 1; c >= 0; --c) {
+        const int bin = NC * lane + c;
+        A[c] = hist[0][bin];
+        if constexpr (WIDE) A[c] += (uint64_t)hist[1][bin] << SEARCH_LOW_BITS;
+        Bc[c] = hist[2][bin];
+        if (c < NC - 1) {
+            A[c] += A[c + 1];
+            Bc[c] += Bc[c + 1];
+        }
+    }
+    Sum ta = A[0];  // sums over this and the higher lanes
+    uint32_t tb = Bc[0];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const Sum oa = __shfl_down_sync(0xffffffffu, ta, o);
+        const uint32_t ob = __shfl_down_sync(0xffffffffu, tb, o);
+        if (lane + o < 32) {
+            ta += oa;
+            tb += ob;
+        }
+    }
+    ta += base_a - A[0];
+    tb += sum_b - Bc[0];
+    // in units of s0 and of s0 times the last place: D / s0^2 = b^2 B - 2 b (unit / s0) A
+    const double unit = __longlong_as_double((long long)(1023 - 25 + (int)emin) << 52);  // value of the smallest weight's last place
+    const float two_u = (float)(2.0 * unit / s0);
+    float d[NC], tol[NC], upper = 3e38f;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+        const float b = 0.01f * (float)(NC * lane + 1 + c);
+        const float cross = b * two_u * (float)(A[c] + ta);
+        const float square = b * b * (float)(Bc[c] + tb);
+        d[c] = square - cross;
+        tol[c] = SEARCH_TOL32 * (square + cross);
+        if (NC * lane + 1 + c > 200) d[c] = 3e38f;
+        upper = fminf(upper, d[c] + tol[c]);
+    }
+    for (int o = 16; o; o >>= 1) upper = fminf(upper, __shfl_xor_sync(0xffffffffu, upper, o));
+    uint32_t flags = 0;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) flags |= d[c] - tol[c] <= upper ? 1u << c : 0u;
+    if (__reduce_add_sync(0xffffffffu, (uint32_t)__popc(flags)) > 1u) {
+        // E_k(i) <= E_k(2i) + 1, with equality for all k (candidate 2i only renames the levels: the same sums, term by term) iff
+        // B(i) = 4 B(2i); the smaller one wins
+        __syncwarp();
+#pragma unroll
+        for (int c = 0; c < NC; ++c) hist[0][NC * lane + c] = (flags >> c) & 1u ? Bc[c] + tb : 0u;
+        __syncwarp();
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            const int i = NC * lane + 1 + c;
+            if (((flags >> c) & 1u) && (i & 1) == 0 && hist[0][i / 2 - 1] == 4u * (Bc[c] + tb)) flags &= ~(1u << c);
+        }
+    }
+    if (__reduce_add_sync(0xffffffffu, (uint32_t)__popc(flags)) > 1u) {
+        double low[NC], up = 1e300;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            low[c] = 0.0;
+            if ((flags >> c) & 1u) {
+                const double sc = search_scale(s0, NC * lane + 1 + c);
+                const double cross = 2.0 * sc * ((double)(A[c] + ta) * unit), square = sc * sc * (double)(Bc[c] + tb);
+                const double t = SEARCH_TOL64 * (square + cross);
+                low[c] = (square - cross) - t;
+                up = fmin(up, (square - cross) + t);
+            }
+        }
+        for (int o = 16; o; o >>= 1) up = fmin(up, __shfl_xor_sync(0xffffffffu, up, o));
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+            if (low[c] > up) flags &= ~(1u << c);
+    }
+    return flags;
+}
+
+template <int BITS, int PER>  // PER = G / 32 weights per lane
+__global__ void __launch_bounds__(256) pot_search_kernel(const uint16_t* __restrict__ W, int64_t ngroups,
+                                                         uint16_t* __restrict__ S, uint32_t* __restrict__ packed) {
+    constexpr int QMAX = qmax_of(BITS), NC = SEARCH_NC;
+    __shared__ __align__(16) uint32_t hist_s[8][3][SEARCH_BINS];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t gi = (int64_t)blockIdx.x * 8 + warp;
+    if (gi >= ngroups) return;
+    uint32_t h[PER];
+    if constexpr (PER == 4) {
+        const uint2 q = __ldg(reinterpret_cast<const uint2*>(W + gi * 128) + lane);
+        h[0] = q.x & 0xFFFFu; h[1] = q.x >> 16; h[2] = q.y & 0xFFFFu; h[3] = q.y >> 16;
+    } else {
+        const uint32_t q = __ldg(reinterpret_cast<const uint32_t*>(W + gi * 64) + lane);
+        h[0] = q & 0xFFFFu; h[1] = q >> 16;
+    }
+    uint4* hz = reinterpret_cast<uint4*>(&hist_s[warp][0][0]);
+#pragma unroll
+    for (int z = 0; z < 3 * SEARCH_BINS / 4; z += 32)
+        if (z + lane < 3 * SEARCH_BINS / 4) hz[z + lane] = make_uint4(0, 0, 0, 0);
+
+    uint32_t mag = 0, top = 0, low = 0x7FFFu;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        const uint32_t m = h[j] & 0x7FFFu;
+        top = max(top, m);
+        mag = max(mag, m > 0x7C00u ? 0u : m);  // (a NaN does not take part)
+        if (m != 0) low = min(low, m);
+    }
+    mag = __reduce_max_sync(0xffffffffu, mag);
+    top = __reduce_max_sync(0xffffffffu, top);
+    low = __reduce_min_sync(0xffffffffu, low);
+    const double s0 = (double)__half2float(__ushort_as_half((uint16_t)mag)) / (double)((1 << QMAX) - 1);
+    __syncwarp();
+
+    uint32_t flags;
+    if (top == 0) flags = lane == 0 ? 1u : 0u;                                                  // all sums are zero: the first candidate
+    else if (top >= 0x7C00u) flags = lane < 28 ? 0x7Fu : (lane == 28 ? 0xFu : 0u);              // a NaN or an infinity: every candidate
+    else {
+        const uint32_t emin = max(low >> 10, 1u), emax = max(top >> 10, 1u);
+        // 2^(11 + emax - emin) in units of the last place, 2^7 weights, 2^QMAX
+        const bool wide = 11 + (emax - emin) + 7 + QMAX > 32;
+        flags = wide ? search_candidates<BITS, PER, true>(h, emin, s0, hist_s[warp], lane)
+                     : search_candidates<BITS, PER, false>(h, emin, s0, hist_s[warp], lane);
+    }
+    const unsigned who = __ballot_sync(0xffffffffu, flags != 0);
+    int best = __shfl_sync(0xffffffffu, NC * lane + __ffs(flags), who ? __ffs(who) - 1 : 0);
+    if (__reduce_add_sync(0xffffffffu, (uint32_t)__popc(flags)) != 1u) {
+        // the sequential loop over the candidates that are left
+        double qmin = 1e300;
+        best = 1;
+        for (int c = 0; c < NC; ++c) {
+            const bool mine = (flags >> c) & 1u;
+            if (!__any_sync(0xffffffffu, mine)) continue;
+            const int i = NC * lane + 1 + c;
+            const double sc = search_scale(s0, i), s2 = __dmul_rn(sc, sc);
+            double q1 = 0.0;
+            for (int src = 0; src < 32; ++src) {
+#pragma unroll
+                for (int j = 0; j < PER; ++j) {
+                    const double wk = (double)__half2float(__ushort_as_half((uint16_t)__shfl_sync(0xffffffffu, h[j], src)));
+                    const double w2 = __dmul_rn(wk, wk);
+                    int E = 0;
+#pragma unroll
+                    for (int k = 0; k < QMAX; ++k) E += (w2 > __dmul_rn(s2, (double)(1 << (2 * k + 1)))) ? 1 : 0;
+                    double rec = __dmul_rn(sc, (double)(1 << E));
+                    if (wk < 0.0) rec = -rec;
+                    const double d = (sc > 0.0) ? __dsub_rn(wk, rec) : wk;
+                    q1 = __dadd_rn(q1, __dmul_rn(d, d));
+                }
+            }
+            if (mine && q1 < qmin) { qmin = q1; best = i; }
+        }
+        for (int o = 16; o; o >>= 1) {  // smallest Q1, ties to the smaller i
+            const double qo = __shfl_xor_sync(0xffffffffu, qmin, o);
+            const int bo = __shfl_xor_sync(0xffffffffu, best, o);
+            if (qo < qmin || (qo == qmin && bo < best)) { qmin = qo; best = bo; }
+        }
+    }
+    const uint16_t sb = clamp_scale_bits(__half_as_ushort(__double2half(search_scale(s0, best))), BITS);
+    if (lane == 0) S[gi] = sb;
+
+    // codes: PER BITS bits per lane -> 8 codes per lane group -> whole words
+    const float two_s2 = pot_two_s2(sb);
+    uint32_t bits = 0;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) bits |= pot_code<BITS>(h[j], two_s2) << (j * BITS);
+    constexpr int LANES8 = 8 / PER;  // lanes that hold 8 codes
+#pragma unroll
+    for (int o = 1; o < LANES8; o <<= 1) {
+        const uint32_t other = __shfl_xor_sync(0xffffffffu, bits, o);
+        bits = (lane & o) ? (bits << (o * PER * BITS)) | other : bits | (other << (o * PER * BITS));
+    }
+    constexpr int WORDS = PER * BITS;  // 32 PER codes of BITS bits
+    int piece = lane, shift = 0;
+    if constexpr (BITS == 2) piece = 2 * lane;
+    if constexpr (BITS == 3) { piece = lane / 3 * 4 + lane % 3; shift = 8 * (lane % 3); }
+    const uint32_t a = __shfl_sync(0xffffffffu, bits, (piece * LANES8) & 31);
+    const uint32_t b = __shfl_sync(0xffffffffu, bits, ((piece + 1) * LANES8) & 31);
+    const uint32_t word = BITS == 4 ? a : (BITS == 2 ? a | (b << 16) : (a >> shift) | (b << (24 - shift)));
+    if (lane < WORDS) packed[gi * WORDS + lane] = word;
+}
+
+// uniform twin: one warp per group; codes are staged in shared memory, then packed 32 bits at a time
+template <int BITS>
+__global__ void __launch_bounds__(256) uint_quantize_kernel(const __half* __restrict__ W, int64_t N, int64_t K, int G,
+                                                            __half* __restrict__ S, __half* __restrict__ Z,
+                                                            uint32_t* __restrict__ packed) {
     __shared__ uint8_t codes_s[8][128];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t ngroups = N * (K / G);
@@ -28,100 +362,30 @@ __global__ void __launch_bounds__(256) quantize_kernel(const __half* __restrict_
     const __half* wg = W + gi * G;
     const int per = G / 32;  // 2 or 4 elements per lane
     double w[4];
-    double amax = 0.0, mn = 1e300, mx = -1e300;
+    double mn = 1e300, mx = -1e300;
     for (int i = 0; i < per; ++i) {
         w[i] = (double)__half2float(wg[lane * per + i]);
-        amax = fmax(amax, fabs(w[i]));
         mn = fmin(mn, w[i]);
         mx = fmax(mx, w[i]);
     }
     for (int o = 16; o; o >>= 1) {
-        amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
         mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, o));
         mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     }
-    constexpr int QMAX = qmax_of(BITS);
-    if constexpr (!UNIFORM) {
-        uint16_t sb;
-        if (rule == POT_SCALE_GIVEN) {
-            sb = __half_as_ushort(S[gi]);
-        } else if (rule == POT_SCALE_SEARCH) {
-            // Algorithm 1: s0 = max|w| / (2^q_max - 1); b = 0.01 i, i = 1..200; keep the first minimiser of
-            // Q1(b) = sum_k (w_k - s0 b sign(w_k) 2^E_k(b))^2.  The 200 candidates are spread over the lanes
-            // (lane l takes i = l + 1, l + 33, ...), every lane adds the G terms of its candidates in the order
-            // k = 0 .. G-1 with separately rounded multiply and add -- the order and rounding of a plain sequential
-            // loop -- and the warp takes the smallest (Q1, i) pair.  The weights travel by shuffle.
-            const double s0 = amax / (double)((1 << QMAX) - 1);
-            constexpr int NC = 7;  // ceil(200 / 32)
-            double sc[NC], q1[NC];
-#pragma unroll
-            for (int c = 0; c < NC; ++c) {
-                sc[c] = __dmul_rn(s0, __dmul_rn(0.01, (double)(lane + 1 + 32 * c)));
-                q1[c] = 0.0;
-            }
-            for (int src = 0; src < 32; ++src) {
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    if (j < per) {
-                        const double wk = __shfl_sync(0xffffffffu, w[j], src);
-                        const double w2 = __dmul_rn(wk, wk);
-#pragma unroll
-                        for (int c = 0; c < NC; ++c) {
-                            const double s2 = __dmul_rn(sc[c], sc[c]);
-                            int E = 0;
-#pragma unroll
-                            for (int k = 0; k < QMAX; ++k) E += (w2 > __dmul_rn(s2, (double)(1 << (2 * k + 1)))) ? 1 : 0;
-                            double rec = __dmul_rn(sc[c], (double)(1 << E));
-                            if (wk < 0.0) rec = -rec;
-                            const double d = (sc[c] > 0.0) ? __dsub_rn(wk, rec) : wk;
-                            q1[c] = __dadd_rn(q1[c], __dmul_rn(d, d));
-                        }
-                    }
-                }
-            }
-            double qmin = 1e300;
-            int best = 1;
-#pragma unroll
-            for (int c = 0; c < NC; ++c) {
-                const int i = lane + 1 + 32 * c;
-                if (i <= 200 && q1[c] < qmin) { qmin = q1[c]; best = i; }
-            }
-            for (int o = 16; o; o >>= 1) {  // smallest Q1, ties to the smaller i
-                const double qo = __shfl_xor_sync(0xffffffffu, qmin, o);
-                const int bo = __shfl_xor_sync(0xffffffffu, best, o);
-                if (qo < qmin || (qo == qmin && bo < best)) { qmin = qo; best = bo; }
-            }
-            sb = clamp_scale_bits(__half_as_ushort(__double2half(__dmul_rn(s0, __dmul_rn(0.01, (double)best)))), BITS);
-            if (lane == 0) S[gi] = __ushort_as_half(sb);
-        } else {
-            const double s = (rule == POT_SCALE_TOP) ? ldexp(amax, -QMAX) : amax / (double)((1 << QMAX) - 1);
-            sb = clamp_scale_bits(__half_as_ushort(__double2half(s)), BITS);
-            if (lane == 0) S[gi] = __ushort_as_half(sb);
-        }
-        const double Sd = (double)__half2float(__ushort_as_half(sb));
-        for (int i = 0; i < per; ++i) {
-            int E = 0;
-            // E >= k+1  <=>  |w|/S > 2^(k+1/2)  <=>  w^2 > 2^(2k+1) S^2   (exact in FP64 for FP16 inputs)
-            for (int k = 0; k < QMAX; ++k) E += (w[i] * w[i] > ldexp(Sd * Sd, 2 * k + 1)) ? 1 : 0;
-            const int sign = w[i] < 0.0 ? 1 : 0;
-            codes_s[warp][lane * per + i] = (uint8_t)((sign << (BITS - 1)) | E);
-        }
-    } else {
-        const double levels = (double)((1 << BITS) - 1);
-        uint16_t sb = __half_as_ushort(__double2half((mx - mn) / levels));
-        if (sb < 0x0400) sb = 0x0400;
-        const double s = (double)__half2float(__ushort_as_half(sb));
-        double z = rint(-mn / s);
-        z = fmin(fmax(z, 0.0), levels);
-        if (lane == 0) {
-            S[gi] = __ushort_as_half(sb);
-            Z[gi] = __double2half(z);
-        }
-        for (int i = 0; i < per; ++i) {
-            double q = rint(w[i] / s) + z;
-            q = fmin(fmax(q, 0.0), levels);
-            codes_s[warp][lane * per + i] = (uint8_t)q;
-        }
+    const double levels = (double)((1 << BITS) - 1);
+    uint16_t sb = __half_as_ushort(__double2half((mx - mn) / levels));
+    if (sb < 0x0400) sb = 0x0400;
+    const double s = (double)__half2float(__ushort_as_half(sb));
+    double z = rint(-mn / s);
+    z = fmin(fmax(z, 0.0), levels);
+    if (lane == 0) {
+        S[gi] = __ushort_as_half(sb);
+        Z[gi] = __double2half(z);
+    }
+    for (int i = 0; i < per; ++i) {
+        double q = rint(w[i] / s) + z;
+        q = fmin(fmax(q, 0.0), levels);
+        codes_s[warp][lane * per + i] = (uint8_t)q;
     }
     __syncwarp();
     const int words = G * BITS / 32;
@@ -241,15 +505,26 @@ extern "C" pot_status_t pot_quantize_ref(const void* W, int64_t N, int64_t K, in
     if (st != POT_OK) return st;
     if ((int)rule < 0 || (int)rule > 3) return POT_ERR_UNSUPPORTED;
     if (!aligned16(W) || !aligned16(scales) || !aligned16(packed)) return POT_ERR_ALIGN;
-    const int64_t ngroups = N * (K / group);
-    const unsigned grid = (unsigned)((ngroups + 7) / 8);
     cudaStream_t s = (cudaStream_t)stream;
-    auto* Wp = (const __half*)W;
-    auto* Sp = (__half*)scales;
+    if (rule == POT_SCALE_SEARCH) {
+        const int64_t ngroups = N * (K / group);
+        auto run = [&](auto kernel) {
+            kernel<<<(unsigned)((ngroups + 7) / 8), 256, 0, s>>>((const uint16_t*)W, ngroups, (uint16_t*)scales, (uint32_t*)packed);
+        };
+        if (bits == 2) group == 128 ? run(pot_search_kernel<2, 4>) : run(pot_search_kernel<2, 2>);
+        else if (bits == 3) group == 128 ? run(pot_search_kernel<3, 4>) : run(pot_search_kernel<3, 2>);
+        else group == 128 ? run(pot_search_kernel<4, 4>) : run(pot_search_kernel<4, 2>);
+        return launched();
+    }
+    const int64_t pieces = N * (K / 8);
+    const unsigned grid = (unsigned)((pieces + QZ_THREADS * QZ_UNROLL - 1) / (QZ_THREADS * QZ_UNROLL));
+    const int ppg_shift = group == 128 ? 4 : 3;  // log2 of the 8-weight pieces per group
+    auto* Wp = (const uint4*)W;
+    auto* Sp = (uint16_t*)scales;
     auto* Pp = (uint32_t*)packed;
-    if (bits == 2) quantize_kernel<2, false><<<grid, 256, 0, s>>>(Wp, N, K, group, (int)rule, Sp, nullptr, Pp);
-    else if (bits == 3) quantize_kernel<3, false><<<grid, 256, 0, s>>>(Wp, N, K, group, (int)rule, Sp, nullptr, Pp);
-    else quantize_kernel<4, false><<<grid, 256, 0, s>>>(Wp, N, K, group, (int)rule, Sp, nullptr, Pp);
+    if (bits == 2) pot_quantize_kernel<2><<<grid, QZ_THREADS, 0, s>>>(Wp, pieces, ppg_shift, (int)rule, Sp, Pp);
+    else if (bits == 3) pot_quantize_kernel<3><<<grid, QZ_THREADS, 0, s>>>(Wp, pieces, ppg_shift, (int)rule, Sp, Pp);
+    else pot_quantize_kernel<4><<<grid, QZ_THREADS, 0, s>>>(Wp, pieces, ppg_shift, (int)rule, Sp, Pp);
     return launched();
 }
 
@@ -266,9 +541,9 @@ extern "C" pot_status_t uint_quantize_ref(const void* W, int64_t N, int64_t K, i
     auto* Sp = (__half*)scales;
     auto* Zp = (__half*)zeros;
     auto* Pp = (uint32_t*)packed;
-    if (bits == 2) quantize_kernel<2, true><<<grid, 256, 0, s>>>(Wp, N, K, group, 0, Sp, Zp, Pp);
-    else if (bits == 3) quantize_kernel<3, true><<<grid, 256, 0, s>>>(Wp, N, K, group, 0, Sp, Zp, Pp);
-    else quantize_kernel<4, true><<<grid, 256, 0, s>>>(Wp, N, K, group, 0, Sp, Zp, Pp);
+    if (bits == 2) uint_quantize_kernel<2><<<grid, 256, 0, s>>>(Wp, N, K, group, Sp, Zp, Pp);
+    else if (bits == 3) uint_quantize_kernel<3><<<grid, 256, 0, s>>>(Wp, N, K, group, Sp, Zp, Pp);
+    else uint_quantize_kernel<4><<<grid, 256, 0, s>>>(Wp, N, K, group, Sp, Zp, Pp);
     return launched();
 }
 

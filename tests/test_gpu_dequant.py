@@ -70,6 +70,34 @@ def test_scale_search_rule_matches_algorithm_1(B, oracle, bits):
 
 @pytest.mark.parametrize("bits", [2, 3, 4])
 @pytest.mark.parametrize("G", [64, 128])
+def test_scale_search_where_sums_tie_or_span_the_whole_range(B, oracle, bits, G):
+    """Groups whose candidates have equal sums (the plain loop decides), sums that do not fit in 32 bits, weights on thresholds."""
+    rng = np.random.default_rng(100 * bits + G)
+    N, K = 24, 2 * G * 64 // G * 2
+    f16 = lambda a: np.asarray(a, dtype=np.float64).astype(np.float16).view(np.uint16)
+    W = np.zeros((N, K), dtype=np.uint16)                              # rows 0, 1: zeros of both signs
+    W[1] = 0x8000
+    W[2], W[3], W[4] = 0x3C00, 0x0001, 0x7BFF                          # one value: the smallest, the largest
+    W[5] = f16(np.where(rng.random(K) < 0.5, -0.75, 0.75))
+    W[6] = f16(rng.choice([0.0, 0.5, -0.5], K))
+    W[7] = f16(2.0 ** -rng.integers(0, 8, K))                          # powers of two: exact reconstructions, many ties
+    W[8] = f16(2.0 ** -rng.integers(0, 24, K))
+    W[9] = f16(rng.choice([1.0, 1.41421356, 2.0, 2.82842712], K))      # next to thresholds
+    W[10:14] = rng.integers(0, 0x7C00, (4, K)).astype(np.uint16)       # every exponent in one group
+    W[14:18] = rng.integers(0, 0x0400, (4, K)).astype(np.uint16) | 0x8000
+    W[18, ::G] = 0x7BFF                                                # one large weight, the others tiny
+    W[18, 1::2] = 0x0003
+    W[19:] = f16(rng.standard_t(2, (N - 19, K)) * 0.02)
+    W[20, ::3] = 0
+    S_ref, _ = oracle.scale_search(W, bits, G)
+    packed, S = B.pot_quantize_ref(f16_dev(W), bits, G, B.SCALE_SEARCH)
+    assert np.array_equal(bits_of(S), S_ref), np.argwhere(bits_of(S) != S_ref)[:5]
+    codes, _ = oracle.quantize(W, bits, G, oracle.RULE_GIVEN, S_ref)
+    assert np.array_equal(packed.cpu().numpy(), oracle.pack(codes, bits))
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("G", [64, 128])
 @pytest.mark.parametrize("dtype", [0, 1])
 def test_pot_dequant_bit_exact(B, oracle, bits, G, dtype):
     for i, (N, K) in enumerate(SHAPES):
