@@ -45,14 +45,14 @@ struct BitPos {
 };
 
 // where bit b of code q is stored inside the record (b < n-1: exponent bits, b = n-1: sign, for PoT)
-__host__ __device__ inline BitPos record_bit(int bits, int kind, int q, int b) {
-    BitPos r;
+__host__ __device__ constexpr BitPos record_bit(int bits, int kind, int q, int b) {
+    BitPos r{0, 0};
     if (kind == KIND_POT) {
         const int T = q >> 5, c = q & 31;
         const int i = c >> 2;                                       // decoded word
         const int l = ((c & 1) << 1) | ((c >> 1) & 1);              // byte lane: perm is its own inverse
         const bool sign = (b == bits - 1);
-        int k, pos;
+        int k = 0, pos = 0;
         if (bits == 2) {
             k = i >> 2;
             pos = 8 * l + 2 * (i & 3) + (sign ? 5 : 0);

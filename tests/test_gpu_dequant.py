@@ -165,3 +165,23 @@ def test_repack_is_a_bijection(B, oracle, bits):
             w, bit = B.pot_layout_bit(bits, 0, q, b)
             idx = (rb * ncb + cb) * 16 * nw + (w >> 2) * 64 + r * 4 + (w & 3)
             assert (int(tiled[idx]) >> bit) & 1 == (int(codes[i, k]) >> b) & 1
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("K", [128, 512, 640])
+def test_repack_puts_every_bit_where_the_layout_map_says(B, oracle, bits, K):
+    """Both kinds of codes, one column block, whole and partly filled blocks of four: every bit, not a sample."""
+    N = 32
+    packed = np.random.default_rng(K + bits).integers(0, 256, (N, K * bits // 8)).astype(np.uint8)
+    codes = oracle.unpack(packed, K, bits).astype(np.uint32)
+    ncb, nw = K // 128, 4 * bits
+    for kind, repack in ((0, B.pot_repack), (1, B.uint_repack)):
+        ref = np.zeros((N // 16, ncb, bits, 16, 4), dtype=np.uint32)
+        for q in range(128):
+            for b in range(bits):
+                w, bit = B.pot_layout_bit(bits, kind, q, b)
+                v = ((codes[:, q::128] >> b) & 1) << bit               # [N, ncb]
+                ref[:, :, w >> 2, :, w & 3] |= v.reshape(N // 16, 16, ncb).transpose(0, 2, 1)
+        tiled = repack(to_dev(packed), K, bits, 0)
+        assert np.array_equal(tiled.cpu().numpy().view(np.uint32).ravel(), ref.ravel())
+        assert np.array_equal(repack(tiled, K, bits, 1).cpu().numpy(), packed)
