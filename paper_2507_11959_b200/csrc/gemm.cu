@@ -9,7 +9,8 @@
 //    lanes' column blocks: lane (gid, tig) feeds codes 4j..4j+3 of its record (rows gid and
 //    gid+8, column block 4*chunk + tig) into k-slots {2tig, 2tig+1, 2tig+8, 2tig+9} of step j,
 //    and the B fragment reads x at the same columns.
-//  * any M, canonical layout: a plain shared-memory tiled mma.sync kernel (the fallback).
+//  * canonical layout: the canonical GEMV kernel for one token, else the tcgen05 kernel of gemm_prefill.cu with producers that
+//    decode canonical codes.
 //  * otherwise, tiled layout: the tcgen05 kernel in gemm_prefill.cu.
 #include "common.cuh"
 #include "layout.cuh"
@@ -17,108 +18,14 @@
 
 namespace pot {
 
-// ------------------------------------------------------------------------------------------
-// fallback: canonical layout, any M.  64 tokens x 64 rows x 128 columns per CTA step.
-// ------------------------------------------------------------------------------------------
-constexpr int FB_LD = 136;  // padded leading dimension (halves) -> conflict-free fragment loads
-
-template <int BITS, int DT = 0>  // DT = 1: BF16 activations, weights (scale rounded once to BF16) and output
-__global__ void __launch_bounds__(128) pot_gemm_fallback_kernel(const uint32_t* __restrict__ packed,
-                                                                const uint16_t* __restrict__ scales, int64_t N, int64_t K,
-                                                                int G, const __half* __restrict__ X, int64_t M,
-                                                                uint16_t* __restrict__ Y) {
-    constexpr int EBIT = DT == 0 ? 10 : 7;
-    constexpr uint32_t CM = (1u << BITS) - 1u;
-    constexpr uint32_t QM2 = (uint32_t)qmax_of(BITS) * 0x10001u;
-    constexpr uint32_t SM2 = (1u << (BITS - 1)) * 0x10001u;
-    __shared__ __align__(16) __half Xs[64 * FB_LD];
-    __shared__ __align__(16) __half Ws[64 * FB_LD];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int gid = lane >> 2, tig = lane & 3;
-    const int wm = (warp & 1) * 32, wn = (warp >> 1) * 32;
-    const int64_t n0 = (int64_t)blockIdx.x * 64, m0 = (int64_t)blockIdx.y * 64;
-    float acc[2][4][4];
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) acc[a][b][i] = 0.f;
-
-    pdl_wait();
-    for (int64_t kb = 0; kb < K / 128; ++kb) {
-        __syncthreads();
-        for (int idx = threadIdx.x; idx < 64 * 16; idx += 128) {
-            const int r = idx >> 4, pc = idx & 15;
-            uint4 xv = make_uint4(0, 0, 0, 0);
-            if (m0 + r < M) xv = ld_dependent16(reinterpret_cast<const uint4*>(X + (m0 + r) * K + kb * 128) + pc);
-            *reinterpret_cast<uint4*>(&Xs[r * FB_LD + pc * 8]) = xv;
-            uint4 wv = make_uint4(0, 0, 0, 0);
-            const int64_t row = n0 + r;
-            if (row < N) {
-                const int64_t k = kb * 128 + pc * 8;
-                const uint32_t v = read_bits(packed + row * (K * BITS / 32), k * BITS, 8 * BITS);
-                uint32_t s16 = __ldg(scales + row * (K / G) + k / G);
-                if (DT == 1) s16 = __bfloat16_as_ushort(__float2bfloat16_rn(__half2float(__ushort_as_half((uint16_t)s16))));
-                const uint32_t sc2 = s16 * 0x10001u;
-                uint32_t o[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const uint32_t t = v >> (2 * j * BITS);
-                    const uint32_t pr = (t & CM) | ((t << (16 - BITS)) & (CM << 16));
-                    o[j] = sc2 + (((pr & QM2) << EBIT) | ((pr & SM2) << (16 - BITS)));
-                }
-                wv = make_uint4(o[0], o[1], o[2], o[3]);
-            }
-            *reinterpret_cast<uint4*>(&Ws[r * FB_LD + pc * 8]) = wv;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int ks = 0; ks < 8; ++ks) {
-            const int k0 = ks * 16 + 2 * tig;
-            uint32_t a[2][4], b[4][2];
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const int r = wm + 16 * i + gid;
-                a[i][0] = *reinterpret_cast<const uint32_t*>(&Xs[r * FB_LD + k0]);
-                a[i][1] = *reinterpret_cast<const uint32_t*>(&Xs[(r + 8) * FB_LD + k0]);
-                a[i][2] = *reinterpret_cast<const uint32_t*>(&Xs[r * FB_LD + k0 + 8]);
-                a[i][3] = *reinterpret_cast<const uint32_t*>(&Xs[(r + 8) * FB_LD + k0 + 8]);
-            }
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int r = wn + 8 * j + gid;
-                b[j][0] = *reinterpret_cast<const uint32_t*>(&Ws[r * FB_LD + k0]);
-                b[j][1] = *reinterpret_cast<const uint32_t*>(&Ws[r * FB_LD + k0 + 8]);
-            }
-#pragma unroll
-            for (int i = 0; i < 2; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    if (DT == 0) sk_mma(acc[i][j], a[i][0], a[i][1], a[i][2], a[i][3], b[j][0], b[j][1]);
-                    else sk_mma_bf16(acc[i][j], a[i][0], a[i][1], a[i][2], a[i][3], b[j][0], b[j][1]);
-                }
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-                const int64_t token = m0 + wm + 16 * i + gid + 8 * hh;
-                const int64_t row = n0 + wn + 8 * j + 2 * tig;
-                if (token < M) {
-                    if (row < N) Y[token * N + row] = sk_out<DT>(acc[i][j][2 * hh]);
-                    if (row + 1 < N) Y[token * N + row + 1] = sk_out<DT>(acc[i][j][2 * hh + 1]);
-                }
-            }
-}
-
 pot_status_t gemm_prefill_launch(const void* packed, const void* scales, int64_t N, int64_t K, int bits, int group,
                                  const void* X, int64_t M, void* Y, void* workspace, size_t ws_bytes, cudaStream_t s, int dt);
 size_t gemm_prefill_workspace(int64_t M, int64_t N, int64_t K, int bits, int group);
 bool gemm_prefill_supported(int64_t M, int64_t N, int64_t K, int bits, int group);
+pot_status_t gemm_canonical_launch(const void* packed, const void* scales, int64_t N, int64_t K, int bits, int group,
+                                   const void* X, int64_t M, void* Y, cudaStream_t s, int dt);
+pot_status_t gemv_canonical_launch(const void* packed, const void* scales, int64_t N, int64_t K, int bits, int group, const void* x,
+                                   void* y, cudaStream_t s, int dt);
 pot_status_t gemv_stream_launch(const void* packed, const void* scales, int64_t N, int64_t K, int bits, int group, const void* x,
                                 void* y, void* workspace, cudaStream_t s, int dt);
 
@@ -180,13 +87,9 @@ static pot_status_t gemm_impl(const void* packed, const void* scales, int64_t N,
         if (!gemm_prefill_supported(M, N, K, bits, group)) return POT_ERR_UNSUPPORTED;
         return gemm_prefill_launch(packed, scales, N, K, bits, group, X, M, Y, workspace, ws_bytes, s, DT);
     }
-    if ((M + 63) / 64 > 65535) return POT_ERR_SHAPE;  // the fallback kernel's token tiles ride on gridDim.y
-    const dim3 grid((unsigned)((N + 63) / 64), (unsigned)((M + 63) / 64)), block(128);
-    auto* P = (const uint32_t*)packed;
-    auto* S = (const uint16_t*)scales;
-    if (bits == 2) return launch_pdl(pot_gemm_fallback_kernel<2, DT>, grid, block, 0, s, P, S, N, K, group, (const __half*)X, M, (uint16_t*)Y);
-    if (bits == 3) return launch_pdl(pot_gemm_fallback_kernel<3, DT>, grid, block, 0, s, P, S, N, K, group, (const __half*)X, M, (uint16_t*)Y);
-    return launch_pdl(pot_gemm_fallback_kernel<4, DT>, grid, block, 0, s, P, S, N, K, group, (const __half*)X, M, (uint16_t*)Y);
+    if ((M + 63) / 64 > 65535) return POT_ERR_SHAPE;
+    if (M == 1) return gemv_canonical_launch(packed, scales, N, K, bits, group, X, Y, s, DT);
+    return gemm_canonical_launch(packed, scales, N, K, bits, group, X, M, Y, s, DT);
 }
 
 extern "C" pot_status_t pot_gemm(const void* packed, const void* scales, int64_t N, int64_t K, int bits, int group,

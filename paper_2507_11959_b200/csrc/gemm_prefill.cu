@@ -129,6 +129,21 @@ __device__ __forceinline__ uint32_t pf_ldg_u16(const uint16_t* p) {
     asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(v) : "l"(p));
     return (uint32_t)v;
 }
+__device__ __forceinline__ void pf_cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+    __syncwarp();
+}
+// address of this CTA's shared-memory location in the CTA with the given rank of the cluster
+__device__ __forceinline__ uint32_t pf_cluster_addr(uint32_t addr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ uint32_t pf_ld_cluster(uint32_t addr) {
+    uint32_t v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    return v;
+}
 __device__ __forceinline__ void pf_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
@@ -304,7 +319,12 @@ __device__ __forceinline__ void pf_issue(uint32_t smem0, uint32_t bar0, uint32_t
 // <bits, 6, 2, 2, 2, dt, 1>: 256 accumulator columns + 6 x 32 columns of A = 448 of the 512 columns.
 // NGP of the NG groups decode, the others only take part in the epilogue (measured slower than NGP = NG = 2 -- the
 // waiting groups poll the accumulator barrier through the whole main loop -- and not instantiated).
-template <int BITS, int PF_STAGES, int NG, int NI, int MT, int DT = 0, int AT = 0, int NGP = NG, int WIDE = 0>  // DT = 1: BF16 activations, weights and output
+// CANON = 1: canonical codes and row-major scales (the 128-column stages only): a producer thread reads its row's 16 BITS
+// contiguous bytes per column block and decodes them with byte look-ups (potl::CanonLut).  There is no workspace on this
+// route: the items of a tile that is cut along K are the CTAs of a thread-block cluster, which add their partial sums through
+// distributed shared memory.  200 tokens x 4099 x 11008, 3 bits: 672 us on the mma.sync kernel that this replaced, 29.6 us
+// (clusters of 4, 132 CTAs; about half of it is latency per 128-column stage with three stages in flight).
+template <int BITS, int PF_STAGES, int NG, int NI, int MT, int DT = 0, int AT = 0, int NGP = NG, int WIDE = 0, int CANON = 0>  // DT = 1: BF16 activations, weights and output
 __global__ void __launch_bounds__(pf_threads(NG, NI), 1)
 pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* __restrict__ packed,
                         const uint16_t* __restrict__ scales, int64_t N, int64_t K, int G, int64_t M,
@@ -314,6 +334,7 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
     // 1024-byte alignment: the swizzle atoms and the matrix descriptors assume it
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     static_assert(AT == 0 || NI == 2, "the tensor-memory weight tile is built for two issuers");
+    static_assert(!CANON || (AT && pf_bks(MT, AT, WIDE) == 2), "canonical codes: 128-column stages, the weight tile in tensor memory");
     constexpr bool AT2 = AT && MT == 2;   // both issuers on every stage, one token tile each (else: alternate stages)
     constexpr int BKS = pf_bks(MT, AT, WIDE);   // 64-column sub-blocks per stage
     constexpr int STAGE_BYTES = pf_stage_bytes(MT, AT, WIDE);
@@ -382,7 +403,16 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
             const int64_t cbx = cb0 + (BKS == 2 ? kb : (kb >> 1));   // the stage's column block
             // tiled scales: the unit's values sit together, rows r and r + 8 of a group in one word
             const int64_t so = (rb * ncb + cbx) * (16 * spg);
-            if constexpr (BKS == 2) {
+            if constexpr (CANON) {
+                const uint4* rowp = packed + (n * ncb + cbx) * BITS;
+#pragma unroll
+                for (int t = 0; t < BITS; ++t) {
+                    const uint4 q = pf_ldg_v4(rowp + t);
+                    rec[buf][4 * t + 0] = q.x; rec[buf][4 * t + 1] = q.y; rec[buf][4 * t + 2] = q.z; rec[buf][4 * t + 3] = q.w;
+                }
+                sc2[buf][0] = pf_ldg_u16(scales + (n * ncb + cbx) * spg);
+                sc2[buf][BKS - 1] = pf_ldg_u16(scales + (n * ncb + cbx) * spg + spg - 1);
+            } else if constexpr (BKS == 2) {
                 const uint4* unit = packed + (rb * ncb + cbx) * (16 * BITS);
 #pragma unroll
                 for (int t = 0; t < BITS; ++t) {
@@ -506,12 +536,14 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
                         uint32_t sh = sc2[buf][hb];
                         if (DT == 1) sh = __bfloat16_as_ushort(__float2bfloat16_rn(__half2float(__ushort_as_half((uint16_t)sh))));
                         const uint32_t sh2 = sh * 0x10001u;
+                        const potl::CanonLut<BITS, DT> lut(sh);
                         uint32_t wa[32];
 #pragma unroll
                         for (int T2 = 0; T2 < 2; ++T2) {
                             uint32_t w2[16];
                             if (row_ok) {
-                                if (DT == 0) potl::pot_decode32<BITS, 4>(rec[buf], 2 * hb + T2, sh2, w2);
+                                if constexpr (CANON) potl::canon_decode32<BITS, DT>(rec[buf] + (2 * hb + T2) * BITS, lut, w2);
+                                else if (DT == 0) potl::pot_decode32<BITS, 4>(rec[buf], 2 * hb + T2, sh2, w2);
                                 else potl::pot_decode32_bf16<BITS, 4>(rec[buf], 2 * hb + T2, sh2, w2);
                             } else {
 #pragma unroll
@@ -601,12 +633,7 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
         // (chunks part, part + NG, ... of the tile's 32-column chunks; the one-tile kernel holds at most PF_SMALL_TOKENS tokens)
         constexpr int NCH = MT == 1 ? PF_SMALL_TOKENS / 32 : MT * PF_BM / 32;
         constexpr int CH = (NCH + NG - 1) / NG;
-#pragma unroll
-        for (int cc = 0; cc < CH; ++cc) {
-            if (part + cc * NG >= NCH) break;
-            const int col = (part + cc * NG) * 32;
-            if (m0 + col >= M) break;             // (warp-uniform) no token in these columns
-            uint32_t v[32];
+        auto sums = [&](int col, uint32_t (&v)[32]) {  // the complete sums of 32 token columns of this item
             pf_ld32(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)col, v);
             if (NI == 2 && !AT2 && nkb > 1) {     // add the second issuer's sums (odd K blocks) to the first's: a fixed order
                                                   // (an item of a single stage -- K = 128 with 128-column stages -- has none)
@@ -618,12 +645,56 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
             } else {
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
             }
-            if (feat < N && !gave_up && in_range(m0 + col < M && m0 >= 0 && feat >= 0 && (splits == 1 || (tail_index >= 0 && zsplit >= 0 && zsplit < splits)), err, 0x60)) {
-                if (splits == 1) {  // a warp stores 32 consecutive features (64 bytes) of one token at a time
-                    uint16_t* dst = Y + (m0 + col) * N + feat;
+        };
+        auto store = [&](int col, const uint32_t (&v)[32]) {  // a warp stores 32 consecutive features (64 bytes) of one token at a time
+            uint16_t* dst = Y + (m0 + col) * N + feat;
 #pragma unroll
-                    for (int i = 0; i < 32; ++i)
-                        if (m0 + col + i < M) dst[(int64_t)i * N] = pf_out<DT>(__uint_as_float(v[i]));
+            for (int i = 0; i < 32; ++i)
+                if (m0 + col + i < M) dst[(int64_t)i * N] = pf_out<DT>(__uint_as_float(v[i]));
+        };
+        if constexpr (CANON) {
+            if (splits > 1) {
+                // The items of the tile are the CTAs of this cluster.  Token chunk c belongs to CTA c % splits: every CTA leaves
+                // the other chunks' sums in its own shared memory (the ring is empty: all MMAs have completed), and after a
+                // cluster barrier each CTA adds its chunks in split order and writes them.
+                static_assert(NCH * 32 * PF_BN * 4 <= PF_STAGES * STAGE_BYTES, "the partial sums fit in the ring");
+                float* red = reinterpret_cast<float*>(smem) + 32 * q + lane;   // [token column][128 features]
+#pragma unroll 1
+                for (int c = part; c < NCH && m0 + c * 32 < M; c += NG) {
+                    if (c % splits == zsplit) continue;
+                    uint32_t v[32];
+                    sums(c * 32, v);
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) red[(c * 32 + i) * PF_BN] = __uint_as_float(v[i]);
+                }
+                pf_cluster_sync();
+#pragma unroll 1
+                for (int c = zsplit + splits * part; c < NCH && m0 + c * 32 < M; c += splits * NG) {
+                    uint32_t own[32], v[32];
+                    sums(c * 32, own);
+                    for (int z = 0; z < splits; ++z) {
+                        uint32_t p[32];
+                        const uint32_t src = pf_cluster_addr(smem_u32(red + c * 32 * PF_BN), (uint32_t)z);
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) p[i] = z == zsplit ? own[i] : pf_ld_cluster(src + (uint32_t)(i * PF_BN * 4));
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) v[i] = z == 0 ? p[i] : __float_as_uint(__uint_as_float(v[i]) + __uint_as_float(p[i]));
+                    }
+                    if (feat < N && !gave_up) store(c * 32, v);
+                }
+            }
+        }
+#pragma unroll
+        for (int cc = 0; cc < CH; ++cc) {
+            if (CANON && splits > 1) break;
+            if (part + cc * NG >= NCH) break;
+            const int col = (part + cc * NG) * 32;
+            if (m0 + col >= M) break;             // (warp-uniform) no token in these columns
+            uint32_t v[32];
+            sums(col, v);
+            if (feat < N && !gave_up && in_range(m0 + col < M && m0 >= 0 && feat >= 0 && (splits == 1 || (tail_index >= 0 && zsplit >= 0 && zsplit < splits)), err, 0x60)) {
+                if (splits == 1) {
+                    store(col, v);
                 } else {  // this split's partial sums: [tail tile][split][token of the tile][128 features] FP32
                     float* dst = partial + (((int64_t)tail_index * splits + zsplit) * rows_alloc + col) * PF_BN + (32 * q + lane);
 #pragma unroll
@@ -632,7 +703,7 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
                 }
             }
         }
-        if (splits > 1 && !gave_up && in_range(tail_index >= 0 && partial != nullptr && counters != nullptr, err, 0x61)) {
+        if (!CANON && splits > 1 && !gave_up && in_range(tail_index >= 0 && partial != nullptr && counters != nullptr, err, 0x61)) {
             // The CTA that delivers the last split of a tile (an arrival counter tells it) adds the splits in
             // ascending order -- the result does not depend on timing -- and writes Y.
             __shared__ unsigned s_prev;
@@ -674,6 +745,12 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
                 }
                 if (threadIdx.x == 32 * PROD_WARP0) counters[tail_index] = 0u;  // leave the workspace ready for the next call
             }
+        }
+    }
+    if constexpr (CANON) {  // every thread of the cluster arrives at both barriers: the epilogue warps at the first one above
+        if (tail_splits > 1) {
+            if (warp < PROD_WARP0) pf_cluster_sync();
+            pf_cluster_sync();  // nobody leaves while its partial sums are being read
         }
     }
     // ---------------- teardown: everyone is done with tensor memory, the allocating warp frees it --------
@@ -742,6 +819,7 @@ static PrefillPlan prefill_plan(int64_t M, int64_t N, int64_t K) {
 size_t gemm_prefill_workspace(int64_t M, int64_t N, int64_t K, int, int) { return prefill_plan(M, N, K).ws_bytes; }
 
 static int* prefill_error_ptr();
+static bool encode_x_map(CUtensorMap* xmap, const void* X, int64_t M, int64_t K);
 
 // Where the large-M kernel keeps the decoded weight tile: in tensor memory (the producers write it with tcgen05.st, the
 // MMAs read their A operand there).  That takes a third of the traffic off shared memory, and a stage of shared memory
@@ -765,17 +843,8 @@ pot_status_t gemm_prefill_launch(const void* packed, const void* scales, int64_t
     if (pl.ws_bytes > 0 && (!workspace || ws_bytes < pl.ws_bytes)) return POT_ERR_WORKSPACE;
     unsigned* counters = (unsigned*)workspace;
     float* partial = pl.ws_bytes > 0 ? (float*)((char*)workspace + pl.counter_bytes) : nullptr;
-    EncodeTiledFn encode = encode_tiled_fn();
-    if (!encode) return POT_ERR_CUDA;
     CUtensorMap xmap;
-    const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)M};
-    const cuuint64_t strides[1] = {(cuuint64_t)K * 2};
-    const cuuint32_t box[2] = {64, (cuuint32_t)(M <= PF_SMALL_TOKENS ? M : PF_BM)};  // the one-tile kernel: no padding rows
-    const cuuint32_t estr[2] = {1, 1};
-    if (encode(&xmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(X), dims, strides, box, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return POT_ERR_CUDA;
+    if (!encode_x_map(&xmap, X, M, K)) return POT_ERR_CUDA;
     const dim3 grid((unsigned)(pl.n_full + pl.n_tail * pl.splits));
     auto run = [&](auto kernel, int stages, int mt, int at = 0, int ng = 4, int wide = 0) -> pot_status_t {
         const size_t smem = pf_smem_bytes(stages, mt, at, wide);
@@ -841,6 +910,75 @@ pot_status_t gemm_prefill_launch(const void* packed, const void* scales, int64_t
 }
 
 static int* prefill_error_ptr() { return error_ptr(ERR_PREFILL); }
+
+static bool encode_x_map(CUtensorMap* xmap, const void* X, int64_t M, int64_t K) {
+    EncodeTiledFn encode = encode_tiled_fn();
+    if (!encode) return false;
+    const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)M};
+    const cuuint64_t strides[1] = {(cuuint64_t)K * 2};
+    const cuuint32_t box[2] = {64, (cuuint32_t)(M <= PF_SMALL_TOKENS ? M : PF_BM)};  // the one-tile kernel: no padding rows
+    const cuuint32_t estr[2] = {1, 1};
+    return encode(xmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(X), dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// Canonical codes: one CTA per tile, or a cluster of up to 8 CTAs that share a tile's K range while the tiles leave SMs idle
+// (at least four column blocks per CTA).  The largest cluster size with which all tiles are resident at once is taken: a
+// cluster lives inside one GPC, so that fewer CTAs fit the larger it is (cudaOccupancyMaxActiveClusters on a B200 with one CTA
+// per SM: 148, 74, 45, 33, 26, 22, 15 clusters of 1, 2, 3, 4, 5, 6, 8); a second wave of clusters costs more than the idle
+// SMs (37 tiles, 128 tokens, K = 8192: 40 us with clusters of 4).
+static int canonical_splits(int64_t tiles, int64_t K) {
+    constexpr int kSizes[] = {8, 6, 5, 4, 3, 2}, kResident[] = {15, 22, 26, 33, 45, 74};
+    for (int i = 0; i < 6; ++i)
+        if (tiles <= kResident[i] && K / 128 >= 4 * kSizes[i]) return kSizes[i];
+    return 1;
+}
+pot_status_t gemm_canonical_launch(const void* packed, const void* scales, int64_t N, int64_t K, int bits, int group,
+                                   const void* X, int64_t M, void* Y, cudaStream_t s, int dt) {
+    const bool small = M <= PF_SMALL_TOKENS;
+    const int64_t tiles_m = small ? 1 : (M + PF_BM * PF_MT - 1) / (PF_BM * PF_MT);
+    const int64_t tiles = tiles_m * ((N + PF_BN - 1) / PF_BN);
+    if (tiles > 0x7fffffff / 8) return POT_ERR_SHAPE;
+    const int splits = canonical_splits(tiles, K);
+    CUtensorMap xmap;
+    if (!encode_x_map(&xmap, X, M, K)) return POT_ERR_CUDA;
+    auto run = [&](auto kernel, int stages, int mt, int wide) -> pot_status_t {
+        if (!allow_max_dynamic_smem(kernel)) return POT_ERR_CUDA;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(tiles * splits));
+        cfg.blockDim = dim3((unsigned)pf_threads(3, 2));
+        cfg.dynamicSmemBytes = pf_smem_bytes(stages, mt, 1, wide);
+        cfg.stream = s;
+        cudaLaunchAttribute attr[2];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = (unsigned)splits;
+        attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = splits > 1 ? 2 : 1;
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, xmap, (const uint4*)packed, (const uint16_t*)scales, N, K, group, M,
+                                                 (uint16_t*)Y, (float*)nullptr, (unsigned*)nullptr, (int)tiles_m,
+                                                 (int)(splits > 1 ? 0 : tiles), splits, prefill_error_ptr());
+        g_launches.fetch_add(1, std::memory_order_relaxed);
+        return e == cudaSuccess ? POT_OK : POT_ERR_CUDA;
+    };
+    auto pick = [&](auto b, auto d) -> pot_status_t {
+        constexpr int B = decltype(b)::value, D = decltype(d)::value;
+        if (small) return run(pot_gemm_prefill_kernel<B, 6, 3, 2, 1, D, 1, 3, 0, 1>, 6, 1, 0);
+        return run(pot_gemm_prefill_kernel<B, 3, 3, 2, 2, D, 1, 3, 1, 1>, 3, 2, 1);
+    };
+    using std::integral_constant;
+    if (dt == 0) {
+        if (bits == 2) return pick(integral_constant<int, 2>(), integral_constant<int, 0>());
+        if (bits == 3) return pick(integral_constant<int, 3>(), integral_constant<int, 0>());
+        return pick(integral_constant<int, 4>(), integral_constant<int, 0>());
+    }
+    if (bits == 2) return pick(integral_constant<int, 2>(), integral_constant<int, 1>());
+    if (bits == 3) return pick(integral_constant<int, 3>(), integral_constant<int, 1>());
+    return pick(integral_constant<int, 4>(), integral_constant<int, 1>());
+}
 
 }  // namespace pot
 

@@ -115,7 +115,24 @@ static pot_status_t launch_gemv_stream(const void* packed, const void* scales, c
 #undef POT_SG
 }
 
-// the tiled FP16 / BF16 GEMV for pot_gemm's single-token case
+template <int DT>
+static pot_status_t launch_gemv_canonical(const void* packed, const void* scales, int64_t N, int64_t K, int bits, int group,
+                                          const void* x, void* y, cudaStream_t s) {
+    const dim3 grid((unsigned)((N + 7) / 8)), block(256);
+    auto* P = (const uint32_t*)packed;
+    auto* S = (const uint16_t*)scales;
+    const uint16_t* Z = nullptr;
+    if (bits == 2) return launch_pdl(gemv_canonical_kernel<2, false, DT>, grid, block, 0, s, P, S, Z, N, K, group, (const uint4*)x, (uint16_t*)y);
+    if (bits == 3) return launch_pdl(gemv_canonical_kernel<3, false, DT>, grid, block, 0, s, P, S, Z, N, K, group, (const uint4*)x, (uint16_t*)y);
+    return launch_pdl(gemv_canonical_kernel<4, false, DT>, grid, block, 0, s, P, S, Z, N, K, group, (const uint4*)x, (uint16_t*)y);
+}
+
+// the FP16 / BF16 GEMV for pot_gemm's single-token case
+pot_status_t gemv_canonical_launch(const void* packed, const void* scales, int64_t N, int64_t K, int bits, int group, const void* x,
+                                   void* y, cudaStream_t s, int dt) {
+    return dt == 0 ? launch_gemv_canonical<0>(packed, scales, N, K, bits, group, x, y, s)
+                   : launch_gemv_canonical<1>(packed, scales, N, K, bits, group, x, y, s);
+}
 pot_status_t gemv_stream_launch(const void* packed, const void* scales, int64_t N, int64_t K, int bits, int group, const void* x,
                                 void* y, void* workspace, cudaStream_t s, int dt) {
     if (dt == 0) return launch_gemv_stream<SK_POT, 0>(packed, scales, nullptr, N, K, bits, group, x, y, workspace, s);
@@ -184,15 +201,7 @@ static pot_status_t gemv_impl(const void* packed, const void* scales, int64_t N,
     const pot_status_t st = check_gemv_args(packed, scales, N, K, bits, group, layout, x, y, workspace, ws_bytes);
     if (st != POT_OK) return st;
     cudaStream_t s = (cudaStream_t)stream;
-    if (layout == POT_LAYOUT_CANONICAL) {
-        const dim3 grid((unsigned)((N + 7) / 8)), block(256);
-        auto* P = (const uint32_t*)packed;
-        auto* S = (const uint16_t*)scales;
-        const uint16_t* Z = nullptr;
-        if (bits == 2) return launch_pdl(gemv_canonical_kernel<2, false, DT>, grid, block, 0, s, P, S, Z, N, K, group, (const uint4*)x, (uint16_t*)y);
-        if (bits == 3) return launch_pdl(gemv_canonical_kernel<3, false, DT>, grid, block, 0, s, P, S, Z, N, K, group, (const uint4*)x, (uint16_t*)y);
-        return launch_pdl(gemv_canonical_kernel<4, false, DT>, grid, block, 0, s, P, S, Z, N, K, group, (const uint4*)x, (uint16_t*)y);
-    }
+    if (layout == POT_LAYOUT_CANONICAL) return launch_gemv_canonical<DT>(packed, scales, N, K, bits, group, x, y, s);
     return launch_gemv_stream<SK_POT, DT>(packed, scales, nullptr, N, K, bits, group, x, y, workspace, s);
 }
 

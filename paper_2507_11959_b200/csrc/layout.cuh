@@ -226,6 +226,103 @@ __device__ __forceinline__ void pot_decode32_bf16(const uint32_t* rec, int T, ui
 }
 
 // ---------------------------------------------------------------------------------------------
+// Canonical codes (a little-endian stream of n-bit fields): byte look-ups.  The integer add E << 10 changes only the upper
+// byte of an FP16 scale, and a permute instruction is a table of eight bytes: a group's table of upper bytes (scale and
+// code added up, sign included for n <= 3) is made once, codes spread to four bits each are its selectors, and one more permute
+// per pair joins two looked-up bytes with the scale's lower byte.  For BF16, where E << 7 straddles the bytes, there is a
+// second table for the lower bytes.  About 3.5 (FP16) and 4 (BF16) instructions per pair of weights; masks, shifts and adds on
+// the fields take 7.
+// ---------------------------------------------------------------------------------------------
+// prmt: byte i of the result is byte (sel >> 4i) & 7 of {b, a}; bit 3 of the selector nibble replicates that byte's top bit
+// (the __byte_perm intrinsic clears that bit)
+__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
+    uint32_t d;
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
+    return d;
+}
+template <int BITS, int DT>
+struct CanonLut {
+    uint32_t h0, h1, l0, l1;  // upper bytes, lower bytes (FP16: l0 = the scale's lower byte) by code (n = 4: by exponent)
+    // s: bit pattern of the scale in the output type
+    __device__ __forceinline__ explicit CanonLut(uint32_t s) {
+        if constexpr (DT == 0) {
+            const uint32_t rep = (s >> 8) * 0x01010101u;
+            h0 = (BITS == 2 ? 0x84800400u : 0x0C080400u) + rep;
+            h1 = (BITS == 3 ? 0x8C888480u : 0x1C181410u) + rep;
+            l0 = s & 0xFFu;
+            l1 = 0;
+        } else {
+            const uint32_t p01 = s * 0x10001u + 0x00800000u, p23 = p01 + 0x01000100u;  // {s, s + 2^7}, {s + 2 2^7, s + 3 2^7}
+            if constexpr (BITS == 2) {
+                h0 = __byte_perm(p01, p01 ^ 0x80008000u, 0x7531);
+                l0 = __byte_perm(p01, p01, 0x6420);
+                h1 = l1 = 0;
+            } else {
+                h0 = __byte_perm(p01, p23, 0x7531);
+                l0 = __byte_perm(p01, p23, 0x6420);
+                const uint32_t p45 = p23 + 0x01000100u, p67 = p45 + 0x01000100u;
+                h1 = BITS == 3 ? h0 ^ 0x80808080u : __byte_perm(p45, p67, 0x7531);
+                l1 = BITS == 3 ? l0 : __byte_perm(p45, p67, 0x6420);
+            }
+        }
+    }
+    // four codes, one per nibble of the lower half of y (n <= 3: bit 3 of every nibble is zero) -> two pairs
+    __device__ __forceinline__ void four(uint32_t y, uint32_t& o0, uint32_t& o1) const {
+        uint32_t hb;
+        if constexpr (BITS == 4) {
+            // bit 3 (the sign) makes the permute replicate the top bit of the looked-up byte: 0x80 or 0xFF here
+            const uint32_t sg = prmt(0x80808080u, 0x80808080u, y);
+            y &= 0x7777u;
+            hb = prmt(h0, h1, y) | ((sg << 1) & 0x80808080u);
+        } else {
+            hb = prmt(h0, h1, y);
+        }
+        if constexpr (DT == 0) {
+            o0 = prmt(hb, l0, 0x1404);
+            o1 = prmt(hb, l0, 0x3424);
+        } else {
+            const uint32_t lb = prmt(l0, l1, y);
+            o0 = prmt(hb, lb, 0x1504);
+            o1 = prmt(hb, lb, 0x3726);
+        }
+    }
+};
+// eight codes in the low 8n bits of v (whatever is above them) -> one code per nibble
+template <int BITS>
+__device__ __forceinline__ uint32_t canon_nibbles(uint32_t v) {
+    if constexpr (BITS == 2) {
+        v = __byte_perm(v, 0, 0x4140);
+        v = (v | (v << 4)) & 0x0F0F0F0Fu;
+        return (v | (v << 2)) & 0x33333333u;
+    } else if constexpr (BITS == 3) {
+        v = sel(v, v << 4, 0x0000FFFFu);
+        v = sel(v, v << 2, 0x00FF00FFu);
+        return sel(v, v << 1, 0x0F0F0F0Fu) & 0x77777777u;
+    } else {
+        return v;
+    }
+}
+// 32 consecutive codes (BITS words) -> 16 pairs, in order
+template <int BITS, int DT>
+__device__ __forceinline__ void canon_decode32(const uint32_t* w, const CanonLut<BITS, DT>& lut, uint32_t (&out)[16]) {
+    uint32_t v[4];
+    if constexpr (BITS == 2) {
+        v[0] = w[0]; v[1] = w[0] >> 16; v[2] = w[1]; v[3] = w[1] >> 16;
+    } else if constexpr (BITS == 3) {
+        v[0] = w[0]; v[1] = __funnelshift_r(w[0], w[1], 24); v[2] = __funnelshift_r(w[1], w[2], 16); v[3] = w[2] >> 8;
+    } else {
+#pragma unroll
+        for (int p = 0; p < 4; ++p) v[p] = w[p];
+    }
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+        const uint32_t y = canon_nibbles<BITS>(v[p]);
+        lut.four(y, out[4 * p], out[4 * p + 1]);
+        lut.four(y >> 16, out[4 * p + 2], out[4 * p + 3]);
+    }
+}
+
+// ---------------------------------------------------------------------------------------------
 // Uniform-INT twin on the same tiled layout: w~ = (q - z) * s with q spliced under the exponent
 // of 1024 (0x6400 | q = 1024 + q as FP16), an exact subtraction, and one rounding multiply.
 // zm2 = half2(1024 + z), s2 = half2(s).  A field that sits at mantissa bit b > 0 gives

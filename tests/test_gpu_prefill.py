@@ -3,7 +3,7 @@ import numpy as np
 import pytest
 
 from paper_2507_11959_b200 import synth
-from tests.gpu_util import PotCase, bits_of, f16_dev, gate
+from tests.gpu_util import PotCase, bf16_dev, bits_of, f16_bits_to_bf16_bits, f16_dev, gate
 
 pytestmark = pytest.mark.gpu
 
@@ -103,3 +103,44 @@ def test_prefill_config5_shape_sampled(B, oracle):
     Y, A = oracle.matmul(c.packed, c.S, K, bits, G, X, rows)
     ok, worst, tight = gate(Yg[:, rows], Y, A)
     assert ok and tight < 4.0, (worst, tight)
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("G", [64, 128])
+@pytest.mark.parametrize("dt", ["f16", "bf16"])
+def test_canonical_gemm_matches_oracle(B, oracle, bits, G, dt):
+    """Canonical codes on the tcgen05 kernel: row counts that are no multiple of anything, either side of the 64-token and
+    128 / 256-token tile boundaries, one CTA per tile and clusters of 2 (K = 1024), 4 (K = 2048), 5, 6 (K = 2560, 3072) and 8 CTAs (K >= 4096)."""
+    shapes = [(2, 1, 128), (5, 37, 4096), (16, 129, 1024), (64, 131, 2048), (65, 127, 4224), (128, 130, 640), (129, 255, 1024),
+              (200, 257, 2048), (256, 33, 128), (257, 300, 4096), (520, 140, 1152), (70, 200, 2560), (30, 20, 3072), (140, 5700, 2048), (20, 3400, 2688)]
+    for i, (M, N, K) in enumerate(shapes):
+        c = PotCase(N, K, bits, G, dist="t5" if i % 2 else "normal", sigma=0.015, seed=(5, 400 + 10 * bits + i))
+        X = synth.activations(synth.rng_for(5, 500 + i), M, K, outliers=(i % 2 == 1))
+        if dt == "bf16":
+            X = f16_bits_to_bf16_bits(X)
+        Y, A = oracle.matmul(c.packed, c.S, K, bits, G, X, dtype=oracle.BF16 if dt == "bf16" else oracle.F16)
+        dX = bf16_dev(X) if dt == "bf16" else f16_dev(X)
+        y1 = bits_of(B.pot_gemm(c.d_packed, c.d_S, K, bits, G, dX, B.CANONICAL))
+        y2 = bits_of(B.pot_gemm(c.d_packed, c.d_S, K, bits, G, dX, B.CANONICAL))
+        assert B.pot_debug_errors() == (0, 0, 0)
+        ok, worst, tight = gate(y1, Y, A, bf16=dt == "bf16")
+        assert ok and tight < 4.0, (M, N, K, worst, tight)
+        assert np.array_equal(y1, y2), (M, N, K)   # the splits are added in a fixed order
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("dt", ["f16", "bf16"])
+def test_canonical_one_hot_tokens_return_dequantized_columns(B, oracle, bits, dt):
+    """Every column of a 128-column block through the canonical decode, with scales at both ends of the legal range."""
+    G, N, K = 64, 70, 384
+    c = PotCase(N, K, bits, G, dist="normal", seed=(5, 600 + bits))
+    S = c.S.copy()
+    S[::3] = 0x0400
+    S[1::3] = ((30 - (2 ** (bits - 1) - 1)) << 10) | 0x3FF
+    deq, _ = oracle.dequant(c.packed, S, K, bits, G, oracle.BF16 if dt == "bf16" else oracle.F16)
+    for cols in (np.arange(128), np.arange(130, 190)):
+        X = np.zeros((len(cols), K), dtype=np.uint16)
+        X[np.arange(len(cols)), cols] = 0x3F80 if dt == "bf16" else 0x3C00
+        dX = bf16_dev(X) if dt == "bf16" else f16_dev(X)
+        got = bits_of(B.pot_gemm(c.d_packed, f16_dev(S), K, bits, G, dX, B.CANONICAL))
+        assert np.array_equal(got, deq[:, cols].T)
