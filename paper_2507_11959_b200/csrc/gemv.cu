@@ -4,8 +4,9 @@
 //    range of 16-row x 128-column units through a private shared-memory ring (bulk copies), decodes the codes in
 //    registers with the mask / shift / integer-add of Sec. 4.2 and feeds them, as A fragments, to warp-level
 //    tensor-core MMAs whose B columns all hold x; row blocks that span warps are combined in a fixed order.
-//  * canonical layout (any N): a CUDA-core kernel, one warp per row, 8 codes per lane per step, products
-//    accumulated in FP32 with the mixed-precision FMA and reduced across lanes with warp shuffles.
+//  * canonical layout (any N): warps of 16 rows on the same MMAs, codes straight from global memory into registers and decoded
+//    with byte look-ups; the uniform twin, and vectors too long for shared memory, run on CUDA cores with one warp per row, 8
+//    codes per lane per step, products accumulated in FP32 with the mixed-precision FMA and reduced with warp shuffles.
 //
 // Programmatic dependent launch: weights and scales do not depend on the previous kernel in the stream, x does.
 // The kernels request their first weights before they execute griddepcontrol.wait, and touch x, y and the
@@ -87,6 +88,159 @@ __global__ void __launch_bounds__(256) gemv_canonical_kernel(const uint32_t* __r
     if (lane == 0) y[row] = sk_out<DT>(acc);
 }
 
+// ------------------------------------------------------------------------------------------
+// canonical layout, PoT: 16 rows per warp on the tensor cores
+// ------------------------------------------------------------------------------------------
+// Lane (gid, tig) holds its part of the A fragments of m16n8k16 MMAs: rows gid and gid + 8.  The order of the K columns is
+// free as long as A and B agree, so in a step of 512 columns lane tig takes the WHOLE column block 4 step + tig of its two rows:
+// BITS 16-byte loads per row from contiguous memory, and each register is loaded for the next step as soon as it has been
+// decoded.  x is staged in shared memory (272 bytes per column block: the four blocks that the lanes of a fragment read lie
+// in different banks) and sits in every column of B; at 2 bits in the order in which the codes leave the words most cheaply.
+// CTAs of eight warps, two per SM: while one of them finishes, another (of the next launch, too) sets itself up.  The steps of
+// a row block are dealt to 1, 2, 4 or 8 warps of a CTA and, where few row blocks leave SMs idle, to the CTAs of a cluster; the sums are
+// added in warp order, then in CTA order.  (One CTA of 16 warps per SM with a contiguous, equal share of the steps per warp was
+// 5 - 20 % slower: its launches do not overlap.)
+// Bound by instruction issue (16 rows x 128 columns: 70 - 110 instructions to decode, 8 MMAs, 12 loads) and by fixed latencies (launch, x,
+// codes).  HBM-cold, 10007 x 4096: 9.2 us at 2 bits, 11.2 us at 3, 13.0 us at 4 bits in BF16 (one warp per row on CUDA cores: 26.5,
+// 31.9, 26.5 us); 4099 x 11008 at 3 bits: 36.1 -> 11.3 us.
+constexpr int GC_WARPS = 8;
+constexpr int GC_X_STRIDE = 272;                 // bytes per staged column block
+constexpr int64_t GC_MAX_K = 64 * 1024;          // x takes 136 KB at this length
+struct CanonPlan { int wk_shift, cluster; unsigned grid; };  // log2 of the warps per row block, CTAs per row block
+static CanonPlan plan_canonical(int64_t N, int64_t K) {
+    const int64_t rbs = (N + 15) / 16, steps = (K / 128 + 3) / 4;
+    CanonPlan p{0, 1, 0};
+    while (p.wk_shift < 3 && (rbs << p.wk_shift) < 2 * GC_WARPS * kSmCount && (2 << p.wk_shift) <= steps) ++p.wk_shift;
+    while (p.cluster < 4 && p.wk_shift == 3 && rbs * p.cluster * 2 <= kSmCount && 2 * p.cluster * GC_WARPS <= steps) p.cluster *= 2;
+    const int64_t per_cta = GC_WARPS >> p.wk_shift;
+    p.grid = (unsigned)((rbs + per_cta - 1) / per_cta * p.cluster);
+    return p;
+}
+
+template <int BITS, int DT>
+__global__ void __launch_bounds__(GC_WARPS * 32, 2) gemv_canonical_mma_kernel(const uint4* __restrict__ packed, const uint16_t* __restrict__ scales,
+                                                                              int64_t N, int ncb, int spg, const uint4* __restrict__ x,
+                                                                              uint16_t* __restrict__ y, int wk_shift, int cluster) {
+    extern __shared__ __align__(16) unsigned char xs[];
+    __shared__ float part[GC_WARPS][16];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int gid = lane >> 2, tig = lane & 3;
+    const int WK = 1 << wk_shift;
+    const int crank = (int)blockIdx.x % cluster;
+    const int64_t rb = (int64_t)(blockIdx.x / cluster) * (GC_WARPS >> wk_shift) + (warp >> wk_shift);
+    const int64_t row0 = min(rb * 16 + gid, N - 1), row1 = min(rb * 16 + gid + 8, N - 1);  // (rows past the end repeat the last one and are not stored)
+    const int steps = (ncb + 3) / 4, stride = WK * cluster;
+    pdl_wait();
+    pdl_launch_dependents();
+
+    uint32_t w[2][4 * BITS], sc[2][2];
+    const uint4* src[2];
+    const uint16_t* ssrc[2];
+    auto point = [&](int step) {  // the codes and scales of this lane's column block (a block past the end repeats the last one)
+        const int cb = min(4 * step + tig, ncb - 1);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int64_t block = (h ? row1 : row0) * ncb + cb;
+            src[h] = packed + block * BITS;
+            ssrc[h] = scales + block * spg;
+        }
+    };
+    auto load_codes = [&](int t) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const uint4 q = __ldg(src[h] + t);
+            w[h][4 * t + 0] = q.x; w[h][4 * t + 1] = q.y; w[h][4 * t + 2] = q.z; w[h][4 * t + 3] = q.w;
+        }
+    };
+    auto load_scales = [&](int hb) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) sc[h][hb] = __ldg(ssrc[h] + (spg == 2 ? hb : 0));
+    };
+    int step = crank * WK + (warp & (WK - 1));
+    if (step < steps) {
+        point(step);
+#pragma unroll
+        for (int t = 0; t < BITS; ++t) load_codes(t);
+        load_scales(0);
+        load_scales(1);
+    }
+    if constexpr (BITS == 2) {  // the order of canon_decode32_any
+        for (int i = threadIdx.x; i < ncb * 8; i += GC_WARPS * 32) {
+            const uint4 a = ld_dependent16(x + 2 * i), b = ld_dependent16(x + 2 * i + 1);
+            uint4* dst = reinterpret_cast<uint4*>(xs + (i >> 3) * GC_X_STRIDE + (i & 7) * 32);
+            dst[0] = make_uint4(potl::prmt(a.x, a.y, 0x5410), potl::prmt(a.z, a.w, 0x5410), potl::prmt(b.x, b.y, 0x5410), potl::prmt(b.z, b.w, 0x5410));
+            dst[1] = make_uint4(potl::prmt(a.x, a.y, 0x7632), potl::prmt(a.z, a.w, 0x7632), potl::prmt(b.x, b.y, 0x7632), potl::prmt(b.z, b.w, 0x7632));
+        }
+    } else {
+        for (int i = threadIdx.x; i < ncb * 16; i += GC_WARPS * 32)
+            *reinterpret_cast<uint4*>(xs + (i >> 4) * GC_X_STRIDE + (i & 15) * 16) = ld_dependent16(x + i);
+    }
+    if (threadIdx.x < 16) *reinterpret_cast<uint4*>(xs + ncb * GC_X_STRIDE + threadIdx.x * 16) = make_uint4(0, 0, 0, 0);  // x of the block past the end
+    __syncthreads();
+
+    float acc[2][4] = {};
+    for (; step < steps; step += stride) {
+        const unsigned char* xb = xs + min(4 * step + tig, ncb) * GC_X_STRIDE;
+        const bool more = step + stride < steps;
+        if (more) point(step + stride);
+#pragma unroll
+        for (int hb = 0; hb < 2; ++hb) {
+            uint32_t s0 = sc[0][hb], s1 = sc[1][hb];
+            if (DT == 1) {
+                s0 = __bfloat16_as_ushort(__float2bfloat16_rn(__half2float(__ushort_as_half((uint16_t)s0))));
+                s1 = __bfloat16_as_ushort(__float2bfloat16_rn(__half2float(__ushort_as_half((uint16_t)s1))));
+            }
+            const potl::CanonLut<BITS, DT> lut0(s0), lut1(s1);
+            if (more) load_scales(hb);
+#pragma unroll
+            for (int T = 2 * hb; T < 2 * hb + 2; ++T) {
+                uint32_t lo[16], hi[16], xq[16];
+                potl::canon_decode32_any<BITS, DT>(w[0] + T * BITS, lut0, lo);
+                potl::canon_decode32_any<BITS, DT>(w[1] + T * BITS, lut1, hi);
+                if (more) {  // the 16-byte pieces whose last word belongs to this quarter
+#pragma unroll
+                    for (int t = 0; t < BITS; ++t)
+                        if ((4 * t + 3) / BITS == T) load_codes(t);
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const uint4 v = *reinterpret_cast<const uint4*>(xb + T * 64 + i * 16);
+                    xq[4 * i + 0] = v.x; xq[4 * i + 1] = v.y; xq[4 * i + 2] = v.z; xq[4 * i + 3] = v.w;
+                }
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    if constexpr (DT == 0) sk_mma(acc[j & 1], lo[2 * j], hi[2 * j], lo[2 * j + 1], hi[2 * j + 1], xq[2 * j], xq[2 * j + 1]);
+                    else sk_mma_bf16(acc[j & 1], lo[2 * j], hi[2 * j], lo[2 * j + 1], hi[2 * j + 1], xq[2 * j], xq[2 * j + 1]);
+            }
+        }
+    }
+    if (tig == 0) {
+        part[warp][gid] = acc[0][0] + acc[1][0];
+        part[warp][gid + 8] = acc[0][2] + acc[1][2];
+    }
+    __syncthreads();
+    // the first warp of a row block adds the sums of its warps, the first CTA of a cluster those of its CTAs
+    float sum = 0.f;
+    const bool first = (warp & (WK - 1)) == 0 && lane < 16;
+    if (first)
+        for (int q = 0; q < WK; ++q) sum += part[warp + q][lane];
+    if (cluster > 1) {
+        __syncthreads();
+        if (first) part[warp][lane] = sum;
+        asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+        if (first && crank == 0)
+            for (int z = 1; z < cluster; ++z) {
+                uint32_t addr;
+                float v;
+                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(smem_u32(&part[warp][lane])), "r"(z));
+                asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+                sum += v;
+            }
+        asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");  // the sums have been read
+    }
+    if (first && crank == 0 && rb * 16 + lane < N) y[rb * 16 + lane] = sk_out<DT>(sum);
+}
+
 // CTAs per SM of the streaming GEMV (16 consumer warps each).  Two: the next launch in the stream becomes resident,
 // sets itself up and fills its rings while this one computes, which hides the launch and the prologue (about 2.5 us);
 // the price is 64 registers per thread and half the ring, i.e. a slower loop (about 15 %).  Worth it while a CTA's
@@ -118,6 +272,33 @@ static pot_status_t launch_gemv_stream(const void* packed, const void* scales, c
 template <int DT>
 static pot_status_t launch_gemv_canonical(const void* packed, const void* scales, int64_t N, int64_t K, int bits, int group,
                                           const void* x, void* y, cudaStream_t s) {
+    if (K <= GC_MAX_K) {
+        const CanonPlan p = plan_canonical(N, K);
+        auto run = [&](auto kernel) -> pot_status_t {
+            const size_t smem = (size_t)(K / 128 + 1) * GC_X_STRIDE;
+            if (smem > 46 * 1024 && !allow_max_dynamic_smem(kernel)) return POT_ERR_CUDA;
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(p.grid);
+            cfg.blockDim = dim3(GC_WARPS * 32);
+            cfg.dynamicSmemBytes = smem;
+            cfg.stream = s;
+            cudaLaunchAttribute attr[2];
+            attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            attr[0].val.programmaticStreamSerializationAllowed = 1;
+            attr[1].id = cudaLaunchAttributeClusterDimension;
+            attr[1].val.clusterDim.x = (unsigned)p.cluster;
+            attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = p.cluster > 1 ? 2 : 1;
+            const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, (const uint4*)packed, (const uint16_t*)scales, N, (int)(K / 128),
+                                                     128 / group, (const uint4*)x, (uint16_t*)y, p.wk_shift, p.cluster);
+            g_launches.fetch_add(1, std::memory_order_relaxed);
+            return e == cudaSuccess ? POT_OK : POT_ERR_CUDA;
+        };
+        if (bits == 2) return run(gemv_canonical_mma_kernel<2, DT>);
+        if (bits == 3) return run(gemv_canonical_mma_kernel<3, DT>);
+        return run(gemv_canonical_mma_kernel<4, DT>);
+    }
     const dim3 grid((unsigned)((N + 7) / 8)), block(256);
     auto* P = (const uint32_t*)packed;
     auto* S = (const uint16_t*)scales;

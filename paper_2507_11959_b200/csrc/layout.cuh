@@ -322,6 +322,23 @@ __device__ __forceinline__ void canon_decode32(const uint32_t* w, const CanonLut
     }
 }
 
+// The same 16 pairs in the order that is cheapest to decode, for kernels that can hold the activations in that order: as above
+// for n = 3, 4; for n = 2, where every other code of a word is in a nibble of its own already, the 16 codes of a word leave as
+// (0,2) (4,6) (8,10) (12,14) (1,3) (5,7) (9,11) (13,15).
+template <int BITS, int DT>
+__device__ __forceinline__ void canon_decode32_any(const uint32_t* w, const CanonLut<BITS, DT>& lut, uint32_t (&out)[16]) {
+    if constexpr (BITS != 2) {
+        canon_decode32<BITS, DT>(w, lut, out);
+    } else {
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+            const uint32_t y = (w[p >> 1] >> (2 * (p & 1))) & 0x33333333u;
+            lut.four(y, out[4 * p], out[4 * p + 1]);
+            lut.four(y >> 16, out[4 * p + 2], out[4 * p + 3]);
+        }
+    }
+}
+
 // ---------------------------------------------------------------------------------------------
 // Uniform-INT twin on the same tiled layout: w~ = (q - z) * s with q spliced under the exponent
 // of 1024 (0x6400 | q = 1024 + q as FP16), an exact subtraction, and one rounding multiply.

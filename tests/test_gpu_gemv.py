@@ -4,7 +4,7 @@ import pytest
 import torch
 
 from paper_2507_11959_b200 import synth
-from tests.gpu_util import PotCase, UintCase, bits_of, f16_dev, gate, to_dev
+from tests.gpu_util import PotCase, UintCase, bf16_dev, bits_of, f16_bits_to_bf16_bits, f16_dev, gate, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -153,3 +153,23 @@ def test_gemv_with_activations_too_long_for_shared_memory(B, oracle):
     ok, worst, tight = gate(bits_of(y), Y[0], A[0])
     assert ok and tight < 4.0, ("uint", worst, tight)
     assert B.pot_debug_errors() == (0, 0, 0)
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("dt", ["f16", "bf16"])
+def test_canonical_gemv_over_every_way_to_share_a_row_block(B, oracle, bits, dt):
+    """1, 2, 4 and 8 warps per row block and clusters of 2 and 4 CTAs; last steps that are partly past the end; one row; rows that
+    are no multiple of 16; x at and beyond the longest one that is staged in shared memory."""
+    for i, (N, K, G) in enumerate([(1, 128, 64), (17, 640, 128), (38001, 512, 128), (18993, 1152, 64), (9601, 2048, 64), (1001, 4096, 128), (555, 11008, 64),
+                                   (1030, 14336, 128), (96, 28672, 64), (9, 65536, 128), (5, 65664, 64)]):
+        c = PotCase(N, K, bits, G, dist="t5", seed=(4, 1000 + 10 * bits + i))
+        X = acts(1, K, 1100 + i)
+        if dt == "bf16":
+            X = f16_bits_to_bf16_bits(X)
+        rows = np.unique(np.concatenate([np.arange(min(N, 40)), np.arange(max(0, N - 40), N), np.linspace(0, N - 1, 50).astype(np.int64)]))
+        Y, A = oracle.matmul(c.packed, c.S, K, bits, G, X, rows=rows, dtype=oracle.BF16 if dt == "bf16" else oracle.F16)
+        dx = bf16_dev(X[0]) if dt == "bf16" else f16_dev(X[0])
+        y = bits_of(B.pot_gemv(c.d_packed, c.d_S, K, bits, G, dx, B.CANONICAL))
+        ok, worst, tight = gate(y[rows], Y[0], A[0], bf16=dt == "bf16")
+        assert ok and tight < 4.0, (N, K, worst, tight)
+        assert np.array_equal(y, bits_of(B.pot_gemv(c.d_packed, c.d_S, K, bits, G, dx, B.CANONICAL)))
