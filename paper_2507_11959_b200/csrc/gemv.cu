@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(256) gemv_canonical_kernel(const uint32_t* __r
 // added in warp order, then in CTA order.  (One CTA of 16 warps per SM with a contiguous, equal share of the steps per warp was
 // 5 - 20 % slower: its launches do not overlap.)
 // Bound by instruction issue (16 rows x 128 columns: 70 - 110 instructions to decode, 8 MMAs, 12 loads) and by fixed latencies (launch, x,
-// codes).  HBM-cold, 10007 x 4096: 9.2 us at 2 bits, 11.2 us at 3, 13.0 us at 4 bits in BF16 (one warp per row on CUDA cores: 26.5,
+// codes).  HBM-cold, 10007 x 4096: 8.8 us at 2 bits, 11.7 us at 3, 13.0 us at 4 bits in BF16 (one warp per row on CUDA cores: 26.5,
 // 31.9, 26.5 us); 4099 x 11008 at 3 bits: 36.1 -> 11.3 us.
 constexpr int GC_WARPS = 8;
 constexpr int GC_X_STRIDE = 272;                 // bytes per staged column block
