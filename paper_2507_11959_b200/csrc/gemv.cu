@@ -246,8 +246,8 @@ __global__ void __launch_bounds__(GC_WARPS * 32, 2) gemv_canonical_mma_kernel(co
 // the price is 64 registers per thread and half the ring, i.e. a slower loop (about 15 %).  Worth it while a CTA's
 // share of the matrix is small; one CTA per SM otherwise, and whenever the half-size ring could not hold two slots.
 constexpr size_t kTwoCtaMaxShare = 300 * 1024;  // bytes of codes + scales per CTA
-static int gemv_occupancy(int64_t N, int64_t K, int bits, int group, int kind) {
-    const StreamPlan p2 = plan_stream(N, K, 1, bits, group, kind, 1, 16, 2);
+static int gemv_occupancy(int64_t N, int64_t K, int bits, int group, int kind, int dt = 0) {
+    const StreamPlan p2 = plan_stream(N, K, 1, bits, group, kind, 1, 16, 2, dt);
     if (!p2.ok || !p2.x_in_smem || p2.ring_capacity < 2 || p2.grid < kSmCount) return 1;
     const size_t share = (size_t)(N / 16) * (size_t)(K / 128) * (size_t)sk_unit_total_bytes(bits, group, kind) / (size_t)p2.grid;
     return share <= kTwoCtaMaxShare ? 2 : 1;
@@ -258,7 +258,7 @@ static pot_status_t launch_gemv_stream(const void* packed, const void* scales, c
                                        int bits, int group, const void* x, void* y, void* workspace, cudaStream_t s) {
     int* err = error_ptr(ERR_GEMV);
 #define POT_SG(B, O) return launch_stream<B, KIND, 1, 16, O, DT>(packed, scales, zeros, N, K, group, x, 1, y, workspace, err, s)
-    if (gemv_occupancy(N, K, bits, group, KIND) == 2) {
+    if (gemv_occupancy(N, K, bits, group, KIND, DT) == 2) {
         if (bits == 2) POT_SG(2, 2);
         if (bits == 3) POT_SG(3, 2);
         POT_SG(4, 2);

@@ -192,6 +192,63 @@ __device__ __forceinline__ void pot_decode32(const uint32_t* rec, int T, uint32_
     }
 }
 
+// The same 32 codes without the scale, for kernels that multiply a group's FP32 sums by it: out[p] = half2{ +-2^(E - 7), +-2^(E - 7) },
+// the masked fields under a constant exponent of 8: ONE logic operation, (word & mask) | bias, instead of a mask and a
+// multiply-add, provided that the bias sits in a register (an instruction takes one constant: with two, mask and bias become
+// two instructions, +24 % time).  Left shifts are multiplications by 2^n read from constant memory (p2[n] = 2^n, which the
+// compiler must not know), because the multiply-add pipe has cycles to spare and the ALU pipe has none: 2 - 3 % faster than
+// shifts.  Right rotations stay on the ALU pipe: as 64-bit products they were 15 - 20 % slower.
+//   lower byte lanes (0, 2) of a word that has to be rotated right by s and then shifted left by 8: their bits lie below bit 29
+//   and move left by 8 - s, so that nothing wraps and no rotation is needed.
+constexpr uint32_t POT_UNIT_BIAS = 0x20002000u;  // exponent field 8: E <= 7 fits below
+constexpr float POT_UNIT_SCALE = 128.f;          // weights of pot_units32 times this are +-2^E
+constexpr int POT_UNIT_SHIFTS = 11;              // p2[0 .. 10]
+
+template <int BITS>
+__device__ __forceinline__ void pot_units32(const uint32_t (&w)[BITS], const uint32_t* __restrict__ p2, uint32_t bias, uint32_t (&out)[16]) {
+    constexpr uint32_t MB = PotLanes<BITS>::MASK & 0xFF00FF00u;
+    auto in_place = [&](uint32_t t) {  // (t & MB) | bias
+        uint32_t d;
+        asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(d) : "r"(t), "r"(MB), "r"(bias));
+        return d;
+    };
+    auto shl = [&](uint32_t v, int n) { return n == 0 ? v : mad(v, p2[n], 0u); };
+    // a word whose fields sit `low` positions below their place
+    auto plain = [&](int i, uint32_t v, int low) {
+        out[2 * i] = in_place(shl(v, 8 + low));
+        out[2 * i + 1] = in_place(shl(v, low));
+    };
+    auto rotated = [&](int i, uint32_t v, int s) {
+        out[2 * i] = in_place(shl(v, 8 - s));
+        out[2 * i + 1] = in_place(rotr(v, s));
+    };
+    if constexpr (BITS == 2) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            plain(4 * k + 0, w[k], 2);
+            plain(4 * k + 1, w[k], 0);
+            rotated(4 * k + 2, w[k], 2);
+            rotated(4 * k + 3, w[k], 4);
+        }
+    } else if constexpr (BITS == 3) {
+        plain(0, w[0], 1);
+        rotated(1, w[0], 1);
+        rotated(2, w[1], 2);
+        rotated(3, w[1], 4);
+        rotated(4, w[2], 3);
+        rotated(5, w[2], 5);
+        plain(6, sel(sel(w[0], w[1], 0x80808080u), w[2], 0x84848484u), 0);
+        plain(7, sel(sel(w[0], w[1], 0x20202020u), w[2], 0x21212121u), 2);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            plain(2 * k, w[k], 0);
+            // E0, E1 and the sign move up by 2, E2 down by 2, inside their byte lanes
+            plain(2 * k + 1, sel(shl(w[k], 2), w[k] >> 2, 0x8C8C8C8Cu), 0);
+        }
+    }
+}
+
 // t * c (upper 32 bits of the product) + s as one instruction: a right shift by 32 - log2(c) fused with the add
 __device__ __forceinline__ uint32_t madhi(uint32_t t, uint32_t c, uint32_t s) {
     uint32_t d;

@@ -12,10 +12,12 @@
 // are requested before the kernel waits for its predecessor in the stream (the weights are constants).
 //
 // Arithmetic.  Lane (gid, tig) of a warp owns quarter tig (32 columns) of rows gid and gid + 8 of a unit: exactly its
-// share of the A fragments of eight m16n8k16 MMAs.  It decodes its 2 x 32 codes in registers (mask, shift and integer add
-// into the group scale's bit pattern, Sec. 4.2 of the paper) and issues the MMAs against B fragments that hold the
-// activation vector in every column (GEMV) or one token per column (small batch).  The FP32 accumulators stay in
-// registers for as long as the warp stays inside one row block.
+// share of the A fragments of eight m16n8k16 MMAs.  It decodes its 2 x 32 codes in registers to +-2^E under a constant
+// exponent and issues the MMAs against B fragments that hold the activation vector in every column (GEMV) or one token per
+// column (small batch); the group's scale multiplies the unit's FP32 sums.  (Where a unit's sums mix two groups -- several tokens
+// with G = 64 --, where x does not fit in shared memory and in the uniform twin the scale goes into the weights: mask, shift and
+// integer add into its bit pattern, Sec. 4.2 of the paper.)  The FP32 accumulators stay in registers for as long as the warp
+// stays inside one row block.
 //
 // Delivery.  A warp that covered a whole row block writes Y.  Otherwise its sums go to slot (row block, position of the
 // warp among the row block's contributors) of the workspace; a per-row-block arrival counter tells the last contributor,
@@ -24,6 +26,8 @@
 #include "common.cuh"
 #include "layout.cuh"
 #include "sync.cuh"
+
+#include <type_traits>
 
 namespace pot {
 
@@ -55,6 +59,7 @@ struct StreamPlan {
     int ring_capacity;    // slots per warp that would fit
     int tok;              // B columns in use: 1 (GEMV) or 8 (small batch)
     bool x_in_smem;
+    bool unscaled;        // decode without the scale, which multiplies the group's sums instead
     int token_shift;      // log2 of the token slots of the staged activations (0 for the GEMV)
     size_t x_bytes, smem_bytes;
     int max_slots;        // partial-sum slots per row block
@@ -64,7 +69,12 @@ struct StreamPlan {
     bool ok;              // false: the shape cannot run on this kernel (too many units)
 };
 
-inline StreamPlan plan_stream(int64_t N, int64_t K, int64_t M, int bits, int group, int kind, int tok, int warps, int occ = 1) {
+// bytes that the unscaled kernel keeps behind the activations: 256 zeros (GEMV) and, for BF16, one FP32 factor per unit and token slot
+__host__ __device__ constexpr int sk_x_extra(int ncb, int tok, int token_shift, int dt) {
+    return (tok == 1 ? 256 : 0) + (dt == 1 ? (ncb << token_shift) * 4 : 0);
+}
+
+inline StreamPlan plan_stream(int64_t N, int64_t K, int64_t M, int bits, int group, int kind, int tok, int warps, int occ = 1, int dt = 0) {
     StreamPlan p = {};
     const int64_t nrb = N / 16, ncb = K / 128, U = nrb * ncb;
     p.ok = U > 0 && U < (int64_t(1) << 31) && ncb < (1 << 24);
@@ -90,7 +100,8 @@ inline StreamPlan plan_stream(int64_t N, int64_t K, int64_t M, int bits, int gro
     const size_t hdr = (size_t)sk_header_bytes(warps, tok);
     // multi-token kernel: the staged block has 2, 4 or 8 token slots per 16-byte chunk position (the smallest that holds M)
     p.token_shift = tok > 1 ? (M <= 2 ? 1 : (M <= 4 ? 2 : 3)) : 0;
-    const size_t xb = ((size_t)K * 2) << p.token_shift;
+    p.unscaled = kind == SK_POT && (tok == 1 || group == 128);
+    const size_t xb = (((size_t)K * 2) << p.token_shift) + (p.unscaled ? (size_t)sk_x_extra((int)ncb, tok, p.token_shift, dt) : 0);
     // slots of 4 units unless the ring could then hold only one of them next to the staged activations
     int q = SK_QMAX;
     if (hdr + xb + (size_t)warps * 2 * (size_t)sk_slot_bytes(bits, group, kind, q) > budget) q = 2;
@@ -100,6 +111,7 @@ inline StreamPlan plan_stream(int64_t N, int64_t K, int64_t M, int bits, int gro
     const size_t slot = (size_t)sk_slot_bytes(bits, group, kind, q);
     const size_t ring2 = (size_t)warps * 2 * slot;  // at least two slots per warp
     p.x_in_smem = hdr + xb + ring2 <= budget;
+    p.unscaled = p.unscaled && p.x_in_smem;
     p.x_bytes = p.x_in_smem ? (xb + 127) / 128 * 128 : 0;
     int64_t st = (int64_t)((budget - hdr - p.x_bytes) / ((size_t)warps * slot));
     p.ring_capacity = (int)(st > 8 ? 8 : st);
@@ -132,6 +144,8 @@ struct StreamArgs {
     int token_shift;               // log2 of the token slots of the staged activations
     int fits32;                    // U * gw_total < 2^32: 32-bit range arithmetic
     int aligned, nrb;              // row-block split (see the kernel), number of row blocks
+    uint32_t bias;                 // potl::POT_UNIT_BIAS and
+    uint32_t p2[potl::POT_UNIT_SHIFTS];  // p2[n] = 2^n
 #ifdef SK_TRACE
     unsigned long long* trace;     // [launch slot][cta][8] globaltimer stamps
 #endif
@@ -160,6 +174,32 @@ __device__ __forceinline__ uint16_t sk_out(float v) {
 }
 __device__ __forceinline__ uint32_t sk_lds32(const unsigned char* p) { return *reinterpret_cast<const uint32_t*>(p); }
 __device__ __forceinline__ uint4 sk_lds128(const unsigned char* p) { return *reinterpret_cast<const uint4*>(p); }
+// Eight BF16 numbers -> FP16 numbers relative to the largest finite one of the 16 lanes that differ in the bits of `lanes`
+// (brought to 2^14 .. 2^15); returns the factor that undoes it.  All 32 lanes take part; !ok: the lane holds nothing.
+__device__ __forceinline__ float sk_normalize(uint4& v, bool ok, int lanes) {
+    uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    uint32_t e = 0x80u;  // exponent field 1, at bit 7
+    if (ok) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t lo = w[i] & 0x7F80u, hi = (w[i] >> 16) & 0x7F80u;
+            e = max(e, lo == 0x7F80u ? 0u : lo);
+            e = max(e, hi == 0x7F80u ? 0u : hi);
+        }
+    }
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1)
+        if (lanes & o) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+    const uint32_t up = min(268u - (e >> 7), 253u);  // exponent field of the factor (253: its inverse is still a normal number)
+    const float f = __uint_as_float(up << 23);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const __half2 h = __floats2half2_rn(__uint_as_float(w[i] << 16) * f, __uint_as_float(w[i] & 0xFFFF0000u) * f);
+        w[i] = *reinterpret_cast<const uint32_t*>(&h);
+    }
+    v = make_uint4(w[0], w[1], w[2], w[3]);
+    return __uint_as_float((254u - up) << 23);
+}
 // floor(a * b / c) for a * b that may need 64 bits
 __device__ __forceinline__ uint32_t sk_muldiv(uint32_t a, uint32_t b, uint32_t c, bool fits32) {
     if (fits32) return (a * b) / c;
@@ -172,7 +212,12 @@ __device__ __forceinline__ uint32_t sk_muldiv(uint32_t a, uint32_t b, uint32_t c
 // XSMEM: the activations are staged in shared memory in fragment order (else they are read through L1 from global).
 // W consumer warps per CTA; OCC = 2 leaves room for a second CTA on the SM (64 registers per thread, half the shared
 // memory), so that the next launch in the stream can become resident and fill its rings while this one still computes.
-template <int BITS, int KIND, int TOK, bool XSMEM, int W, int OCC, int SK_Q, int DT>
+// UNSC: the codes are decoded without their scale (pot_units32) and a unit's FP32 sums are multiplied by it.  With two groups per
+// unit (G = 64, GEMV only) columns 0-3 of B hold x of the first group's quarters and zeros for the others, columns 4-7 the
+// opposite, so that the two groups' sums come out in different lanes.  BF16 activations are staged as FP16 numbers relative to
+// the largest of their unit (2^14 .. 2^15), whose factor the unit's sums are multiplied by: the error, 2^-25 in those units where
+// FP16 runs out of exponents, is 2^-39 of the unit's largest |x|, against which every weight of the group counts at least 2^-7.
+template <int BITS, int KIND, int TOK, bool XSMEM, int W, int OCC, int SK_Q, int DT, bool UNSC>
 __device__ __forceinline__ void stream_body(const StreamArgs& sa, int* __restrict__ err) {
     constexpr int UB = sk_unit_bytes(BITS);
     constexpr bool UNIFORM = (KIND == SK_UINT);
@@ -207,6 +252,7 @@ __device__ __forceinline__ void stream_body(const StreamArgs& sa, int* __restric
     unsigned* lcnt = reinterpret_cast<unsigned*>(smem + W * 96);               // local arrival counters
     float* lslots = reinterpret_cast<float*>(smem + W * 96 + W * 4);           // [warp][first, last][16 TOK]
     const unsigned char* xs = smem + HDR;
+    float* xfac = reinterpret_cast<float*>(smem + HDR + ((sa.K * 2) << sa.token_shift) + (TOK == 1 ? 256 : 0));  // UNSC, BF16: [unit][token slot]
     const unsigned char* ringp = xs + sa.x_bytes + (uint32_t)warp * (uint32_t)S * slot_bytes;  // this warp's ring
     const uint32_t ring = smem0 + (uint32_t)HDR + (uint32_t)sa.x_bytes + (uint32_t)warp * (uint32_t)S * slot_bytes;
 
@@ -282,10 +328,12 @@ __device__ __forceinline__ void stream_body(const StreamArgs& sa, int* __restric
         uint4* dst = reinterpret_cast<uint4*>(smem + HDR);
         const uint4* src = reinterpret_cast<const uint4*>(sa.X);
         const int kc = (int)(sa.K / 8);  // 16-byte chunks per token
+        if constexpr (UNSC && TOK == 1)
+            if (threadIdx.x < 16) *reinterpret_cast<uint4*>(smem + HDR + sa.K * 2 + threadIdx.x * 16) = make_uint4(0, 0, 0, 0);
         if constexpr (TOK == 1) {
             // chunk (quarter t, part j) of a unit goes to position j * 4 + t: lanes tig = 0..3 read 64 contiguous bytes
             // (four loads in flight per thread before the first store: one round trip for K <= 32 * 32 W)
-            for (int i0 = threadIdx.x; i0 < kc; i0 += 4 * W * 32) {
+            for (int i0 = threadIdx.x; (i0 & ~31) < kc; i0 += 4 * W * 32) {  // (whole warps)
                 uint4 v[4];
 #pragma unroll
                 for (int p = 0; p < 4; ++p)
@@ -293,6 +341,10 @@ __device__ __forceinline__ void stream_body(const StreamArgs& sa, int* __restric
 #pragma unroll
                 for (int p = 0; p < 4; ++p) {
                     const int i = i0 + p * W * 32;
+                    if constexpr (UNSC && DT == 1) {  // lanes 0-15 and 16-31 hold one unit each
+                        const float f = sk_normalize(v[p], i < kc, 0x0F);
+                        if (i < kc && (i & 15) == 0) xfac[i >> 4] = f;
+                    }
                     if (i < kc) dst[(i & ~15) | ((i & 3) << 2) | ((i >> 2) & 3)] = v[p];
                 }
             }
@@ -306,7 +358,7 @@ __device__ __forceinline__ void stream_body(const StreamArgs& sa, int* __restric
             // token's parity, then j -- a warp loads the 256 contiguous bytes of a unit for two tokens.
             const int ts = sa.token_shift;
             const int total = kc << ts;
-            for (int e0 = threadIdx.x; e0 < total; e0 += 8 * W * 32) {  // eight loads in flight per thread
+            for (int e0 = threadIdx.x; (e0 & ~31) < total; e0 += 8 * W * 32) {  // eight loads in flight per thread, whole warps
                 uint4 v[8];
 #pragma unroll
                 for (int p = 0; p < 8; ++p) {
@@ -320,6 +372,10 @@ __device__ __forceinline__ void stream_body(const StreamArgs& sa, int* __restric
                     const int e = e0 + p * W * 32;
                     const int t = e & 3, par = (e >> 2) & 1, j = (e >> 3) & 3, hi = (e >> 5) & ((1 << (ts - 1)) - 1), unit_ = e >> (4 + ts);
                     const int token = (hi << 1) | par;
+                    if constexpr (UNSC && DT == 1) {  // a warp holds one unit of two tokens: t in bits 0-1 of the lane, j in bits 3-4
+                        const float f = sk_normalize(v[p], e < total && token < sa.M, 0x1B);
+                        if (e < total && (e & 0x1B) == 0) xfac[(unit_ << ts) + token] = f;
+                    }
                     if (e < total && token < sa.M) dst[(((unit_ << 2) + j) << (2 + ts)) + (hi << 3) + (par << 2) + t] = v[p];
                 }
             }
@@ -342,6 +398,16 @@ __device__ __forceinline__ void stream_body(const StreamArgs& sa, int* __restric
             v[e] = acc[0][e] + acc[1][e];
             acc[0][e] = 0.f;
             acc[1][e] = 0.f;
+        }
+        if constexpr (UNSC) {
+            if constexpr (TOK == 1) {
+                if (spg == 2) {  // the second group's sums sit in lanes tig = 2, 3
+                    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+                    v[2] += __shfl_xor_sync(0xffffffffu, v[2], 2);
+                }
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) v[e] *= potl::POT_UNIT_SCALE;
         }
         const bool first = rbd == wst[2];
         const uint32_t expect = first ? wst[5] : (rbd == wst[3] ? wst[6] : 0u);
@@ -441,6 +507,11 @@ __device__ __forceinline__ void stream_body(const StreamArgs& sa, int* __restric
             for (int h = 0; h < 2; ++h)
 #pragma unroll
                 for (int k = 0; k < BITS; ++k) w[h][k] = sk_lds32(code + (uint32_t)(k * 256 + h * 128) + (uint32_t)lane * 4u);
+            if constexpr (UNSC) {
+                potl::pot_units32<BITS>(w[0], sa.p2, sa.bias, lo);
+                potl::pot_units32<BITS>(w[1], sa.p2, sa.bias, hi);
+                return;
+            }
             const uint32_t scw = sk_lds32(param + poff);  // {row gid, row gid + 8}
             if constexpr (DT == 0) {
                 potl::pot_decode32<BITS, 1>(w[0], 0, __byte_perm(scw, 0, 0x1010), lo);
@@ -479,11 +550,15 @@ __device__ __forceinline__ void stream_body(const StreamArgs& sa, int* __restric
             }
         }
     };
-    auto multiply = [&](const uint32_t (&lo)[16], const uint32_t (&hi)[16], uint32_t cbu) {
+    // this lane's column of B (GEMV): x, or zeros if the column belongs to the other group
+    const bool zero_column = UNSC && TOK == 1 && spg == 2 && (gid >> 2) != (tig >> 1);
+    const unsigned char* xcol = zero_column ? xs + sa.K * 2 + tig * 16 : xs + tig * 16;
+    const uint32_t xstep = zero_column ? 0u : 256u;
+    auto multiply = [&](const uint32_t (&lo)[16], const uint32_t (&hi)[16], const unsigned char* param, uint32_t cbu) {
         // activations of quarter tig (of token gid): the B fragments of the eight MMAs
         uint32_t xq[16];
         if constexpr (XSMEM) {
-            const unsigned char* xa = TOK == 1 ? xs + cbu * 256u + (uint32_t)tig * 16u
+            const unsigned char* xa = TOK == 1 ? xcol + cbu * xstep
                                                : xs + ((((cbu * 16u) << sa.token_shift) + ((((uint32_t)gid & ((1u << sa.token_shift) - 1u)) >> 1) << 3) +
                                                         (((uint32_t)gid & 1u) << 2) + (uint32_t)tig) << 4);
 #pragma unroll
@@ -502,6 +577,35 @@ __device__ __forceinline__ void stream_body(const StreamArgs& sa, int* __restric
                 xq[4 * i + 0] = v.x; xq[4 * i + 1] = v.y; xq[4 * i + 2] = v.z; xq[4 * i + 3] = v.w;
             }
         }
+        if constexpr (UNSC) {
+            float c[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int j = 0; j < 8; ++j) sk_mma(c, lo[2 * j], hi[2 * j], lo[2 * j + 1], hi[2 * j + 1], xq[2 * j], xq[2 * j + 1]);
+            const uint32_t scw = sk_lds32(param + ((spg == 2 ? (uint32_t)(tig >> 1) * 8u : 0u) + (uint32_t)gid) * 4u);  // {row gid, row gid + 8}
+            float2 sc = __half22float2(*reinterpret_cast<const __half2*>(&scw));
+            if constexpr (DT == 0) {
+                acc[0][0] = fmaf(c[0], sc.x, acc[0][0]);
+                acc[0][2] = fmaf(c[2], sc.y, acc[0][2]);
+                if constexpr (TOK > 1) {
+                    acc[0][1] = fmaf(c[1], sc.x, acc[0][1]);
+                    acc[0][3] = fmaf(c[3], sc.y, acc[0][3]);
+                }
+            } else {  // the FP16 scale rounded once to BF16; times the unit's factor last, so that no product leaves FP32's range early
+                sc = __bfloat1622float2(__float22bfloat162_rn(sc));
+                if constexpr (TOK == 1) {
+                    const float f = xfac[cbu];
+                    acc[0][0] = fmaf(c[0] * sc.x, f, acc[0][0]);
+                    acc[0][2] = fmaf(c[2] * sc.y, f, acc[0][2]);
+                } else {
+                    const float2 f = *reinterpret_cast<const float2*>(xfac + (cbu << sa.token_shift) + ((2 * tig) & ((1 << sa.token_shift) - 1)));
+                    acc[0][0] = fmaf(c[0] * sc.x, f.x, acc[0][0]);
+                    acc[0][1] = fmaf(c[1] * sc.x, f.y, acc[0][1]);
+                    acc[0][2] = fmaf(c[2] * sc.y, f.x, acc[0][2]);
+                    acc[0][3] = fmaf(c[3] * sc.y, f.y, acc[0][3]);
+                }
+            }
+            return;
+        }
 #pragma unroll
         for (int j = 0; j < 8; ++j)  // two accumulators: half the length of the dependent chain
             if constexpr (DT == 0) sk_mma(acc[j & 1], lo[2 * j], hi[2 * j], lo[2 * j + 1], hi[2 * j + 1], xq[2 * j], xq[2 * j + 1]);
@@ -511,7 +615,7 @@ __device__ __forceinline__ void stream_body(const StreamArgs& sa, int* __restric
         if (!unit_ok(code, param, cbu)) return;
         uint32_t lo[16], hi[16];
         decode(code, param, lo, hi);
-        multiply(lo, hi, cbu);
+        multiply(lo, hi, param, cbu);
     };
 
     // ---- main loop over this warp's chunks --------------------------------------------------------------------
@@ -572,9 +676,9 @@ __device__ __forceinline__ void stream_body(const StreamArgs& sa, int* __restric
     stamp(6);
 }
 
-template <int BITS, int KIND, int TOK, bool XSMEM, int W, int OCC = 1, int SK_Q = SK_QMAX, int DT = 0>
-__global__ void __launch_bounds__(W * 32, OCC) stream_kernel(const StreamArgs sa, int* __restrict__ err) {
-    stream_body<BITS, KIND, TOK, XSMEM, W, OCC, SK_Q, DT>(sa, err);
+template <int BITS, int KIND, int TOK, bool XSMEM, int W, int OCC, int SK_Q, int DT, bool UNSC>
+__global__ void __launch_bounds__(W * 32, OCC) stream_kernel(const __grid_constant__ StreamArgs sa, int* __restrict__ err) {
+    stream_body<BITS, KIND, TOK, XSMEM, W, OCC, SK_Q, DT, UNSC>(sa, err);
 }
 #endif  // __CUDACC__
 
@@ -609,6 +713,8 @@ inline StreamArgs stream_args(const StreamPlan& p, const void* packed, const voi
     sa.trace = g_sk_trace;
     if (g_sk_trace) g_sk_trace += 148 * 2 * 8;
 #endif
+    sa.bias = potl::POT_UNIT_BIAS;
+    for (int i = 0; i < potl::POT_UNIT_SHIFTS; ++i) sa.p2[i] = 1u << i;
     sa.fits32 = ((uint64_t)p.units + 1) * ((uint64_t)sa.gw_total + 1) < (uint64_t(1) << 32) ? 1 : 0;
     return sa;
 }
@@ -617,22 +723,26 @@ inline StreamArgs stream_args(const StreamPlan& p, const void* packed, const voi
 template <int BITS, int KIND, int TOK, int W, int OCC = 1, int DT = 0>
 pot_status_t launch_stream(const void* packed, const void* scales, const void* zeros, int64_t N, int64_t K, int group,
                            const void* X, int M, void* Y, void* workspace, int* err, cudaStream_t s) {
-    const StreamPlan p = plan_stream(N, K, M, BITS, group, KIND, TOK, W, OCC);
+    const StreamPlan p = plan_stream(N, K, M, BITS, group, KIND, TOK, W, OCC, DT);
     if (!p.ok) return POT_ERR_SHAPE;
     const StreamArgs sa = stream_args(p, packed, scales, zeros, N, K, group, X, M, Y, workspace);
     auto run = [&](auto kernel) -> pot_status_t {
         if (!allow_max_dynamic_smem(kernel)) return POT_ERR_CUDA;
         return launch_pdl(kernel, dim3((unsigned)p.grid), dim3(W * 32), p.smem_bytes, s, sa, err);
     };
-    if (p.q == 2) {
-        if (p.x_in_smem) return run(stream_kernel<BITS, KIND, TOK, true, W, OCC, 2, DT>);
-        return run(stream_kernel<BITS, KIND, TOK, false, W, OCC, 2, DT>);
-    }
-    if constexpr (OCC == 1 && TOK == 1) {
-        if (p.q == 8) return run(stream_kernel<BITS, KIND, TOK, true, W, OCC, 8, DT>);  // only chosen with x in shared memory
-    }
-    if (p.x_in_smem) return run(stream_kernel<BITS, KIND, TOK, true, W, OCC, SK_QMAX, DT>);
-    return run(stream_kernel<BITS, KIND, TOK, false, W, OCC, SK_QMAX, DT>);
+    constexpr bool POT = KIND == SK_POT;
+    auto pick = [&](auto q) -> pot_status_t {  // q units per slot
+        constexpr int Q = decltype(q)::value;
+        if constexpr (POT)
+            if (p.unscaled) return run(stream_kernel<BITS, KIND, TOK, true, W, OCC, Q, DT, true>);
+        if constexpr (!(POT && TOK == 1))
+            if (p.x_in_smem) return run(stream_kernel<BITS, KIND, TOK, true, W, OCC, Q, DT, false>);
+        return run(stream_kernel<BITS, KIND, TOK, false, W, OCC, Q, DT, false>);
+    };
+    if (p.q == 2) return pick(std::integral_constant<int, 2>());
+    if constexpr (OCC == 1 && TOK == 1)
+        if (p.q == 8) return pick(std::integral_constant<int, 8>());
+    return pick(std::integral_constant<int, SK_QMAX>());
 }
 #endif
 

@@ -63,3 +63,40 @@ def test_bf16_gemm_matches_oracle(B, oracle, bits, M):
             Yg = B.pot_gemm(P, S, K, bits, G, bf16_dev(Xb), layout)
             ok, worst, tight = gate(bits_of(Yg), Y, A, bf16=True)
             assert ok and tight < 4.0, (layout, N, K, M, worst, tight)
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("G", [64, 128])
+@pytest.mark.parametrize("M", [1, 3, 8])
+def test_bf16_activations_over_the_whole_exponent_range(B, oracle, bits, G, M):
+    """The streaming kernels hold BF16 activations as FP16 numbers relative to the largest of 128 columns: units far apart in size,
+    elements far below their unit's largest, all zeros, the smallest and the largest magnitudes -- and infinities and NaN, which
+    come out as the sum of the products has them."""
+    N, K = 64, 1152
+    c = PotCase(N, K, bits, G, dist="normal", seed=(7, 800 + bits))
+    rng = np.random.default_rng(10 * bits + M)
+    X = f16_bits_to_bf16_bits(synth.activations(synth.rng_for(7, 900 + M), M, K)).copy()
+    X[:, 0:128] = rng.integers(1, 0x0200, (M, 128))                               # subnormal and the smallest normal numbers
+    X[:, 128:256] = 0
+    X[:, 256:384] = (rng.integers(60, 190, (M, 128)) << 7) | rng.integers(0, 0x80, (M, 128))   # 2^-67 .. 2^62 in one unit
+    X[:, 512] = 0x5F80                                                            # 2^64
+    X ^= (rng.integers(0, 2, X.shape) << 15).astype(X.dtype)
+    Y, A = oracle.matmul(c.packed, c.S, K, bits, G, X, dtype=oracle.BF16)
+    got = bits_of(B.pot_gemm(c.tiled(), c.tiled_S(), K, bits, G, bf16_dev(X), B.TILED)).reshape(M, N)
+    ok, worst, tight = gate(got, Y, A, bf16=True)
+    assert ok and tight < 4.0, (worst, tight)
+    Xt = np.zeros((M, K), dtype=np.uint16)                                        # tiny numbers alone: nothing may be flushed early
+    Xt[:, 128:256] = rng.integers(0x0A00, 0x0D00, (M, 128))                       # 2^-107 .. 2^-101
+    Y, A = oracle.matmul(c.packed, c.S, K, bits, G, Xt, dtype=oracle.BF16)
+    got = bits_of(B.pot_gemm(c.tiled(), c.tiled_S(), K, bits, G, bf16_dev(Xt), B.TILED)).reshape(M, N)
+    val = (got.astype(np.uint32) << 16).view(np.float32).astype(np.float64)
+    assert np.all(np.abs(val - Y) <= 1e-3 * A + 2.0 ** -8 * np.abs(Y) + 2.0 ** -130)
+    for bad in (0x7F80, 0xFF80, 0x7FC0):
+        Xb = X.copy()
+        Xb[M - 1, 700] = bad
+        w = oracle.dequant(c.packed, c.S, K, bits, G, oracle.BF16)[0][:, 700]
+        got = bits_of(B.pot_gemm(c.tiled(), c.tiled_S(), K, bits, G, bf16_dev(Xb), B.TILED)).reshape(M, N)[M - 1]
+        if bad == 0x7FC0:
+            assert np.all((got & 0x7FFF) > 0x7F80)
+        else:
+            assert np.array_equal(got, np.where((w ^ bad) & 0x8000, 0xFF80, 0x7F80).astype(np.uint16))
