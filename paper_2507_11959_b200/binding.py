@@ -91,16 +91,18 @@ def _check(status: int, what: str) -> None:
 
 
 def _ptr(t):
-    if t is None:
-        return None
-    if isinstance(t, int):
-        return ctypes.c_void_p(t)
-    return ctypes.c_void_p(t.data_ptr())
+    """Address for a void* argument (None, an address, or a tensor)."""
+    return t if t is None or isinstance(t, int) else t.data_ptr()
 
 
 def _stream(stream=None):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    """Raw handle of the given stream, or of the current stream of the current device (asked for without building a Stream
+    object, which costs 3 us: as much as a small launch)."""
+    if stream is not None:
+        return stream.cuda_stream
+    if torch.cuda.is_initialized():
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def pot_status_string(status: int) -> str:
@@ -202,9 +204,8 @@ def pot_gemv(packed, scales, K: int, bits: int, group: int, x: torch.Tensor, lay
     if y is None:
         y = torch.empty(N, dtype=x.dtype, device=x.device)
     assert y.dtype == x.dtype
-    need = pot_gemv_workspace_bytes(N, K, bits, group) if layout == TILED else 0
-    if need and workspace is None:
-        workspace = new_workspace(need, x.device)
+    if workspace is None and layout == TILED:
+        workspace = new_workspace(pot_gemv_workspace_bytes(N, K, bits, group), x.device)
     fn = lib().pot_gemv if x.dtype == torch.float16 else lib().pot_gemv_bf16
     _check(fn(_ptr(packed), _ptr(scales), N, K, bits, group, layout, _ptr(x), _ptr(y), _ptr(workspace),
               0 if workspace is None else workspace.numel(), _stream(stream)), "pot_gemv")
@@ -228,9 +229,8 @@ def pot_gemm(packed, scales, K: int, bits: int, group: int, X: torch.Tensor, lay
     if Y is None:
         Y = torch.empty((M, N), dtype=X.dtype, device=X.device)
     assert Y.dtype == X.dtype
-    need = pot_gemm_workspace_bytes(M, N, K, bits, group) if layout == TILED else 0
-    if need and workspace is None:
-        workspace = new_workspace(need, X.device)
+    if workspace is None and layout == TILED:
+        workspace = new_workspace(pot_gemm_workspace_bytes(M, N, K, bits, group), X.device)
     fn = lib().pot_gemm if X.dtype == torch.float16 else lib().pot_gemm_bf16
     _check(fn(_ptr(packed), _ptr(scales), N, K, bits, group, layout, _ptr(X), M, _ptr(Y), _ptr(workspace),
               0 if workspace is None else workspace.numel(), _stream(stream)), "pot_gemm")
@@ -262,9 +262,8 @@ def uint_gemv(packed, scales, zeros, K: int, bits: int, group: int, x: torch.Ten
     N = packed.shape[0]
     if y is None:
         y = torch.empty(N, dtype=torch.float16, device=x.device)
-    need = pot_gemv_workspace_bytes(N, K, bits, group) if layout == TILED else 0
-    if need and workspace is None:
-        workspace = new_workspace(need, x.device)
+    if workspace is None and layout == TILED:
+        workspace = new_workspace(pot_gemv_workspace_bytes(N, K, bits, group), x.device)
     _check(lib().uint_gemv(_ptr(packed), _ptr(scales), _ptr(zeros), N, K, bits, group, layout, _ptr(x), _ptr(y),
                            _ptr(workspace), 0 if workspace is None else workspace.numel(), _stream(stream)), "uint_gemv")
     return y

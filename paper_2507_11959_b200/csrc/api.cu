@@ -32,6 +32,29 @@ int error_fetch(int which) {
 }
 }  // namespace pot
 
+namespace pot {
+bool allow_max_dynamic_smem(const void* kernel) {
+    // open addressing by the kernel's address; bit d of a slot: set on device d.  More kernels or devices than fit: set every time.
+    constexpr int kSlots = 512, kProbes = 16;
+    static std::atomic<const void*> keys[kSlots];
+    static std::atomic<uint64_t> done[kSlots];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    const size_t h = (reinterpret_cast<uintptr_t>(kernel) >> 4) * 0x9E3779B97F4A7C15ull >> 40;
+    for (int p = 0; p < kProbes && dev < 64; ++p) {
+        const size_t i = (h + p) % kSlots;
+        const void* k = keys[i].load(std::memory_order_acquire);
+        if (!k && keys[i].compare_exchange_strong(k, kernel)) k = kernel;
+        if (k != kernel) continue;
+        if (done[i].load(std::memory_order_acquire) >> dev & 1u) return true;
+        if (!set_max_dynamic_smem(kernel)) return false;
+        done[i].fetch_or(uint64_t(1) << dev, std::memory_order_release);
+        return true;
+    }
+    return set_max_dynamic_smem(kernel);
+}
+}  // namespace pot
+
 extern "C" int pot_debug_gemv_error(void) { return error_fetch(ERR_GEMV); }
 extern "C" int pot_debug_gemm_error(void) { return error_fetch(ERR_GEMM); }
 extern "C" int pot_debug_prefill_error(void) { return error_fetch(ERR_PREFILL); }

@@ -34,15 +34,11 @@ inline pot_status_t launched(int n = 1) {
 constexpr int kSmCount = 148;  // B200: 2 dies x 74 SMs
 
 #ifdef __CUDACC__
-// Launch with programmatic stream serialization: the kernel may start while the previous kernel
-// in the stream is still draining; it must execute griddepcontrol.wait before touching anything
-// the previous kernel wrote (and before writing anything the previous kernel may still read).
 // Largest dynamic shared memory a CTA may ask for on sm_100a.  Kernels opt in to this maximum rather than to the
 // size of the current launch: a launch recorded in a CUDA graph must still fit the function's attribute when the
 // graph is replayed, whatever other shapes were launched in between.
 constexpr int kMaxDynamicSmem = 227 * 1024;
-template <typename K>
-inline bool allow_max_dynamic_smem(K kernel) {
+inline bool set_max_dynamic_smem(const void* kernel) {
     cudaFuncAttributes fa;
     if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) return false;
     const int room = kMaxDynamicSmem - (int)fa.sharedSizeBytes;  // static shared memory counts against the same limit
@@ -50,22 +46,42 @@ inline bool allow_max_dynamic_smem(K kernel) {
         return false;
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, room) == cudaSuccess;
 }
+// The attributes belong to (kernel, device) and outlast the call, so they are set on a kernel's first launch per device only
+// (the three runtime calls cost about as much as the launch).  False: the runtime refused.
+bool allow_max_dynamic_smem(const void* kernel);
 
+// Launch with programmatic stream serialization: the kernel may start while the previous kernel
+// in the stream is still draining; it must execute griddepcontrol.wait before touching anything
+// the previous kernel wrote (and before writing anything the previous kernel may still read).
+// cluster > 1: CTAs per thread-block cluster.  big_smem: the kernel needs allow_max_dynamic_smem.
 template <typename... Args>
-inline pot_status_t launch_pdl(void (*kernel)(Args...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {
+inline pot_status_t launch_pdl_cluster(void (*kernel)(Args...), dim3 grid, dim3 block, size_t smem, int cluster, bool big_smem, cudaStream_t s, Args... args) {
+    if (big_smem && !allow_max_dynamic_smem((const void*)kernel)) return POT_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
+    if (e == cudaErrorInvalidValue && big_smem) {  // the attributes are gone (the device was reset, another context is current): once more
+        cudaGetLastError();
+        if (!set_max_dynamic_smem((const void*)kernel)) return POT_ERR_CUDA;
+        e = cudaLaunchKernelEx(&cfg, kernel, args...);
+    }
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return e == cudaSuccess ? POT_OK : POT_ERR_CUDA;
+}
+template <typename... Args>
+inline pot_status_t launch_pdl(void (*kernel)(Args...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {
+    return launch_pdl_cluster(kernel, grid, block, smem, 1, false, s, args...);
 }
 #endif
 

@@ -849,8 +849,7 @@ pot_status_t gemm_prefill_launch(const void* packed, const void* scales, int64_t
     auto run = [&](auto kernel, int stages, int mt, int at = 0, int ng = 4, int wide = 0) -> pot_status_t {
         const size_t smem = pf_smem_bytes(stages, mt, at, wide);
         const dim3 block((unsigned)pf_threads(ng, 2));
-        if (!allow_max_dynamic_smem(kernel)) return POT_ERR_CUDA;
-        return launch_pdl(kernel, grid, block, smem, s, xmap, (const uint4*)packed, (const uint16_t*)scales, N, K, group, M,
+        return launch_pdl_cluster(kernel, grid, block, smem, 1, true, s, xmap, (const uint4*)packed, (const uint16_t*)scales, N, K, group, M,
                           (uint16_t*)Y, partial, counters, pl.tiles_m, pl.n_full, pl.splits, prefill_error_ptr());
     };
     // two issuers, one CTA per SM; for batches of up to 64 tokens: one token tile, three producer groups, six stages of a whole
@@ -944,25 +943,9 @@ pot_status_t gemm_canonical_launch(const void* packed, const void* scales, int64
     CUtensorMap xmap;
     if (!encode_x_map(&xmap, X, M, K)) return POT_ERR_CUDA;
     auto run = [&](auto kernel, int stages, int mt, int wide) -> pot_status_t {
-        if (!allow_max_dynamic_smem(kernel)) return POT_ERR_CUDA;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)(tiles * splits));
-        cfg.blockDim = dim3((unsigned)pf_threads(3, 2));
-        cfg.dynamicSmemBytes = pf_smem_bytes(stages, mt, 1, wide);
-        cfg.stream = s;
-        cudaLaunchAttribute attr[2];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        attr[1].id = cudaLaunchAttributeClusterDimension;
-        attr[1].val.clusterDim.x = (unsigned)splits;
-        attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = splits > 1 ? 2 : 1;
-        const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, xmap, (const uint4*)packed, (const uint16_t*)scales, N, K, group, M,
-                                                 (uint16_t*)Y, (float*)nullptr, (unsigned*)nullptr, (int)tiles_m,
-                                                 (int)(splits > 1 ? 0 : tiles), splits, prefill_error_ptr());
-        g_launches.fetch_add(1, std::memory_order_relaxed);
-        return e == cudaSuccess ? POT_OK : POT_ERR_CUDA;
+        return launch_pdl_cluster(kernel, dim3((unsigned)(tiles * splits)), dim3((unsigned)pf_threads(3, 2)), pf_smem_bytes(stages, mt, 1, wide),
+                                  splits, true, s, xmap, (const uint4*)packed, (const uint16_t*)scales, N, K, group, M, (uint16_t*)Y,
+                                  (float*)nullptr, (unsigned*)nullptr, (int)tiles_m, (int)(splits > 1 ? 0 : tiles), splits, prefill_error_ptr());
     };
     auto pick = [&](auto b, auto d) -> pot_status_t {
         constexpr int B = decltype(b)::value, D = decltype(d)::value;

@@ -276,24 +276,8 @@ static pot_status_t launch_gemv_canonical(const void* packed, const void* scales
         const CanonPlan p = plan_canonical(N, K);
         auto run = [&](auto kernel) -> pot_status_t {
             const size_t smem = (size_t)(K / 128 + 1) * GC_X_STRIDE;
-            if (smem > 46 * 1024 && !allow_max_dynamic_smem(kernel)) return POT_ERR_CUDA;
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(p.grid);
-            cfg.blockDim = dim3(GC_WARPS * 32);
-            cfg.dynamicSmemBytes = smem;
-            cfg.stream = s;
-            cudaLaunchAttribute attr[2];
-            attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-            attr[0].val.programmaticStreamSerializationAllowed = 1;
-            attr[1].id = cudaLaunchAttributeClusterDimension;
-            attr[1].val.clusterDim.x = (unsigned)p.cluster;
-            attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
-            cfg.attrs = attr;
-            cfg.numAttrs = p.cluster > 1 ? 2 : 1;
-            const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, (const uint4*)packed, (const uint16_t*)scales, N, (int)(K / 128),
-                                                     128 / group, (const uint4*)x, (uint16_t*)y, p.wk_shift, p.cluster);
-            g_launches.fetch_add(1, std::memory_order_relaxed);
-            return e == cudaSuccess ? POT_OK : POT_ERR_CUDA;
+            return launch_pdl_cluster(kernel, dim3(p.grid), dim3(GC_WARPS * 32), smem, p.cluster, smem > 46 * 1024, s, (const uint4*)packed,
+                                      (const uint16_t*)scales, N, (int)(K / 128), 128 / group, (const uint4*)x, (uint16_t*)y, p.wk_shift, p.cluster);
         };
         if (bits == 2) return run(gemv_canonical_mma_kernel<2, DT>);
         if (bits == 3) return run(gemv_canonical_mma_kernel<3, DT>);

@@ -727,8 +727,7 @@ pot_status_t launch_stream(const void* packed, const void* scales, const void* z
     if (!p.ok) return POT_ERR_SHAPE;
     const StreamArgs sa = stream_args(p, packed, scales, zeros, N, K, group, X, M, Y, workspace);
     auto run = [&](auto kernel) -> pot_status_t {
-        if (!allow_max_dynamic_smem(kernel)) return POT_ERR_CUDA;
-        return launch_pdl(kernel, dim3((unsigned)p.grid), dim3(W * 32), p.smem_bytes, s, sa, err);
+        return launch_pdl_cluster(kernel, dim3((unsigned)p.grid), dim3(W * 32), p.smem_bytes, 1, true, s, sa, err);
     };
     constexpr bool POT = KIND == SK_POT;
     auto pick = [&](auto q) -> pot_status_t {  // q units per slot
