@@ -16,6 +16,8 @@
 //                        the stage back to the producers.  One issuing thread leaves the tensor pipe idle for several
 //                        hundred cycles per stage (barrier test, fence, commit, the pipe's start-up after a gap); two
 //                        threads fill each other's gaps.
+// (The 256-token tile is the general case: with the weight tile in tensor memory, below, a tile has two X tiles of h tokens, h a
+// multiple of 16 up to 192 that is chosen per launch, see prefill_plan.)
 // After the last K block each issuer commits to a common barrier; the producer warps read the accumulators with
 // tcgen05.ld (each warp its own 32-lane quarter), add the two issuers' sums in a fixed order, convert to FP16 and
 // store (a warp writes 32 consecutive features of one token at a time).  The weights are re-decoded once per 256-token
@@ -65,11 +67,14 @@ __host__ __device__ constexpr int pf_x_bytes(int mt) { return mt == 1 ? PF_SMALL
 // pipe set the pace)
 __host__ __device__ constexpr int pf_bks(int mt, int at, int wide = 0) { return (at && (mt == 1 || wide)) ? 2 : 1; }
 __host__ __device__ constexpr int pf_stage_bytes(int mt, int at = 0, int wide = 0) { return pf_x_bytes(mt) * pf_bks(mt, at, wide) + (at ? 0 : PF_ATOM_BYTES); }
+constexpr size_t pf_smem_bytes_h(int stages, int h, int bks) { return 1024 + (size_t)stages * 2 * h * 128 * bks + 256; }  // tiles of 2 h tokens
 constexpr size_t pf_smem_bytes(int stages, int mt, int at = 0, int wide = 0) { return 1024 /*align slack*/ + (size_t)stages * pf_stage_bytes(mt, at, wide) + 256 /*barriers*/; }
-constexpr int PF_AT_ACC_COLS = 256;   // at = 1, 256-token tiles: accumulator columns (token t of the tile = column t), then 32 columns per stage of A
+// at = 1, tiles of up to 384 tokens: two X tiles of h tokens (h a multiple of 16, chosen per launch), accumulator columns 0 .. 2h - 1
+// (token t of the tile = column t), then 32 columns per 64-column stage of A: six stages up to h = 128, four up to h = 192
+constexpr int PF_MAX_H = 192;
 // at = 1, the one-tile kernel (up to 64 tokens): the two issuers' accumulators take 64 columns each, the A ring follows
 constexpr int PF_AT1_ACC_STRIDE = PF_SMALL_TOKENS;
-__host__ __device__ constexpr int pf_at_ring_col0(int mt) { return mt == 2 ? PF_AT_ACC_COLS : 2 * PF_AT1_ACC_STRIDE; }
+constexpr int PF_AT1_RING_COL0 = 2 * PF_AT1_ACC_STRIDE;
 
 // UMMA instruction descriptor: FP16 x FP16 -> FP32, both operands K-major, M = 128 (the weight rows of the tile are the
 // A operand), N = n token rows of the X tile (the B operand), 16 <= n <= 256, n % 16 == 0
@@ -169,6 +174,12 @@ __device__ __forceinline__ void pf_mma_ta(uint32_t d_tmem, uint32_t a_tmem, uint
         "r"(a_tmem), "r"(blo), "r"(hi), "r"(idesc), "r"(accumulate)
         : "memory");
 }
+__device__ __forceinline__ void pf_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr)
+                 : "memory");
+}
 __device__ __forceinline__ void pf_st32(uint32_t taddr, const uint32_t (&r)[32]) {
     asm volatile(
         "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,"
@@ -181,23 +192,24 @@ __device__ __forceinline__ void pf_st32(uint32_t taddr, const uint32_t (&r)[32])
 }
 
 // Issuer J of the variant that keeps the decoded weight tile in tensor memory: it takes EVERY stage, multiplies the tile
-// (A, from tensor memory: 128 weight rows x 64) by token tile J of the stage (B, 128 tokens, from shared memory) and
-// accumulates into columns 128 J .. 128 J + 127 -- the two issuers share the weight tile and never the accumulator, so
+// (A, from tensor memory: 128 weight rows x 64) by token tile J of the stage (B, h tokens of which the first n are
+// multiplied, from shared memory) and accumulates into columns h J .. h J + n - 1 -- the two issuers share the weight tile and never the accumulator, so
 // the order of the additions is fixed.  A stage is free again when every active issuer's MMAs on it have completed.
 template <int J, int PF_STAGES, int DT, int BKS = 1>
-__device__ __forceinline__ void pf_issue_at(uint32_t smem0, uint32_t bar0, uint32_t tmem_base, int nkb, int* err) {
+__device__ __forceinline__ void pf_issue_at(uint32_t smem0, uint32_t bar0, uint32_t tmem_base, int nkb, uint32_t h, uint32_t n, int* err) {
     auto full = [&](int s) { return bar0 + 8u * s; };
     auto empty = [&](int s) { return bar0 + 8u * (PF_STAGES + s); };
     const uint32_t accum = bar0 + 8u * (2 * PF_STAGES);
-    uint32_t blo[PF_STAGES];
+    uint32_t blo[PF_STAGES][BKS];   // [stage][64-column sub-block]
 #pragma unroll
     for (int s = 0; s < PF_STAGES; ++s)
-        blo[s] = (uint32_t)pf_smem_desc(smem0 + (uint32_t)s * pf_stage_bytes(PF_MT, 1, BKS == 2) + (uint32_t)J * PF_ATOM_BYTES);
+#pragma unroll
+        for (int b = 0; b < BKS; ++b) blo[s][b] = (uint32_t)pf_smem_desc(smem0 + (uint32_t)((s * BKS + b) * PF_MT + J) * (h * 128u));
     constexpr uint32_t desc_hi = (uint32_t)(PF_DESC_CONST >> 32);
     constexpr uint32_t SLOT = 32u * BKS;   // tensor-memory columns of a stage's weights
-    const uint32_t d0 = tmem_base + (uint32_t)(J * PF_BM);
-    const uint32_t a0 = tmem_base + (uint32_t)PF_AT_ACC_COLS;
-    const uint32_t idesc = pf_idesc(PF_BM, DT);
+    const uint32_t d0 = tmem_base + (uint32_t)J * h;
+    const uint32_t a0 = tmem_base + 2 * h;
+    const uint32_t idesc = pf_idesc(n, DT);
     uint32_t ready = mbar_test(full(0), 0);
     uint32_t ph = 0;
     for (int kb0 = 0; kb0 < nkb; kb0 += PF_STAGES, ph ^= 1u) {
@@ -212,9 +224,9 @@ __device__ __forceinline__ void pf_issue_at(uint32_t smem0, uint32_t bar0, uint3
             if (kb + 1 < nkb) ready = mbar_test(full((s + 1) % PF_STAGES), s + 1 >= PF_STAGES ? ph ^ 1u : ph);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-            for (int ks = 0; ks < BKS * (PF_BK / 16); ++ks)   // sub-block ks / 4: its X tiles follow the first sub-block's
+            for (int ks = 0; ks < BKS * (PF_BK / 16); ++ks)   // sub-block ks / 4
                 pf_mma_ta(d0, a0 + SLOT * (uint32_t)s + (uint32_t)(8 * ks),
-                          blo[s] + (uint32_t)(((ks >> 2) * PF_MT * PF_ATOM_BYTES + (ks & 3) * 32) >> 4), desc_hi, idesc,
+                          blo[s][ks >> 2] + (uint32_t)(((ks & 3) * 32) >> 4), desc_hi, idesc,
                           (s != 0 || ks != 0) ? 1u : (uint32_t)(kb0 != 0));
             pf_commit(empty(s));
         }
@@ -236,7 +248,7 @@ __device__ __forceinline__ void pf_issue_at1(uint32_t smem0, uint32_t bar0, uint
     constexpr int BKS = pf_bks(1, 1);                       // 64-column sub-blocks per stage
     constexpr uint32_t SLOT = 32u * BKS;                    // tensor-memory columns of a stage's weights
     const uint32_t d0 = tmem_base + (uint32_t)(J * PF_AT1_ACC_STRIDE);
-    const uint32_t a0 = tmem_base + (uint32_t)pf_at_ring_col0(1);
+    const uint32_t a0 = tmem_base + (uint32_t)PF_AT1_RING_COL0;
     const uint32_t idesc = pf_idesc(n_tok, DT);
     uint32_t ready = mbar_test(full(J), 0);
     uint32_t ph = 0;
@@ -322,14 +334,15 @@ __device__ __forceinline__ void pf_issue(uint32_t smem0, uint32_t bar0, uint32_t
 // CANON = 1: canonical codes and row-major scales (the 128-column stages only): a producer thread reads its row's 16 BITS
 // contiguous bytes per column block and decodes them with byte look-ups (potl::CanonLut).  There is no workspace on this
 // route: the items of a tile that is cut along K are the CTAs of a thread-block cluster, which add their partial sums through
-// distributed shared memory.  200 tokens x 4099 x 11008, 3 bits: 672 us on the mma.sync kernel that this replaced, 29.6 us
-// (clusters of 4, 132 CTAs; about half of it is latency per 128-column stage with three stages in flight).
+// distributed shared memory.  200 tokens x 4099 x 11008, 3 bits: 672 us on the mma.sync kernel that this replaced, 27.3 us
+// (clusters of 4, 132 CTAs; about half of it is latency per 128-column stage with three stages in flight; 29.6 us with the 32-token
+// chunks of a tile dealt to the CTAs instead of 8-token groups, and X tiles of 128 tokens).
 template <int BITS, int PF_STAGES, int NG, int NI, int MT, int DT = 0, int AT = 0, int NGP = NG, int WIDE = 0, int CANON = 0>  // DT = 1: BF16 activations, weights and output
 __global__ void __launch_bounds__(pf_threads(NG, NI), 1)
 pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* __restrict__ packed,
                         const uint16_t* __restrict__ scales, int64_t N, int64_t K, int G, int64_t M,
                         uint16_t* __restrict__ Y, float* __restrict__ partial, unsigned* __restrict__ counters,
-                        int tiles_m, int n_full, int tail_splits, int* __restrict__ err) {
+                        int tiles_m, int n_full, int tail_splits, int tok_h, int* __restrict__ err) {
     extern __shared__ unsigned char smem_raw[];
     // 1024-byte alignment: the swizzle atoms and the matrix descriptors assume it
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -337,7 +350,10 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
     static_assert(!CANON || (AT && pf_bks(MT, AT, WIDE) == 2), "canonical codes: 128-column stages, the weight tile in tensor memory");
     constexpr bool AT2 = AT && MT == 2;   // both issuers on every stage, one token tile each (else: alternate stages)
     constexpr int BKS = pf_bks(MT, AT, WIDE);   // 64-column sub-blocks per stage
-    constexpr int STAGE_BYTES = pf_stage_bytes(MT, AT, WIDE);
+    const int h = AT2 ? tok_h : PF_BM;                      // tokens per X tile
+    const int x_tile_bytes = AT2 ? h * 128 : PF_ATOM_BYTES;
+    const int STAGE_BYTES = AT2 ? MT * BKS * x_tile_bytes : pf_stage_bytes(MT, AT, WIDE);
+    const int ring_col0 = AT2 ? 2 * h : PF_AT1_RING_COL0;   // AT: first tensor-memory column of the weight ring
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)PF_STAGES * STAGE_BYTES);
     // bars: full[S] (TMA bytes + one arrival per producer warp), empty[S], accum, then the tensor-memory base address
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * PF_STAGES + 1);
@@ -349,8 +365,7 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
     constexpr int PROD_WARP0 = pf_prod_warp0(NI);
     constexpr int NPT = NG * 128;                       // producer / epilogue threads
     constexpr int TMEM_COLS = AT ? 512 : NI * PF_BN * MT;  // MT accumulators per issuer; AT: 256 accumulator columns + the A ring
-    static_assert((NGP % 2 == 0 || BKS == 2) && NGP <= NG && (AT2 || PF_STAGES % NI == 0) && PF_STAGES % NGP == 0,
-                  "a group always decodes the same half of a column block; a stage buffer belongs to one issuer and one group");
+    static_assert(NGP <= NG && (AT2 || PF_STAGES % NI == 0) && PF_STAGES % NGP == 0, "a stage buffer belongs to one issuer and one group");
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // Work items in launch order: the first n_full are whole output tiles; each of the remaining ("tail") tiles is cut
     // into tail_splits items along K, so that the last, partly filled wave of CTAs is short.  Tiles are numbered
@@ -367,15 +382,15 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
     {
         int tile, zsplit, splits;
         item(tile, zsplit, splits);
-        m0 = (int64_t)(tile % tiles_m) * (PF_BM * MT);
+        m0 = (int64_t)(tile % tiles_m) * (h * MT);
         n0 = (int64_t)(tile / tiles_m) * PF_BN;
         // split item z of a tile owns column blocks [cb0, cb1), two stages each
         cb0 = (int64_t)zsplit * (K / 128) / splits;
         cb1 = ((int64_t)zsplit + 1) * (K / 128) / splits;
     }
     const int64_t ncb = K / 128;
-    // a tile with at most 128 real tokens (decode batches, the ragged last token tile) uses one accumulator only
-    const int n_mt = M - m0 > PF_BM ? MT : 1;
+    // a tile with at most h real tokens (decode batches, the ragged last token tile) uses one accumulator only
+    const int n_mt = M - m0 > h ? MT : 1;
     // token rows the MMA reads from the X stage: whole tiles, or (one-tile kernel) the batch rounded up to the MMA's N step
     const uint32_t n_tok = MT == 1 ? (uint32_t)((M + 15) & ~(int64_t)15) : (uint32_t)(n_mt * PF_BM);  // MT == 1: M <= 64
     const int nkb = (int)((2 / BKS) * (cb1 - cb0));   // stages of this item
@@ -383,10 +398,9 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
 
     // ---- dequant producers, part 1 (before the set-up below, so that the first loads of codes and scales -- constants,
     // they do not depend on the previous kernel -- are in flight while the barriers and the tensor memory are set up and
-    // the kernel waits for its predecessor): thread = one weight row; group g owns the stages with kb % NGP == g, hence
-    // (NGP is even) always the same half of the records.
+    // the kernel waits for its predecessor): thread = one weight row; group g owns the stages with kb % NGP == g.
     const int pt = threadIdx.x - 32 * PROD_WARP0;          // 0 .. NPT-1 for the producer warps
-    const int grp = pt >> 7, row = pt & 127, half = grp & 1;
+    const int grp = pt >> 7, row = pt & 127;
     const int64_t n = n0 + row;
     const bool row_ok = n < N;
     const int64_t rb = n >> 4;
@@ -422,6 +436,7 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
                 sc2[buf][0] = pf_ldg_u16(scales + so + potl::scale_tile_index(r, 0));
                 sc2[buf][BKS - 1] = pf_ldg_u16(scales + so + potl::scale_tile_index(r, spg == 2 ? 1 : 0));
             } else {
+                const int half = NGP % 2 == 0 ? grp & 1 : kb & 1;   // half of the column block
                 const uint2* unit = reinterpret_cast<const uint2*>(packed + (rb * ncb + cbx) * (16 * BITS));
 #pragma unroll
                 for (int t = 0; t < BITS; ++t) {
@@ -473,22 +488,22 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
                 ready = (kn < nkb && kn >= PF_STAGES) ? mbar_test(empty(kn % PF_STAGES), (uint32_t)((kn / PF_STAGES - 1) & 1)) : 0u;
                 // MT == 1 (M <= 64): the box holds exactly the M token rows -- the TMA unit spends time on every row of a
                 // box, in range or not; the rows of the tile that nothing writes belong to tokens that are never stored
-                mbar_expect_tx(full(s), MT == 1 ? (uint32_t)M * 128u * BKS : (uint32_t)n_mt * PF_ATOM_BYTES * BKS);
+                mbar_expect_tx(full(s), MT == 1 ? (uint32_t)M * 128u * BKS : (uint32_t)(n_mt * x_tile_bytes * BKS));
                 const uint32_t a = smem_u32(smem + (size_t)s * STAGE_BYTES);
                 if constexpr (BKS == 2 && MT == 1) {  // (one-tile kernel) the two 64-column tiles of the stage's column block
                     pf_tma_load_2d(a, &xmap, (kb0 + kb) * 2 * PF_BK, (int)m0, full(s));
                     pf_tma_load_2d(a + pf_x_bytes(1), &xmap, (kb0 + kb) * 2 * PF_BK + PF_BK, (int)m0, full(s));
-                } else if constexpr (BKS == 2) {      // [sub-block][token tile] tiles of 16 KB
+                } else if constexpr (BKS == 2) {      // [sub-block][token tile]
 #pragma unroll
                     for (int sub = 0; sub < 2; ++sub)
 #pragma unroll
                         for (int mt = 0; mt < MT; ++mt)
                             if (mt < n_mt)
-                                pf_tma_load_2d(a + (sub * MT + mt) * PF_ATOM_BYTES, &xmap, ((kb0 + kb) * 2 + sub) * PF_BK, (int)m0 + mt * PF_BM, full(s));
+                                pf_tma_load_2d(a + (sub * MT + mt) * x_tile_bytes, &xmap, ((kb0 + kb) * 2 + sub) * PF_BK, (int)m0 + mt * h, full(s));
                 } else {
 #pragma unroll
                     for (int mt = 0; mt < MT; ++mt)
-                        if (mt < n_mt) pf_tma_load_2d(a + mt * PF_ATOM_BYTES, &xmap, (kb0 + kb) * PF_BK, (int)m0 + mt * PF_BM, full(s));
+                        if (mt < n_mt) pf_tma_load_2d(a + mt * x_tile_bytes, &xmap, (kb0 + kb) * PF_BK, (int)m0 + mt * h, full(s));
                 }
             }
         }
@@ -496,8 +511,10 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
         // ---------------- MMA issuers (one thread each) ------------------------------------------------
         if (lane == 0) {
             if constexpr (AT2) {
-                if (warp == 1) pf_issue_at<0, PF_STAGES, DT, BKS>(smem_u32(smem), bar0, tmem_base, nkb, err);
-                else if (n_mt == 2) pf_issue_at<1, PF_STAGES, DT, BKS>(smem_u32(smem), bar0, tmem_base, nkb, err);
+                // (the tokens of an X tile, rounded up to the MMA's N step, from uniform values: the descriptor stays in a uniform register)
+                auto n_of = [&](int64_t left) { return (uint32_t)(left < h ? (left + 15) & ~(int64_t)15 : h); };
+                if (warp == 1) pf_issue_at<0, PF_STAGES, DT, BKS>(smem_u32(smem), bar0, tmem_base, nkb, (uint32_t)h, n_of(M - m0), err);
+                else if (n_mt == 2) pf_issue_at<1, PF_STAGES, DT, BKS>(smem_u32(smem), bar0, tmem_base, nkb, (uint32_t)h, n_of(M - m0 - h), err);
             } else if constexpr (AT) {
                 if (warp == 1) pf_issue_at1<0, NI, PF_STAGES, DT>(smem_u32(smem), bar0, tmem_base, nkb, n_tok, err);
                 else pf_issue_at1<NI - 1, NI, PF_STAGES, DT>(smem_u32(smem), bar0, tmem_base, nkb, n_tok, err);
@@ -519,32 +536,33 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
                 const int kb = NGP * i + grp;
                 if (i + PF_DEPTH - 1 < nmine) load(kb + NGP * (PF_DEPTH - 1), (buf + PF_DEPTH - 1) % PF_DEPTH);
                 const int s = kb % PF_STAGES;
-                if (kb >= PF_STAGES) {
-                    // Every lane polls (the warp is about to WRITE the stage).  One polling lane + __syncwarp() left the
-                    // warp running as two groups (lane 0 / the rest) through the whole decode in some builds: every
-                    // load and store issued twice.
-                    if (!mbar_wait(empty(s), (uint32_t)((kb / PF_STAGES - 1) & 1))) {
-                        if (err && lane == 0) atomicCAS(err, 0, 0x30 | (kb << 8));
+                auto wait_stage = [&]() {
+                    if (kb >= PF_STAGES) {
+                        // Every lane polls (the warp is about to WRITE the stage).  One polling lane + __syncwarp() left the
+                        // warp running as two groups (lane 0 / the rest) through the whole decode in some builds: every
+                        // load and store issued twice.
+                        if (!mbar_wait(empty(s), (uint32_t)((kb / PF_STAGES - 1) & 1))) {
+                            if (err && lane == 0) atomicCAS(err, 0, 0x30 | (kb << 8));
+                        }
+                        __syncwarp();
                     }
-                    __syncwarp();
-                }
-                if constexpr (AT && BKS == 2) {
-                    // a whole record: the two 64-column halves in turn, 32 packed pairs = 32 columns of this thread's lane each
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");  // (behind the wait for the stage)
-#pragma unroll
-                    for (int hb = 0; hb < 2; ++hb) {
+                };
+                if constexpr (AT) {
+                    // 64 weights of the row at a time = 32 packed pairs = 32 columns of this thread's tensor-memory lane; the first
+                    // (BKS = 1: only) half is decoded before the wait for the stage, so that a stage that has become free is
+                    // filled at once
+                    auto decode = [&](int hb, uint32_t (&wa)[32]) {
                         uint32_t sh = sc2[buf][hb];
                         if (DT == 1) sh = __bfloat16_as_ushort(__float2bfloat16_rn(__half2float(__ushort_as_half((uint16_t)sh))));
-                        const uint32_t sh2 = sh * 0x10001u;
+                        const uint32_t sh2 = sh * 0x10001u;  // scale pattern in both halves
                         const potl::CanonLut<BITS, DT> lut(sh);
-                        uint32_t wa[32];
 #pragma unroll
                         for (int T2 = 0; T2 < 2; ++T2) {
                             uint32_t w2[16];
                             if (row_ok) {
                                 if constexpr (CANON) potl::canon_decode32<BITS, DT>(rec[buf] + (2 * hb + T2) * BITS, lut, w2);
-                                else if (DT == 0) potl::pot_decode32<BITS, 4>(rec[buf], 2 * hb + T2, sh2, w2);
-                                else potl::pot_decode32_bf16<BITS, 4>(rec[buf], 2 * hb + T2, sh2, w2);
+                                else if (DT == 0) potl::pot_decode32<BITS, 2 * BKS>(rec[buf], 2 * hb + T2, sh2, w2);
+                                else potl::pot_decode32_bf16<BITS, 2 * BKS>(rec[buf], 2 * hb + T2, sh2, w2);
                             } else {
 #pragma unroll
                                 for (int q = 0; q < 16; ++q) w2[q] = 0u;
@@ -552,7 +570,19 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
 #pragma unroll
                             for (int q = 0; q < 16; ++q) wa[16 * T2 + q] = w2[q];
                         }
-                        pf_st32(tmem_base + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(pf_at_ring_col0(MT) + 64 * s + 32 * hb), wa);
+                    };
+                    const uint32_t slot = tmem_base + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(ring_col0 + 32 * BKS * s);
+                    uint32_t wa[32];
+                    decode(0, wa);
+#pragma unroll
+                    for (int q = 0; q < 32; ++q) asm volatile("" : "+r"(wa[q]));  // (here, not behind the wait)
+                    wait_stage();
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");  // (behind the wait for the stage)
+                    pf_st32(slot, wa);
+                    if constexpr (BKS == 2) {
+                        uint32_t wb[32];
+                        decode(1, wb);
+                        pf_st32(slot + 32, wb);
                     }
                     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -560,33 +590,10 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
                     if (lane == 0) mbar_arrive(full(s));
                     continue;
                 }
+                wait_stage();
                 uint32_t s16 = sc2[buf][0];
                 if (DT == 1) s16 = __bfloat16_as_ushort(__float2bfloat16_rn(__half2float(__ushort_as_half((uint16_t)s16))));
                 const uint32_t s2 = s16 * 0x10001u;  // scale pattern in both halves
-                if constexpr (AT) {
-                    // the row's 64 weights of this stage = 32 packed pairs = 32 columns of this thread's tensor-memory lane
-                    uint32_t wa[32];
-#pragma unroll
-                    for (int T2 = 0; T2 < 2; ++T2) {
-                        uint32_t w2[16];
-                        if (row_ok) {
-                            if (DT == 0) potl::pot_decode32<BITS, 2>(rec[buf], T2, s2, w2);
-                            else potl::pot_decode32_bf16<BITS, 2>(rec[buf], T2, s2, w2);
-                        } else {
-#pragma unroll
-                            for (int q = 0; q < 16; ++q) w2[q] = 0u;
-                        }
-#pragma unroll
-                        for (int q = 0; q < 16; ++q) wa[16 * T2 + q] = w2[q];
-                    }
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");  // (behind the wait for the stage)
-                    pf_st32(tmem_base + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(pf_at_ring_col0(MT) + 32 * s), wa);
-                    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(full(s));
-                    continue;
-                }
                 unsigned char* brow = smem + (size_t)s * STAGE_BYTES + pf_x_bytes(MT) + row * 128;
 #pragma unroll
                 for (int T2 = 0; T2 < 2; ++T2) {
@@ -627,12 +634,11 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
         int tile, zsplit, splits;  // recomputed here rather than kept in registers across the main loop
         item(tile, zsplit, splits);
         const int tail_index = tile - n_full;   // index of the tile among the split ones
-        const int64_t rows_alloc = M < PF_BM * MT ? M : PF_BM * MT;  // token rows kept per tile in the workspace
+        const int64_t rows_alloc = M < h * MT ? M : h * MT;  // token rows kept per tile in the workspace
         // 32-column chunks per warp: the NG warps of a lane quarter share the tile's columns (the one-tile kernel holds at
         // most PF_SMALL_TOKENS tokens: two chunks, whatever NG is)
         // (chunks part, part + NG, ... of the tile's 32-column chunks; the one-tile kernel holds at most PF_SMALL_TOKENS tokens)
-        constexpr int NCH = MT == 1 ? PF_SMALL_TOKENS / 32 : MT * PF_BM / 32;
-        constexpr int CH = (NCH + NG - 1) / NG;
+        const int nch = MT == 1 ? PF_SMALL_TOKENS / 32 : MT * h / 32;
         auto sums = [&](int col, uint32_t (&v)[32]) {  // the complete sums of 32 token columns of this item
             pf_ld32(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)col, v);
             if (NI == 2 && !AT2 && nkb > 1) {     // add the second issuer's sums (odd K blocks) to the first's: a fixed order
@@ -654,41 +660,66 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
         };
         if constexpr (CANON) {
             if (splits > 1) {
-                // The items of the tile are the CTAs of this cluster.  Token chunk c belongs to CTA c % splits: every CTA leaves
-                // the other chunks' sums in its own shared memory (the ring is empty: all MMAs have completed), and after a
-                // cluster barrier each CTA adds its chunks in split order and writes them.
-                static_assert(NCH * 32 * PF_BN * 4 <= PF_STAGES * STAGE_BYTES, "the partial sums fit in the ring");
+                // The items of the tile are the CTAs of this cluster.  Group g of 8 token columns belongs to CTA g % splits: every
+                // CTA leaves the other groups' sums in its own shared memory (the ring is empty: all MMAs have completed; it
+                // holds at least 512 bytes per token of the tile), and after a cluster barrier each CTA adds its groups in
+                // split order -- all peers' numbers of a group in flight at once -- and writes them.
                 float* red = reinterpret_cast<float*>(smem) + 32 * q + lane;   // [token column][128 features]
 #pragma unroll 1
-                for (int c = part; c < NCH && m0 + c * 32 < M; c += NG) {
-                    if (c % splits == zsplit) continue;
+                for (int c = part; c < nch && m0 + c * 32 < M; c += NG) {
                     uint32_t v[32];
                     sums(c * 32, v);
 #pragma unroll
-                    for (int i = 0; i < 32; ++i) red[(c * 32 + i) * PF_BN] = __uint_as_float(v[i]);
+                    for (int g = 0; g < 4; ++g) {
+                        if ((4 * c + g) % splits == zsplit) continue;
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) red[(c * 32 + 8 * g + i) * PF_BN] = __uint_as_float(v[8 * g + i]);
+                    }
                 }
                 pf_cluster_sync();
 #pragma unroll 1
-                for (int c = zsplit + splits * part; c < NCH && m0 + c * 32 < M; c += splits * NG) {
-                    uint32_t own[32], v[32];
-                    sums(c * 32, own);
-                    for (int z = 0; z < splits; ++z) {
-                        uint32_t p[32];
-                        const uint32_t src = pf_cluster_addr(smem_u32(red + c * 32 * PF_BN), (uint32_t)z);
+                for (int g = zsplit + splits * part; g < 4 * nch && m0 + g * 8 < M; g += splits * NG) {
+                    uint32_t p[8][8], own[8];
+                    const uint32_t mine = smem_u32(red + g * 8 * PF_BN);
 #pragma unroll
-                        for (int i = 0; i < 32; ++i) p[i] = z == zsplit ? own[i] : pf_ld_cluster(src + (uint32_t)(i * PF_BN * 4));
+                    for (int z = 0; z < 8; ++z) {
+                        if (z >= splits || z == zsplit) continue;
+                        const uint32_t src = pf_cluster_addr(mine, (uint32_t)z);
 #pragma unroll
-                        for (int i = 0; i < 32; ++i) v[i] = z == 0 ? p[i] : __float_as_uint(__uint_as_float(v[i]) + __uint_as_float(p[i]));
+                        for (int i = 0; i < 8; ++i) p[z][i] = pf_ld_cluster(src + (uint32_t)(i * PF_BN * 4));
                     }
-                    if (feat < N && !gave_up) store(c * 32, v);
+                    pf_ld8(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(8 * g), own);
+                    if (!AT2 && nkb > 1) {
+                        uint32_t second[8];
+                        pf_ld8(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(PF_AT1_ACC_STRIDE + 8 * g), second);
+                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) own[i] = __float_as_uint(__uint_as_float(own[i]) + __uint_as_float(second[i]));
+                    } else {
+                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    }
+                    float v[8];
+#pragma unroll
+                    for (int z = 0; z < 8; ++z) {
+                        if (z >= splits) continue;
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            const float t = __uint_as_float(z == zsplit ? own[i] : p[z][i]);
+                            v[i] = z == 0 ? t : v[i] + t;
+                        }
+                    }
+                    if (feat < N && !gave_up) {
+                        uint16_t* dst = Y + (m0 + g * 8) * N + feat;
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            if (m0 + g * 8 + i < M) dst[(int64_t)i * N] = pf_out<DT>(v[i]);
+                    }
                 }
             }
         }
-#pragma unroll
-        for (int cc = 0; cc < CH; ++cc) {
-            if (CANON && splits > 1) break;
-            if (part + cc * NG >= NCH) break;
-            const int col = (part + cc * NG) * 32;
+#pragma unroll 1
+        for (int c = part; c < nch && !(CANON && splits > 1); c += NG) {
+            const int col = c * 32;
             if (m0 + col >= M) break;             // (warp-uniform) no token in these columns
             uint32_t v[32];
             sums(col, v);
@@ -788,13 +819,20 @@ bool gemm_prefill_supported(int64_t M, int64_t N, int64_t K, int bits, int group
 // tiles when they cover at most half of the SMs -- are cut along K into `splits` items each (FP32 partial sums + an
 // arrival counter per such tile in the workspace), at least four column blocks per item.
 struct PrefillPlan {
+    int h;                // tokens per X tile, two X tiles per output tile
     int tiles_m, tiles, n_full, n_tail, splits;
     int64_t rows_alloc;
     size_t counter_bytes, ws_bytes;
 };
-static PrefillPlan prefill_plan(int64_t M, int64_t N, int64_t K) {
+// h for tiles_m token tiles of (nearly) equal size; a single tile of at most 128 tokens has one X tile
+static int even_h(int64_t M, int64_t tiles_m) {
+    if (M <= PF_BM) return PF_BM;
+    return (int)(((M + 2 * tiles_m - 1) / (2 * tiles_m) + 15) / 16 * 16);
+}
+static PrefillPlan prefill_items(int64_t M, int64_t N, int64_t K, int h) {
     PrefillPlan p{};
-    p.tiles_m = (int)((M + PF_BM * PF_MT - 1) / (PF_BM * PF_MT));
+    p.h = h;
+    p.tiles_m = (int)((M + 2 * h - 1) / (2 * h));
     p.tiles = p.tiles_m * (int)((N + PF_BN - 1) / PF_BN);
     const int slots = kSmCount;
     const int rem = p.tiles % slots;
@@ -810,16 +848,44 @@ static PrefillPlan prefill_plan(int64_t M, int64_t N, int64_t K) {
     p.splits = (int)s;
     p.n_tail = tail;
     p.n_full = p.tiles - tail;
-    p.rows_alloc = M < PF_BM * PF_MT ? M : PF_BM * PF_MT;
+    p.rows_alloc = M < 2 * h ? M : 2 * h;
     p.counter_bytes = tail ? ((size_t)tail * 4 + 255) / 256 * 256 : 0;
     p.ws_bytes = tail ? p.counter_bytes + (size_t)tail * (size_t)s * (size_t)p.rows_alloc * PF_BN * 4 : 0;
     return p;
+}
+static bool prefill_weight_tile_in_tmem();
+// The number of token tiles, hence h = half a tile's tokens (a multiple of 16, at most PF_MAX_H), whose work items take the
+// least time: waves of CTAs x (stages x pace + fixed cost), in cycles.  A 64-column stage takes 4 h cycles on the tensor pipe, as
+// many to bring in 2 h tokens of X at 64 bytes per clock, and not less than 500 (the roles' hand-offs); the CTA that adds up
+// the splits of a tile takes a round to memory per 16 KB of every other split.  Against equal tiles of 256 tokens: 301 tokens x 15360 x
+// 5120, one tile instead of two: 55.5 -> 35.6 us; x 11024 x 4096 (BF16), one: 47.7 -> 30.8 us; 512 x 5120 x 13824, three: 74 ->
+// 61 us.
+static PrefillPlan prefill_plan(int64_t M, int64_t N, int64_t K) {
+    if (!prefill_weight_tile_in_tmem()) return prefill_items(M, N, K, PF_BM);
+    if (M <= 2 * PF_BM) return prefill_items(M, N, K, even_h(M, 1));
+    PrefillPlan best{};
+    int64_t best_cost = INT64_MAX;
+    const int64_t t0 = (M + 2 * PF_MAX_H - 1) / (2 * PF_MAX_H);
+    for (int64_t t = t0; t <= t0 + 8 && t <= (M + PF_BM - 1) / PF_BM; ++t) {
+        const int h = even_h(M, t);
+        if (h > PF_MAX_H) continue;
+        const PrefillPlan p = prefill_items(M, N, K, h);
+        const int64_t pace = 46 * h / 10 > 500 ? 46 * h / 10 : 500, fixed = 7000 + 20 * h, stages = K / 64;
+        const int64_t waves = (p.n_full + kSmCount - 1) / kSmCount;
+        const int64_t add_up = 3000 + 20 * h + (p.rows_alloc + 31) / 32 * ((p.splits + 1) / 2) * 1600;
+        const int64_t cost = waves * (stages * pace + fixed) + (p.n_tail ? stages / p.splits * pace + fixed + add_up : 0);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = p;
+        }
+    }
+    return best;
 }
 // arrival counters (must start at zero; the kernel leaves them at zero) + FP32 partial sums of the split tiles
 size_t gemm_prefill_workspace(int64_t M, int64_t N, int64_t K, int, int) { return prefill_plan(M, N, K).ws_bytes; }
 
 static int* prefill_error_ptr();
-static bool encode_x_map(CUtensorMap* xmap, const void* X, int64_t M, int64_t K);
+static bool encode_x_map(CUtensorMap* xmap, const void* X, int64_t M, int64_t K, int h);
 
 // Where the large-M kernel keeps the decoded weight tile: in tensor memory (the producers write it with tcgen05.st, the
 // MMAs read their A operand there).  That takes a third of the traffic off shared memory, and a stage of shared memory
@@ -837,6 +903,16 @@ static bool prefill_wide_stages_allowed() {
     return !(e && strcmp(e, "tmem-narrow") == 0);
 }
 
+// f(integral_constant<bits>, integral_constant<0: FP16, 1: BF16>)
+template <typename F>
+static pot_status_t with_bits_and_type(int bits, int dt, F f) {
+    using std::integral_constant;
+    auto with_type = [&](auto b) { return dt == 0 ? f(b, integral_constant<int, 0>()) : f(b, integral_constant<int, 1>()); };
+    if (bits == 2) return with_type(integral_constant<int, 2>());
+    if (bits == 3) return with_type(integral_constant<int, 3>());
+    return with_type(integral_constant<int, 4>());
+}
+
 pot_status_t gemm_prefill_launch(const void* packed, const void* scales, int64_t N, int64_t K, int bits, int group,
                                  const void* X, int64_t M, void* Y, void* workspace, size_t ws_bytes, cudaStream_t s, int dt) {
     const PrefillPlan pl = prefill_plan(M, N, K);
@@ -844,78 +920,48 @@ pot_status_t gemm_prefill_launch(const void* packed, const void* scales, int64_t
     unsigned* counters = (unsigned*)workspace;
     float* partial = pl.ws_bytes > 0 ? (float*)((char*)workspace + pl.counter_bytes) : nullptr;
     CUtensorMap xmap;
-    if (!encode_x_map(&xmap, X, M, K)) return POT_ERR_CUDA;
+    if (!encode_x_map(&xmap, X, M, K, pl.h)) return POT_ERR_CUDA;
     const dim3 grid((unsigned)(pl.n_full + pl.n_tail * pl.splits));
-    auto run = [&](auto kernel, int stages, int mt, int at = 0, int ng = 4, int wide = 0) -> pot_status_t {
-        const size_t smem = pf_smem_bytes(stages, mt, at, wide);
-        const dim3 block((unsigned)pf_threads(ng, 2));
-        return launch_pdl_cluster(kernel, grid, block, smem, 1, true, s, xmap, (const uint4*)packed, (const uint16_t*)scales, N, K, group, M,
-                          (uint16_t*)Y, partial, counters, pl.tiles_m, pl.n_full, pl.splits, prefill_error_ptr());
+    auto run = [&](auto kernel, int ng, size_t smem) -> pot_status_t {
+        return launch_pdl_cluster(kernel, grid, dim3((unsigned)pf_threads(ng, 2)), smem, 1, true, s, xmap, (const uint4*)packed,
+                                  (const uint16_t*)scales, N, K, group, M, (uint16_t*)Y, partial, counters, pl.tiles_m, pl.n_full,
+                                  pl.splits, pl.h, prefill_error_ptr());
     };
-    // two issuers, one CTA per SM; for batches of up to 64 tokens: one token tile, three producer groups, six stages of a whole
-    // 128-column block with the weight ring in tensor memory (four groups, eight 24 KB stages with the tile in shared memory)
-    if (dt == 1) {
-        if (M <= PF_SMALL_TOKENS && prefill_weight_tile_in_tmem()) {
-            if (bits == 2) return run(pot_gemm_prefill_kernel<2, 6, 3, 2, 1, 1, 1>, 6, 1, 1, 3);
-            if (bits == 3) return run(pot_gemm_prefill_kernel<3, 6, 3, 2, 1, 1, 1>, 6, 1, 1, 3);
-            return run(pot_gemm_prefill_kernel<4, 6, 3, 2, 1, 1, 1>, 6, 1, 1, 3);
-        }
-        if (M <= PF_SMALL_TOKENS) {
-            if (bits == 2) return run(pot_gemm_prefill_kernel<2, 8, 4, 2, 1, 1>, 8, 1);
-            if (bits == 3) return run(pot_gemm_prefill_kernel<3, 8, 4, 2, 1, 1>, 8, 1);
-            return run(pot_gemm_prefill_kernel<4, 8, 4, 2, 1, 1>, 8, 1);
-        }
-        if (prefill_weight_tile_in_tmem() && grid.x <= (unsigned)kSmCount && prefill_wide_stages_allowed()) {
-            if (bits == 2) return run(pot_gemm_prefill_kernel<2, 3, 3, 2, 2, 1, 1, 3, 1>, 3, 2, 1, 3, 1);
-            if (bits == 3) return run(pot_gemm_prefill_kernel<3, 3, 3, 2, 2, 1, 1, 3, 1>, 3, 2, 1, 3, 1);
-            return run(pot_gemm_prefill_kernel<4, 3, 3, 2, 2, 1, 1, 3, 1>, 3, 2, 1, 3, 1);
-        }
-        if (prefill_weight_tile_in_tmem()) {
-            if (bits == 2) return run(pot_gemm_prefill_kernel<2, 6, 2, 2, 2, 1, 1>, 6, 2, 1, 2);
-            if (bits == 3) return run(pot_gemm_prefill_kernel<3, 6, 2, 2, 2, 1, 1>, 6, 2, 1, 2);
-            return run(pot_gemm_prefill_kernel<4, 6, 2, 2, 2, 1, 1>, 6, 2, 1, 2);
-        }
-        if (bits == 2) return run(pot_gemm_prefill_kernel<2, 4, 4, 2, 2, 1>, 4, 2);
-        if (bits == 3) return run(pot_gemm_prefill_kernel<3, 4, 4, 2, 2, 1>, 4, 2);
-        return run(pot_gemm_prefill_kernel<4, 4, 4, 2, 2, 1>, 4, 2);
-    }
-    if (M <= PF_SMALL_TOKENS && prefill_weight_tile_in_tmem()) {  // six stages of a whole 128-column block (16 KB of X), three producer groups; the A ring fills tensor memory
-        if (bits == 2) return run(pot_gemm_prefill_kernel<2, 6, 3, 2, 1, 0, 1>, 6, 1, 1, 3);
-        if (bits == 3) return run(pot_gemm_prefill_kernel<3, 6, 3, 2, 1, 0, 1>, 6, 1, 1, 3);
-        return run(pot_gemm_prefill_kernel<4, 6, 3, 2, 1, 0, 1>, 6, 1, 1, 3);
-    }
-    if (M <= PF_SMALL_TOKENS) {
-        if (bits == 2) return run(pot_gemm_prefill_kernel<2, 8, 4, 2, 1>, 8, 1);
-        if (bits == 3) return run(pot_gemm_prefill_kernel<3, 8, 4, 2, 1>, 8, 1);
-        return run(pot_gemm_prefill_kernel<4, 8, 4, 2, 1>, 8, 1);
-    }
-    // A single wave of CTAs (65 .. 256 tokens on decode-sized matrices) is paced by the stage visits, not by the tensor
-    // pipe: three stages of a whole 128-column block (64 KB of X, 64 columns of weights, three producer groups), as in the
-    // one-tile kernel (15360 x 5120 at 65 .. 128 tokens: 27.5 - 28.5 -> 22.2 - 23.1 us).
+    const bool tmem = prefill_weight_tile_in_tmem();
     const bool one_wave = grid.x <= (unsigned)kSmCount && prefill_wide_stages_allowed();
-    if (prefill_weight_tile_in_tmem() && one_wave) {
-        if (bits == 2) return run(pot_gemm_prefill_kernel<2, 3, 3, 2, 2, 0, 1, 3, 1>, 3, 2, 1, 3, 1);
-        if (bits == 3) return run(pot_gemm_prefill_kernel<3, 3, 3, 2, 2, 0, 1, 3, 1>, 3, 2, 1, 3, 1);
-        return run(pot_gemm_prefill_kernel<4, 3, 3, 2, 2, 0, 1, 3, 1>, 3, 2, 1, 3, 1);
-    }
-    if (prefill_weight_tile_in_tmem()) {  // two producer groups, six stages (32 KB of X each), the A ring in tensor memory
-        if (bits == 2) return run(pot_gemm_prefill_kernel<2, 6, 2, 2, 2, 0, 1>, 6, 2, 1, 2);
-        if (bits == 3) return run(pot_gemm_prefill_kernel<3, 6, 2, 2, 2, 0, 1>, 6, 2, 1, 2);
-        return run(pot_gemm_prefill_kernel<4, 6, 2, 2, 2, 0, 1>, 6, 2, 1, 2);
-    }
-    if (bits == 2) return run(pot_gemm_prefill_kernel<2, 4, 4, 2, 2>, 4, 2);
-    if (bits == 3) return run(pot_gemm_prefill_kernel<3, 4, 4, 2, 2>, 4, 2);
-    return run(pot_gemm_prefill_kernel<4, 4, 4, 2, 2>, 4, 2);
+    // two issuers, one CTA per SM
+    return with_bits_and_type(bits, dt, [&](auto b, auto d) -> pot_status_t {
+        constexpr int B = decltype(b)::value, D = decltype(d)::value;
+        if (M <= PF_SMALL_TOKENS) {
+            // one token tile, three producer groups, six stages of a whole 128-column block with the weight ring in tensor memory
+            // (four groups, eight 24 KB stages with the tile in shared memory)
+            if (tmem) return run(pot_gemm_prefill_kernel<B, 6, 3, 2, 1, D, 1>, 3, pf_smem_bytes(6, 1, 1));
+            return run(pot_gemm_prefill_kernel<B, 8, 4, 2, 1, D>, 4, pf_smem_bytes(8, 1));
+        }
+        if (!tmem) return run(pot_gemm_prefill_kernel<B, 4, 4, 2, 2, D>, 4, pf_smem_bytes(4, 2));
+        // Two producer groups keep up with the tensor pipe; BF16, whose decode takes longer, needs more (11024 x 4096 at 4 bits: 1024 tokens
+        // 80 -> 69 us, 2048 tokens 151 -> 141 us with three).
+        if (pl.h > PF_BM) {  // more than 256 tokens per tile: four stages, paced by the tensor pipe (4 h cycles per stage) whatever the matrix
+            constexpr int NG = D == 1 ? 4 : 2;
+            return run(pot_gemm_prefill_kernel<B, 4, NG, 2, 2, D, 1>, NG, pf_smem_bytes_h(4, pl.h, 1));
+        }
+        // A single wave of CTAs (65 .. 256 tokens on decode-sized matrices) is paced by the stage visits, not by the tensor
+        // pipe: three stages of a whole 128-column block (64 KB of X, 64 columns of weights, three producer groups), as in the
+        // one-tile kernel (15360 x 5120 at 65 .. 128 tokens: 27.5 - 28.5 -> 22.2 - 23.1 us).
+        if (one_wave) return run(pot_gemm_prefill_kernel<B, 3, 3, 2, 2, D, 1, 3, 1>, 3, pf_smem_bytes_h(3, pl.h, 2));
+        constexpr int NG = D == 1 ? 3 : 2;   // six stages (32 KB of X each)
+        return run(pot_gemm_prefill_kernel<B, 6, NG, 2, 2, D, 1>, NG, pf_smem_bytes_h(6, pl.h, 1));
+    });
 }
 
 static int* prefill_error_ptr() { return error_ptr(ERR_PREFILL); }
 
-static bool encode_x_map(CUtensorMap* xmap, const void* X, int64_t M, int64_t K) {
+static bool encode_x_map(CUtensorMap* xmap, const void* X, int64_t M, int64_t K, int h) {
     EncodeTiledFn encode = encode_tiled_fn();
     if (!encode) return false;
     const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)M};
     const cuuint64_t strides[1] = {(cuuint64_t)K * 2};
-    const cuuint32_t box[2] = {64, (cuuint32_t)(M <= PF_SMALL_TOKENS ? M : PF_BM)};  // the one-tile kernel: no padding rows
+    const cuuint32_t box[2] = {64, (cuuint32_t)(M <= PF_SMALL_TOKENS ? M : h)};  // the one-tile kernel: no padding rows
     const cuuint32_t estr[2] = {1, 1};
     return encode(xmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(X), dims, strides, box, estr,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -936,31 +982,23 @@ static int canonical_splits(int64_t tiles, int64_t K) {
 pot_status_t gemm_canonical_launch(const void* packed, const void* scales, int64_t N, int64_t K, int bits, int group,
                                    const void* X, int64_t M, void* Y, cudaStream_t s, int dt) {
     const bool small = M <= PF_SMALL_TOKENS;
-    const int64_t tiles_m = small ? 1 : (M + PF_BM * PF_MT - 1) / (PF_BM * PF_MT);
+    const int64_t tiles_m = (M + 2 * PF_BM - 1) / (2 * PF_BM);
     const int64_t tiles = tiles_m * ((N + PF_BN - 1) / PF_BN);
     if (tiles > 0x7fffffff / 8) return POT_ERR_SHAPE;
     const int splits = canonical_splits(tiles, K);
+    const int h = even_h(M, tiles_m);
     CUtensorMap xmap;
-    if (!encode_x_map(&xmap, X, M, K)) return POT_ERR_CUDA;
-    auto run = [&](auto kernel, int stages, int mt, int wide) -> pot_status_t {
-        return launch_pdl_cluster(kernel, dim3((unsigned)(tiles * splits)), dim3((unsigned)pf_threads(3, 2)), pf_smem_bytes(stages, mt, 1, wide),
-                                  splits, true, s, xmap, (const uint4*)packed, (const uint16_t*)scales, N, K, group, M, (uint16_t*)Y,
-                                  (float*)nullptr, (unsigned*)nullptr, (int)tiles_m, (int)(splits > 1 ? 0 : tiles), splits, prefill_error_ptr());
+    if (!encode_x_map(&xmap, X, M, K, h)) return POT_ERR_CUDA;
+    auto run = [&](auto kernel, size_t smem) -> pot_status_t {
+        return launch_pdl_cluster(kernel, dim3((unsigned)(tiles * splits)), dim3((unsigned)pf_threads(3, 2)), smem, splits, true, s, xmap,
+                                  (const uint4*)packed, (const uint16_t*)scales, N, K, group, M, (uint16_t*)Y, (float*)nullptr,
+                                  (unsigned*)nullptr, (int)tiles_m, (int)(splits > 1 ? 0 : tiles), splits, h, prefill_error_ptr());
     };
-    auto pick = [&](auto b, auto d) -> pot_status_t {
+    return with_bits_and_type(bits, dt, [&](auto b, auto d) -> pot_status_t {
         constexpr int B = decltype(b)::value, D = decltype(d)::value;
-        if (small) return run(pot_gemm_prefill_kernel<B, 6, 3, 2, 1, D, 1, 3, 0, 1>, 6, 1, 0);
-        return run(pot_gemm_prefill_kernel<B, 3, 3, 2, 2, D, 1, 3, 1, 1>, 3, 2, 1);
-    };
-    using std::integral_constant;
-    if (dt == 0) {
-        if (bits == 2) return pick(integral_constant<int, 2>(), integral_constant<int, 0>());
-        if (bits == 3) return pick(integral_constant<int, 3>(), integral_constant<int, 0>());
-        return pick(integral_constant<int, 4>(), integral_constant<int, 0>());
-    }
-    if (bits == 2) return pick(integral_constant<int, 2>(), integral_constant<int, 1>());
-    if (bits == 3) return pick(integral_constant<int, 3>(), integral_constant<int, 1>());
-    return pick(integral_constant<int, 4>(), integral_constant<int, 1>());
+        if (small) return run(pot_gemm_prefill_kernel<B, 6, 3, 2, 1, D, 1, 3, 0, 1>, pf_smem_bytes(6, 1, 1));
+        return run(pot_gemm_prefill_kernel<B, 3, 3, 2, 2, D, 1, 3, 1, 1>, pf_smem_bytes_h(3, h, 2));
+    });
 }
 
 }  // namespace pot

@@ -106,13 +106,35 @@ def test_prefill_config5_shape_sampled(B, oracle):
 
 
 @pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("dt", ["f16", "bf16"])
+def test_token_tiles_of_every_height(B, oracle, bits, dt):
+    """Two X tiles of h tokens, h a multiple of 16 up to 192: full, ragged and nearly empty second tiles, more than 256 tokens per
+    tile (four stages), K of one, a few and more stages than the ring has, whole tiles and tiles cut along K."""
+    G = 128
+    for i, (M, N, K) in enumerate([(130, 48, 128), (161, 144, 640), (177, 128, 1152), (225, 272, 384), (257, 16, 128), (273, 400, 256), (289, 144, 1152),
+                                   (305, 272, 2048), (321, 128, 640), (350, 144, 384), (384, 272, 896), (385, 48, 1152), (600, 128, 640), (750, 160, 512),
+                                   (300, 9600, 256), (384, 9600, 128)]):
+        c = PotCase(N, K, bits, G, dist="t5" if i % 2 else "normal", sigma=0.015, seed=(5, 700 + 10 * bits + i))
+        X = synth.activations(synth.rng_for(5, 800 + i), M, K, outliers=(i % 2 == 1))
+        if dt == "bf16":
+            X = f16_bits_to_bf16_bits(X)
+        rows = np.unique(np.concatenate([np.arange(min(N, 160)), np.arange(max(0, N - 160), N)]))
+        Y, A = oracle.matmul(c.packed, c.S, K, bits, G, X, rows=rows, dtype=oracle.BF16 if dt == "bf16" else oracle.F16)
+        dX = bf16_dev(X) if dt == "bf16" else f16_dev(X)
+        y = bits_of(B.pot_gemm(c.tiled(), c.tiled_S(), K, bits, G, dX, B.TILED))
+        assert B.pot_debug_errors() == (0, 0, 0)
+        ok, worst, tight = gate(y[:, rows], Y, A, bf16=dt == "bf16")
+        assert ok and tight < 4.0, (M, N, K, worst, tight)
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4])
 @pytest.mark.parametrize("G", [64, 128])
 @pytest.mark.parametrize("dt", ["f16", "bf16"])
 def test_canonical_gemm_matches_oracle(B, oracle, bits, G, dt):
     """Canonical codes on the tcgen05 kernel: row counts that are no multiple of anything, either side of the 64-token and
     128 / 256-token tile boundaries, one CTA per tile and clusters of 2 (K = 1024), 4 (K = 2048), 5, 6 (K = 2560, 3072) and 8 CTAs (K >= 4096)."""
     shapes = [(2, 1, 128), (5, 37, 4096), (16, 129, 1024), (64, 131, 2048), (65, 127, 4224), (128, 130, 640), (129, 255, 1024),
-              (200, 257, 2048), (256, 33, 128), (257, 300, 4096), (520, 140, 1152), (70, 200, 2560), (30, 20, 3072), (140, 5700, 2048), (20, 3400, 2688)]
+              (200, 257, 2048), (256, 33, 128), (257, 300, 4096), (520, 140, 1152), (800, 200, 640), (70, 200, 2560), (30, 20, 3072), (140, 5700, 2048), (20, 3400, 2688)]
     for i, (M, N, K) in enumerate(shapes):
         c = PotCase(N, K, bits, G, dist="t5" if i % 2 else "normal", sigma=0.015, seed=(5, 400 + 10 * bits + i))
         X = synth.activations(synth.rng_for(5, 500 + i), M, K, outliers=(i % 2 == 1))
