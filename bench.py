@@ -719,7 +719,7 @@ def extras(args, B, torch, dev, stream, f16, capture, time_graph, peaks, build_c
             fl = 2.0 * synth.PREFILL_M * pr.N * pr.K
             row = {"shape": f"70B {pr.name} {pr.K}->{pr.N}", "M": synth.PREFILL_M, "bits": bits, "ms": t,
                    "TFLOPs": fl / t / 1e9, "frac_tensor_burst": fl / t / 1e9 / peaks["bf16_tflops"],
-                   "kernel": "tcgen05" if layout == B.TILED else "mma.sync fallback"}
+                   "kernel": "tcgen05"}
             if bits == HEADLINE_BITS and pr.name == "gate_or_up":
                 # the same launch ~600 times back to back: about half a second under the power cap, the regime in
                 # which the sustained cuBLAS figure was measured

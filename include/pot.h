@@ -251,12 +251,13 @@ pot_status_t pot_gemv_noalloc(const void* packed_tiled, const void* scales_f16, 
  * accumulation, FP16 output.  M = 1 runs pot_gemv's kernel.  2 <= M <= 8 (decode batches) runs the streaming
  * tensor-core kernel of pot_gemv with one token per MMA column, the weights decoded straight into MMA
  * fragments (5 <= M <= 8 only while 16 K bytes of activations fit in shared memory beside the rings: K <= 8192 or so);
- * larger M runs the tcgen05 kernel: TMA loads of X tiles, weights decoded into swizzled shared-memory tiles,
- * accumulators in tensor memory (two issuing threads with an accumulator each, added in a fixed
+ * larger M runs the tcgen05 kernel: TMA loads of X tiles, weights decoded into tensor memory,
+ * accumulators beside them (two issuing threads with an accumulator each, added in a fixed
  * order: the result does not depend on timing); the tiles of a last, at most half-filled wave
  * of CTAs -- or all tiles when they cover at most half of the SMs -- are split along K (FP32
- * partial sums and arrival counters in `workspace`, added in a fixed order).  The tcgen05
- * kernel requires layout == POT_LAYOUT_TILED.
+ * partial sums and arrival counters in `workspace`, added in a fixed order).
+ * POT_LAYOUT_CANONICAL (any N, no workspace): M = 1 runs pot_gemv's kernel, larger M the tcgen05 kernel with
+ * producers that decode canonical codes; few tiles are split along K over the CTAs of a cluster.
  *   workspace >= pot_gemm_workspace_bytes(M,N,K,bits,group), 16-byte aligned, zero before its
  *   first use (the kernels leave the counters at zero); may be NULL when that size is 0.
  */
@@ -265,8 +266,8 @@ pot_status_t pot_gemm(const void* packed, const void* scales_f16, int64_t N, int
                       void* workspace, size_t workspace_bytes, void* stream);
 
 /* pot_gemm_bf16 -- pot_gemm with BF16 activations X_bf16 [M,K], BF16 reconstruction (see pot_gemv_bf16) and BF16
- * output Y_bf16 [M,N]; same routes (streaming kernel, tcgen05 kernel with the BF16 instruction kind, canonical
- * fallback), same workspace sizes.                                                                              */
+ * output Y_bf16 [M,N]; same routes (streaming kernel, tcgen05 kernel with the BF16 instruction kind), same
+ * workspace sizes.                                                                                              */
 pot_status_t pot_gemm_bf16(const void* packed, const void* scales_f16, int64_t N, int64_t K, int bits,
                            int group, pot_layout_t layout, const void* X_bf16, int64_t M, void* Y_bf16,
                            void* workspace, size_t workspace_bytes, void* stream);
