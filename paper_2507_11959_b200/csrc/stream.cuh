@@ -14,10 +14,10 @@
 // Arithmetic.  Lane (gid, tig) of a warp owns quarter tig (32 columns) of rows gid and gid + 8 of a unit: exactly its
 // share of the A fragments of eight m16n8k16 MMAs.  It decodes its 2 x 32 codes in registers to +-2^E under a constant
 // exponent and issues the MMAs against B fragments that hold the activation vector in every column (GEMV) or one token per
-// column (small batch); the group's scale multiplies the unit's FP32 sums.  (Where a unit's sums mix two groups -- several tokens
-// with G = 64 --, where x does not fit in shared memory and in the uniform twin the scale goes into the weights: mask, shift and
-// integer add into its bit pattern, Sec. 4.2 of the paper.)  The FP32 accumulators stay in registers for as long as the warp
-// stays inside one row block.
+// column (small batch); the group's scale multiplies the unit's FP32 sums.  (With BF16 activations, where a unit's sums mix two
+// groups -- several tokens with G = 64 --, where x does not fit in shared memory and in the uniform twin the scale goes into the
+// weights: mask, shift and integer add into its bit pattern, Sec. 4.2 of the paper.)  The FP32 accumulators stay in registers for
+// as long as the warp stays inside one row block.
 //
 // Delivery.  A warp that covered a whole row block writes Y.  Otherwise its sums go to slot (row block, position of the
 // warp among the row block's contributors) of the workspace; a per-row-block arrival counter tells the last contributor,
@@ -69,10 +69,7 @@ struct StreamPlan {
     bool ok;              // false: the shape cannot run on this kernel (too many units)
 };
 
-// bytes that the unscaled kernel keeps behind the activations: 256 zeros (GEMV) and, for BF16, one FP32 factor per unit and token slot
-__host__ __device__ constexpr int sk_x_extra(int ncb, int tok, int token_shift, int dt) {
-    return (tok == 1 ? 256 : 0) + (dt == 1 ? (ncb << token_shift) * 4 : 0);
-}
+constexpr int SK_ZERO_BYTES = 256;  // zeros that the unscaled GEMV keeps behind the activations
 
 inline StreamPlan plan_stream(int64_t N, int64_t K, int64_t M, int bits, int group, int kind, int tok, int warps, int occ = 1, int dt = 0) {
     StreamPlan p = {};
@@ -100,8 +97,9 @@ inline StreamPlan plan_stream(int64_t N, int64_t K, int64_t M, int bits, int gro
     const size_t hdr = (size_t)sk_header_bytes(warps, tok);
     // multi-token kernel: the staged block has 2, 4 or 8 token slots per 16-byte chunk position (the smallest that holds M)
     p.token_shift = tok > 1 ? (M <= 2 ? 1 : (M <= 4 ? 2 : 3)) : 0;
-    p.unscaled = kind == SK_POT && (tok == 1 || group == 128);
-    const size_t xb = (((size_t)K * 2) << p.token_shift) + (p.unscaled ? (size_t)sk_x_extra((int)ncb, tok, p.token_shift, dt) : 0);
+    // (BF16: every BF16 number has to stay an exact operand, and FP16 codes cannot meet them in one MMA)
+    p.unscaled = kind == SK_POT && dt == 0 && (tok == 1 || group == 128);
+    const size_t xb = (((size_t)K * 2) << p.token_shift) + (p.unscaled && tok == 1 ? SK_ZERO_BYTES : 0);
     // slots of 4 units unless the ring could then hold only one of them next to the staged activations
     int q = SK_QMAX;
     if (hdr + xb + (size_t)warps * 2 * (size_t)sk_slot_bytes(bits, group, kind, q) > budget) q = 2;
@@ -174,32 +172,6 @@ __device__ __forceinline__ uint16_t sk_out(float v) {
 }
 __device__ __forceinline__ uint32_t sk_lds32(const unsigned char* p) { return *reinterpret_cast<const uint32_t*>(p); }
 __device__ __forceinline__ uint4 sk_lds128(const unsigned char* p) { return *reinterpret_cast<const uint4*>(p); }
-// Eight BF16 numbers -> FP16 numbers relative to the largest finite one of the 16 lanes that differ in the bits of `lanes`
-// (brought to 2^14 .. 2^15); returns the factor that undoes it.  All 32 lanes take part; !ok: the lane holds nothing.
-__device__ __forceinline__ float sk_normalize(uint4& v, bool ok, int lanes) {
-    uint32_t w[4] = {v.x, v.y, v.z, v.w};
-    uint32_t e = 0x80u;  // exponent field 1, at bit 7
-    if (ok) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const uint32_t lo = w[i] & 0x7F80u, hi = (w[i] >> 16) & 0x7F80u;
-            e = max(e, lo == 0x7F80u ? 0u : lo);
-            e = max(e, hi == 0x7F80u ? 0u : hi);
-        }
-    }
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1)
-        if (lanes & o) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
-    const uint32_t up = min(268u - (e >> 7), 253u);  // exponent field of the factor (253: its inverse is still a normal number)
-    const float f = __uint_as_float(up << 23);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const __half2 h = __floats2half2_rn(__uint_as_float(w[i] << 16) * f, __uint_as_float(w[i] & 0xFFFF0000u) * f);
-        w[i] = *reinterpret_cast<const uint32_t*>(&h);
-    }
-    v = make_uint4(w[0], w[1], w[2], w[3]);
-    return __uint_as_float((254u - up) << 23);
-}
 // floor(a * b / c) for a * b that may need 64 bits
 __device__ __forceinline__ uint32_t sk_muldiv(uint32_t a, uint32_t b, uint32_t c, bool fits32) {
     if (fits32) return (a * b) / c;
@@ -214,14 +186,15 @@ __device__ __forceinline__ uint32_t sk_muldiv(uint32_t a, uint32_t b, uint32_t c
 // memory), so that the next launch in the stream can become resident and fill its rings while this one still computes.
 // UNSC: the codes are decoded without their scale (pot_units32) and a unit's FP32 sums are multiplied by it.  With two groups per
 // unit (G = 64, GEMV only) columns 0-3 of B hold x of the first group's quarters and zeros for the others, columns 4-7 the
-// opposite, so that the two groups' sums come out in different lanes.  BF16 activations are staged as FP16 numbers relative to
-// the largest of their unit (2^14 .. 2^15), whose factor the unit's sums are multiplied by: the error, 2^-25 in those units where
-// FP16 runs out of exponents, is 2^-39 of the unit's largest |x|, against which every weight of the group counts at least 2^-7.
+// opposite, so that the two groups' sums come out in different lanes.  FP16 only: BF16 activations staged as FP16 numbers
+// relative to the largest of 128 columns took 29 instead of 38 us on 28672 x 8192 at 4 bits, but numbers more than 2^29 below
+// that largest one lost bits, which shows where the large terms cancel or stand under another group's small scale.
 template <int BITS, int KIND, int TOK, bool XSMEM, int W, int OCC, int SK_Q, int DT, bool UNSC>
 __device__ __forceinline__ void stream_body(const StreamArgs& sa, int* __restrict__ err) {
     constexpr int UB = sk_unit_bytes(BITS);
     constexpr bool UNIFORM = (KIND == SK_UINT);
     constexpr int NPARAM = UNIFORM ? 2 : 1;
+    static_assert(!UNSC || (!UNIFORM && DT == 0 && XSMEM), "the decode without the scale: PoT codes, FP16, x in shared memory");
     extern __shared__ __align__(128) unsigned char smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int gid = lane >> 2, tig = lane & 3;  // MMA fragment coordinates: rows gid and gid + 8, quarter tig
@@ -252,7 +225,6 @@ __device__ __forceinline__ void stream_body(const StreamArgs& sa, int* __restric
     unsigned* lcnt = reinterpret_cast<unsigned*>(smem + W * 96);               // local arrival counters
     float* lslots = reinterpret_cast<float*>(smem + W * 96 + W * 4);           // [warp][first, last][16 TOK]
     const unsigned char* xs = smem + HDR;
-    float* xfac = reinterpret_cast<float*>(smem + HDR + ((sa.K * 2) << sa.token_shift) + (TOK == 1 ? 256 : 0));  // UNSC, BF16: [unit][token slot]
     const unsigned char* ringp = xs + sa.x_bytes + (uint32_t)warp * (uint32_t)S * slot_bytes;  // this warp's ring
     const uint32_t ring = smem0 + (uint32_t)HDR + (uint32_t)sa.x_bytes + (uint32_t)warp * (uint32_t)S * slot_bytes;
 
@@ -329,11 +301,11 @@ __device__ __forceinline__ void stream_body(const StreamArgs& sa, int* __restric
         const uint4* src = reinterpret_cast<const uint4*>(sa.X);
         const int kc = (int)(sa.K / 8);  // 16-byte chunks per token
         if constexpr (UNSC && TOK == 1)
-            if (threadIdx.x < 16) *reinterpret_cast<uint4*>(smem + HDR + sa.K * 2 + threadIdx.x * 16) = make_uint4(0, 0, 0, 0);
+            if (threadIdx.x < SK_ZERO_BYTES / 16) *reinterpret_cast<uint4*>(smem + HDR + sa.K * 2 + threadIdx.x * 16) = make_uint4(0, 0, 0, 0);
         if constexpr (TOK == 1) {
             // chunk (quarter t, part j) of a unit goes to position j * 4 + t: lanes tig = 0..3 read 64 contiguous bytes
             // (four loads in flight per thread before the first store: one round trip for K <= 32 * 32 W)
-            for (int i0 = threadIdx.x; (i0 & ~31) < kc; i0 += 4 * W * 32) {  // (whole warps)
+            for (int i0 = threadIdx.x; i0 < kc; i0 += 4 * W * 32) {
                 uint4 v[4];
 #pragma unroll
                 for (int p = 0; p < 4; ++p)
@@ -341,10 +313,6 @@ __device__ __forceinline__ void stream_body(const StreamArgs& sa, int* __restric
 #pragma unroll
                 for (int p = 0; p < 4; ++p) {
                     const int i = i0 + p * W * 32;
-                    if constexpr (UNSC && DT == 1) {  // lanes 0-15 and 16-31 hold one unit each
-                        const float f = sk_normalize(v[p], i < kc, 0x0F);
-                        if (i < kc && (i & 15) == 0) xfac[i >> 4] = f;
-                    }
                     if (i < kc) dst[(i & ~15) | ((i & 3) << 2) | ((i >> 2) & 3)] = v[p];
                 }
             }
@@ -358,7 +326,7 @@ __device__ __forceinline__ void stream_body(const StreamArgs& sa, int* __restric
             // token's parity, then j -- a warp loads the 256 contiguous bytes of a unit for two tokens.
             const int ts = sa.token_shift;
             const int total = kc << ts;
-            for (int e0 = threadIdx.x; (e0 & ~31) < total; e0 += 8 * W * 32) {  // eight loads in flight per thread, whole warps
+            for (int e0 = threadIdx.x; e0 < total; e0 += 8 * W * 32) {  // eight loads in flight per thread
                 uint4 v[8];
 #pragma unroll
                 for (int p = 0; p < 8; ++p) {
@@ -372,10 +340,6 @@ __device__ __forceinline__ void stream_body(const StreamArgs& sa, int* __restric
                     const int e = e0 + p * W * 32;
                     const int t = e & 3, par = (e >> 2) & 1, j = (e >> 3) & 3, hi = (e >> 5) & ((1 << (ts - 1)) - 1), unit_ = e >> (4 + ts);
                     const int token = (hi << 1) | par;
-                    if constexpr (UNSC && DT == 1) {  // a warp holds one unit of two tokens: t in bits 0-1 of the lane, j in bits 3-4
-                        const float f = sk_normalize(v[p], e < total && token < sa.M, 0x1B);
-                        if (e < total && (e & 0x1B) == 0) xfac[(unit_ << ts) + token] = f;
-                    }
                     if (e < total && token < sa.M) dst[(((unit_ << 2) + j) << (2 + ts)) + (hi << 3) + (par << 2) + t] = v[p];
                 }
             }
@@ -582,27 +546,12 @@ __device__ __forceinline__ void stream_body(const StreamArgs& sa, int* __restric
 #pragma unroll
             for (int j = 0; j < 8; ++j) sk_mma(c, lo[2 * j], hi[2 * j], lo[2 * j + 1], hi[2 * j + 1], xq[2 * j], xq[2 * j + 1]);
             const uint32_t scw = sk_lds32(param + ((spg == 2 ? (uint32_t)(tig >> 1) * 8u : 0u) + (uint32_t)gid) * 4u);  // {row gid, row gid + 8}
-            float2 sc = __half22float2(*reinterpret_cast<const __half2*>(&scw));
-            if constexpr (DT == 0) {
-                acc[0][0] = fmaf(c[0], sc.x, acc[0][0]);
-                acc[0][2] = fmaf(c[2], sc.y, acc[0][2]);
-                if constexpr (TOK > 1) {
-                    acc[0][1] = fmaf(c[1], sc.x, acc[0][1]);
-                    acc[0][3] = fmaf(c[3], sc.y, acc[0][3]);
-                }
-            } else {  // the FP16 scale rounded once to BF16; times the unit's factor last, so that no product leaves FP32's range early
-                sc = __bfloat1622float2(__float22bfloat162_rn(sc));
-                if constexpr (TOK == 1) {
-                    const float f = xfac[cbu];
-                    acc[0][0] = fmaf(c[0] * sc.x, f, acc[0][0]);
-                    acc[0][2] = fmaf(c[2] * sc.y, f, acc[0][2]);
-                } else {
-                    const float2 f = *reinterpret_cast<const float2*>(xfac + (cbu << sa.token_shift) + ((2 * tig) & ((1 << sa.token_shift) - 1)));
-                    acc[0][0] = fmaf(c[0] * sc.x, f.x, acc[0][0]);
-                    acc[0][1] = fmaf(c[1] * sc.x, f.y, acc[0][1]);
-                    acc[0][2] = fmaf(c[2] * sc.y, f.x, acc[0][2]);
-                    acc[0][3] = fmaf(c[3] * sc.y, f.y, acc[0][3]);
-                }
+            const float2 sc = __half22float2(*reinterpret_cast<const __half2*>(&scw));
+            acc[0][0] = fmaf(c[0], sc.x, acc[0][0]);
+            acc[0][2] = fmaf(c[2], sc.y, acc[0][2]);
+            if constexpr (TOK > 1) {
+                acc[0][1] = fmaf(c[1], sc.x, acc[0][1]);
+                acc[0][3] = fmaf(c[3], sc.y, acc[0][3]);
             }
             return;
         }
@@ -732,9 +681,9 @@ pot_status_t launch_stream(const void* packed, const void* scales, const void* z
     constexpr bool POT = KIND == SK_POT;
     auto pick = [&](auto q) -> pot_status_t {  // q units per slot
         constexpr int Q = decltype(q)::value;
-        if constexpr (POT)
+        if constexpr (POT && DT == 0)
             if (p.unscaled) return run(stream_kernel<BITS, KIND, TOK, true, W, OCC, Q, DT, true>);
-        if constexpr (!(POT && TOK == 1))
+        if constexpr (!(POT && DT == 0 && TOK == 1))
             if (p.x_in_smem) return run(stream_kernel<BITS, KIND, TOK, true, W, OCC, Q, DT, false>);
         return run(stream_kernel<BITS, KIND, TOK, false, W, OCC, Q, DT, false>);
     };

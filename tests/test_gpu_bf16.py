@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 
 from paper_2507_11959_b200 import synth
-from tests.gpu_util import GuardedBinding, PotCase, bf16_dev, bits_of, f16_bits_to_bf16_bits, gate
+from tests.gpu_util import GuardedBinding, PotCase, bf16_dev, bits_of, f16_bits_to_bf16_bits, f16_dev, gate, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -69,9 +69,8 @@ def test_bf16_gemm_matches_oracle(B, oracle, bits, M):
 @pytest.mark.parametrize("G", [64, 128])
 @pytest.mark.parametrize("M", [1, 3, 8])
 def test_bf16_activations_over_the_whole_exponent_range(B, oracle, bits, G, M):
-    """The streaming kernels hold BF16 activations as FP16 numbers relative to the largest of 128 columns: units far apart in size,
-    elements far below their unit's largest, all zeros, the smallest and the largest magnitudes -- and infinities and NaN, which
-    come out as the sum of the products has them."""
+    """Units of 128 columns far apart in size, elements far below their unit's largest, all zeros, the smallest and the largest
+    magnitudes -- and infinities and NaN, which come out as the sum of the products has them."""
     N, K = 64, 1152
     c = PotCase(N, K, bits, G, dist="normal", seed=(7, 800 + bits))
     rng = np.random.default_rng(10 * bits + M)
@@ -100,3 +99,43 @@ def test_bf16_activations_over_the_whole_exponent_range(B, oracle, bits, G, M):
             assert np.all((got & 0x7FFF) > 0x7F80)
         else:
             assert np.array_equal(got, np.where((w ^ bad) & 0x8000, 0xFF80, 0x7F80).astype(np.uint16))
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("G", [64, 128])
+@pytest.mark.parametrize("M", [1, 3, 8, 12])
+def test_bf16_activations_are_exact_operands(B, oracle, bits, G, M):
+    """Activations 2^36 and more below the largest of their 128 columns count in full: (a) two large terms that cancel exactly, in one
+    MMA that multiplies nothing else (columns 32 q .. 32 q + 3 belong together in the streaming and canonical kernels, at 2 bits the even
+    ones of 32 q .. 32 q + 7 in the canonical one, 16 neighbours in the tcgen05 kernel: columns 0 and 2 always do); (b) a large
+    activation under a group's smallest scale beside small ones under the largest."""
+    N, K = 64, 512
+    rng = np.random.default_rng(100 * bits + G + M)
+    c = PotCase(N, K, bits, G, dist="normal", seed=(7, 1000 + bits))
+
+    def run(codes, S, X, Y, A):
+        packed, dS = to_dev(oracle.pack(codes, bits)), f16_dev(S)
+        tiled, tS = B.pot_repack(packed, K, bits, 0), B.pot_repack_scales(dS, K, G, 0)
+        for layout, P, Sd in ((B.TILED, tiled, tS), (B.CANONICAL, packed, dS)):
+            got = bits_of(B.pot_gemm(P, Sd, K, bits, G, bf16_dev(X), layout)).reshape(M, N)
+            ok, worst, tight = gate(got, Y, A, bf16=True)
+            assert ok and tight < 4.0, (layout, worst, tight)
+
+    codes = c.codes.copy()
+    codes[:, 2] = codes[:, 0]
+    X = ((rng.integers(117, 120, (M, K)) << 7) | rng.integers(0, 0x80, (M, K)) | (rng.integers(0, 2, (M, K)) << 15)).astype(np.uint16)
+    X[:, np.arange(K) % 32 < 8] = 0
+    X[:, :16] = 0
+    Y, A = oracle.matmul(oracle.pack(codes, bits), c.S, K, bits, G, X, dtype=oracle.BF16)  # (of the small ones alone)
+    X[:, 0], X[:, 2] = 0x4E80, 0xCE80                                                      # 2^30, -2^30
+    run(codes, c.S, X, Y, A)
+
+    codes = np.zeros_like(c.codes)
+    codes[:, 64:] = 2 ** (bits - 1) - 1
+    S = np.full((N, K // G), ((30 - (2 ** (bits - 1) - 1)) << 10) | 0x200, dtype=np.uint16)
+    S[:, 0] = 0x0400 if G == 64 else S[0, 0]
+    X = np.zeros((M, K), dtype=np.uint16)
+    X[:, 0] = (127 + 39) << 7
+    X[:, 64:128] = 0x3F80
+    Y, A = oracle.matmul(oracle.pack(codes, bits), S, K, bits, G, X, dtype=oracle.BF16)
+    run(codes, S, X, Y, A)

@@ -96,6 +96,20 @@ def test_scale_search_where_sums_tie_or_span_the_whole_range(B, oracle, bits, G)
     assert np.array_equal(packed.cpu().numpy(), oracle.pack(codes, bits))
 
 
+def test_scale_search_between_sums_closer_than_the_loops_roundings(B, oracle):
+    """An outlier above all levels: Q1 is five times s^2 B + 2 s A, and the sums of candidates 2 and 3 differ by less than the
+    sequential loop rounds.  The exact sum of candidate 3 is the smaller one; the loop takes candidate 2."""
+    group = np.array([0x788F] + [0x5E5B] * 117 + [0x4DF6, 0x1E66, 0x001A] + [0] * 7, dtype=np.uint16)
+    W = np.tile(group, (8, 2))
+    W[1::2] |= 0x8000
+    S_ref, best = oracle.scale_search(W, 2, 128)
+    assert np.all(best == 2)
+    packed, S = B.pot_quantize_ref(f16_dev(W), 2, 128, B.SCALE_SEARCH)
+    assert np.array_equal(bits_of(S), S_ref)
+    codes, _ = oracle.quantize(W, 2, 128, oracle.RULE_GIVEN, S_ref)
+    assert np.array_equal(packed.cpu().numpy(), oracle.pack(codes, 2))
+
+
 @pytest.mark.parametrize("bits", [2, 3, 4])
 @pytest.mark.parametrize("G", [64, 128])
 @pytest.mark.parametrize("dtype", [0, 1])
