@@ -106,16 +106,18 @@ __global__ void __launch_bounds__(QZ_THREADS) pot_quantize_kernel(const uint4* _
 // sums of it.  I_k = I_0 >> k, because s_i scales exactly when i is doubled.  I_0 comes from one FP32 multiplication; where
 // that is too close to an integer the comparison of the sequential loop itself decides.  A and B are integers (A in units of
 // the last place of the group's smallest weight), hence exact.
-// D is evaluated in FP32, off by at most SEARCH_TOL32 T, T = s^2 B + 2 s A (7 roundings of 2^-24 T and the sequential loop's
-// own 131 2^-53 Q1).  A candidate whose lower bound is above the smallest upper bound cannot be the minimiser.  Mostly one
-// candidate is left; else the same bounds in FP64 (SEARCH_TOL64: 16 + 131 roundings of 2^-53), and if several are left even
-// then (equal or all but equal sums) the sequential loop decides between those: the result is that of the plain loop
-// bit for bit.
+// A candidate whose lower bound is above the smallest upper bound cannot be the one that the loop takes.  The loop's own
+// roundings, 131 2^-53 Q1, belong to the bounds: relative to Q1 = W2 + D, not to T = s^2 B + 2 s A, of which Q1 is several
+// times as much where an outlier lies above all levels.  D is evaluated in FP32, off by at most SEARCH_TOL32 T (7 roundings
+// of 2^-24 T; the loop's share fits into what is left, because W2 <= 6400 T for any group: T >= 2 s A >= 0.02 s0 max|w| sum|w| / max|w|
+// and s0 >= max|w| / 127).  Mostly one candidate is left; else the bounds are taken in FP64, off by SEARCH_EPS (16 T + 132 Q1), and
+// if several are left even then (equal or all but equal sums) the sequential loop decides between those: the result is that
+// of the plain loop bit for bit.
 // What bounds it: instruction issue (82 % of the issue slots, 750 instructions per group of 128 at 3 bits, two thirds of them the
 // histogram's entries and the 200 evaluations).  11008 x 4096, groups of 128 (64), 3 bits: 9184 us term by term, 280 us so;
-// 4 bits 12424 (12873), 476 (631) us; 2 bits, groups of 64: 5974, 376 us.
+// 4 bits 12424 (12873), 476 (631) us; 2 bits, groups of 64: 5974, 376 us; Q1 in the FP64 bounds: 0 - 2 % more.
 constexpr float SEARCH_TOL32 = 6e-7f;
-constexpr double SEARCH_TOL64 = 2e-14;
+constexpr double SEARCH_EPS = 1.1102230246251565e-16;  // 2^-53
 constexpr int SEARCH_BINS = 224;     // 7 candidates per lane; 201 .. 224 stay empty
 constexpr int SEARCH_NC = 7;         // candidates per lane: i = 7 lane + 1 .. 7 lane + 7
 constexpr int SEARCH_LOW_BITS = 22;  // WIDE: A's bins are two 32-bit sums, and no bin of 128 weights x QMAX entries overflows
@@ -228,15 +230,23 @@ __device__ __forceinline__ uint32_t search_candidates(const uint32_t (&h)[PER], 
     }
     if (__reduce_add_sync(0xffffffffu, (uint32_t)__popc(flags)) > 1u) {
         double low[NC], up = 1e300;
+        float w2 = 0.f;
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            const float w = __half2float(__ushort_as_half((uint16_t)h[j]));
+            w2 = fmaf(w, w, w2);
+        }
+        for (int o = 16; o; o >>= 1) w2 += __shfl_xor_sync(0xffffffffu, w2, o);
+        w2 *= 1.0001f;  // (above W2, whatever the roundings of this sum)
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
             low[c] = 0.0;
             if ((flags >> c) & 1u) {
                 const double sc = search_scale(s0, NC * lane + 1 + c);
                 const double cross = 2.0 * sc * ((double)(A[c] + ta) * unit), square = sc * sc * (double)(Bc[c] + tb);
-                const double t = SEARCH_TOL64 * (square + cross);
-                low[c] = (square - cross) - t;
-                up = fmin(up, (square - cross) + t);
+                const double D = square - cross, t = SEARCH_EPS * (16.0 * (square + cross) + 132.0 * ((double)w2 + D));
+                low[c] = D - t;
+                up = fmin(up, D + t);
             }
         }
         for (int o = 16; o; o >>= 1) up = fmin(up, __shfl_xor_sync(0xffffffffu, up, o));
