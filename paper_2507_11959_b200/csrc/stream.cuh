@@ -142,12 +142,18 @@ struct StreamArgs {
     int token_shift;               // log2 of the token slots of the staged activations
     int fits32;                    // U * gw_total < 2^32: 32-bit range arithmetic
     int aligned, nrb;              // row-block split (see the kernel), number of row blocks
-    uint32_t bias;                 // potl::POT_UNIT_BIAS and
-    uint32_t p2[potl::POT_UNIT_SHIFTS];  // p2[n] = 2^n
 #ifdef SK_TRACE
     unsigned long long* trace;     // [launch slot][cta][8] globaltimer stamps
 #endif
 };
+// What only the decode without the scale reads (a type of its own: with twelve more words the parameters of
+// stream_kernel_by_value no longer fit in its registers).
+struct StreamArgsUnscaled : StreamArgs {
+    uint32_t bias;                       // potl::POT_UNIT_BIAS
+    uint32_t p2[potl::POT_UNIT_SHIFTS];  // p2[n] = 2^n
+};
+template <bool UNSC>
+using StreamKernelArgs = typename std::conditional<UNSC, StreamArgsUnscaled, StreamArgs>::type;
 
 #ifdef __CUDACC__
 __device__ __forceinline__ void sk_mma(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
@@ -190,7 +196,7 @@ __device__ __forceinline__ uint32_t sk_muldiv(uint32_t a, uint32_t b, uint32_t c
 // relative to the largest of 128 columns took 29 instead of 38 us on 28672 x 8192 at 4 bits, but numbers more than 2^29 below
 // that largest one lost bits, which shows where the large terms cancel or stand under another group's small scale.
 template <int BITS, int KIND, int TOK, bool XSMEM, int W, int OCC, int SK_Q, int DT, bool UNSC>
-__device__ __forceinline__ void stream_body(const StreamArgs& sa, int* __restrict__ err) {
+__device__ __forceinline__ void stream_body(const StreamKernelArgs<UNSC>& sa, int* __restrict__ err) {
     constexpr int UB = sk_unit_bytes(BITS);
     constexpr bool UNIFORM = (KIND == SK_UINT);
     constexpr int NPARAM = UNIFORM ? 2 : 1;
@@ -626,8 +632,20 @@ __device__ __forceinline__ void stream_body(const StreamArgs& sa, int* __restric
 }
 
 template <int BITS, int KIND, int TOK, bool XSMEM, int W, int OCC, int SK_Q, int DT, bool UNSC>
-__global__ void __launch_bounds__(W * 32, OCC) stream_kernel(const __grid_constant__ StreamArgs sa, int* __restrict__ err) {
+__global__ void __launch_bounds__(W * 32, OCC) stream_kernel(const __grid_constant__ StreamKernelArgs<UNSC> sa, int* __restrict__ err) {
     stream_body<BITS, KIND, TOK, XSMEM, W, OCC, SK_Q, DT, UNSC>(sa, err);
+}
+// The same with the parameters by value, for the uniform twin at 2 bits: read from constant memory they cost its two-CTA build
+// (64 registers) spills of 96 / 112 bytes, 4096 x 4096 4.2 -> 5.7 us, 12288 x 4096 9.6 -> 12.2 us.  At 3 bits constant memory is 3 %
+// the faster one (14.1 -> 13.7 us), at 4 bits between 3 % slower and 2 % faster.
+template <int BITS, int KIND, int TOK, bool XSMEM, int W, int OCC, int SK_Q, int DT, bool UNSC>
+__global__ void __launch_bounds__(W * 32, OCC) stream_kernel_by_value(const StreamArgs sa, int* __restrict__ err) {
+    stream_body<BITS, KIND, TOK, XSMEM, W, OCC, SK_Q, DT, UNSC>(sa, err);
+}
+template <int BITS, int KIND, int TOK, bool XSMEM, int W, int OCC, int SK_Q, int DT, bool UNSC>
+constexpr auto stream_kernel_of() {
+    if constexpr (KIND == SK_UINT && BITS == 2) return stream_kernel_by_value<BITS, KIND, TOK, XSMEM, W, OCC, SK_Q, DT, UNSC>;
+    else return stream_kernel<BITS, KIND, TOK, XSMEM, W, OCC, SK_Q, DT, UNSC>;
 }
 #endif  // __CUDACC__
 
@@ -662,8 +680,6 @@ inline StreamArgs stream_args(const StreamPlan& p, const void* packed, const voi
     sa.trace = g_sk_trace;
     if (g_sk_trace) g_sk_trace += 148 * 2 * 8;
 #endif
-    sa.bias = potl::POT_UNIT_BIAS;
-    for (int i = 0; i < potl::POT_UNIT_SHIFTS; ++i) sa.p2[i] = 1u << i;
     sa.fits32 = ((uint64_t)p.units + 1) * ((uint64_t)sa.gw_total + 1) < (uint64_t(1) << 32) ? 1 : 0;
     return sa;
 }
@@ -674,18 +690,23 @@ pot_status_t launch_stream(const void* packed, const void* scales, const void* z
                            const void* X, int M, void* Y, void* workspace, int* err, cudaStream_t s) {
     const StreamPlan p = plan_stream(N, K, M, BITS, group, KIND, TOK, W, OCC, DT);
     if (!p.ok) return POT_ERR_SHAPE;
-    const StreamArgs sa = stream_args(p, packed, scales, zeros, N, K, group, X, M, Y, workspace);
+    StreamArgsUnscaled args;
+    static_cast<StreamArgs&>(args) = stream_args(p, packed, scales, zeros, N, K, group, X, M, Y, workspace);
+    args.bias = potl::POT_UNIT_BIAS;
+    for (int i = 0; i < potl::POT_UNIT_SHIFTS; ++i) args.p2[i] = 1u << i;
     auto run = [&](auto kernel) -> pot_status_t {
-        return launch_pdl_cluster(kernel, dim3((unsigned)p.grid), dim3(W * 32), p.smem_bytes, 1, true, s, sa, err);
+        auto launch = [&](const auto& a) { return launch_pdl_cluster(kernel, dim3((unsigned)p.grid), dim3(W * 32), p.smem_bytes, 1, true, s, a, err); };
+        if constexpr (std::is_same<decltype(kernel), void (*)(StreamArgs, int*)>::value) return launch(static_cast<const StreamArgs&>(args));
+        else return launch(args);
     };
     constexpr bool POT = KIND == SK_POT;
     auto pick = [&](auto q) -> pot_status_t {  // q units per slot
         constexpr int Q = decltype(q)::value;
         if constexpr (POT && DT == 0)
-            if (p.unscaled) return run(stream_kernel<BITS, KIND, TOK, true, W, OCC, Q, DT, true>);
+            if (p.unscaled) return run(stream_kernel_of<BITS, KIND, TOK, true, W, OCC, Q, DT, true>());
         if constexpr (!(POT && DT == 0 && TOK == 1))
-            if (p.x_in_smem) return run(stream_kernel<BITS, KIND, TOK, true, W, OCC, Q, DT, false>);
-        return run(stream_kernel<BITS, KIND, TOK, false, W, OCC, Q, DT, false>);
+            if (p.x_in_smem) return run(stream_kernel_of<BITS, KIND, TOK, true, W, OCC, Q, DT, false>());
+        return run(stream_kernel_of<BITS, KIND, TOK, false, W, OCC, Q, DT, false>());
     };
     if (p.q == 2) return pick(std::integral_constant<int, 2>());
     if constexpr (OCC == 1 && TOK == 1)
