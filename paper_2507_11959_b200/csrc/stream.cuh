@@ -69,7 +69,7 @@ struct StreamPlan {
     bool ok;              // false: the shape cannot run on this kernel (too many units)
 };
 
-constexpr int SK_ZERO_BYTES = 256;  // zeros that the unscaled GEMV keeps behind the activations
+constexpr int SK_ZERO_BYTES = 256;  // zeros that the unscaled GEMV keeps behind the activations (two groups per unit)
 
 inline StreamPlan plan_stream(int64_t N, int64_t K, int64_t M, int bits, int group, int kind, int tok, int warps, int occ = 1, int dt = 0) {
     StreamPlan p = {};
@@ -99,7 +99,7 @@ inline StreamPlan plan_stream(int64_t N, int64_t K, int64_t M, int bits, int gro
     p.token_shift = tok > 1 ? (M <= 2 ? 1 : (M <= 4 ? 2 : 3)) : 0;
     // (BF16: every BF16 number has to stay an exact operand, and FP16 codes cannot meet them in one MMA)
     p.unscaled = kind == SK_POT && dt == 0 && (tok == 1 || group == 128);
-    const size_t xb = (((size_t)K * 2) << p.token_shift) + (p.unscaled && tok == 1 ? SK_ZERO_BYTES : 0);
+    const size_t xb = (((size_t)K * 2) << p.token_shift) + (p.unscaled && tok == 1 && group == 64 ? SK_ZERO_BYTES : 0);
     // slots of 4 units unless the ring could then hold only one of them next to the staged activations
     int q = SK_QMAX;
     if (hdr + xb + (size_t)warps * 2 * (size_t)sk_slot_bytes(bits, group, kind, q) > budget) q = 2;
@@ -307,7 +307,7 @@ __device__ __forceinline__ void stream_body(const StreamKernelArgs<UNSC>& sa, in
         const uint4* src = reinterpret_cast<const uint4*>(sa.X);
         const int kc = (int)(sa.K / 8);  // 16-byte chunks per token
         if constexpr (UNSC && TOK == 1)
-            if (threadIdx.x < SK_ZERO_BYTES / 16) *reinterpret_cast<uint4*>(smem + HDR + sa.K * 2 + threadIdx.x * 16) = make_uint4(0, 0, 0, 0);
+            if (spg == 2 && threadIdx.x < SK_ZERO_BYTES / 16) *reinterpret_cast<uint4*>(smem + HDR + sa.K * 2 + threadIdx.x * 16) = make_uint4(0, 0, 0, 0);
         if constexpr (TOK == 1) {
             // chunk (quarter t, part j) of a unit goes to position j * 4 + t: lanes tig = 0..3 read 64 contiguous bytes
             // (four loads in flight per thread before the first store: one round trip for K <= 32 * 32 W)

@@ -117,3 +117,12 @@ def test_tiled_layout_map_is_a_bijection_with_pairs_16_apart(L, bits, kind):
             assert w0 == w1 and (b1 - b0) % 32 == 16
     with pytest.raises(binding.PotError):
         binding.pot_layout_bit(bits, kind, 128, 0)
+
+
+def test_units_of_one_group_reserve_nothing_beside_the_activations(L):
+    """K at the edge of what fits beside the rings: with G = 128 the GEMV keeps no zeros behind x, which would cost the longer
+    slots at one K, the second CTA per SM at another and x its place in shared memory at a third."""
+    from paper_2507_11959_b200 import binding
+    assert binding.pot_debug_gemv_plan(1024, 4736, 3, 128)["units_per_slot"] == 4
+    assert binding.pot_debug_gemv_plan(1024, 30336, 3, 128)["ctas_per_sm"] == 2
+    assert binding.pot_debug_gemv_plan(1024, 95360, 2, 128)["x_in_smem"] == 1
