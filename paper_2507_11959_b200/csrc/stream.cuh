@@ -706,7 +706,9 @@ pot_status_t launch_stream(const void* packed, const void* scales, const void* z
             if (p.unscaled) return run(stream_kernel_of<BITS, KIND, TOK, true, W, OCC, Q, DT, true>());
         if constexpr (!(POT && DT == 0 && TOK == 1))
             if (p.x_in_smem) return run(stream_kernel_of<BITS, KIND, TOK, true, W, OCC, Q, DT, false>());
-        return run(stream_kernel_of<BITS, KIND, TOK, false, W, OCC, Q, DT, false>());
+        // (x that does not fit in shared memory leaves no room for longer slots, and is never planned with two CTAs per SM)
+        if constexpr (OCC == 1 && Q == 2) return run(stream_kernel_of<BITS, KIND, TOK, false, W, OCC, Q, DT, false>());
+        else return POT_ERR_SHAPE;
     };
     if (p.q == 2) return pick(std::integral_constant<int, 2>());
     if constexpr (OCC == 1 && TOK == 1)
