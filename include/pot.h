@@ -102,6 +102,9 @@ int pot_debug_gemv_error(void);
  * in shared memory.                                                                                                  */
 pot_status_t pot_debug_gemv_plan(int64_t N, int64_t K, int bits, int group, int uniform, int* ctas_per_sm,
                                  int* row_block_split, int* ring_slots, int* units_per_slot, int* x_in_smem);
+/* Host arithmetic only: the number of CTAs (one cluster) that share a tile's K range where codes are canonical, if
+ * resident[0 .. 5] clusters of 8, 6, 5, 4, 3 and 2 CTAs fit on the GPU at once; 0 on invalid arguments.               */
+int pot_debug_canonical_splits(int64_t tiles, int64_t K, const int* resident);
 int pot_debug_gemm_error(void);
 int pot_debug_prefill_error(void);
 

@@ -22,6 +22,7 @@ pot_status_t gemm_prefill_launch(const void* packed, const void* scales, int64_t
                                  const void* X, int64_t M, void* Y, void* workspace, size_t ws_bytes, cudaStream_t s, int dt);
 size_t gemm_prefill_workspace(int64_t M, int64_t N, int64_t K, int bits, int group);
 bool gemm_prefill_supported(int64_t M, int64_t N, int64_t K, int bits, int group);
+int canonical_splits(int64_t tiles, int64_t K, const int (&resident)[6]);
 pot_status_t gemm_canonical_launch(const void* packed, const void* scales, int64_t N, int64_t K, int bits, int group,
                                    const void* X, int64_t M, void* Y, cudaStream_t s, int dt);
 pot_status_t gemv_canonical_launch(const void* packed, const void* scales, int64_t N, int64_t K, int bits, int group, const void* x,
@@ -56,6 +57,14 @@ extern "C" size_t pot_gemm_workspace_bytes(int64_t M, int64_t N, int64_t K, int 
         return tok8 > tok1 ? tok8 : tok1;
     }
     return gemm_prefill_workspace(M, N, K, bits, group);
+}
+
+// Host arithmetic only: into how many CTAs of a cluster a tile of a canonical product is cut, where `resident` clusters of 8,
+// 6, 5, 4, 3 and 2 CTAs are resident at once.
+extern "C" int pot_debug_canonical_splits(int64_t tiles, int64_t K, const int* resident) {
+    if (!resident || tiles <= 0 || K <= 0) return 0;
+    const int r[6] = {resident[0], resident[1], resident[2], resident[3], resident[4], resident[5]};
+    return canonical_splits(tiles, K, r);
 }
 
 template <int DT>

@@ -970,14 +970,45 @@ static bool encode_x_map(CUtensorMap* xmap, const void* X, int64_t M, int64_t K,
 
 // Canonical codes: one CTA per tile, or a cluster of up to 8 CTAs that share a tile's K range while the tiles leave SMs idle
 // (at least four column blocks per CTA).  The largest cluster size with which all tiles are resident at once is taken: a
-// cluster lives inside one GPC, so that fewer CTAs fit the larger it is (cudaOccupancyMaxActiveClusters on a B200 with one CTA
-// per SM: 148, 74, 45, 33, 26, 22, 15 clusters of 1, 2, 3, 4, 5, 6, 8); a second wave of clusters costs more than the idle
-// SMs (37 tiles, 128 tokens, K = 8192: 40 us with clusters of 4).
-static int canonical_splits(int64_t tiles, int64_t K) {
-    constexpr int kSizes[] = {8, 6, 5, 4, 3, 2}, kResident[] = {15, 22, 26, 33, 45, 74};
+// cluster lives inside one GPC, so that fewer CTAs fit the larger it is, and how many depends on which SMs of which GPC a
+// chip has (one CTA per SM, on the B200s that this was measured on: 148, 74, 45, 33, 26, 22, 15 clusters of 1, 2, 3, 4, 5, 6, 8); a
+// second wave of clusters costs more than the idle SMs (37 tiles, 128 tokens, K = 8192: 40 us with clusters of 4, 24.5 us with 3).
+constexpr int kClusterSizes[] = {8, 6, 5, 4, 3, 2};
+int canonical_splits(int64_t tiles, int64_t K, const int (&resident)[6]) {
     for (int i = 0; i < 6; ++i)
-        if (tiles <= kResident[i] && K / 128 >= 4 * kSizes[i]) return kSizes[i];
+        if (tiles <= resident[i] && K / 128 >= 4 * kClusterSizes[i]) return kClusterSizes[i];
     return 1;
+}
+// How many clusters of each size are resident at once, asked of the runtime once per device.  All kernels on canonical
+// codes take an SM per CTA (512 threads, more than 64 registers), so that one answer holds for all of them.
+static bool resident_clusters(const void* kernel, dim3 block, size_t smem, int (&resident)[6]) {
+    constexpr int kDevices = 64;
+    static std::atomic<uint64_t> answers[kDevices];  // eight bits per size, the top byte marks an answer
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    uint64_t a = dev < kDevices ? answers[dev].load(std::memory_order_relaxed) : 0;
+    if (a == 0) {
+        if (!allow_max_dynamic_smem(kernel)) return false;
+        for (int i = 0; i < 6; ++i) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3((unsigned)kClusterSizes[i]);
+            cfg.blockDim = block;
+            cfg.dynamicSmemBytes = smem;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = (unsigned)kClusterSizes[i];
+            attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            int n = 0;
+            if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) return false;
+            a |= (uint64_t)(n < 255 ? n : 255) << (8 * i);
+        }
+        a |= uint64_t(1) << 56;
+        if (dev < kDevices) answers[dev].store(a, std::memory_order_relaxed);
+    }
+    for (int i = 0; i < 6; ++i) resident[i] = (int)(a >> (8 * i) & 0xFF);
+    return true;
 }
 pot_status_t gemm_canonical_launch(const void* packed, const void* scales, int64_t N, int64_t K, int bits, int group,
                                    const void* X, int64_t M, void* Y, cudaStream_t s, int dt) {
@@ -985,12 +1016,15 @@ pot_status_t gemm_canonical_launch(const void* packed, const void* scales, int64
     const int64_t tiles_m = (M + 2 * PF_BM - 1) / (2 * PF_BM);
     const int64_t tiles = tiles_m * ((N + PF_BN - 1) / PF_BN);
     if (tiles > 0x7fffffff / 8) return POT_ERR_SHAPE;
-    const int splits = canonical_splits(tiles, K);
     const int h = even_h(M, tiles_m);
     CUtensorMap xmap;
     if (!encode_x_map(&xmap, X, M, K, h)) return POT_ERR_CUDA;
     auto run = [&](auto kernel, size_t smem) -> pot_status_t {
-        return launch_pdl_cluster(kernel, dim3((unsigned)(tiles * splits)), dim3((unsigned)pf_threads(3, 2)), smem, splits, true, s, xmap,
+        const dim3 block((unsigned)pf_threads(3, 2));
+        int resident[6];
+        if (!resident_clusters((const void*)kernel, block, smem, resident)) return POT_ERR_CUDA;
+        const int splits = canonical_splits(tiles, K, resident);
+        return launch_pdl_cluster(kernel, dim3((unsigned)(tiles * splits)), block, smem, splits, true, s, xmap,
                                   (const uint4*)packed, (const uint16_t*)scales, N, K, group, M, (uint16_t*)Y, (float*)nullptr,
                                   (unsigned*)nullptr, (int)tiles_m, (int)(splits > 1 ? 0 : tiles), splits, h, prefill_error_ptr());
     };

@@ -126,3 +126,13 @@ def test_units_of_one_group_reserve_nothing_beside_the_activations(L):
     assert binding.pot_debug_gemv_plan(1024, 4736, 3, 128)["units_per_slot"] == 4
     assert binding.pot_debug_gemv_plan(1024, 30336, 3, 128)["ctas_per_sm"] == 2
     assert binding.pot_debug_gemv_plan(1024, 95360, 2, 128)["x_in_smem"] == 1
+
+
+def test_canonical_tiles_are_cut_into_clusters_that_are_resident_at_once(L):
+    """How many clusters fit depends on the chip's GPCs: a tile more than that takes the next smaller cluster."""
+    from paper_2507_11959_b200 import binding
+    usual, fewer = [15, 22, 26, 33, 45, 74], [12, 18, 24, 32, 44, 72]
+    splits = lambda tiles, K, r: binding.pot_debug_canonical_splits(tiles, K, r)
+    assert [splits(t, 11008, usual) for t in (1, 15, 16, 22, 23, 26, 27, 33, 34, 45, 46, 74, 75, 5000)] == [8, 8, 6, 6, 5, 5, 4, 4, 3, 3, 2, 2, 1, 1]
+    assert [splits(t, 11008, fewer) for t in (12, 13, 32, 33, 73)] == [8, 6, 4, 3, 1]
+    assert [splits(1, K, usual) for K in (128, 896, 1024, 1536, 2048, 2560, 3072, 4096)] == [1, 1, 2, 3, 4, 5, 6, 8]  # four column blocks per CTA
