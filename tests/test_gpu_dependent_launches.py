@@ -161,3 +161,61 @@ def test_weights_written_just_before_the_tcgen05_gemm_are_complete(oracle, M):
         Y, _, _ = run(Ws[r], False)
         assert torch.equal(Y, ref[r][0]), (it, r)
     assert B.pot_debug_errors() == (0, 0, 0)
+
+
+@pytest.mark.parametrize("dt", [torch.float16, torch.bfloat16])
+def test_canonical_products_behind_one_another_follow_their_inputs(oracle, dt):
+    """The canonical kernels release their dependents early, and the GEMM fetches codes ahead of its wait: quantize -> products
+    of 1, 16 and 200 tokens, each reading what the one before it wrote, nothing synchronised, new weights and inputs every
+    time -- eagerly, and replayed from a graph -- against the same sequence run step by step."""
+    bits, G, K, R = 3, 128, 2048, 6
+    Ws = [f16_dev(synth.weights(synth.rng_for(8, 510 + r), K, K, "normal")) for r in range(R)]
+    Xs = [f16_dev(synth.activations(synth.rng_for(8, 520 + r), 200, K)).to(dt) for r in range(R)]
+    W, X = torch.empty_like(Ws[0]), torch.empty_like(Xs[0])
+    bufs = [torch.empty((m, K), dtype=dt, device=DEV) for m in (200, 16, 1, 1, 16, 200)]
+
+    def chain(sync):
+        packed, S = B.pot_quantize_ref(W, bits, G, B.SCALE_TOP)
+        cur = X
+        for Y in bufs:
+            if sync:
+                torch.cuda.synchronize()
+            m = Y.shape[0]
+            src = cur if cur.shape[0] >= m else cur.repeat((m + cur.shape[0] - 1) // cur.shape[0], 1)
+            B.pot_gemm(packed, S, K, bits, G, src[:m], B.CANONICAL, Y=Y)
+            cur = Y
+        return packed, S
+
+    ref = []
+    for r in range(R):
+        W.copy_(Ws[r])
+        X.copy_(Xs[r])
+        packed, S = chain(True)
+        torch.cuda.synchronize()
+        ref.append([y.clone() for y in bufs])
+        if r == 0:
+            bf16 = dt == torch.bfloat16
+            Yo, A = oracle.matmul(packed.cpu().numpy(), bits_of(S), K, bits, G, bits_of(X), dtype=oracle.BF16 if bf16 else oracle.F16)
+            ok, worst, tight = gate(bits_of(ref[0][0]), Yo, A, bf16=bf16)
+            assert ok and tight < 4.0, (worst, tight)
+    assert not torch.equal(ref[0][5], ref[1][5])
+    for it in range(4 * R):
+        r = (5 * it) % R
+        W.copy_(Ws[r])
+        X.copy_(Xs[r])
+        chain(False)
+        assert all(torch.equal(a, b) for a, b in zip(bufs, ref[r])), (it, r)
+    st = torch.cuda.Stream()
+    st.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(st):
+        gr = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(gr, stream=st):
+            chain(False)
+        for it in range(2 * R):
+            r = (5 * it + 1) % R
+            W.copy_(Ws[r])
+            X.copy_(Xs[r])
+            gr.replay()
+            st.synchronize()
+            assert all(torch.equal(a, b) for a, b in zip(bufs, ref[r])), ("graph", it, r)
+    assert B.pot_debug_errors() == (0, 0, 0)
