@@ -102,6 +102,13 @@ int pot_debug_gemv_error(void);
  * in shared memory.                                                                                                  */
 pot_status_t pot_debug_gemv_plan(int64_t N, int64_t K, int bits, int group, int uniform, int* ctas_per_sm,
                                  int* row_block_split, int* ring_slots, int* units_per_slot, int* x_in_smem);
+/* Host arithmetic only: how pot_gemm (bf16 = 0) / pot_gemm_bf16 (bf16 = 1) would run M tokens on a tiled shape: on the
+ * streaming kernel (streaming = 1, the others 0), or on the tcgen05 kernel with output tiles of 128 rows x tile_tokens
+ * tokens, ring_stages stages of stage_columns columns of K, producer_groups groups of four decoding warps, and
+ * split_tiles of its `tiles` tiles cut along K into `splits` work items each.                                         */
+pot_status_t pot_debug_gemm_plan(int64_t M, int64_t N, int64_t K, int bits, int group, int bf16, int* streaming,
+                                 int* tile_tokens, int* ring_stages, int* stage_columns, int* producer_groups,
+                                 int* tiles, int* split_tiles, int* splits);
 /* Host arithmetic only: the number of CTAs (one cluster) that share a tile's K range where codes are canonical, if
  * resident[0 .. 5] clusters of 8, 6, 5, 4, 3 and 2 CTAs fit on the GPU at once; 0 on invalid arguments.               */
 int pot_debug_canonical_splits(int64_t tiles, int64_t K, const int* resident);

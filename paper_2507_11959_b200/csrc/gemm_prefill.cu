@@ -903,6 +903,37 @@ static bool prefill_wide_stages_allowed() {
     return !(e && strcmp(e, "tmem-narrow") == 0);
 }
 
+// The instantiation that a launch takes.
+struct PrefillVariant { bool in_tmem; int stages, stage_columns, groups; };
+static PrefillVariant prefill_variant(const PrefillPlan& pl, int64_t M, int dt) {
+    const bool tmem = prefill_weight_tile_in_tmem();
+    // one token tile, three producer groups, six stages of a whole 128-column block with the weight ring in tensor memory
+    // (four groups, eight 24 KB stages with the tile in shared memory)
+    if (M <= PF_SMALL_TOKENS) return tmem ? PrefillVariant{true, 6, 128, 3} : PrefillVariant{false, 8, 64, 4};
+    if (!tmem) return {false, 4, 64, 4};
+    // Two producer groups keep up with the tensor pipe; BF16, whose decode takes longer, needs more (11024 x 4096 at 4 bits: 1024 tokens
+    // 80 -> 69 us, 2048 tokens 151 -> 141 us with three).
+    // more than 256 tokens per tile: four stages, paced by the tensor pipe (4 h cycles per stage) whatever the matrix
+    if (pl.h > PF_BM) return {true, 4, 64, dt == 1 ? 4 : 2};
+    // A single wave of CTAs (65 .. 256 tokens on decode-sized matrices) is paced by the stage visits, not by the tensor
+    // pipe: three stages of a whole 128-column block (64 KB of X, 64 columns of weights, three producer groups), as in the
+    // one-tile kernel (15360 x 5120 at 65 .. 128 tokens: 27.5 - 28.5 -> 22.2 - 23.1 us).
+    if (pl.n_full + (int64_t)pl.n_tail * pl.splits <= kSmCount && prefill_wide_stages_allowed()) return {true, 3, 128, 3};
+    return {true, 6, 64, dt == 1 ? 3 : 2};  // 32 KB of X per stage
+}
+void gemm_prefill_plan_query(int64_t M, int64_t N, int64_t K, int dt, int* tile_tokens, int* ring_stages, int* stage_columns, int* producer_groups,
+                             int* tiles, int* split_tiles, int* splits) {
+    const PrefillPlan pl = prefill_plan(M, N, K);
+    const PrefillVariant v = prefill_variant(pl, M, dt);
+    *tile_tokens = M <= PF_SMALL_TOKENS ? PF_SMALL_TOKENS : 2 * pl.h;
+    *ring_stages = v.stages;
+    *stage_columns = v.stage_columns;
+    *producer_groups = v.groups;
+    *tiles = pl.tiles;
+    *split_tiles = pl.n_tail;
+    *splits = pl.splits;
+}
+
 // f(integral_constant<bits>, integral_constant<0: FP16, 1: BF16>)
 template <typename F>
 static pot_status_t with_bits_and_type(int bits, int dt, F f) {
@@ -927,30 +958,19 @@ pot_status_t gemm_prefill_launch(const void* packed, const void* scales, int64_t
                                   (const uint16_t*)scales, N, K, group, M, (uint16_t*)Y, partial, counters, pl.tiles_m, pl.n_full,
                                   pl.splits, pl.h, prefill_error_ptr());
     };
-    const bool tmem = prefill_weight_tile_in_tmem();
-    const bool one_wave = grid.x <= (unsigned)kSmCount && prefill_wide_stages_allowed();
+    const PrefillVariant v = prefill_variant(pl, M, dt);
     // two issuers, one CTA per SM
     return with_bits_and_type(bits, dt, [&](auto b, auto d) -> pot_status_t {
         constexpr int B = decltype(b)::value, D = decltype(d)::value;
         if (M <= PF_SMALL_TOKENS) {
-            // one token tile, three producer groups, six stages of a whole 128-column block with the weight ring in tensor memory
-            // (four groups, eight 24 KB stages with the tile in shared memory)
-            if (tmem) return run(pot_gemm_prefill_kernel<B, 6, 3, 2, 1, D, 1>, 3, pf_smem_bytes(6, 1, 1));
+            if (v.in_tmem) return run(pot_gemm_prefill_kernel<B, 6, 3, 2, 1, D, 1>, 3, pf_smem_bytes(6, 1, 1));
             return run(pot_gemm_prefill_kernel<B, 8, 4, 2, 1, D>, 4, pf_smem_bytes(8, 1));
         }
-        if (!tmem) return run(pot_gemm_prefill_kernel<B, 4, 4, 2, 2, D>, 4, pf_smem_bytes(4, 2));
-        // Two producer groups keep up with the tensor pipe; BF16, whose decode takes longer, needs more (11024 x 4096 at 4 bits: 1024 tokens
-        // 80 -> 69 us, 2048 tokens 151 -> 141 us with three).
-        if (pl.h > PF_BM) {  // more than 256 tokens per tile: four stages, paced by the tensor pipe (4 h cycles per stage) whatever the matrix
-            constexpr int NG = D == 1 ? 4 : 2;
-            return run(pot_gemm_prefill_kernel<B, 4, NG, 2, 2, D, 1>, NG, pf_smem_bytes_h(4, pl.h, 1));
-        }
-        // A single wave of CTAs (65 .. 256 tokens on decode-sized matrices) is paced by the stage visits, not by the tensor
-        // pipe: three stages of a whole 128-column block (64 KB of X, 64 columns of weights, three producer groups), as in the
-        // one-tile kernel (15360 x 5120 at 65 .. 128 tokens: 27.5 - 28.5 -> 22.2 - 23.1 us).
-        if (one_wave) return run(pot_gemm_prefill_kernel<B, 3, 3, 2, 2, D, 1, 3, 1>, 3, pf_smem_bytes_h(3, pl.h, 2));
-        constexpr int NG = D == 1 ? 3 : 2;   // six stages (32 KB of X each)
-        return run(pot_gemm_prefill_kernel<B, 6, NG, 2, 2, D, 1>, NG, pf_smem_bytes_h(6, pl.h, 1));
+        if (!v.in_tmem) return run(pot_gemm_prefill_kernel<B, 4, 4, 2, 2, D>, 4, pf_smem_bytes(4, 2));
+        constexpr int NG4 = D == 1 ? 4 : 2, NG6 = D == 1 ? 3 : 2;
+        if (v.stages == 4) return run(pot_gemm_prefill_kernel<B, 4, NG4, 2, 2, D, 1>, NG4, pf_smem_bytes_h(4, pl.h, 1));
+        if (v.stages == 3) return run(pot_gemm_prefill_kernel<B, 3, 3, 2, 2, D, 1, 3, 1>, 3, pf_smem_bytes_h(3, pl.h, 2));
+        return run(pot_gemm_prefill_kernel<B, 6, NG6, 2, 2, D, 1>, NG6, pf_smem_bytes_h(6, pl.h, 1));
     });
 }
 

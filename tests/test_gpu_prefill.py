@@ -3,7 +3,7 @@ import numpy as np
 import pytest
 
 from paper_2507_11959_b200 import synth
-from tests.gpu_util import PotCase, bf16_dev, bits_of, f16_bits_to_bf16_bits, f16_dev, gate
+from tests.gpu_util import PotCase, bf16_dev, bits_of, f16_bits_to_bf16_bits, f16_dev, gate, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -108,8 +108,9 @@ def test_prefill_config5_shape_sampled(B, oracle):
 @pytest.mark.parametrize("bits", [2, 3, 4])
 @pytest.mark.parametrize("dt", ["f16", "bf16"])
 def test_token_tiles_of_every_height(B, oracle, bits, dt):
-    """Two X tiles of h tokens, h a multiple of 16 up to 192: full, ragged and nearly empty second tiles, more than 256 tokens per
-    tile (four stages), K of one, a few and more stages than the ring has, whole tiles and tiles cut along K."""
+    """Two X tiles of h tokens on small matrices, which run a single wave of CTAs (three stages of 128 columns, h up to 128): full,
+    ragged and nearly empty second tiles, K of one, a few and more stages than the ring has, whole tiles and tiles cut along K.
+    The last two run more than 256 tokens per tile on a K of a few stages; test_tiles_of_large_launches runs the rest."""
     G = 128
     for i, (M, N, K) in enumerate([(130, 48, 128), (161, 144, 640), (177, 128, 1152), (225, 272, 384), (257, 16, 128), (273, 400, 256), (289, 144, 1152),
                                    (305, 272, 2048), (321, 128, 640), (350, 144, 384), (384, 272, 896), (385, 48, 1152), (600, 128, 640), (750, 160, 512),
@@ -166,3 +167,40 @@ def test_canonical_one_hot_tokens_return_dequantized_columns(B, oracle, bits, dt
         dX = bf16_dev(X) if dt == "bf16" else f16_dev(X)
         got = bits_of(B.pot_gemm(c.d_packed, f16_dev(S), K, bits, G, dX, B.CANONICAL))
         assert np.array_equal(got, deq[:, cols].T)
+
+
+# (M, N, K), the plan with FP16 activations, producer groups with BF16.  More than 256 tokens per tile run four stages of 64
+# columns; more than one wave of CTAs run six.  64 K blocks of 64 columns use the ring many times over; last token tiles are
+# ragged (whose MMAs are narrower than the tile) or one X tile short; the tail tiles of the last wave are cut along K.
+LARGE = [
+    ((301, 11024, 4096), dict(tile_tokens=320, ring_stages=4, tiles=87, split_tiles=0), 4),
+    ((700, 19200, 1152), dict(tile_tokens=352, ring_stages=4, tiles=300, split_tiles=4, splits=2), 4),
+    ((1000, 9600, 2048), dict(tile_tokens=352, ring_stages=4, tiles=225, split_tiles=0), 4),
+    ((600, 6400, 2048), dict(tile_tokens=320, ring_stages=4, tiles=100, split_tiles=0), 4),
+    ((384, 9600, 3072), dict(tile_tokens=384, ring_stages=4, tiles=75, split_tiles=0), 4),
+    ((200, 19200, 1152), dict(tile_tokens=224, ring_stages=6, tiles=150, split_tiles=2, splits=2), 3),
+    ((640, 11024, 2048), dict(tile_tokens=224, ring_stages=6, tiles=261, split_tiles=0), 3),
+]
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("dt", ["f16", "bf16"])
+def test_tiles_of_large_launches(B, oracle, bits, dt):
+    bf16 = dt == "bf16"
+    for i, ((M, N, K), want, bf16_groups) in enumerate(LARGE):
+        G = 64 if i % 2 else 128
+        plan = B.pot_debug_gemm_plan(M, N, K, bits, G, bf16)
+        assert plan["streaming"] == 0 and plan["stage_columns"] == 64 and plan["producer_groups"] == (bf16_groups if bf16 else 2), plan
+        assert all(plan[k] == v for k, v in want.items()), (M, N, K, plan)
+        c = PotCase(176, K, bits, G, dist="t5" if i % 2 else "normal", sigma=0.015, seed=(5, 1100 + 10 * bits + i))
+        row = np.random.default_rng(i).integers(0, c.N, N)      # the matrix repeats the rows of a small one in random order
+        packed, S = to_dev(c.packed[row]), f16_dev(c.S[row])
+        X = synth.activations(synth.rng_for(5, 1200 + i), M, K, outliers=(i % 2 == 1))
+        if bf16:
+            X = f16_bits_to_bf16_bits(X)
+        Y, A = oracle.matmul(c.packed, c.S, K, bits, G, X, dtype=oracle.BF16 if bf16 else oracle.F16)
+        dX = bf16_dev(X) if bf16 else f16_dev(X)
+        y = bits_of(B.pot_gemm(B.pot_repack(packed, K, bits, 0), B.pot_repack_scales(S, K, G, 0), K, bits, G, dX, B.TILED))
+        assert B.pot_debug_errors() == (0, 0, 0)
+        ok, worst, tight = gate(y, Y[:, row], A[:, row], bf16=bf16)
+        assert ok and tight < 4.0, (M, N, K, worst, tight)
