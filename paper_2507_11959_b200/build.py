@@ -33,8 +33,8 @@ def _deps_mtime() -> float:
 
 
 def build(force: bool = False, verbose: bool = False, checked: bool = False) -> Path:
-    """Build the library; checked=True builds the variant whose kernels verify their indices before every store,
-    atomic and streamed shared-memory read and report a violation through the error words instead of accessing."""
+    """Build the library; checked=True builds the variant whose GEMV and GEMM kernels verify their indices before stores,
+    atomics and shape-dependent shared-memory accesses and report a violation through the error words instead of accessing."""
     LIB = LIB_CHECKED if checked else globals()["LIB"]
     OBJ_DIR = HERE / ("build_checked" if checked else "build")
     sources = [s for s in SOURCES if (CSRC / s).exists()]

@@ -109,8 +109,8 @@ __device__ __forceinline__ uint32_t signed_exponent(uint32_t c, int ebit) {
     return e | s;
 }
 
-// Checked build (-DPOT_CHECKED): device-side index checks in front of stores, atomics and the streaming kernels'
-// shared-memory reads.  A failed check records `code` in the kernel family's error word (first failure wins) and the
+// Checked build (-DPOT_CHECKED): device-side index checks in the GEMV and GEMM kernels, in front of stores to global memory,
+// atomics, and the shared-memory offsets that depend on the shape.  A failed check records `code` in the kernel family's error word (first failure wins) and the
 // access is skipped; nothing traps.  In the normal build the checks compile to nothing.
 #ifdef POT_CHECKED
 __device__ __forceinline__ bool in_range(bool ok, int* err, int code) {
@@ -120,6 +120,11 @@ __device__ __forceinline__ bool in_range(bool ok, int* err, int code) {
 #else
 __device__ __forceinline__ bool in_range(bool, int*, int) { return true; }
 #endif
+__device__ __forceinline__ uint32_t dynamic_smem_bytes() {
+    uint32_t n;
+    asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(n));
+    return n;
+}
 
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // 16-byte load of data that the previous kernel in the stream may have written (activations, mostly).  Such data is

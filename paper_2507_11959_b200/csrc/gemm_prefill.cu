@@ -669,6 +669,7 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
                 for (int c = part; c < nch && m0 + c * 32 < M; c += NG) {
                     uint32_t v[32];
                     sums(c * 32, v);
+                    if (!in_range((c + 1) * 32 * PF_BN * 4 <= PF_STAGES * STAGE_BYTES && zsplit < splits, err, 0x62)) continue;
 #pragma unroll
                     for (int g = 0; g < 4; ++g) {
                         if ((4 * c + g) % splits == zsplit) continue;
@@ -708,7 +709,7 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
                             v[i] = z == 0 ? t : v[i] + t;
                         }
                     }
-                    if (feat < N && !gave_up) {
+                    if (feat < N && !gave_up && in_range(m0 + g * 8 < M && m0 >= 0 && feat >= 0, err, 0x63)) {
                         uint16_t* dst = Y + (m0 + g * 8) * N + feat;
 #pragma unroll
                         for (int i = 0; i < 8; ++i)

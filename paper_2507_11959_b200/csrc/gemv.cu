@@ -120,7 +120,7 @@ static CanonPlan plan_canonical(int64_t N, int64_t K) {
 template <int BITS, int DT>
 __global__ void __launch_bounds__(GC_WARPS * 32, 2) gemv_canonical_mma_kernel(const uint4* __restrict__ packed, const uint16_t* __restrict__ scales,
                                                                               int64_t N, int ncb, int spg, const uint4* __restrict__ x,
-                                                                              uint16_t* __restrict__ y, int wk_shift, int cluster) {
+                                                                              uint16_t* __restrict__ y, int wk_shift, int cluster, int* __restrict__ err) {
     extern __shared__ __align__(16) unsigned char xs[];
     __shared__ float part[GC_WARPS][16];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -156,7 +156,8 @@ __global__ void __launch_bounds__(GC_WARPS * 32, 2) gemv_canonical_mma_kernel(co
 #pragma unroll
         for (int h = 0; h < 2; ++h) sc[h][hb] = __ldg(ssrc[h] + (spg == 2 ? hb : 0));
     };
-    int step = crank * WK + (warp & (WK - 1));
+    const bool fits = in_range((uint32_t)(ncb + 1) * GC_X_STRIDE <= dynamic_smem_bytes() && WK <= GC_WARPS && crank < cluster, err, 0x160);
+    int step = fits ? crank * WK + (warp & (WK - 1)) : steps;
     if (step < steps) {
         point(step);
 #pragma unroll
@@ -165,17 +166,17 @@ __global__ void __launch_bounds__(GC_WARPS * 32, 2) gemv_canonical_mma_kernel(co
         load_scales(1);
     }
     if constexpr (BITS == 2) {  // the order of canon_decode32_any
-        for (int i = threadIdx.x; i < ncb * 8; i += GC_WARPS * 32) {
+        for (int i = threadIdx.x; fits && i < ncb * 8; i += GC_WARPS * 32) {
             const uint4 a = ld_dependent16(x + 2 * i), b = ld_dependent16(x + 2 * i + 1);
             uint4* dst = reinterpret_cast<uint4*>(xs + (i >> 3) * GC_X_STRIDE + (i & 7) * 32);
             dst[0] = make_uint4(potl::prmt(a.x, a.y, 0x5410), potl::prmt(a.z, a.w, 0x5410), potl::prmt(b.x, b.y, 0x5410), potl::prmt(b.z, b.w, 0x5410));
             dst[1] = make_uint4(potl::prmt(a.x, a.y, 0x7632), potl::prmt(a.z, a.w, 0x7632), potl::prmt(b.x, b.y, 0x7632), potl::prmt(b.z, b.w, 0x7632));
         }
     } else {
-        for (int i = threadIdx.x; i < ncb * 16; i += GC_WARPS * 32)
+        for (int i = threadIdx.x; fits && i < ncb * 16; i += GC_WARPS * 32)
             *reinterpret_cast<uint4*>(xs + (i >> 4) * GC_X_STRIDE + (i & 15) * 16) = ld_dependent16(x + i);
     }
-    if (threadIdx.x < 16) *reinterpret_cast<uint4*>(xs + ncb * GC_X_STRIDE + threadIdx.x * 16) = make_uint4(0, 0, 0, 0);  // x of the block past the end
+    if (fits && threadIdx.x < 16) *reinterpret_cast<uint4*>(xs + ncb * GC_X_STRIDE + threadIdx.x * 16) = make_uint4(0, 0, 0, 0);  // x of the block past the end
     __syncthreads();
 
     float acc[2][4] = {};
@@ -238,7 +239,7 @@ __global__ void __launch_bounds__(GC_WARPS * 32, 2) gemv_canonical_mma_kernel(co
             }
         asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");  // the sums have been read
     }
-    if (first && crank == 0 && rb * 16 + lane < N) y[rb * 16 + lane] = sk_out<DT>(sum);
+    if (first && crank == 0 && rb * 16 + lane < N && in_range(fits && rb >= 0, err, 0x161)) y[rb * 16 + lane] = sk_out<DT>(sum);
 }
 
 // CTAs per SM of the streaming GEMV (16 consumer warps each).  Two: the next launch in the stream becomes resident,
@@ -277,7 +278,7 @@ static pot_status_t launch_gemv_canonical(const void* packed, const void* scales
         auto run = [&](auto kernel) -> pot_status_t {
             const size_t smem = (size_t)(K / 128 + 1) * GC_X_STRIDE;
             return launch_pdl_cluster(kernel, dim3(p.grid), dim3(GC_WARPS * 32), smem, p.cluster, smem > 46 * 1024, s, (const uint4*)packed,
-                                      (const uint16_t*)scales, N, (int)(K / 128), 128 / group, (const uint4*)x, (uint16_t*)y, p.wk_shift, p.cluster);
+                                      (const uint16_t*)scales, N, (int)(K / 128), 128 / group, (const uint4*)x, (uint16_t*)y, p.wk_shift, p.cluster, error_ptr(ERR_GEMV));
         };
         if (bits == 2) return run(gemv_canonical_mma_kernel<2, DT>);
         if (bits == 3) return run(gemv_canonical_mma_kernel<3, DT>);
