@@ -93,6 +93,21 @@ def test_uint_gemv_matches_oracle(B, oracle, bits, G):
 
 
 @pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("G", [64, 128])
+def test_uint_gemv_with_two_ctas_per_sm(B, oracle, bits, G):
+    """The builds with 64 registers per thread: row blocks shared between CTAs or not, slots of 2 and 4 units, rings that are
+    used several times over."""
+    for i, (N, K) in enumerate([(4224, 1152), (592, 8192), (11008, 4096)]):
+        assert B.pot_debug_gemv_plan(N, K, bits, G, uniform=True)["ctas_per_sm"] == 2
+        c = UintCase(N, K, bits, G, dist="t5", seed=(4, 330 + 10 * bits + i))
+        X = acts(1, K, 430 + i)
+        Y, A = oracle.uint_matmul(c.packed, c.S, c.Z, K, bits, G, X)
+        y = B.uint_gemv(c.tiled(), c.tiled_S(), c.tiled_Z(), K, bits, G, f16_dev(X[0]), B.TILED)
+        ok, worst, tight = gate(bits_of(y), Y[0], A[0])
+        assert ok and tight < 4.0, (N, K, worst, tight)
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4])
 @pytest.mark.parametrize("M", [1, 2, 3, 4, 5, 7, 8, 13, 16, 32])
 def test_pot_gemm_small_batch_matches_oracle(B, oracle, bits, M):
     """M = 1: the GEMV kernel; 2 / 3-4 / 5-8 tokens: the streaming kernel with 2 / 4 / 8 token slots (K = 11008 at 5-8
