@@ -99,16 +99,6 @@ __device__ __forceinline__ uint32_t read_bits(const uint32_t* __restrict__ p, in
     return nbits == 32 ? v : (v & ((1u << nbits) - 1u));
 }
 
-// Sec. 4.2, stage 1 on one canonical code c = sign << (n-1) | E:
-//   exponent bits by AND mask, sign moved to the top, OR  ->  [S | 0.. E] as a 6-bit word,
-//   aligned so that E sits at bit `ebit` (10 for FP16, 7 for BF16) and the sign at bit 15.
-template <int BITS>
-__device__ __forceinline__ uint32_t signed_exponent(uint32_t c, int ebit) {
-    const uint32_t e = (c & (uint32_t)qmax_of(BITS)) << ebit;
-    const uint32_t s = (c << (16 - BITS)) & 0x8000u;
-    return e | s;
-}
-
 // Checked build (-DPOT_CHECKED): device-side index checks in the GEMV and GEMM kernels, in front of stores to global memory,
 // atomics, and the shared-memory offsets that depend on the shape.  A failed check records `code` in the kernel family's error word (first failure wins) and the
 // access is skipped; nothing traps.  In the normal build the checks compile to nothing.

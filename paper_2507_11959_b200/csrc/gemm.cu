@@ -6,9 +6,9 @@
 //    to 16 is needed and a warp decodes each record exactly once, straight into the A
 //    fragment registers -- the FP16 weights never exist in shared or global memory.
 //    Because a reduction may visit K in any order, the MMA's k-slots are mapped to the four
-//    lanes' column blocks: lane (gid, tig) feeds codes 4j..4j+3 of its record (rows gid and
-//    gid+8, column block 4*chunk + tig) into k-slots {2tig, 2tig+1, 2tig+8, 2tig+9} of step j,
-//    and the B fragment reads x at the same columns.
+//    quarters of a 128-column unit: lane (gid, tig) feeds codes 4j..4j+3 of quarter tig (rows gid
+//    and gid+8) into k-slots {2tig, 2tig+1, 2tig+8, 2tig+9} of step j, and the B fragment reads x
+//    at the same columns.
 //  * canonical layout: the canonical GEMV kernel for one token, else the tcgen05 kernel of gemm_prefill.cu with producers that
 //    decode canonical codes.
 //  * otherwise, tiled layout: the tcgen05 kernel in gemm_prefill.cu.
@@ -37,8 +37,8 @@ pot_status_t gemv_stream_launch(const void* packed, const void* scales, int64_t 
 using namespace pot;
 
 // The streaming kernel (weights decoded straight into MMA fragments, one token per MMA column) serves up to 8 tokens;
-// the tcgen05 kernel's time is flat in the batch but its floor is higher.  Measured on the 13B shapes: 13 - 23 us for
-// 1 - 8 tokens on the streaming kernel, 25 - 26 us for 8 - 32 tokens on the tcgen05 kernel.
+// the tcgen05 kernel's time is flat in the batch but its floor is higher.  Measured on the 13B shapes: 12.5 - 15.9 us for
+// 2 - 8 tokens on the streaming kernel, 15.9 - 17.7 us for 9 - 32 tokens on the tcgen05 kernel.
 constexpr int64_t kSmallBatchMax = 8;
 // ... and, above four tokens, only while the eight-token activation block fits in shared memory beside the rings
 // (K <= 8192 or so): read through L2 for every unit instead, the streaming kernel loses to the tcgen05 kernel at 8
@@ -110,7 +110,7 @@ static pot_status_t gemm_impl(const void* packed, const void* scales, int64_t N,
         if (!gemm_prefill_supported(M, N, K, bits, group)) return POT_ERR_UNSUPPORTED;
         return gemm_prefill_launch(packed, scales, N, K, bits, group, X, M, Y, workspace, ws_bytes, s, DT);
     }
-    if ((M + 63) / 64 > 65535) return POT_ERR_SHAPE;
+    if ((M + 63) / 64 > 65535) return POT_ERR_SHAPE;  // (canonical codes have never taken more tokens than this)
     if (M == 1) return gemv_canonical_launch(packed, scales, N, K, bits, group, X, Y, s, DT);
     return gemm_canonical_launch(packed, scales, N, K, bits, group, X, M, Y, s, DT);
 }

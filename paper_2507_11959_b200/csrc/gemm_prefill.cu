@@ -322,13 +322,18 @@ __device__ __forceinline__ void pf_issue(uint32_t smem0, uint32_t bar0, uint32_t
 // their own accumulators, MT token tiles of 128 per CTA.  PF_STAGES is a multiple of NG and of NI: a stage buffer is
 // always filled by the same group, loaded by the same TMA thread and read by the same issuer, so every parity wait is
 // made by a thread that has itself seen the barrier's previous phase (a waiter two phases behind could not tell).
-// Instantiated as <bits, 4, 4, 2, 2> (M > 64: 256-token tiles, four 48 KB stages) and <bits, 8, 4, 2, 1> (M <= 64: one
-// tile of up to 64 tokens, eight 24 KB stages -- a stage buffer's round trip producer -> issuer -> tensor pipe ->
-// producer is ~2000 cycles whatever the tile holds, so more buffers = more stages per unit of time).
-// AT = 1 (MT = 2, NI = 2 only): the producers write the decoded weight tile into tensor memory (tcgen05.st) instead of
+// AT = 0 (diagnostic): the decoded weight tile in shared memory.  <bits, 4, 4, 2, 2> (M > 64: 256-token tiles, four 48 KB
+// stages) and <bits, 8, 4, 2, 1> (M <= 64: one tile of up to 64 tokens, eight 24 KB stages -- a stage buffer's round trip
+// producer -> issuer -> tensor pipe -> producer is ~2000 cycles whatever the tile holds, so more buffers = more stages per
+// unit of time).
+// AT = 1 (NI = 2 only): the producers write the decoded weight tile into tensor memory (tcgen05.st) instead of
 // shared memory and the MMAs take their A operand from there, which removes a third of the shared-memory traffic of a
-// stage (16 KB written + 16 KB read of 96 KB); see pf_issue_at for the issuers' division of work.  Instantiated as
-// <bits, 6, 2, 2, 2, dt, 1>: 256 accumulator columns + 6 x 32 columns of A = 448 of the 512 columns.
+// stage (16 KB written + 16 KB read of 96 KB); see pf_issue_at for the issuers' division of work.  Of the 512 columns
+//   <bits, 6, 3, 2, 1, dt, 1>           (M <= 64)           2 x 64 accumulate, 6 x 64 hold stages of 128 columns of K,
+//   <bits, 3, 3, 2, 2, dt, 1, 3, 1>     (one wave of CTAs)  2 h accumulate (h <= 128), 3 x 64 hold stages of 128 columns,
+//   <bits, 6, 2 or 3, 2, 2, dt, 1>      (more waves)        2 h accumulate (h <= 128), 6 x 32 hold stages of 64 columns,
+//   <bits, 4, 2 or 4, 2, 2, dt, 1>      (h > 128)           2 h accumulate (h <= 192), 4 x 32 hold stages of 64 columns;
+// the larger number of producer groups is that of BF16.
 // NGP of the NG groups decode, the others only take part in the epilogue (measured slower than NGP = NG = 2 -- the
 // waiting groups poll the accumulator barrier through the whole main loop -- and not instantiated).
 // CANON = 1: canonical codes and row-major scales (the 128-column stages only): a producer thread reads its row's 16 BITS

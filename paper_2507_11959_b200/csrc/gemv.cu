@@ -9,8 +9,8 @@
 //    codes per lane per step, products accumulated in FP32 with the mixed-precision FMA and reduced with warp shuffles.
 //
 // Programmatic dependent launch: weights and scales do not depend on the previous kernel in the stream, x does.
-// The kernels request their first weights before they execute griddepcontrol.wait, and touch x, y and the
-// workspace only after it.
+// The streaming kernel requests its first weights before it executes griddepcontrol.wait, and touches x, y and the
+// workspace only after it; the canonical kernels wait first.
 #include "common.cuh"
 #include "layout.cuh"
 #include "stream.cuh"
