@@ -7,9 +7,10 @@ One "step" = one decode token through the linear layers of a Llama-2-7B-shaped m
 160 fused dequant+GEMV launches over 3-bit, group-128 PoT codes (2.53 GB of codes + scales, so
 every step streams its weights from HBM: the inputs are ~20x larger than L2).  The metric is the
 achieved algorithmic GB/s (codes + scales + x + y bytes per step / step time).  The same JSON
-line carries: the 2-bit chain, the standalone dequant throughput next to the uniform-INT twin,
-the small-batch and prefill GEMM figures, the roofline fraction of the dominant kernel, the
-oracle timed on the host cores, and an end-to-end figure with activations/results in host memory.
+line carries the roofline fraction of the dominant kernel, the oracle timed on the host cores and
+an end-to-end figure with activations/results in host memory; a JSON line on stderr holds the
+2-bit chain, the standalone dequant throughput next to the uniform-INT twin, the small-batch and
+the prefill GEMM figures (--no-extras skips it).
 
 With --gpus N > 1 (launched by torch.distributed.run) every rank runs its own replica of the
 chain (the path needs no exchange step); the value is the sum over ranks / max time.
@@ -329,7 +330,9 @@ def main():
     }
 
     if rank == 0 and world == 1 and not args.no_extras:
-        out["extras"] = extras(args, B, torch, dev, stream, f16, capture, time_graph, peaks, build_chain, enqueue_chain)
+        # the per-config tables go to stderr: the one line on stdout stays short enough to be read from the end of a log
+        tables = extras(args, B, torch, dev, stream, f16, capture, time_graph, peaks, build_chain, enqueue_chain)
+        print(json.dumps({"extras": tables}), file=sys.stderr, flush=True)
         out["cpu_baseline"] = cpu_baseline()
     del layers3
     if rank == 0:
