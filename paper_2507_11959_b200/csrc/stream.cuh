@@ -151,6 +151,7 @@ struct StreamArgs {
 struct StreamArgsUnscaled : StreamArgs {
     uint32_t bias;                       // potl::POT_UNIT_BIAS
     uint32_t p2[potl::POT_UNIT_SHIFTS];  // p2[n] = 2^n
+    uint32_t zeros_at;                   // shared-memory offset of SK_ZERO_BYTES that are cleared (one group per unit: any that are free)
 };
 template <bool UNSC>
 using StreamKernelArgs = typename std::conditional<UNSC, StreamArgsUnscaled, StreamArgs>::type;
@@ -307,11 +308,12 @@ __device__ __forceinline__ void stream_body(const StreamKernelArgs<UNSC>& sa, in
         const uint4* src = reinterpret_cast<const uint4*>(sa.X);
         const int kc = (int)(sa.K / 8);  // 16-byte chunks per token
         if constexpr (UNSC && TOK == 1)
-            if (spg == 2 && threadIdx.x < SK_ZERO_BYTES / 16) *reinterpret_cast<uint4*>(smem + HDR + sa.K * 2 + threadIdx.x * 16) = make_uint4(0, 0, 0, 0);
+            if (threadIdx.x < SK_ZERO_BYTES / 16) *reinterpret_cast<uint4*>(smem + sa.zeros_at + threadIdx.x * 16) = make_uint4(0, 0, 0, 0);
         if constexpr (TOK == 1) {
             // chunk (quarter t, part j) of a unit goes to position j * 4 + t: lanes tig = 0..3 read 64 contiguous bytes
             // (four loads in flight per thread before the first store: one round trip for K <= 32 * 32 W)
-            for (int i0 = threadIdx.x; i0 < kc; i0 += 4 * W * 32) {
+            // (a bound for whole warps, here and below: 0.5 - 0.8 % of an eight-layer token in the two-CTA build)
+            for (int i0 = threadIdx.x; (i0 & ~31) < kc; i0 += 4 * W * 32) {
                 uint4 v[4];
 #pragma unroll
                 for (int p = 0; p < 4; ++p)
@@ -332,7 +334,7 @@ __device__ __forceinline__ void stream_body(const StreamKernelArgs<UNSC>& sa, in
             // token's parity, then j -- a warp loads the 256 contiguous bytes of a unit for two tokens.
             const int ts = sa.token_shift;
             const int total = kc << ts;
-            for (int e0 = threadIdx.x; e0 < total; e0 += 8 * W * 32) {  // eight loads in flight per thread
+            for (int e0 = threadIdx.x; (e0 & ~31) < total; e0 += 8 * W * 32) {  // eight loads in flight per thread
                 uint4 v[8];
 #pragma unroll
                 for (int p = 0; p < 8; ++p) {
@@ -521,8 +523,12 @@ __device__ __forceinline__ void stream_body(const StreamKernelArgs<UNSC>& sa, in
         }
     };
     // this lane's column of B (GEMV): x, or zeros if the column belongs to the other group
+    auto zeros = [&]() -> const unsigned char* {
+        if constexpr (UNSC) return smem + sa.zeros_at;
+        else return xs;
+    };
     const bool zero_column = UNSC && TOK == 1 && spg == 2 && (gid >> 2) != (tig >> 1);
-    const unsigned char* xcol = zero_column ? xs + sa.K * 2 + tig * 16 : xs + tig * 16;
+    const unsigned char* xcol = zero_column ? zeros() + tig * 16 : xs + tig * 16;
     const uint32_t xstep = zero_column ? 0u : 256u;
     auto multiply = [&](const uint32_t (&lo)[16], const uint32_t (&hi)[16], const unsigned char* param, uint32_t cbu) {
         // activations of quarter tig (of token gid): the B fragments of the eight MMAs
@@ -693,6 +699,10 @@ pot_status_t launch_stream(const void* packed, const void* scales, const void* z
     StreamArgsUnscaled args;
     static_cast<StreamArgs&>(args) = stream_args(p, packed, scales, zeros, N, K, group, X, M, Y, workspace);
     args.bias = potl::POT_UNIT_BIAS;
+    // (cleared whether needed or not: a condition in the kernel cost 0.7 % of an eight-layer token with G = 64.  With one group per
+    // unit that is the start of the slots of partial sums, which are written after the prologue's barrier)
+    args.zeros_at = group == 64 ? (uint32_t)sk_header_bytes(W, TOK) + (uint32_t)K * 2 : (uint32_t)W * 100;
+    static_assert(W * 2 * 16 * TOK * 4 >= SK_ZERO_BYTES && W * 100 % 16 == 0, "the zeros fit into the partial-sum slots");
     for (int i = 0; i < potl::POT_UNIT_SHIFTS; ++i) args.p2[i] = 1u << i;
     auto run = [&](auto kernel) -> pot_status_t {
         auto launch = [&](const auto& a) { return launch_pdl_cluster(kernel, dim3((unsigned)p.grid), dim3(W * 32), p.smem_bytes, 1, true, s, a, err); };
