@@ -1047,8 +1047,8 @@ pot_status_t gemm_canonical_launch(const void* packed, const void* scales, int64
     if (!encode_x_map(&xmap, X, M, K, h)) return POT_ERR_CUDA;
     auto run = [&](auto kernel, size_t smem) -> pot_status_t {
         const dim3 block((unsigned)pf_threads(3, 2));
-        int resident[6];
-        if (!resident_clusters((const void*)kernel, block, smem, resident)) return POT_ERR_CUDA;
+        int resident[6] = {};
+        if (!resident_clusters((const void*)kernel, block, smem, resident)) cudaGetLastError();  // no answer: one CTA per tile
         const int splits = canonical_splits(tiles, K, resident);
         return launch_pdl_cluster(kernel, dim3((unsigned)(tiles * splits)), block, smem, splits, true, s, xmap,
                                   (const uint4*)packed, (const uint16_t*)scales, N, K, group, M, (uint16_t*)Y, (float*)nullptr,
