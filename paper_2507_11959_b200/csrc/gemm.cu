@@ -42,8 +42,9 @@ using namespace pot;
 constexpr int64_t kSmallBatchMax = 8;
 // ... and, above four tokens, only while the eight-token activation block fits in shared memory beside the rings
 // (K <= 8192 or so): read through L2 for every unit instead, the streaming kernel loses to the tcgen05 kernel at 8
-// tokens (27.7 against 26.1 us at 13824 -> 5120) and still wins at 4 (20.3 against 25.8 us).  One token always takes
-// the GEMV kernel.
+// tokens.  At 2 tokens it wins wherever x is (8192 x 28672, 3 bits: 39 against 44 us, BF16 49 against 55; 5120 x 27648: 26 against
+// 31, BF16 31 against 38); at 4, with x read through L2, only BF16 at the narrower of these two does (FP16 51 against 44 and
+// 32 against 31, BF16 55 against 55 and 35 against 38).  One token always takes the GEMV kernel.
 static bool use_small(int64_t M, int64_t N, int64_t K, pot_layout_t layout, int bits = 3, int group = 128) {
     if (layout != POT_LAYOUT_TILED || M > kSmallBatchMax || N % 16 != 0) return false;
     if (M == 1) return true;
