@@ -109,8 +109,8 @@ __global__ void __launch_bounds__(QZ_THREADS) pot_quantize_kernel(const uint4* _
 // A candidate whose lower bound is above the smallest upper bound cannot be the one that the loop takes.  The loop's own
 // roundings, 131 2^-53 Q1, belong to the bounds: relative to Q1 = W2 + D, not to T = s^2 B + 2 s A, of which Q1 is several
 // times as much where an outlier lies above all levels.  D is evaluated in FP32, off by at most SEARCH_TOL32 T (7 roundings
-// of 2^-24 T; the loop's share fits into what is left, because W2 <= 6400 T for any group: T >= 2 s A >= 0.02 s0 max|w| sum|w| / max|w|
-// and s0 >= max|w| / 127).  Mostly one candidate is left; else the bounds are taken in FP64, off by SEARCH_EPS (16 T + 132 Q1), and
+// of 2^-24 T; the loop's share fits into what is left, because W2 <= 6350 T for any group: T >= 2 s A >= 0.02 s0 sum|w|,
+// s0 >= max|w| / 127 and W2 <= max|w| sum|w|).  Mostly one candidate is left; else the bounds are taken in FP64, off by SEARCH_EPS (16 T + 132 Q1), and
 // if several are left even then (equal or all but equal sums) the sequential loop decides between those: the result is that
 // of the plain loop bit for bit.
 // What bounds it: instruction issue (82 % of the issue slots, 750 instructions per group of 128 at 3 bits, two thirds of them the
