@@ -108,77 +108,96 @@ __global__ void __launch_bounds__(QZ_THREADS) pot_quantize_kernel(const uint4* _
 // the last place of the group's smallest weight), hence exact.
 // A candidate whose lower bound is above the smallest upper bound cannot be the one that the loop takes.  The loop's own
 // roundings, 131 2^-53 Q1, belong to the bounds: relative to Q1 = W2 + D, not to T = s^2 B + 2 s A, of which Q1 is several
-// times as much where an outlier lies above all levels.  D is evaluated in FP32, off by at most SEARCH_TOL32 T (7 roundings
-// of 2^-24 T; the loop's share fits into what is left, because W2 <= 6350 T for any group: T >= 2 s A >= 0.02 s0 sum|w|,
+// times as much where an outlier lies above all levels.  D is evaluated in FP32, off by at most SEARCH_TOL32 T = 15 2^-24 T (2 s A:
+// 11 roundings of 2^-24, four of them those of a 2-ulp division; D and the bound itself: one each; the loop's share fits into
+// what is left, because W2 <= 6350 T for any group: T >= 2 s A >= 0.02 s0 sum|w|,
 // s0 >= max|w| / 127 and W2 <= max|w| sum|w|).  Mostly one candidate is left; else the bounds are taken in FP64, off by SEARCH_EPS (16 T + 132 Q1), and
 // if several are left even then (equal or all but equal sums) the sequential loop decides between those: the result is that
 // of the plain loop bit for bit.
-// What bounds it: instruction issue (82 % of the issue slots, 750 instructions per group of 128 at 3 bits, two thirds of them the
-// histogram's entries and the 200 evaluations).  11008 x 4096, groups of 128 (64), 3 bits: 9184 us term by term, 280 us so;
-// 4 bits 12424 (12873), 476 (631) us; 2 bits, groups of 64: 5974, 376 us; Q1 in the FP64 bounds: 0 - 2 % more.
-constexpr float SEARCH_TOL32 = 6e-7f;
+// What bounds it: instruction issue and shared memory (about 600 instructions and 140 wavefronts, half of them the histogram's, per group
+// of 128 at 3 bits; 77 and 63 % of what the SMs take).  11008 x 4096, groups of 128 (64), us: 2 / 3 / 4 bits 205 (382), 245 (402), 440 (541).
+// With one group per warp and launch, entries above bin 200 kept in registers behind a branch, and conversions to find I_0: 226 (382),
+// 278 (445), 480 (633); term by term 9184 at 3 bits.
+constexpr float SEARCH_TOL32 = 9e-7f;
 constexpr double SEARCH_EPS = 1.1102230246251565e-16;  // 2^-53
-constexpr int SEARCH_BINS = 224;     // 7 candidates per lane; 201 .. 224 stay empty
+constexpr int SEARCH_BINS = 232;     // bin I of 0 .. 224: bin 0 counts for nothing, and nothing reads the bins above 200 by themselves
 constexpr int SEARCH_NC = 7;         // candidates per lane: i = 7 lane + 1 .. 7 lane + 7
 constexpr int SEARCH_LOW_BITS = 22;  // WIDE: A's bins are two 32-bit sums, and no bin of 128 weights x QMAX entries overflows
+enum { SEARCH_A = 0, SEARCH_B = 1, SEARCH_A_HI = 2 };
 
 __device__ __forceinline__ double search_scale(double s0, int i) { return __dmul_rn(s0, __dmul_rn(0.01, (double)i)); }
+// a / (2^QMAX - 1) rounded once, for FP16 numbers a (a quotient corrected by its exact remainder; compared with the division for all of them)
+template <int QMAX>
+__device__ __forceinline__ double search_s0(double a) {
+    constexpr double D = (double)((1 << QMAX) - 1), R = 1.0 / D;
+    const double q = a * R;
+    return fma(fma(-D, q, a), R, q);
+}
 
-// The candidates that may be the minimiser: bit c of the result stands for i = 7 lane + 1 + c.  hist: zeroed.
+// The candidates that may be the minimiser: bit c of the result stands for i = 7 lane + 1 + c.  hist: zeroed.  b, b2: the lane's
+// candidates 0.01 i and their squares, rounded once.
 // WIDE = false: 128 weights times the largest one times 2^QMAX is below 2^32 in units of the last place, so that all sums of A
 // are 32-bit numbers.
 template <int BITS, int PER, bool WIDE>
-__device__ __forceinline__ uint32_t search_candidates(const uint32_t (&h)[PER], uint32_t emin, double s0, uint32_t (&hist)[3][SEARCH_BINS], int lane) {
+__device__ __forceinline__ uint32_t search_candidates(const uint32_t (&h)[PER], uint32_t emin, float amax, double s0, const float (&b)[SEARCH_NC],
+                                                      const float (&b2)[SEARCH_NC], uint32_t (&hist)[3][SEARCH_BINS], int lane) {
     constexpr int QMAX = qmax_of(BITS), NC = SEARCH_NC;
     using Sum = typename std::conditional<WIDE, uint64_t, uint32_t>::type;
-    const float inv = __fdiv_rn(1.f, (float)(s0 * 0.014142135623730951));
-    Sum sum_a = 0;  // the parts of A and B that all candidates share: the leading terms and the entries with I_k >= 200
-    uint32_t sum_b = PER;
+    const float inv = __fdividef((float)(((1 << QMAX) - 1) / 0.014142135623730951), amax);  // 1 / (0.01 sqrt(2) s0), 3 ulp
+    const float units = __uint_as_float((152u - emin) << 23);  // one over the value of the smallest weight's last place
+    const int cap = 201 + lane * 3 / 4;  // where I_k > 200 is counted: a bin that few lanes share
+    Sum sum_a = 0;  // the leading terms
+    Sum v[PER];
+    int I0[PER];
+    float w[PER];
+    bool close = false;
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
-        const uint32_t m = h[j] & 0x7FFFu, e = m >> 10;
-        const float w = __half2float(__ushort_as_half((uint16_t)m));
-        const uint32_t v = m == 0 ? 0u : (e ? (m & 0x3FFu) | 0x400u : m);
-        const Sum vj = (Sum)v << (m == 0 ? 0u : max(e, 1u) - emin);
-        sum_a += vj;
-        const float x = w * inv, near = rintf(x);
-        int I0 = (int)x;  // (x is not an integer unless the test below is true: x is within 3 2^-24 of its value)
-        if (fabsf(x - near) < fmaf(x, 2.5e-7f, 1e-6f)) {
-            const double sc = search_scale(s0, (int)near);
-            I0 = (int)near - 1 + ((double)(w * w) > 2.0 * __dmul_rn(sc, sc) ? 1 : 0);
-        }
+        w[j] = __half2float(__ushort_as_half((uint16_t)(h[j] & 0x7FFFu)));
+        if constexpr (WIDE) v[j] = (Sum)(w[j] * units);                                          // exact
+        else v[j] = __float_as_uint(fmaf(w[j], units, 8388608.f)) - 0x4B000000u;                 // (below 2^23)
+        sum_a += v[j];
+        // the nearest integer from the last place of 2^23 + x; I_0 is right where x, 3.6e-7 of its value off, is farther than that from it
+        const float x = w[j] * inv, t = x + 8388608.f, off = x - (t - 8388608.f);
+        I0[j] = (int)(__float_as_uint(t) - 0x4B000000u) - (off < 0.f ? 1 : 0);
+        close = close || fabsf(off) < fmaf(x, 4.5e-7f, 1e-6f);
+    }
+    if (close) {
 #pragma unroll
-        for (int k = 0; k < QMAX; ++k) {
-            const int I = I0 >> k;
-            if (I >= 200) {
-                sum_a += vj << k;
-                sum_b += 3u << (2 * k);
-            } else if (I >= 1) {
-                const Sum vk = vj << k;
-                if constexpr (WIDE) {
-                    atomicAdd(&hist[0][I - 1], (uint32_t)vk & ((1u << SEARCH_LOW_BITS) - 1));
-                    const uint32_t hi = (uint32_t)(vk >> SEARCH_LOW_BITS);
-                    if (hi) atomicAdd(&hist[1][I - 1], hi);
-                } else {
-                    atomicAdd(&hist[0][I - 1], vk);
-                }
-                atomicAdd(&hist[2][I - 1], 3u << (2 * k));
+        for (int j = 0; j < PER; ++j) {
+            const float x = w[j] * inv, near = rintf(x);
+            if (fabsf(x - near) < fmaf(x, 4.5e-7f, 1e-6f)) {
+                const double sc = search_scale(s0, (int)near);
+                I0[j] = max((int)near - 1 + ((double)(w[j] * w[j]) > 2.0 * __dmul_rn(sc, sc) ? 1 : 0), 0);
             }
         }
     }
+#pragma unroll
+    for (int j = 0; j < PER; ++j)
+#pragma unroll
+        for (int k = 0; k < QMAX; ++k) {
+            const int I = min(I0[j] >> k, cap);
+            const Sum vk = v[j] << k;
+            if constexpr (WIDE) {
+                atomicAdd(&hist[SEARCH_A][I], (uint32_t)vk & ((1u << SEARCH_LOW_BITS) - 1));
+                atomicAdd(&hist[SEARCH_A_HI][I], (uint32_t)(vk >> SEARCH_LOW_BITS));
+            } else {
+                atomicAdd(&hist[SEARCH_A][I], vk);
+            }
+            atomicAdd(&hist[SEARCH_B][I], 3u << (2 * k));
+        }
     Sum base_a;
     if constexpr (WIDE) base_a = ((uint64_t)__reduce_add_sync(0xffffffffu, (uint32_t)(sum_a >> 24)) << 24) + __reduce_add_sync(0xffffffffu, (uint32_t)sum_a & 0xFFFFFFu);
     else base_a = __reduce_add_sync(0xffffffffu, sum_a);
-    sum_b = __reduce_add_sync(0xffffffffu, sum_b);
     __syncwarp();
     Sum A[NC];
     uint32_t Bc[NC];
 #pragma unroll
     for (int c = NC - 1; c >= 0; --c) {
-        const int bin = NC * lane + c;
-        A[c] = hist[0][bin];
-        if constexpr (WIDE) A[c] += (uint64_t)hist[1][bin] << SEARCH_LOW_BITS;
-        Bc[c] = hist[2][bin];
+        const int bin = NC * lane + 1 + c;
+        A[c] = hist[SEARCH_A][bin];
+        if constexpr (WIDE) A[c] += (uint64_t)hist[SEARCH_A_HI][bin] << SEARCH_LOW_BITS;
+        Bc[c] = hist[SEARCH_B][bin];
         if (c < NC - 1) {
             A[c] += A[c + 1];
             Bc[c] += Bc[c + 1];
@@ -196,168 +215,193 @@ __device__ __forceinline__ uint32_t search_candidates(const uint32_t (&h)[PER], 
         }
     }
     ta += base_a - A[0];
-    tb += sum_b - Bc[0];
+    tb += 32u * PER - Bc[0];
     // in units of s0 and of s0 times the last place: D / s0^2 = b^2 B - 2 b (unit / s0) A
-    const double unit = __longlong_as_double((long long)(1023 - 25 + (int)emin) << 52);  // value of the smallest weight's last place
-    const float two_u = (float)(2.0 * unit / s0);
-    float d[NC], tol[NC], upper = 3e38f;
+    const float two_u = inv * 0.014142135623730951f * __uint_as_float((103u + emin) << 23);  // (2 units^-1 = 2^(emin - 24))
+    float d[NC], sum[NC], upper = 3e38f;  // (b = 0 and b2 huge where i > 200)
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
-        const float b = 0.01f * (float)(NC * lane + 1 + c);
-        const float cross = b * two_u * (float)(A[c] + ta);
-        const float square = b * b * (float)(Bc[c] + tb);
-        d[c] = square - cross;
-        tol[c] = SEARCH_TOL32 * (square + cross);
-        if (NC * lane + 1 + c > 200) d[c] = 3e38f;
-        upper = fminf(upper, d[c] + tol[c]);
+        const float cross = b[c] * (two_u * (float)(A[c] + ta));
+        d[c] = fmaf(b2[c], (float)(Bc[c] + tb), -cross);
+        sum[c] = fmaf(2.f, cross, d[c]);  // square + cross
+        upper = fminf(upper, fmaf(SEARCH_TOL32, sum[c], d[c]));
     }
     for (int o = 16; o; o >>= 1) upper = fminf(upper, __shfl_xor_sync(0xffffffffu, upper, o));
     uint32_t flags = 0;
 #pragma unroll
-    for (int c = 0; c < NC; ++c) flags |= d[c] - tol[c] <= upper ? 1u << c : 0u;
-    if (__reduce_add_sync(0xffffffffu, (uint32_t)__popc(flags)) > 1u) {
+    for (int c = 0; c < NC; ++c) flags |= fmaf(-SEARCH_TOL32, sum[c], d[c]) <= upper ? 1u << c : 0u;
+    auto several = [&]() {
+        const uint32_t lanes = __ballot_sync(0xffffffffu, flags != 0);
+        return (lanes & (lanes - 1)) != 0 || __any_sync(0xffffffffu, (flags & (flags - 1)) != 0);
+    };
+    if (several()) {
         // E_k(i) <= E_k(2i) + 1, with equality for all k (candidate 2i only renames the levels: the same sums, term by term) iff
         // B(i) = 4 B(2i); the smaller one wins
         __syncwarp();
 #pragma unroll
-        for (int c = 0; c < NC; ++c) hist[0][NC * lane + c] = (flags >> c) & 1u ? Bc[c] + tb : 0u;
+        for (int c = 0; c < NC; ++c) hist[SEARCH_A][NC * lane + 1 + c] = (flags >> c) & 1u ? Bc[c] + tb : 0u;
         __syncwarp();
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
             const int i = NC * lane + 1 + c;
-            if (((flags >> c) & 1u) && (i & 1) == 0 && hist[0][i / 2 - 1] == 4u * (Bc[c] + tb)) flags &= ~(1u << c);
+            if (((flags >> c) & 1u) && (i & 1) == 0 && hist[SEARCH_A][i / 2] == 4u * (Bc[c] + tb)) flags &= ~(1u << c);
         }
-    }
-    if (__reduce_add_sync(0xffffffffu, (uint32_t)__popc(flags)) > 1u) {
-        double low[NC], up = 1e300;
-        float w2 = 0.f;
+        if (several()) {
+            const double unit = __longlong_as_double((long long)(1023 - 25 + (int)emin) << 52);  // value of the smallest weight's last place
+            double low[NC], up = 1e300;
+            float w2 = 0.f;
 #pragma unroll
-        for (int j = 0; j < PER; ++j) {
-            const float w = __half2float(__ushort_as_half((uint16_t)h[j]));
-            w2 = fmaf(w, w, w2);
-        }
-        for (int o = 16; o; o >>= 1) w2 += __shfl_xor_sync(0xffffffffu, w2, o);
-        w2 *= 1.0001f;  // (above W2, whatever the roundings of this sum)
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {
-            low[c] = 0.0;
-            if ((flags >> c) & 1u) {
-                const double sc = search_scale(s0, NC * lane + 1 + c);
-                const double cross = 2.0 * sc * ((double)(A[c] + ta) * unit), square = sc * sc * (double)(Bc[c] + tb);
-                const double D = square - cross, t = SEARCH_EPS * (16.0 * (square + cross) + 132.0 * ((double)w2 + D));
-                low[c] = D - t;
-                up = fmin(up, D + t);
+            for (int j = 0; j < PER; ++j) {
+                const float w = __half2float(__ushort_as_half((uint16_t)h[j]));
+                w2 = fmaf(w, w, w2);
             }
-        }
-        for (int o = 16; o; o >>= 1) up = fmin(up, __shfl_xor_sync(0xffffffffu, up, o));
+            for (int o = 16; o; o >>= 1) w2 += __shfl_xor_sync(0xffffffffu, w2, o);
+            w2 *= 1.0001f;  // (above W2, whatever the roundings of this sum)
 #pragma unroll
-        for (int c = 0; c < NC; ++c)
-            if (low[c] > up) flags &= ~(1u << c);
+            for (int c = 0; c < NC; ++c) {
+                low[c] = 0.0;
+                if ((flags >> c) & 1u) {
+                    const double sc = search_scale(s0, NC * lane + 1 + c);
+                    const double cross = 2.0 * sc * ((double)(A[c] + ta) * unit), square = sc * sc * (double)(Bc[c] + tb);
+                    const double D = square - cross, t = SEARCH_EPS * (16.0 * (square + cross) + 132.0 * ((double)w2 + D));
+                    low[c] = D - t;
+                    up = fmin(up, D + t);
+                }
+            }
+            for (int o = 16; o; o >>= 1) up = fmin(up, __shfl_xor_sync(0xffffffffu, up, o));
+#pragma unroll
+            for (int c = 0; c < NC; ++c)
+                if (low[c] > up) flags &= ~(1u << c);
+        }
     }
     return flags;
 }
 
+// As many CTAs as are resident at once; their warps walk the groups, so that a lane's candidates are constants and the next group's
+// weights are on their way while one is worked through.
+constexpr int SEARCH_CTAS_PER_SM = 4;
 template <int BITS, int PER>  // PER = G / 32 weights per lane
-__global__ void __launch_bounds__(256) pot_search_kernel(const uint16_t* __restrict__ W, int64_t ngroups,
-                                                         uint16_t* __restrict__ S, uint32_t* __restrict__ packed) {
+__global__ void __launch_bounds__(256, SEARCH_CTAS_PER_SM) pot_search_kernel(const uint16_t* __restrict__ W, int64_t ngroups,
+                                                                             uint16_t* __restrict__ S, uint32_t* __restrict__ packed) {
     constexpr int QMAX = qmax_of(BITS), NC = SEARCH_NC;
+    using Raw = typename std::conditional<PER == 4, uint2, uint32_t>::type;
     __shared__ __align__(16) uint32_t hist_s[8][3][SEARCH_BINS];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t gi = (int64_t)blockIdx.x * 8 + warp;
+    const int64_t step = (int64_t)gridDim.x * 8;
+    int64_t gi = (int64_t)blockIdx.x * 8 + warp;
     if (gi >= ngroups) return;
-    uint32_t h[PER];
-    if constexpr (PER == 4) {
-        const uint2 q = __ldg(reinterpret_cast<const uint2*>(W + gi * 128) + lane);
-        h[0] = q.x & 0xFFFFu; h[1] = q.x >> 16; h[2] = q.y & 0xFFFFu; h[3] = q.y >> 16;
-    } else {
-        const uint32_t q = __ldg(reinterpret_cast<const uint32_t*>(W + gi * 64) + lane);
-        h[0] = q & 0xFFFFu; h[1] = q >> 16;
+    float b[NC], b2[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+        const int i = NC * lane + 1 + c;
+        const double v = __dmul_rn(0.01, (double)i);
+        b[c] = i <= 200 ? (float)v : 0.f;
+        b2[c] = i <= 200 ? (float)(v * v) : 1e30f;
     }
-    uint4* hz = reinterpret_cast<uint4*>(&hist_s[warp][0][0]);
+    auto fetch = [&](int64_t g) { return __ldg(reinterpret_cast<const Raw*>(W + g * (32 * PER)) + lane); };
+    Raw next = fetch(gi);
+    for (; gi < ngroups; gi += step) {
+        uint32_t h[PER];
+        if constexpr (PER == 4) {
+            h[0] = next.x & 0xFFFFu; h[1] = next.x >> 16; h[2] = next.y & 0xFFFFu; h[3] = next.y >> 16;
+        } else {
+            h[0] = next & 0xFFFFu; h[1] = next >> 16;
+        }
+        if (gi + step < ngroups) next = fetch(gi + step);
+        uint32_t top = 0, low = 0xFFFFFFFFu;
 #pragma unroll
-    for (int z = 0; z < 3 * SEARCH_BINS / 4; z += 32)
-        if (z + lane < 3 * SEARCH_BINS / 4) hz[z + lane] = make_uint4(0, 0, 0, 0);
-
-    uint32_t mag = 0, top = 0, low = 0x7FFFu;
+        for (int j = 0; j < PER; ++j) {
+            const uint32_t m = h[j] & 0x7FFFu;
+            top = max(top, m);
+            low = min(low, m - 1u);  // (zeros: the largest number there is)
+        }
+        top = __reduce_max_sync(0xffffffffu, top);
+        low = __reduce_min_sync(0xffffffffu, low) + 1u;
+        uint32_t mag = top;
+        if (top > 0x7C00u) {  // a NaN does not take part
+            mag = 0;
 #pragma unroll
-    for (int j = 0; j < PER; ++j) {
-        const uint32_t m = h[j] & 0x7FFFu;
-        top = max(top, m);
-        mag = max(mag, m > 0x7C00u ? 0u : m);  // (a NaN does not take part)
-        if (m != 0) low = min(low, m);
-    }
-    mag = __reduce_max_sync(0xffffffffu, mag);
-    top = __reduce_max_sync(0xffffffffu, top);
-    low = __reduce_min_sync(0xffffffffu, low);
-    const double s0 = (double)__half2float(__ushort_as_half((uint16_t)mag)) / (double)((1 << QMAX) - 1);
-    __syncwarp();
-
-    uint32_t flags;
-    if (top == 0) flags = lane == 0 ? 1u : 0u;                                                  // all sums are zero: the first candidate
-    else if (top >= 0x7C00u) flags = lane < 28 ? 0x7Fu : (lane == 28 ? 0xFu : 0u);              // a NaN or an infinity: every candidate
-    else {
-        const uint32_t emin = max(low >> 10, 1u), emax = max(top >> 10, 1u);
-        // 2^(11 + emax - emin) in units of the last place, 2^7 weights, 2^QMAX
-        const bool wide = 11 + (emax - emin) + 7 + QMAX > 32;
-        flags = wide ? search_candidates<BITS, PER, true>(h, emin, s0, hist_s[warp], lane)
-                     : search_candidates<BITS, PER, false>(h, emin, s0, hist_s[warp], lane);
-    }
-    const unsigned who = __ballot_sync(0xffffffffu, flags != 0);
-    int best = __shfl_sync(0xffffffffu, NC * lane + __ffs(flags), who ? __ffs(who) - 1 : 0);
-    if (__reduce_add_sync(0xffffffffu, (uint32_t)__popc(flags)) != 1u) {
-        // the sequential loop over the candidates that are left
-        double qmin = 1e300;
-        best = 1;
-        for (int c = 0; c < NC; ++c) {
-            const bool mine = (flags >> c) & 1u;
-            if (!__any_sync(0xffffffffu, mine)) continue;
-            const int i = NC * lane + 1 + c;
-            const double sc = search_scale(s0, i), s2 = __dmul_rn(sc, sc);
-            double q1 = 0.0;
-            for (int src = 0; src < 32; ++src) {
+            for (int j = 0; j < PER; ++j) mag = max(mag, (h[j] & 0x7FFFu) > 0x7C00u ? 0u : h[j] & 0x7FFFu);
+            mag = __reduce_max_sync(0xffffffffu, mag);
+        }
+        const float amax = __half2float(__ushort_as_half((uint16_t)mag));
+        const double s0 = mag >= 0x7C00u ? (double)amax : search_s0<QMAX>((double)amax);
+        uint32_t flags;
+        if (top == 0) flags = lane == 0 ? 1u : 0u;                                                  // all sums are zero: the first candidate
+        else if (top >= 0x7C00u) flags = lane < 28 ? 0x7Fu : (lane == 28 ? 0xFu : 0u);              // a NaN or an infinity: every candidate
+        else {
+            const uint32_t emin = max(low >> 10, 1u), emax = max(top >> 10, 1u);
+            // 2^(11 + emax - emin) in units of the last place, at most 2^23; 2^7 weights, 2^QMAX
+            const bool wide = 11 + (emax - emin) + 7 + (QMAX > 2 ? QMAX : 2) > 32;
+            uint4* hz = reinterpret_cast<uint4*>(&hist_s[warp][0][0]);
+            static_assert(SEARCH_A < 2 && SEARCH_B < 2 && 2 * SEARCH_BINS / 4 > 96 && 2 * SEARCH_BINS / 4 <= 128 && 3 * SEARCH_BINS / 4 <= 192, "");
+            __syncwarp();
 #pragma unroll
-                for (int j = 0; j < PER; ++j) {
-                    const double wk = (double)__half2float(__ushort_as_half((uint16_t)__shfl_sync(0xffffffffu, h[j], src)));
-                    const double w2 = __dmul_rn(wk, wk);
-                    int E = 0;
+            for (int z = 0; z < 4; ++z)
+                if (z < 3 || lane + 96 < 2 * SEARCH_BINS / 4) hz[lane + 32 * z] = make_uint4(0, 0, 0, 0);
+            if (wide)
+                for (int z = lane + 96; z < 3 * SEARCH_BINS / 4; z += 32) hz[z] = make_uint4(0, 0, 0, 0);
+            __syncwarp();
+            flags = wide ? search_candidates<BITS, PER, true>(h, emin, amax, s0, b, b2, hist_s[warp], lane)
+                         : search_candidates<BITS, PER, false>(h, emin, amax, s0, b, b2, hist_s[warp], lane);
+        }
+        const unsigned who = __ballot_sync(0xffffffffu, flags != 0);
+        int best = __shfl_sync(0xffffffffu, NC * lane + __ffs(flags), who ? __ffs(who) - 1 : 0);
+        if (who == 0 || (who & (who - 1)) != 0 || __any_sync(0xffffffffu, (flags & (flags - 1)) != 0)) {
+            // the sequential loop over the candidates that are left
+            double qmin = 1e300;
+            best = 1;
+            for (int c = 0; c < NC; ++c) {
+                const bool mine = (flags >> c) & 1u;
+                if (!__any_sync(0xffffffffu, mine)) continue;
+                const int i = NC * lane + 1 + c;
+                const double sc = search_scale(s0, i), s2 = __dmul_rn(sc, sc);
+                double q1 = 0.0;
+                for (int src = 0; src < 32; ++src) {
 #pragma unroll
-                    for (int k = 0; k < QMAX; ++k) E += (w2 > __dmul_rn(s2, (double)(1 << (2 * k + 1)))) ? 1 : 0;
-                    double rec = __dmul_rn(sc, (double)(1 << E));
-                    if (wk < 0.0) rec = -rec;
-                    const double d = (sc > 0.0) ? __dsub_rn(wk, rec) : wk;
-                    q1 = __dadd_rn(q1, __dmul_rn(d, d));
+                    for (int j = 0; j < PER; ++j) {
+                        const double wk = (double)__half2float(__ushort_as_half((uint16_t)__shfl_sync(0xffffffffu, h[j], src)));
+                        const double w2 = __dmul_rn(wk, wk);
+                        int E = 0;
+#pragma unroll
+                        for (int k = 0; k < QMAX; ++k) E += (w2 > __dmul_rn(s2, (double)(1 << (2 * k + 1)))) ? 1 : 0;
+                        double rec = __dmul_rn(sc, (double)(1 << E));
+                        if (wk < 0.0) rec = -rec;
+                        const double d = (sc > 0.0) ? __dsub_rn(wk, rec) : wk;
+                        q1 = __dadd_rn(q1, __dmul_rn(d, d));
+                    }
                 }
+                if (mine && q1 < qmin) { qmin = q1; best = i; }
             }
-            if (mine && q1 < qmin) { qmin = q1; best = i; }
+            for (int o = 16; o; o >>= 1) {  // smallest Q1, ties to the smaller i
+                const double qo = __shfl_xor_sync(0xffffffffu, qmin, o);
+                const int bo = __shfl_xor_sync(0xffffffffu, best, o);
+                if (qo < qmin || (qo == qmin && bo < best)) { qmin = qo; best = bo; }
+            }
         }
-        for (int o = 16; o; o >>= 1) {  // smallest Q1, ties to the smaller i
-            const double qo = __shfl_xor_sync(0xffffffffu, qmin, o);
-            const int bo = __shfl_xor_sync(0xffffffffu, best, o);
-            if (qo < qmin || (qo == qmin && bo < best)) { qmin = qo; best = bo; }
-        }
-    }
-    const uint16_t sb = clamp_scale_bits(__half_as_ushort(__double2half(search_scale(s0, best))), BITS);
-    if (lane == 0) S[gi] = sb;
+        const uint16_t sb = clamp_scale_bits(__half_as_ushort(__double2half(search_scale(s0, best))), BITS);
+        if (lane == 0) S[gi] = sb;
 
-    // codes: PER BITS bits per lane -> 8 codes per lane group -> whole words
-    const float two_s2 = pot_two_s2(sb);
-    uint32_t bits = 0;
+        // codes: PER BITS bits per lane -> 8 codes per lane group -> whole words
+        const float two_s2 = pot_two_s2(sb);
+        uint32_t bits = 0;
 #pragma unroll
-    for (int j = 0; j < PER; ++j) bits |= pot_code<BITS>(h[j], two_s2) << (j * BITS);
-    constexpr int LANES8 = 8 / PER;  // lanes that hold 8 codes
+        for (int j = 0; j < PER; ++j) bits |= pot_code<BITS>(h[j], two_s2) << (j * BITS);
+        constexpr int LANES8 = 8 / PER;  // lanes that hold 8 codes
 #pragma unroll
-    for (int o = 1; o < LANES8; o <<= 1) {
-        const uint32_t other = __shfl_xor_sync(0xffffffffu, bits, o);
-        bits = (lane & o) ? (bits << (o * PER * BITS)) | other : bits | (other << (o * PER * BITS));
+        for (int o = 1; o < LANES8; o <<= 1) {
+            const uint32_t other = __shfl_xor_sync(0xffffffffu, bits, o);
+            bits = (lane & o) ? (bits << (o * PER * BITS)) | other : bits | (other << (o * PER * BITS));
+        }
+        constexpr int WORDS = PER * BITS;  // 32 PER codes of BITS bits
+        int piece = lane, shift = 0;
+        if constexpr (BITS == 2) piece = 2 * lane;
+        if constexpr (BITS == 3) { piece = lane / 3 * 4 + lane % 3; shift = 8 * (lane % 3); }
+        const uint32_t lo8 = __shfl_sync(0xffffffffu, bits, (piece * LANES8) & 31);
+        const uint32_t hi8 = __shfl_sync(0xffffffffu, bits, ((piece + 1) * LANES8) & 31);
+        const uint32_t word = BITS == 4 ? lo8 : (BITS == 2 ? lo8 | (hi8 << 16) : (lo8 >> shift) | (hi8 << (24 - shift)));
+        if (lane < WORDS) packed[gi * WORDS + lane] = word;
     }
-    constexpr int WORDS = PER * BITS;  // 32 PER codes of BITS bits
-    int piece = lane, shift = 0;
-    if constexpr (BITS == 2) piece = 2 * lane;
-    if constexpr (BITS == 3) { piece = lane / 3 * 4 + lane % 3; shift = 8 * (lane % 3); }
-    const uint32_t a = __shfl_sync(0xffffffffu, bits, (piece * LANES8) & 31);
-    const uint32_t b = __shfl_sync(0xffffffffu, bits, ((piece + 1) * LANES8) & 31);
-    const uint32_t word = BITS == 4 ? a : (BITS == 2 ? a | (b << 16) : (a >> shift) | (b << (24 - shift)));
-    if (lane < WORDS) packed[gi * WORDS + lane] = word;
 }
 
 // uniform twin: one warp per group; codes are staged in shared memory, then packed 32 bits at a time
@@ -461,13 +505,12 @@ __device__ __forceinline__ void permute_quarter(const uint32_t (&in)[BITS], uint
 // One thread per quarter: 8 rows x 4 quarters per warp, so that a plane of the tiled unit is written (or read) as 128
 // contiguous bytes per warp; a block covers the 16 rows of a row block in 4 neighbouring column blocks (192 contiguous bytes
 // of a canonical row at 3 bits).  Bound by HBM and the launch (a pass reads and writes BITS / 8 bytes per weight):
-// 11008 x 4096, 3 bits: 17 us, 2446 us when a thread looked every bit of a record up for each output word (back: 339 us).
+// 11008 x 4096, 3 bits: 15 us, 2446 us when a thread looked every bit of a record up for each output word (back: 339 us).
 template <int BITS, int KIND, int DIR>
 __global__ void __launch_bounds__(256) repack_kernel(const uint32_t* __restrict__ src, uint32_t* __restrict__ dst, int64_t N, int64_t K) {
-    const int64_t ncb = K / 128;
-    const int64_t cblocks = (ncb + 3) / 4;
+    const uint32_t ncb = (uint32_t)(K >> 7), cblocks = (ncb + 3) / 4;  // (32-bit divisions: 15.4 -> 14.7 us)
     const int64_t rb = blockIdx.x / cblocks;
-    const int64_t cb = (blockIdx.x - rb * cblocks) * 4 + (threadIdx.x >> 6);
+    const uint32_t cb = (blockIdx.x % cblocks) * 4 + (threadIdx.x >> 6);
     if (cb >= ncb) return;
     const int T = threadIdx.x & 3, r = (threadIdx.x >> 2) & 15;
     const int64_t canon = (rb * 16 + r) * (K * BITS / 32) + (cb * 4 + T) * BITS;
@@ -486,14 +529,16 @@ __global__ void __launch_bounds__(256) repack_kernel(const uint32_t* __restrict_
     }
 }
 
-// per-group parameters: row-major [N, K/G] <-> tiled (see scale_tiled_index); one thread per value
-__global__ void repack_scales_kernel(const uint16_t* __restrict__ src, uint16_t* __restrict__ dst, int64_t N, int64_t K,
-                                     int G, int direction) {
-    const int64_t gpr = K / G, total = N * gpr;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t ti = potl::scale_tiled_index(t / gpr, t % gpr, K, G);
-        if (direction == 0) dst[ti] = src[t];
-        else dst[t] = src[ti];
+// per-group parameters: row-major [N, K/G] <-> tiled (see scale_tiled_index).  One block per row block, whose 16 K / G values are one
+// contiguous range in both orders: indices inside it fit in 32 bits (one thread per value of the whole array, 64-bit divisions: 5.5 us for
+// 11008 x 4096, groups of 128; so 3.5 us).
+__global__ void __launch_bounds__(256) repack_scales_kernel(const uint16_t* __restrict__ src, uint16_t* __restrict__ dst, uint32_t gpr, uint32_t spg_shift, int direction) {
+    const int64_t base = (int64_t)blockIdx.x * 16 * gpr;
+    for (uint32_t e = threadIdx.x; e < 16 * gpr; e += 256) {
+        const uint32_t r = e / gpr, g = e - r * gpr;
+        const uint32_t t = (g >> spg_shift) * (16u << spg_shift) + (uint32_t)potl::scale_tile_index((int)r, (int)(g & ((1u << spg_shift) - 1)));
+        if (direction == 0) dst[base + t] = src[base + e];
+        else dst[base + e] = src[base + t];
     }
 }
 
@@ -509,9 +554,8 @@ extern "C" pot_status_t pot_repack_scales(const void* src, void* dst, int64_t N,
     if (N % 16 != 0) return POT_ERR_SHAPE;
     if (direction != 0 && direction != 1) return POT_ERR_UNSUPPORTED;
     if (!aligned16(src) || !aligned16(dst)) return POT_ERR_ALIGN;
-    const int64_t total = N * (K / group);
-    const unsigned grid = (unsigned)((total + 255) / 256 < 65535 ? (total + 255) / 256 : 65535);
-    repack_scales_kernel<<<grid, 256, 0, (cudaStream_t)stream>>>((const uint16_t*)src, (uint16_t*)dst, N, K, group, direction);
+    repack_scales_kernel<<<(unsigned)(N / 16), 256, 0, (cudaStream_t)stream>>>((const uint16_t*)src, (uint16_t*)dst, (uint32_t)(K / group),
+                                                                              group == 64 ? 1u : 0u, direction);
     return launched();
 }
 
@@ -534,8 +578,9 @@ extern "C" pot_status_t pot_quantize_ref(const void* W, int64_t N, int64_t K, in
     cudaStream_t s = (cudaStream_t)stream;
     if (rule == POT_SCALE_SEARCH) {
         const int64_t ngroups = N * (K / group);
+        const int64_t ctas = (ngroups + 7) / 8, resident = SEARCH_CTAS_PER_SM * kSmCount;
         auto run = [&](auto kernel) {
-            kernel<<<(unsigned)((ngroups + 7) / 8), 256, 0, s>>>((const uint16_t*)W, ngroups, (uint16_t*)scales, (uint32_t*)packed);
+            kernel<<<(unsigned)(ctas < resident ? ctas : resident), 256, 0, s>>>((const uint16_t*)W, ngroups, (uint16_t*)scales, (uint32_t*)packed);
         };
         if (bits == 2) group == 128 ? run(pot_search_kernel<2, 4>) : run(pot_search_kernel<2, 2>);
         else if (bits == 3) group == 128 ? run(pot_search_kernel<3, 4>) : run(pot_search_kernel<3, 2>);

@@ -199,3 +199,24 @@ def test_repack_puts_every_bit_where_the_layout_map_says(B, oracle, bits, K):
         tiled = repack(to_dev(packed), K, bits, 0)
         assert np.array_equal(tiled.cpu().numpy().view(np.uint32).ravel(), ref.ravel())
         assert np.array_equal(repack(tiled, K, bits, 1).cpu().numpy(), packed)
+
+
+@pytest.mark.parametrize("bits, G, N, K", [(2, 64, 96, 4224), (3, 128, 160, 4096), (4, 64, 75, 4096), (3, 64, 1, 64 * 2), (4, 128, 3, 128)])
+def test_scale_search_of_more_and_fewer_groups_than_warps(B, oracle, bits, G, N, K):
+    """The search's warps walk the groups: several groups per warp, a last round that is partly filled, fewer groups than warps; rows of
+    zeros, of one number, of numbers that share a candidate's thresholds and over the type's whole range next to ordinary ones."""
+    from paper_2507_11959_b200 import synth
+    W = synth.weights(synth.rng_for(3, 700 + bits), N, K, "t5", 0.02).copy()
+    rng = np.random.default_rng(bits)
+    if N > 8:
+        W[1] = 0
+        W[2, ::2] = 0
+        W[3] = 0x3C00
+        W[4] = (rng.integers(-60, 61, K) * 0.015625).astype(np.float16).view(np.uint16)
+        W[5] = rng.integers(0, 0x7C00, K).astype(np.uint16) | (rng.integers(0, 2, K) << 15).astype(np.uint16)
+        W[6] = rng.integers(0, 4, K).astype(np.uint16)
+    S_ref, _ = oracle.scale_search(W, bits, G)
+    packed, S = B.pot_quantize_ref(f16_dev(W), bits, G, B.SCALE_SEARCH)
+    assert np.array_equal(bits_of(S), S_ref)
+    codes, _ = oracle.quantize(W, bits, G, oracle.RULE_GIVEN, S_ref)
+    assert np.array_equal(packed.cpu().numpy(), oracle.pack(codes, bits))
