@@ -14,10 +14,11 @@
 // Arithmetic.  Lane (gid, tig) of a warp owns quarter tig (32 columns) of rows gid and gid + 8 of a unit: exactly its
 // share of the A fragments of eight m16n8k16 MMAs.  It decodes its 2 x 32 codes in registers to +-2^E under a constant
 // exponent and issues the MMAs against B fragments that hold the activation vector in every column (GEMV) or one token per
-// column (small batch); the group's scale multiplies the unit's FP32 sums.  (With BF16 activations, where a unit's sums mix two
-// groups -- several tokens with G = 64 --, where x does not fit in shared memory and in the uniform twin the scale goes into the
-// weights: mask, shift and integer add into its bit pattern, Sec. 4.2 of the paper.)  The FP32 accumulators stay in registers for
-// as long as the warp stays inside one row block.
+// column (small batch); the group's scale multiplies the unit's FP32 sums.  One BF16 token is staged as FP16 numbers relative to the
+// largest of each unit where that is exact, and the unit's sums are multiplied by that factor too; the units where it is not are
+// decoded to BF16.  (Where a unit's sums mix two groups -- several tokens with G = 64 --, with several BF16 tokens, on small matrices
+// with BF16, where x does not fit in shared memory and in the uniform twin the scale goes into the weights: mask, shift and integer add
+// into its bit pattern, Sec. 4.2 of the paper.)  The FP32 accumulators stay in registers for as long as the warp stays inside one row block.
 //
 // Delivery.  A warp that covered a whole row block writes Y.  Otherwise its sums go to slot (row block, position of the
 // warp among the row block's contributors) of the workspace; a per-row-block arrival counter tells the last contributor,
@@ -70,6 +71,8 @@ struct StreamPlan {
 };
 
 constexpr int SK_ZERO_BYTES = 256;  // zeros that the unscaled GEMV keeps behind the activations (two groups per unit)
+// Below this many units per warp BF16 activations are not worth making FP16 numbers of (4096 x 4096, 3.5 units, 2 bits: 4.3 -> 4.8 us; 11008 x 4096, 9.3 units: 8.6 -> 8.3).
+constexpr int64_t SK_BF16_MIN_UNITS = 6;
 
 inline StreamPlan plan_stream(int64_t N, int64_t K, int64_t M, int bits, int group, int kind, int tok, int warps, int occ = 1, int dt = 0) {
     StreamPlan p = {};
@@ -97,9 +100,9 @@ inline StreamPlan plan_stream(int64_t N, int64_t K, int64_t M, int bits, int gro
     const size_t hdr = (size_t)sk_header_bytes(warps, tok);
     // multi-token kernel: the staged block has 2, 4 or 8 token slots per 16-byte chunk position (the smallest that holds M)
     p.token_shift = tok > 1 ? (M <= 2 ? 1 : (M <= 4 ? 2 : 3)) : 0;
-    // (BF16: every BF16 number has to stay an exact operand, and FP16 codes cannot meet them in one MMA)
-    p.unscaled = kind == SK_POT && dt == 0 && (tok == 1 || group == 128);
-    const size_t xb = (((size_t)K * 2) << p.token_shift) + (p.unscaled && tok == 1 && group == 64 ? SK_ZERO_BYTES : 0);
+    p.unscaled = kind == SK_POT && (dt == 0 ? tok == 1 || group == 128 : tok == 1 && U >= SK_BF16_MIN_UNITS * GW);
+    const size_t zeros = p.unscaled && tok == 1 && group == 64 ? SK_ZERO_BYTES : 0;
+    const size_t xb = (((size_t)K * 2) << p.token_shift) + (dt == 0 ? zeros : 0);
     // slots of 4 units unless the ring could then hold only one of them next to the staged activations
     int q = SK_QMAX;
     if (hdr + xb + (size_t)warps * 2 * (size_t)sk_slot_bytes(bits, group, kind, q) > budget) q = 2;
@@ -110,7 +113,10 @@ inline StreamPlan plan_stream(int64_t N, int64_t K, int64_t M, int bits, int gro
     const size_t ring2 = (size_t)warps * 2 * slot;  // at least two slots per warp
     p.x_in_smem = hdr + xb + ring2 <= budget;
     p.unscaled = p.unscaled && p.x_in_smem;
-    p.x_bytes = p.x_in_smem ? (xb + 127) / 128 * 128 : 0;
+    // (BF16: without the scale where zeros and factors fit as well; they decide neither where x goes nor the length of the slots)
+    const size_t xf = xb + (dt == 1 ? zeros + (size_t)ncb * 4 : 0);
+    if (dt == 1 && hdr + (xf + 127) / 128 * 128 + ring2 > budget) p.unscaled = false;
+    p.x_bytes = p.x_in_smem ? ((p.unscaled ? xf : xb) + 127) / 128 * 128 : 0;
     int64_t st = (int64_t)((budget - hdr - p.x_bytes) / ((size_t)warps * slot));
     p.ring_capacity = (int)(st > 8 ? 8 : st);
     const int64_t need = (per_warp + q - 1) / q;
@@ -152,6 +158,7 @@ struct StreamArgsUnscaled : StreamArgs {
     uint32_t bias;                       // potl::POT_UNIT_BIAS
     uint32_t p2[potl::POT_UNIT_SHIFTS];  // p2[n] = 2^n
     uint32_t zeros_at;                   // shared-memory offset of SK_ZERO_BYTES that are cleared (one group per unit: any that are free)
+    uint32_t factors_at;                 // BF16: shared-memory offset of one FP32 factor per unit
 };
 template <bool UNSC>
 using StreamKernelArgs = typename std::conditional<UNSC, StreamArgsUnscaled, StreamArgs>::type;
@@ -179,10 +186,63 @@ __device__ __forceinline__ uint16_t sk_out(float v) {
 }
 __device__ __forceinline__ uint32_t sk_lds32(const unsigned char* p) { return *reinterpret_cast<const uint32_t*>(p); }
 __device__ __forceinline__ uint4 sk_lds128(const unsigned char* p) { return *reinterpret_cast<const uint4*>(p); }
+// Eight BF16 numbers -> FP16 numbers relative to the largest one of the half-warp's unit (brought to 2^15 .. 2^16: BF16's largest
+// significand stays below FP16's).  Returns the factor that undoes it, negative if one of the unit's numbers might not be exact: not
+// zero and a subnormal FP16 number or less, 2^-30 of the largest one.  All 32 lanes take part; !ok: the lane holds nothing.
+__device__ __forceinline__ float sk_normalize(uint4& v, bool ok) {
+    uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    auto bf2 = [](uint32_t b) { return *reinterpret_cast<const __nv_bfloat162*>(&b); };
+    __nv_bfloat162 top = __habs2(bf2(w[0]));
+#pragma unroll
+    for (int i = 1; i < 4; ++i) top = __hmax2(top, __habs2(bf2(w[i])));  // (the maximum of a number and a NaN is the number)
+    uint32_t m = *reinterpret_cast<const uint32_t*>(&top);
+    m = max(m & 0xFFFFu, m >> 16);
+    if (!ok || m > 0x7F80u) m = 0;
+#pragma unroll
+    for (int o = 1; o < 16; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    const uint32_t up = min(269u - max(m >> 7, 1u), 253u);  // exponent field of the inverse of the factor (253: both are normal numbers)
+    const float f = __uint_as_float(up << 23), back = __uint_as_float((254u - up) << 23);
+    uint32_t inexact = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const __half2 h = __floats2half2_rn(__uint_as_float(w[i] << 16) * f, __uint_as_float(w[i] & 0xFFFF0000u) * f);
+        inexact |= __hlt2_mask(__habs2(h), __float2half2_rn(6.103515625e-5f)) & __hne2_mask(bf2(w[i]), __float2bfloat162_rn(0.f));
+        w[i] = *reinterpret_cast<const uint32_t*>(&h);
+    }
+    v = make_uint4(w[0], w[1], w[2], w[3]);
+    const uint32_t lanes = __ballot_sync(0xffffffffu, ok && inexact != 0);
+    return (lanes & ((threadIdx.x & 16) ? 0xFFFF0000u : 0xFFFFu)) ? -back : back;
+}
 // floor(a * b / c) for a * b that may need 64 bits
 __device__ __forceinline__ uint32_t sk_muldiv(uint32_t a, uint32_t b, uint32_t c, bool fits32) {
     if (fits32) return (a * b) / c;
     return (uint32_t)(((uint64_t)a * (uint64_t)b) / (uint64_t)c);
+}
+
+// One unit the way of BF16 operands, of which all BF16 numbers are exact: the lane's codes decoded under their scales, x (null: a
+// column of zeros) as it is in global memory.  Returns the sums of rows gid and gid + 8.  Not inlined: the registers of the loop that
+// calls it are few, and it is as good as never called.
+template <int BITS>
+__device__ __noinline__ float2 sk_unit_bf16(const unsigned char* code, const unsigned char* scale, const uint4* x) {
+    const uint32_t scw = sk_lds32(scale);
+    uint32_t w[2][BITS], lo[16], hi[16];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int k = 0; k < BITS; ++k) w[h][k] = sk_lds32(code + k * 256 + h * 128);
+    const __nv_bfloat162 sc = __float22bfloat162_rn(__half22float2(*reinterpret_cast<const __half2*>(&scw)));
+    const uint32_t sb = *reinterpret_cast<const uint32_t*>(&sc);
+    potl::pot_decode32_bf16<BITS, 1>(w[0], 0, __byte_perm(sb, 0, 0x1010), lo);
+    potl::pot_decode32_bf16<BITS, 1>(w[1], 0, __byte_perm(sb, 0, 0x3232), hi);
+    float c[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        uint4 v = make_uint4(0, 0, 0, 0);
+        if (x) v = ld_dependent16(x + i);
+        sk_mma_bf16(c, lo[4 * i], hi[4 * i], lo[4 * i + 1], hi[4 * i + 1], v.x, v.y);
+        sk_mma_bf16(c, lo[4 * i + 2], hi[4 * i + 2], lo[4 * i + 3], hi[4 * i + 3], v.z, v.w);
+    }
+    return make_float2(c[0], c[2]);
 }
 
 // DT = 0: FP16 activations, weights and output; DT = 1: BF16 (PoT codes only: the scale is rounded once to BF16 and the
@@ -193,15 +253,17 @@ __device__ __forceinline__ uint32_t sk_muldiv(uint32_t a, uint32_t b, uint32_t c
 // memory), so that the next launch in the stream can become resident and fill its rings while this one still computes.
 // UNSC: the codes are decoded without their scale (pot_units32) and a unit's FP32 sums are multiplied by it.  With two groups per
 // unit (G = 64, GEMV only) columns 0-3 of B hold x of the first group's quarters and zeros for the others, columns 4-7 the
-// opposite, so that the two groups' sums come out in different lanes.  FP16 only: BF16 activations staged as FP16 numbers
-// relative to the largest of 128 columns took 29 instead of 38 us on 28672 x 8192 at 4 bits, but numbers more than 2^29 below
-// that largest one lost bits, which shows where the large terms cancel or stand under another group's small scale.
+// opposite, so that the two groups' sums come out in different lanes.  BF16: FP16 codes cannot meet BF16 numbers in one MMA, and the
+// decode to BF16 costs 41 instead of 25 logic operations per 32 codes, so that x is staged as FP16 numbers relative to the largest of
+// 128 columns -- where that is exact.  A unit where it might not be (see sk_normalize) goes the other way: its codes are decoded to BF16
+// under their scale and x comes from global memory; a launch whose x has such a unit takes no straight-line chunks.
 template <int BITS, int KIND, int TOK, bool XSMEM, int W, int OCC, int SK_Q, int DT, bool UNSC>
 __device__ __forceinline__ void stream_body(const StreamKernelArgs<UNSC>& sa, int* __restrict__ err) {
     constexpr int UB = sk_unit_bytes(BITS);
     constexpr bool UNIFORM = (KIND == SK_UINT);
     constexpr int NPARAM = UNIFORM ? 2 : 1;
-    static_assert(!UNSC || (!UNIFORM && DT == 0 && XSMEM), "the decode without the scale: PoT codes, FP16, x in shared memory");
+    static_assert(!UNSC || (!UNIFORM && XSMEM && (DT == 0 || TOK == 1)), "the decode without the scale: PoT codes, x in shared memory, BF16 one token");
+    constexpr bool FACTORS = UNSC && DT == 1;
     extern __shared__ __align__(128) unsigned char smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int gid = lane >> 2, tig = lane & 3;  // MMA fragment coordinates: rows gid and gid + 8, quarter tig
@@ -303,6 +365,9 @@ __device__ __forceinline__ void stream_body(const StreamKernelArgs<UNSC>& sa, in
     stamp(1);
     pdl_wait();  // x, Y and the workspace may belong to the previous kernel in the stream
     stamp(2);
+    float* factors = nullptr;  // BF16 without the scale: one per unit
+    if constexpr (FACTORS) factors = reinterpret_cast<float*>(smem + sa.factors_at);
+    bool inexact = false;
     if constexpr (XSMEM) {
         uint4* dst = reinterpret_cast<uint4*>(smem + HDR);
         const uint4* src = reinterpret_cast<const uint4*>(sa.X);
@@ -321,6 +386,11 @@ __device__ __forceinline__ void stream_body(const StreamKernelArgs<UNSC>& sa, in
 #pragma unroll
                 for (int p = 0; p < 4; ++p) {
                     const int i = i0 + p * W * 32;
+                    if constexpr (FACTORS) {  // lanes 0-15 and 16-31 hold one unit each
+                        const float f = sk_normalize(v[p], i < kc);
+                        inexact = inexact || (i < kc && f < 0.f);
+                        if (i < kc && (i & 15) == 0) factors[i >> 4] = f * potl::POT_UNIT_SCALE;
+                    }
                     if (i < kc) dst[(i & ~15) | ((i & 3) << 2) | ((i >> 2) & 3)] = v[p];
                 }
             }
@@ -353,7 +423,8 @@ __device__ __forceinline__ void stream_body(const StreamKernelArgs<UNSC>& sa, in
             }
         }
     }
-    __syncthreads();
+    if constexpr (FACTORS) inexact = __syncthreads_or(inexact);
+    else __syncthreads();
     stamp(3);
 
     float acc[2][4];
@@ -379,7 +450,8 @@ __device__ __forceinline__ void stream_body(const StreamKernelArgs<UNSC>& sa, in
                 }
             }
 #pragma unroll
-            for (int e = 0; e < 4; ++e) v[e] *= potl::POT_UNIT_SCALE;
+            for (int e = 0; e < 4; ++e)
+                if constexpr (!FACTORS) v[e] *= potl::POT_UNIT_SCALE;
         }
         const bool first = rbd == wst[2];
         const uint32_t expect = first ? wst[5] : (rbd == wst[3] ? wst[6] : 0u);
@@ -558,12 +630,19 @@ __device__ __forceinline__ void stream_body(const StreamKernelArgs<UNSC>& sa, in
 #pragma unroll
             for (int j = 0; j < 8; ++j) sk_mma(c, lo[2 * j], hi[2 * j], lo[2 * j + 1], hi[2 * j + 1], xq[2 * j], xq[2 * j + 1]);
             const uint32_t scw = sk_lds32(param + ((spg == 2 ? (uint32_t)(tig >> 1) * 8u : 0u) + (uint32_t)gid) * 4u);  // {row gid, row gid + 8}
-            const float2 sc = __half22float2(*reinterpret_cast<const __half2*>(&scw));
-            acc[0][0] = fmaf(c[0], sc.x, acc[0][0]);
-            acc[0][2] = fmaf(c[2], sc.y, acc[0][2]);
-            if constexpr (TOK > 1) {
-                acc[0][1] = fmaf(c[1], sc.x, acc[0][1]);
-                acc[0][3] = fmaf(c[3], sc.y, acc[0][3]);
+            float2 sc = __half22float2(*reinterpret_cast<const __half2*>(&scw));
+            if constexpr (!FACTORS) {
+                acc[0][0] = fmaf(c[0], sc.x, acc[0][0]);
+                acc[0][2] = fmaf(c[2], sc.y, acc[0][2]);
+                if constexpr (TOK > 1) {
+                    acc[0][1] = fmaf(c[1], sc.x, acc[0][1]);
+                    acc[0][3] = fmaf(c[3], sc.y, acc[0][3]);
+                }
+            } else {  // the FP16 scale rounded once to BF16; times the unit's factor last, so that no product leaves FP32's range early
+                sc = __bfloat1622float2(__float22bfloat162_rn(sc));
+                const float f = factors[cbu];
+                acc[0][0] = fmaf(c[0] * sc.x, f, acc[0][0]);
+                acc[0][2] = fmaf(c[2] * sc.y, f, acc[0][2]);
             }
             return;
         }
@@ -577,6 +656,14 @@ __device__ __forceinline__ void stream_body(const StreamKernelArgs<UNSC>& sa, in
         uint32_t lo[16], hi[16];
         decode(code, param, lo, hi);
         multiply(lo, hi, param, cbu);
+    };
+    // a unit whose activations may not be FP16 numbers times one factor (as good as never)
+    auto unit_bf16 = [&](const unsigned char* code, const unsigned char* param, uint32_t cbu) {
+        if (!unit_ok(code, param, cbu)) return;
+        const float2 v = sk_unit_bf16<BITS>(code + (uint32_t)lane * 4u, param + ((spg == 2 ? (uint32_t)(tig >> 1) * 8u : 0u) + (uint32_t)gid) * 4u,
+                                            zero_column ? nullptr : reinterpret_cast<const uint4*>(sa.X) + (int64_t)cbu * 16 + tig * 4);
+        acc[0][0] += v.x;
+        acc[0][2] += v.y;
     };
 
     // ---- main loop over this warp's chunks --------------------------------------------------------------------
@@ -600,7 +687,7 @@ __device__ __forceinline__ void stream_body(const StreamKernelArgs<UNSC>& sa, in
             return;
         }
         if (j == 0) stamp(4);
-        if (left >= (uint32_t)SK_Q && cb + (uint32_t)SK_Q <= ncb) {
+        if (left >= (uint32_t)SK_Q && cb + (uint32_t)SK_Q <= ncb && !(FACTORS && inexact)) {
             // the common case: a full chunk inside one row block, straight-line code
 #pragma unroll
             for (int i = 0; i < SK_Q; ++i) unit(code + i * UB, param + (uint32_t)i * PB, cb + (uint32_t)i);
@@ -614,7 +701,12 @@ __device__ __forceinline__ void stream_body(const StreamKernelArgs<UNSC>& sa, in
         } else {
             const uint32_t cnt = left < (uint32_t)SK_Q ? left : (uint32_t)SK_Q;
             for (uint32_t i = 0; i < cnt; ++i) {
-                unit(code, param, cb);
+                if constexpr (FACTORS) {
+                    if (inexact && factors[cb] < 0.f) unit_bf16(code, param, cb);
+                    else unit(code, param, cb);
+                } else {
+                    unit(code, param, cb);
+                }
                 code += UB;
                 param += PB;
                 if (++cb == ncb) {
@@ -704,6 +796,7 @@ pot_status_t launch_stream(const void* packed, const void* scales, const void* z
     args.zeros_at = group == 64 ? (uint32_t)sk_header_bytes(W, TOK) + (uint32_t)K * 2 : (uint32_t)W * 100;
     static_assert(W * 2 * 16 * TOK * 4 >= SK_ZERO_BYTES && W * 100 % 16 == 0, "the zeros fit into the partial-sum slots");
     for (int i = 0; i < potl::POT_UNIT_SHIFTS; ++i) args.p2[i] = 1u << i;
+    args.factors_at = (uint32_t)sk_header_bytes(W, TOK) + (uint32_t)K * 2u + (group == 64 ? SK_ZERO_BYTES : 0);
     auto run = [&](auto kernel) -> pot_status_t {
         auto launch = [&](const auto& a) { return launch_pdl_cluster(kernel, dim3((unsigned)p.grid), dim3(W * 32), p.smem_bytes, 1, true, s, a, err); };
         if constexpr (std::is_same<decltype(kernel), void (*)(StreamArgs, int*)>::value) return launch(static_cast<const StreamArgs&>(args));
@@ -712,7 +805,7 @@ pot_status_t launch_stream(const void* packed, const void* scales, const void* z
     constexpr bool POT = KIND == SK_POT;
     auto pick = [&](auto q) -> pot_status_t {  // q units per slot
         constexpr int Q = decltype(q)::value;
-        if constexpr (POT && DT == 0)
+        if constexpr (POT && (DT == 0 || TOK == 1))
             if (p.unscaled) return run(stream_kernel_of<BITS, KIND, TOK, true, W, OCC, Q, DT, true>());
         if constexpr (!(POT && DT == 0 && TOK == 1))
             if (p.x_in_smem) return run(stream_kernel_of<BITS, KIND, TOK, true, W, OCC, Q, DT, false>());

@@ -139,3 +139,38 @@ def test_bf16_activations_are_exact_operands(B, oracle, bits, G, M):
     X[:, 64:128] = 0x3F80
     Y, A = oracle.matmul(oracle.pack(codes, bits), S, K, bits, G, X, dtype=oracle.BF16)
     run(codes, S, X, Y, A)
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("G", [64, 128])
+def test_bf16_gemv_where_some_units_are_no_fp16_numbers(B, oracle, bits, G):
+    """Matrices large enough for the decode without the scale (two CTAs per SM, one, long slots), x with 128-column units that hold two
+    large numbers that cancel and small ones, 2^-50 .. 2^-150 of them (some subnormal), next to ordinary units or to zeros; at either end
+    and over whole slots.  The small numbers count in full.  (Columns 32 q .. 32 q + 3 belong to one MMA.)"""
+    for i, (N, K) in enumerate([(7104, 4096), (2400, 28672)] + ([(9472, 16384)] if bits == 4 and G == 64 else [])):
+        ncb = K // 128
+        rng = np.random.default_rng(100 * bits + G + i)
+        codes = rng.integers(0, 1 << bits, (N, K), dtype=np.uint8)
+        codes[:, 2::128] = codes[:, 0::128]
+        S = rng.integers(0x1000, 0x2400, (N, K // G), dtype=np.uint16)
+        packed = oracle.pack(codes, bits)
+        dP, dS = to_dev(packed), f16_dev(S)
+        tiled, tS = B.pot_repack(dP, K, bits, 0), B.pot_repack_scales(dS, K, G, 0)
+        rows = np.unique(np.linspace(0, N - 1, 200).astype(np.int64))
+        ordinary = f16_bits_to_bf16_bits(synth.activations(synth.rng_for(7, 1250 + i), 1, K))
+        for units, zero in (([], False), ([0], False), ([ncb - 1], True), ([1, 2, 3, 4, ncb // 2], False), ([1, 2, 3, 4, ncb // 2], True)):
+            X = np.zeros_like(ordinary) if zero else ordinary.copy()
+            for u in units:
+                unit = np.zeros(128, dtype=np.uint16)
+                at = np.array([8, 9, 31, 40, 64 + 20, 127])
+                unit[at] = (rng.integers(0, 100, at.size) << 7) | rng.integers(0, 128, at.size)
+                unit[at[u % 6]] = 99 << 7
+                X[0, 128 * u:128 * u + 128] = unit
+            Y, A = oracle.matmul(packed, S, K, bits, G, X, rows=rows, dtype=oracle.BF16)
+            for u in units:
+                X[0, 128 * u], X[0, 128 * u + 2] = 0x5880, 0xD880    # 2^50, -2^50
+            got = bits_of(B.pot_gemv(tiled, tS, K, bits, G, bf16_dev(X[0]), B.TILED))[rows]
+            val = (got.astype(np.uint32) << 16).view(np.float32).astype(np.float64)
+            # sums of FP32 products, rounded to BF16
+            assert np.all(np.abs(val - Y[0]) <= 1e-3 * A[0] + 2.0 ** -8 * np.abs(Y[0])), (N, K, units, zero)
+    assert B.pot_debug_errors() == (0, 0, 0)
