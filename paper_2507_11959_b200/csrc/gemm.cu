@@ -24,7 +24,7 @@ size_t gemm_prefill_workspace(int64_t M, int64_t N, int64_t K, int bits, int gro
 bool gemm_prefill_supported(int64_t M, int64_t N, int64_t K, int bits, int group);
 void gemm_prefill_plan_query(int64_t M, int64_t N, int64_t K, int dt, int* tile_tokens, int* ring_stages, int* stage_columns, int* producer_groups,
                              int* tiles, int* split_tiles, int* splits);
-int canonical_splits(int64_t tiles, int64_t K, const int (&resident)[6]);
+int cluster_splits(int64_t tiles, int64_t K, const int (&resident)[6]);
 pot_status_t gemm_canonical_launch(const void* packed, const void* scales, int64_t N, int64_t K, int bits, int group,
                                    const void* X, int64_t M, void* Y, cudaStream_t s, int dt);
 pot_status_t gemv_canonical_launch(const void* packed, const void* scales, int64_t N, int64_t K, int bits, int group, const void* x,
@@ -79,7 +79,7 @@ extern "C" pot_status_t pot_debug_gemm_plan(int64_t M, int64_t N, int64_t K, int
 extern "C" int pot_debug_canonical_splits(int64_t tiles, int64_t K, const int* resident) {
     if (!resident || tiles <= 0 || K <= 0) return 0;
     const int r[6] = {resident[0], resident[1], resident[2], resident[3], resident[4], resident[5]};
-    return canonical_splits(tiles, K, r);
+    return cluster_splits(tiles, K, r);
 }
 
 template <int DT>

@@ -144,9 +144,9 @@ __device__ __forceinline__ uint32_t pf_cluster_addr(uint32_t addr, uint32_t rank
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
-__device__ __forceinline__ uint32_t pf_ld_cluster(uint32_t addr) {
-    uint32_t v;
-    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+__device__ __forceinline__ uint4 pf_ld_cluster4(uint32_t addr) {
+    uint4 v;
+    asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
     return v;
 }
 __device__ __forceinline__ void pf_commit(uint32_t bar) {
@@ -173,12 +173,6 @@ __device__ __forceinline__ void pf_mma_ta(uint32_t d_tmem, uint32_t a_tmem, uint
         "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %4, p;\n\t}" ::"r"(d_tmem),
         "r"(a_tmem), "r"(blo), "r"(hi), "r"(idesc), "r"(accumulate)
         : "memory");
-}
-__device__ __forceinline__ void pf_ld8(uint32_t taddr, uint32_t (&r)[8]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(taddr)
-                 : "memory");
 }
 __device__ __forceinline__ void pf_st32(uint32_t taddr, const uint32_t (&r)[32]) {
     asm volatile(
@@ -318,6 +312,69 @@ __device__ __forceinline__ void pf_issue(uint32_t smem0, uint32_t bar0, uint32_t
     pf_commit(accum);  // this issuer's accumulators are complete once all its MMAs have finished
 }
 
+// The second half of a cluster's epilogue: warp `warp` of WARPS adds up the tokens of its CTA (rank `zsplit` of `splits`).  (Inlined.
+// As a function, out of the way of the instructions of the kernel's other routes, the call and its stack cost 2 us.)
+struct PfAddUp {
+    const float* sums;     // of the tile: [split][token][128 features]; CANON: in each CTA's shared memory instead
+    uint16_t* Y;
+    int64_t M, N, m0, n0, rows;
+    int tokens, splits, zsplit, warp;
+    bool gave_up;
+};
+template <int DT, int CANON, int WARPS, int Z, int U>  // at most Z splits, U tokens at a time
+__device__ __forceinline__ void pf_add_up_of(const PfAddUp& a, uint32_t smem, int* err) {
+    const int lane = threadIdx.x & 31;
+    const int64_t n4 = a.n0 + 4 * lane;
+    [[maybe_unused]] uint32_t src[Z];
+    [[maybe_unused]] const uint4* first = reinterpret_cast<const uint4*>(a.sums) + lane;
+    if constexpr (CANON) {
+#pragma unroll
+        for (int z = 0; z < Z; ++z) src[z] = pf_cluster_addr(smem + lane * 16, (uint32_t)(z < a.splits ? z : 0));
+    }
+    auto fetch = [&](int z, int t) {
+        if constexpr (CANON) return pf_ld_cluster4(src[z] + (uint32_t)t * (PF_BN * 4));
+        else return __ldcg(first + (z * a.rows + t) * (PF_BN / 4));
+    };
+    const int step = WARPS * a.splits;
+#pragma unroll 1
+    for (int t0 = a.warp * a.splits + a.zsplit; t0 < a.tokens; t0 += U * step) {
+        uint4 p[U][Z];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int z = 0; z < Z; ++z)
+                if (z < a.splits && t0 + u * step < a.tokens) p[u][z] = fetch(z, t0 + u * step);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t t = a.m0 + t0 + u * step;
+            if (t0 + u * step >= a.tokens || a.gave_up || n4 >= a.N || !in_range(t < a.M && a.m0 >= 0, err, 0x63)) continue;
+            float v[4] = {__uint_as_float(p[u][0].x), __uint_as_float(p[u][0].y), __uint_as_float(p[u][0].z), __uint_as_float(p[u][0].w)};
+#pragma unroll
+            for (int z = 1; z < Z; ++z) {
+                if (z >= a.splits) continue;
+                v[0] += __uint_as_float(p[u][z].x);
+                v[1] += __uint_as_float(p[u][z].y);
+                v[2] += __uint_as_float(p[u][z].z);
+                v[3] += __uint_as_float(p[u][z].w);
+            }
+            uint16_t* dst = a.Y + t * a.N + n4;
+            if (a.N % 4 == 0) {
+                *reinterpret_cast<uint2*>(dst) = make_uint2((uint32_t)pf_out<DT>(v[0]) | ((uint32_t)pf_out<DT>(v[1]) << 16),
+                                                            (uint32_t)pf_out<DT>(v[2]) | ((uint32_t)pf_out<DT>(v[3]) << 16));
+            } else {  // (canonical codes: any number of rows)
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (n4 + e < a.N) dst[e] = pf_out<DT>(v[e]);
+            }
+        }
+    }
+}
+template <int DT, int CANON, int WARPS>
+__device__ __forceinline__ void pf_add_up(const PfAddUp& a, uint32_t smem, int* err) {
+    if (a.splits <= 4) pf_add_up_of<DT, CANON, WARPS, 4, 4>(a, smem, err);
+    else pf_add_up_of<DT, CANON, WARPS, 8, 2>(a, smem, err);
+}
+
 // PF_STAGES stages, NG producer groups (K block kb is decoded by group kb % NG into stage kb % PF_STAGES), NI issuers with
 // their own accumulators, MT token tiles of 128 per CTA.  PF_STAGES is a multiple of NG and of NI: a stage buffer is
 // always filled by the same group, loaded by the same TMA thread and read by the same issuer, so every parity wait is
@@ -339,15 +396,16 @@ __device__ __forceinline__ void pf_issue(uint32_t smem0, uint32_t bar0, uint32_t
 // CANON = 1: canonical codes and row-major scales (the 128-column stages only): a producer thread reads its row's 16 BITS
 // contiguous bytes per column block and decodes them with byte look-ups (potl::CanonLut).  There is no workspace on this
 // route: the items of a tile that is cut along K are the CTAs of a thread-block cluster, which add their partial sums through
-// distributed shared memory.  200 tokens x 4099 x 11008, 3 bits: 672 us on the mma.sync kernel that this replaced, 27.3 us
-// (clusters of 4, 132 CTAs; about half of it is latency per 128-column stage with three stages in flight; 29.6 us with the 32-token
-// chunks of a tile dealt to the CTAs instead of 8-token groups, and X tiles of 128 tokens).
-template <int BITS, int PF_STAGES, int NG, int NI, int MT, int DT = 0, int AT = 0, int NGP = NG, int WIDE = 0, int CANON = 0>  // DT = 1: BF16 activations, weights and output
+// distributed shared memory.  200 tokens x 4099 x 11008, 3 bits: 672 us on the mma.sync kernel that this replaced, 26.5 us
+// (clusters of 4, 132 CTAs: the loads of codes, a cache line per row each, and 5 us to add up the sums).
+// CLUSTER = 1: the items of every tile are a cluster (canonical codes: if `clustered`).  An instantiation of its own for tiled codes: with
+// the choice made at run time, launches without clusters took 1 - 3 % longer (301 tokens x 11024 x 4096, BF16: 30.1 -> 31.1 us).
+template <int BITS, int PF_STAGES, int NG, int NI, int MT, int DT = 0, int AT = 0, int NGP = NG, int WIDE = 0, int CANON = 0, int CLUSTER = CANON>  // DT = 1: BF16 activations, weights and output
 __global__ void __launch_bounds__(pf_threads(NG, NI), 1)
 pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* __restrict__ packed,
                         const uint16_t* __restrict__ scales, int64_t N, int64_t K, int G, int64_t M,
                         uint16_t* __restrict__ Y, float* __restrict__ partial, unsigned* __restrict__ counters,
-                        int tiles_m, int n_full, int tail_splits, int tok_h, int* __restrict__ err) {
+                        int tiles_m, int n_full, int tail_splits, int clustered, int tok_h, int* __restrict__ err) {
     extern __shared__ unsigned char smem_raw[];
     // 1024-byte alignment: the swizzle atoms and the matrix descriptors assume it
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -663,68 +721,40 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
             for (int i = 0; i < 32; ++i)
                 if (m0 + col + i < M) dst[(int64_t)i * N] = pf_out<DT>(__uint_as_float(v[i]));
         };
-        if constexpr (CANON) {
-            if (splits > 1) {
-                // The items of the tile are the CTAs of this cluster.  Group g of 8 token columns belongs to CTA g % splits: every
-                // CTA leaves the other groups' sums in its own shared memory (the ring is empty: all MMAs have completed; it
-                // holds at least 512 bytes per token of the tile), and after a cluster barrier each CTA adds its groups in
-                // split order -- all peers' numbers of a group in flight at once -- and writes them.
-                float* red = reinterpret_cast<float*>(smem) + 32 * q + lane;   // [token column][128 features]
+        const bool share = CLUSTER && (!CANON || clustered);   // the tile's items are a cluster
+        if constexpr (CLUSTER) {
+            if (share) {
+                // The items of the tile are the CTAs of this cluster.  Every CTA leaves its sums, [token][128 features], where the others can
+                // read them, and after a cluster barrier CTA z adds up the tokens z, z + splits, ... in split order and writes them: a
+                // warp has the 128 features of a token, 16 bytes per lane, and the numbers of several tokens are in flight at
+                // once.  Tiled codes: in the workspace (L2: 64 bytes per clock and SM).  Canonical codes, which have none: in shared
+                // memory (the ring is empty, all MMAs have completed; it holds at least 512 bytes per token of the tile), where peers
+                // read 16 bytes per clock (a CTA's share of 256 tokens in 4 CTAs: 4.8 us, from L2 2.2 us).
+                float* const mine = CANON ? reinterpret_cast<float*>(smem) : partial + ((int64_t)tile * splits + zsplit) * rows_alloc * PF_BN;
 #pragma unroll 1
                 for (int c = part; c < nch && m0 + c * 32 < M; c += NG) {
                     uint32_t v[32];
                     sums(c * 32, v);
-                    if (!in_range((c + 1) * 32 * PF_BN * 4 <= PF_STAGES * STAGE_BYTES && zsplit < splits, err, 0x62)) continue;
+                    if (!in_range(zsplit < splits && (CANON ? (c + 1) * 32 * PF_BN * 4 <= PF_STAGES * STAGE_BYTES : partial != nullptr && n_full == 0), err, 0x62)) continue;
+                    float* dst = mine + (int64_t)c * 32 * PF_BN + 32 * q + lane;
+                    if (CANON || m0 + c * 32 + 32 <= M) {
 #pragma unroll
-                    for (int g = 0; g < 4; ++g) {
-                        if ((4 * c + g) % splits == zsplit) continue;
+                        for (int i = 0; i < 32; ++i) dst[i * PF_BN] = __uint_as_float(v[i]);
+                    } else {
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) red[(c * 32 + 8 * g + i) * PF_BN] = __uint_as_float(v[8 * g + i]);
+                        for (int i = 0; i < 32; ++i)
+                            if (m0 + c * 32 + i < M) dst[i * PF_BN] = __uint_as_float(v[i]);
                     }
                 }
                 pf_cluster_sync();
-#pragma unroll 1
-                for (int g = zsplit + splits * part; g < 4 * nch && m0 + g * 8 < M; g += splits * NG) {
-                    uint32_t p[8][8], own[8];
-                    const uint32_t mine = smem_u32(red + g * 8 * PF_BN);
-#pragma unroll
-                    for (int z = 0; z < 8; ++z) {
-                        if (z >= splits || z == zsplit) continue;
-                        const uint32_t src = pf_cluster_addr(mine, (uint32_t)z);
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) p[z][i] = pf_ld_cluster(src + (uint32_t)(i * PF_BN * 4));
-                    }
-                    pf_ld8(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(8 * g), own);
-                    if (!AT2 && nkb > 1) {
-                        uint32_t second[8];
-                        pf_ld8(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(PF_AT1_ACC_STRIDE + 8 * g), second);
-                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) own[i] = __float_as_uint(__uint_as_float(own[i]) + __uint_as_float(second[i]));
-                    } else {
-                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                    }
-                    float v[8];
-#pragma unroll
-                    for (int z = 0; z < 8; ++z) {
-                        if (z >= splits) continue;
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const float t = __uint_as_float(z == zsplit ? own[i] : p[z][i]);
-                            v[i] = z == 0 ? t : v[i] + t;
-                        }
-                    }
-                    if (feat < N && !gave_up && in_range(m0 + g * 8 < M && m0 >= 0 && feat >= 0, err, 0x63)) {
-                        uint16_t* dst = Y + (m0 + g * 8) * N + feat;
-#pragma unroll
-                        for (int i = 0; i < 8; ++i)
-                            if (m0 + g * 8 + i < M) dst[(int64_t)i * N] = pf_out<DT>(v[i]);
-                    }
-                }
+                const int64_t left = M - m0;
+                const PfAddUp a{CANON ? nullptr : partial + (int64_t)tile * splits * rows_alloc * PF_BN, Y, M, N, m0, n0, rows_alloc,
+                                MT == 1 ? (int)M : (int)(left < MT * h ? left : MT * h), splits, zsplit, pt >> 5, gave_up};
+                pf_add_up<DT, CANON, 4 * NG>(a, smem_u32(smem), err);
             }
         }
 #pragma unroll 1
-        for (int c = part; c < nch && !(CANON && splits > 1); c += NG) {
+        for (int c = part; c < nch && !share; c += NG) {
             const int col = c * 32;
             if (m0 + col >= M) break;             // (warp-uniform) no token in these columns
             uint32_t v[32];
@@ -740,7 +770,7 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
                 }
             }
         }
-        if (!CANON && splits > 1 && !gave_up && in_range(tail_index >= 0 && partial != nullptr && counters != nullptr, err, 0x61)) {
+        if (splits > 1 && !share && !gave_up && in_range(tail_index >= 0 && partial != nullptr && counters != nullptr, err, 0x61)) {
             // The CTA that delivers the last split of a tile (an arrival counter tells it) adds the splits in
             // ascending order -- the result does not depend on timing -- and writes Y.
             __shared__ unsigned s_prev;
@@ -784,10 +814,10 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
             }
         }
     }
-    if constexpr (CANON) {  // every thread of the cluster arrives at both barriers: the epilogue warps at the first one above
-        if (tail_splits > 1) {
+    if constexpr (CLUSTER) {  // every thread of the cluster arrives at the barriers: the epilogue warps at the first one above
+        if (!CANON || clustered) {
             if (warp < PROD_WARP0) pf_cluster_sync();
-            pf_cluster_sync();  // nobody leaves while its partial sums are being read
+            if constexpr (CANON) pf_cluster_sync();  // nobody leaves while its partial sums are being read
         }
     }
     // ---------------- teardown: everyone is done with tensor memory, the allocating warp frees it --------
@@ -950,63 +980,19 @@ static pot_status_t with_bits_and_type(int bits, int dt, F f) {
     return with_type(integral_constant<int, 4>());
 }
 
-pot_status_t gemm_prefill_launch(const void* packed, const void* scales, int64_t N, int64_t K, int bits, int group,
-                                 const void* X, int64_t M, void* Y, void* workspace, size_t ws_bytes, cudaStream_t s, int dt) {
-    const PrefillPlan pl = prefill_plan(M, N, K);
-    if (pl.ws_bytes > 0 && (!workspace || ws_bytes < pl.ws_bytes)) return POT_ERR_WORKSPACE;
-    unsigned* counters = (unsigned*)workspace;
-    float* partial = pl.ws_bytes > 0 ? (float*)((char*)workspace + pl.counter_bytes) : nullptr;
-    CUtensorMap xmap;
-    if (!encode_x_map(&xmap, X, M, K, pl.h)) return POT_ERR_CUDA;
-    const dim3 grid((unsigned)(pl.n_full + pl.n_tail * pl.splits));
-    auto run = [&](auto kernel, int ng, size_t smem) -> pot_status_t {
-        return launch_pdl_cluster(kernel, grid, dim3((unsigned)pf_threads(ng, 2)), smem, 1, true, s, xmap, (const uint4*)packed,
-                                  (const uint16_t*)scales, N, K, group, M, (uint16_t*)Y, partial, counters, pl.tiles_m, pl.n_full,
-                                  pl.splits, pl.h, prefill_error_ptr());
-    };
-    const PrefillVariant v = prefill_variant(pl, M, dt);
-    // two issuers, one CTA per SM
-    return with_bits_and_type(bits, dt, [&](auto b, auto d) -> pot_status_t {
-        constexpr int B = decltype(b)::value, D = decltype(d)::value;
-        if (M <= PF_SMALL_TOKENS) {
-            if (v.in_tmem) return run(pot_gemm_prefill_kernel<B, 6, 3, 2, 1, D, 1>, 3, pf_smem_bytes(6, 1, 1));
-            return run(pot_gemm_prefill_kernel<B, 8, 4, 2, 1, D>, 4, pf_smem_bytes(8, 1));
-        }
-        if (!v.in_tmem) return run(pot_gemm_prefill_kernel<B, 4, 4, 2, 2, D>, 4, pf_smem_bytes(4, 2));
-        constexpr int NG4 = D == 1 ? 4 : 2, NG6 = D == 1 ? 3 : 2;
-        if (v.stages == 4) return run(pot_gemm_prefill_kernel<B, 4, NG4, 2, 2, D, 1>, NG4, pf_smem_bytes_h(4, pl.h, 1));
-        if (v.stages == 3) return run(pot_gemm_prefill_kernel<B, 3, 3, 2, 2, D, 1, 3, 1>, 3, pf_smem_bytes_h(3, pl.h, 2));
-        return run(pot_gemm_prefill_kernel<B, 6, NG6, 2, 2, D, 1>, NG6, pf_smem_bytes_h(6, pl.h, 1));
-    });
-}
-
-static int* prefill_error_ptr() { return error_ptr(ERR_PREFILL); }
-
-static bool encode_x_map(CUtensorMap* xmap, const void* X, int64_t M, int64_t K, int h) {
-    EncodeTiledFn encode = encode_tiled_fn();
-    if (!encode) return false;
-    const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)M};
-    const cuuint64_t strides[1] = {(cuuint64_t)K * 2};
-    const cuuint32_t box[2] = {64, (cuuint32_t)(M <= PF_SMALL_TOKENS ? M : h)};  // the one-tile kernel: no padding rows
-    const cuuint32_t estr[2] = {1, 1};
-    return encode(xmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(X), dims, strides, box, estr,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// Canonical codes: one CTA per tile, or a cluster of up to 8 CTAs that share a tile's K range while the tiles leave SMs idle
-// (at least four column blocks per CTA).  The largest cluster size with which all tiles are resident at once is taken: a
+// Where the tiles leave SMs idle, a cluster of up to 8 CTAs shares a tile's K range (at least four column
+// blocks per CTA).  The largest cluster size with which all tiles are resident at once is taken: a
 // cluster lives inside one GPC, so that fewer CTAs fit the larger it is, and how many depends on which SMs of which GPC a
 // chip has (one CTA per SM, on the B200s that this was measured on: 148, 74, 45, 33, 26, 22, 15 clusters of 1, 2, 3, 4, 5, 6, 8); a
 // second wave of clusters costs more than the idle SMs (37 tiles, 128 tokens, K = 8192: 40 us with clusters of 4, 24.5 us with 3).
 constexpr int kClusterSizes[] = {8, 6, 5, 4, 3, 2};
-int canonical_splits(int64_t tiles, int64_t K, const int (&resident)[6]) {
+int cluster_splits(int64_t tiles, int64_t K, const int (&resident)[6]) {
     for (int i = 0; i < 6; ++i)
         if (tiles <= resident[i] && K / 128 >= 4 * kClusterSizes[i]) return kClusterSizes[i];
     return 1;
 }
-// How many clusters of each size are resident at once, asked of the runtime once per device.  All kernels on canonical
-// codes take an SM per CTA (512 threads, more than 64 registers), so that one answer holds for all of them.
+// How many clusters of each size are resident at once, asked of the runtime once per device.  All kernels that run in clusters
+// take an SM per CTA (384 threads or more, more than half of the registers), so that one answer holds for all of them.
 static bool resident_clusters(const void* kernel, dim3 block, size_t smem, int (&resident)[6]) {
     constexpr int kDevices = 64;
     static std::atomic<uint64_t> answers[kDevices];  // eight bits per size, the top byte marks an answer
@@ -1036,6 +1022,71 @@ static bool resident_clusters(const void* kernel, dim3 block, size_t smem, int (
     for (int i = 0; i < 6; ++i) resident[i] = (int)(a >> (8 * i) & 0xFF);
     return true;
 }
+// Whether a cluster of CTAs shares a split tile and all of them add its sums up, or pl.splits CTAs deliver to the last one of them.
+// A chip does not hold every number of clusters, so that a cluster may have fewer CTAs than there would be splits: its K ranges are
+// `longer` cycles longer.  Measured, us, last CTA -> cluster: 256 tokens x 4096 x 4096 (4 CTAs) 20.1 -> 15.0, x 2048 x 8192 (9 -> 6) 28.1 ->
+// 15.8, x 1024 x 4096 (8) 22.4 -> 10.3; 32 tokens 8.4 -> 7.9, 9.6 -> 8.3, 7.4 -> 5.4; 9 tokens 7.8 -> 7.7, 8.7 -> 8.6, 6.5 -> 5.3.  Where the last
+// CTA is kept: 32 tokens x 1024 x 28672 (16 -> 8) 12.4 -> 13.3, 400 tokens x 2048 x 8192 (3 -> 2) 22.1 -> 22.7.
+static bool clusters_win(const PrefillPlan& pl, int64_t K, int cluster) {
+    if (cluster < 2 || cluster > pl.splits) return false;  // (the workspace holds pl.splits items' sums per tile)
+    const int64_t rows = pl.rows_alloc, pace = 92 * rows / 20 > 650 ? 92 * rows / 20 : 650;  // cycles per 128 columns
+    const int64_t longer = (K / 128) * pace * (pl.splits - cluster) / ((int64_t)cluster * pl.splits);
+    return 2900 + 10 * rows * pl.splits > longer;
+}
+pot_status_t gemm_prefill_launch(const void* packed, const void* scales, int64_t N, int64_t K, int bits, int group,
+                                 const void* X, int64_t M, void* Y, void* workspace, size_t ws_bytes, cudaStream_t s, int dt) {
+    const PrefillPlan pl = prefill_plan(M, N, K);
+    if (pl.ws_bytes > 0 && (!workspace || ws_bytes < pl.ws_bytes)) return POT_ERR_WORKSPACE;
+    unsigned* counters = (unsigned*)workspace;
+    float* partial = pl.ws_bytes > 0 ? (float*)((char*)workspace + pl.counter_bytes) : nullptr;
+    CUtensorMap xmap;
+    if (!encode_x_map(&xmap, X, M, K, pl.h)) return POT_ERR_CUDA;
+    const PrefillVariant v = prefill_variant(pl, M, dt);
+    auto run = [&](auto kernel, int ng, size_t smem, int cluster) -> pot_status_t {
+        const int splits = cluster > 1 ? cluster : pl.splits;
+        return launch_pdl_cluster(kernel, dim3((unsigned)(pl.n_full + pl.n_tail * splits)), dim3((unsigned)pf_threads(ng, 2)), smem, cluster, true, s,
+                                  xmap, (const uint4*)packed, (const uint16_t*)scales, N, K, group, M, (uint16_t*)Y, partial, counters,
+                                  pl.tiles_m, pl.n_full, splits, cluster > 1 ? 1 : 0, pl.h, prefill_error_ptr());
+    };
+    // every tile is cut: a cluster of CTAs for each, if that is faster (the kernel without clusters if the runtime gives no answer)
+    auto run_split = [&](auto kernel, auto clustered, int ng, size_t smem) -> pot_status_t {
+        if (pl.n_full > 0 || pl.n_tail == 0) return run(kernel, ng, smem, 1);
+        int resident[6] = {};
+        if (!resident_clusters((const void*)clustered, dim3((unsigned)pf_threads(ng, 2)), smem, resident)) cudaGetLastError();
+        const int cluster = cluster_splits(pl.tiles, K, resident);
+        return clusters_win(pl, K, cluster) ? run(clustered, ng, smem, cluster) : run(kernel, ng, smem, 1);
+    };
+    // two issuers, one CTA per SM
+    return with_bits_and_type(bits, dt, [&](auto b, auto d) -> pot_status_t {
+        constexpr int B = decltype(b)::value, D = decltype(d)::value;
+        if (M <= PF_SMALL_TOKENS) {
+            if (v.in_tmem) return run_split(pot_gemm_prefill_kernel<B, 6, 3, 2, 1, D, 1>, pot_gemm_prefill_kernel<B, 6, 3, 2, 1, D, 1, 3, 0, 0, 1>, 3, pf_smem_bytes(6, 1, 1));
+            return run(pot_gemm_prefill_kernel<B, 8, 4, 2, 1, D>, 4, pf_smem_bytes(8, 1), 1);
+        }
+        if (!v.in_tmem) return run(pot_gemm_prefill_kernel<B, 4, 4, 2, 2, D>, 4, pf_smem_bytes(4, 2), 1);
+        constexpr int NG4 = D == 1 ? 4 : 2, NG6 = D == 1 ? 3 : 2;
+        if (v.stages == 4)
+            return run_split(pot_gemm_prefill_kernel<B, 4, NG4, 2, 2, D, 1>, pot_gemm_prefill_kernel<B, 4, NG4, 2, 2, D, 1, NG4, 0, 0, 1>, NG4, pf_smem_bytes_h(4, pl.h, 1));
+        if (v.stages == 3)
+            return run_split(pot_gemm_prefill_kernel<B, 3, 3, 2, 2, D, 1, 3, 1>, pot_gemm_prefill_kernel<B, 3, 3, 2, 2, D, 1, 3, 1, 0, 1>, 3, pf_smem_bytes_h(3, pl.h, 2));
+        return run(pot_gemm_prefill_kernel<B, 6, NG6, 2, 2, D, 1>, NG6, pf_smem_bytes_h(6, pl.h, 1), 1);
+    });
+}
+
+static int* prefill_error_ptr() { return error_ptr(ERR_PREFILL); }
+
+static bool encode_x_map(CUtensorMap* xmap, const void* X, int64_t M, int64_t K, int h) {
+    EncodeTiledFn encode = encode_tiled_fn();
+    if (!encode) return false;
+    const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)M};
+    const cuuint64_t strides[1] = {(cuuint64_t)K * 2};
+    const cuuint32_t box[2] = {64, (cuuint32_t)(M <= PF_SMALL_TOKENS ? M : h)};  // the one-tile kernel: no padding rows
+    const cuuint32_t estr[2] = {1, 1};
+    return encode(xmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(X), dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 pot_status_t gemm_canonical_launch(const void* packed, const void* scales, int64_t N, int64_t K, int bits, int group,
                                    const void* X, int64_t M, void* Y, cudaStream_t s, int dt) {
     const bool small = M <= PF_SMALL_TOKENS;
@@ -1049,10 +1100,10 @@ pot_status_t gemm_canonical_launch(const void* packed, const void* scales, int64
         const dim3 block((unsigned)pf_threads(3, 2));
         int resident[6] = {};
         if (!resident_clusters((const void*)kernel, block, smem, resident)) cudaGetLastError();  // no answer: one CTA per tile
-        const int splits = canonical_splits(tiles, K, resident);
+        const int splits = cluster_splits(tiles, K, resident);
         return launch_pdl_cluster(kernel, dim3((unsigned)(tiles * splits)), block, smem, splits, true, s, xmap,
                                   (const uint4*)packed, (const uint16_t*)scales, N, K, group, M, (uint16_t*)Y, (float*)nullptr,
-                                  (unsigned*)nullptr, (int)tiles_m, (int)(splits > 1 ? 0 : tiles), splits, h, prefill_error_ptr());
+                                  (unsigned*)nullptr, (int)tiles_m, (int)(splits > 1 ? 0 : tiles), splits, splits > 1 ? 1 : 0, h, prefill_error_ptr());
     };
     return with_bits_and_type(bits, dt, [&](auto b, auto d) -> pot_status_t {
         constexpr int B = decltype(b)::value, D = decltype(d)::value;

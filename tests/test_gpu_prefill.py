@@ -204,3 +204,30 @@ def test_tiles_of_large_launches(B, oracle, bits, dt):
         assert B.pot_debug_errors() == (0, 0, 0)
         ok, worst, tight = gate(y, Y[:, row], A[:, row], bf16=bf16)
         assert ok and tight < 4.0, (M, N, K, worst, tight)
+
+
+@pytest.mark.parametrize("bits, dt", [(2, "bf16"), (3, "f16"), (4, "f16")])
+@pytest.mark.parametrize("K, splits", [(1024, 2), (1536, 3), (2048, 4), (2560, 5), (3072, 6), (4096, 8)])
+def test_tiles_cut_by_clusters_of_every_size(B, oracle, bits, dt, K, splits):
+    """Two feature tiles (the second of 16 rows) whose K range is shared by a cluster: one or two X tiles of every raggedness, their tokens
+    dealt to the CTAs unevenly.  The arrival counters, which only the way without clusters uses, stay untouched (as does all of
+    the workspace behind the sums of the tiles)."""
+    N, G = 144, 64 if bits == 4 else 128
+    c = PotCase(N, K, bits, G, dist="normal", sigma=0.015, seed=(5, 900 + bits))
+    tiled, tS = c.tiled(), c.tiled_S()
+    X = synth.activations(synth.rng_for(5, 950 + bits), 300, K, outliers=True)
+    if dt == "bf16":
+        X = f16_bits_to_bf16_bits(X)
+    Y, A = oracle.matmul(c.packed, c.S, K, bits, G, X, dtype=oracle.BF16 if dt == "bf16" else oracle.F16)
+    for M in (65, 100, 128, 129, 200, 256, 300):
+        plan = B.pot_debug_gemm_plan(M, N, K, bits, G, dt == "bf16")
+        assert plan["split_tiles"] == plan["tiles"] and plan["splits"] >= splits
+        need = B.pot_gemm_workspace_bytes(M, N, K, bits, G)
+        ws = B.new_workspace(need)
+        dX = (bf16_dev if dt == "bf16" else f16_dev)(np.ascontiguousarray(X[:M]))
+        got = [bits_of(B.pot_gemm(tiled, tS, K, bits, G, dX, B.TILED, workspace=ws)) for _ in range(2)]
+        assert not bool(ws[:256].any())
+        ok, worst, tight = gate(got[0], Y[:M], A[:M], bf16=dt == "bf16")
+        assert ok and tight < 4.0, (M, worst, tight)
+        assert np.array_equal(got[0], got[1])
+    assert B.pot_debug_errors() == (0, 0, 0)
