@@ -189,7 +189,9 @@ __device__ __forceinline__ void pf_st32(uint32_t taddr, const uint32_t (&r)[32])
 // (A, from tensor memory: 128 weight rows x 64) by token tile J of the stage (B, h tokens of which the first n are
 // multiplied, from shared memory) and accumulates into columns h J .. h J + n - 1 -- the two issuers share the weight tile and never the accumulator, so
 // the order of the additions is fixed.  A stage is free again when every active issuer's MMAs on it have completed.
-template <int J, int PF_STAGES, int DT, int BKS = 1>
+// KSPLIT (stages of two sub-blocks, a tile of at most h tokens): issuer J multiplies sub-block J by the one X tile, into columns h J ...
+// again, and the epilogue adds the two (one issuer alone leaves the pipe idle half of the time: 100 tokens x 15360 x 5120 23.7 -> 20.7 us).
+template <int J, int PF_STAGES, int DT, int BKS = 1, bool KSPLIT = false>
 __device__ __forceinline__ void pf_issue_at(uint32_t smem0, uint32_t bar0, uint32_t tmem_base, int nkb, uint32_t h, uint32_t n, int* err) {
     auto full = [&](int s) { return bar0 + 8u * s; };
     auto empty = [&](int s) { return bar0 + 8u * (PF_STAGES + s); };
@@ -198,7 +200,7 @@ __device__ __forceinline__ void pf_issue_at(uint32_t smem0, uint32_t bar0, uint3
 #pragma unroll
     for (int s = 0; s < PF_STAGES; ++s)
 #pragma unroll
-        for (int b = 0; b < BKS; ++b) blo[s][b] = (uint32_t)pf_smem_desc(smem0 + (uint32_t)((s * BKS + b) * PF_MT + J) * (h * 128u));
+        for (int b = 0; b < BKS; ++b) blo[s][b] = (uint32_t)pf_smem_desc(smem0 + (uint32_t)((s * BKS + b) * PF_MT + (KSPLIT ? 0 : J)) * (h * 128u));
     constexpr uint32_t desc_hi = (uint32_t)(PF_DESC_CONST >> 32);
     constexpr uint32_t SLOT = 32u * BKS;   // tensor-memory columns of a stage's weights
     const uint32_t d0 = tmem_base + (uint32_t)J * h;
@@ -218,10 +220,10 @@ __device__ __forceinline__ void pf_issue_at(uint32_t smem0, uint32_t bar0, uint3
             if (kb + 1 < nkb) ready = mbar_test(full((s + 1) % PF_STAGES), s + 1 >= PF_STAGES ? ph ^ 1u : ph);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-            for (int ks = 0; ks < BKS * (PF_BK / 16); ++ks)   // sub-block ks / 4
+            for (int ks = KSPLIT ? 4 * J : 0; ks < (KSPLIT ? 4 * J + 4 : BKS * (PF_BK / 16)); ++ks)   // sub-block ks / 4
                 pf_mma_ta(d0, a0 + SLOT * (uint32_t)s + (uint32_t)(8 * ks),
                           blo[s][ks >> 2] + (uint32_t)(((ks & 3) * 32) >> 4), desc_hi, idesc,
-                          (s != 0 || ks != 0) ? 1u : (uint32_t)(kb0 != 0));
+                          (s != 0 || ks != (KSPLIT ? 4 * J : 0)) ? 1u : (uint32_t)(kb0 != 0));
             pf_commit(empty(s));
         }
     }
@@ -454,6 +456,12 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
     const int64_t ncb = K / 128;
     // a tile with at most h real tokens (decode batches, the ragged last token tile) uses one accumulator only
     const int n_mt = M - m0 > h ? MT : 1;
+    // ... unless all tokens fit in one X tile and a stage has two sub-blocks: then each issuer takes one of these (a ragged last tile of
+    // many is no longer than the others as it is: 400 tokens x 2048 x 8192 22.1 us, 22.7 with its stages shared)
+    const bool ksplit = AT2 && BKS == 2 && M <= PF_BM;
+    const int n_acc = AT2 ? (ksplit ? 2 : n_mt) : NI;      // issuers at work
+    // bytes of an X tile that a stage brings in (at most 128 tokens: the box holds exactly these)
+    const int box_bytes = M <= PF_BM ? (int)M * 128 : x_tile_bytes;
     // token rows the MMA reads from the X stage: whole tiles, or (one-tile kernel) the batch rounded up to the MMA's N step
     const uint32_t n_tok = MT == 1 ? (uint32_t)((M + 15) & ~(int64_t)15) : (uint32_t)(n_mt * PF_BM);  // MT == 1: M <= 64
     const int nkb = (int)((2 / BKS) * (cb1 - cb0));   // stages of this item
@@ -518,9 +526,9 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
     if (threadIdx.x == 0) {
         for (int s = 0; s < PF_STAGES; ++s) {
             mbar_init(full(s), 1 + 4);  // the TMA thread's expect_tx arrival + one arrival per warp of the group that fills the stage
-            mbar_init(empty(s), AT2 ? n_mt : 1);  // AT2: every active issuer reads every stage
+            mbar_init(empty(s), AT2 ? n_acc : 1);  // AT2: every active issuer reads every stage
         }
-        mbar_init(accum, AT2 ? n_mt : NI);
+        mbar_init(accum, n_acc);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {  // allocate the accumulator columns of tensor memory (whole warp), base address lands in shared memory
@@ -551,7 +559,7 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
                 ready = (kn < nkb && kn >= PF_STAGES) ? mbar_test(empty(kn % PF_STAGES), (uint32_t)((kn / PF_STAGES - 1) & 1)) : 0u;
                 // MT == 1 (M <= 64): the box holds exactly the M token rows -- the TMA unit spends time on every row of a
                 // box, in range or not; the rows of the tile that nothing writes belong to tokens that are never stored
-                mbar_expect_tx(full(s), MT == 1 ? (uint32_t)M * 128u * BKS : (uint32_t)(n_mt * x_tile_bytes * BKS));
+                mbar_expect_tx(full(s), MT == 1 ? (uint32_t)M * 128u * BKS : (uint32_t)(n_mt * box_bytes * BKS));
                 const uint32_t a = smem_u32(smem + (size_t)s * STAGE_BYTES);
                 if constexpr (BKS == 2 && MT == 1) {  // (one-tile kernel) the two 64-column tiles of the stage's column block
                     pf_tma_load_2d(a, &xmap, (kb0 + kb) * 2 * PF_BK, (int)m0, full(s));
@@ -576,7 +584,12 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
             if constexpr (AT2) {
                 // (the tokens of an X tile, rounded up to the MMA's N step, from uniform values: the descriptor stays in a uniform register)
                 auto n_of = [&](int64_t left) { return (uint32_t)(left < h ? (left + 15) & ~(int64_t)15 : h); };
-                if (warp == 1) pf_issue_at<0, PF_STAGES, DT, BKS>(smem_u32(smem), bar0, tmem_base, nkb, (uint32_t)h, n_of(M - m0), err);
+                if (ksplit) {
+                    if constexpr (BKS == 2) {
+                        if (warp == 1) pf_issue_at<0, PF_STAGES, DT, BKS, true>(smem_u32(smem), bar0, tmem_base, nkb, (uint32_t)h, n_of(M - m0), err);
+                        else pf_issue_at<1, PF_STAGES, DT, BKS, true>(smem_u32(smem), bar0, tmem_base, nkb, (uint32_t)h, n_of(M - m0), err);
+                    }
+                } else if (warp == 1) pf_issue_at<0, PF_STAGES, DT, BKS>(smem_u32(smem), bar0, tmem_base, nkb, (uint32_t)h, n_of(M - m0), err);
                 else if (n_mt == 2) pf_issue_at<1, PF_STAGES, DT, BKS>(smem_u32(smem), bar0, tmem_base, nkb, (uint32_t)h, n_of(M - m0 - h), err);
             } else if constexpr (AT) {
                 if (warp == 1) pf_issue_at1<0, NI, PF_STAGES, DT>(smem_u32(smem), bar0, tmem_base, nkb, n_tok, err);
@@ -704,10 +717,10 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
         const int nch = MT == 1 ? PF_SMALL_TOKENS / 32 : MT * h / 32;
         auto sums = [&](int col, uint32_t (&v)[32]) {  // the complete sums of 32 token columns of this item
             pf_ld32(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)col, v);
-            if (NI == 2 && !AT2 && nkb > 1) {     // add the second issuer's sums (odd K blocks) to the first's: a fixed order
-                                                  // (an item of a single stage -- K = 128 with 128-column stages -- has none)
+            if (AT2 ? ksplit : NI == 2 && nkb > 1) {  // add the second issuer's sums (odd K blocks) to the first's: a fixed order
+                                                      // (an item of a single stage -- K = 128 with 128-column stages -- has none)
                 uint32_t v1[32];
-                pf_ld32(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)((AT ? PF_AT1_ACC_STRIDE : PF_BM * MT) + col), v1);
+                pf_ld32(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)((AT2 ? h : AT ? PF_AT1_ACC_STRIDE : PF_BM * MT) + col), v1);
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
                 for (int i = 0; i < 32; ++i) v[i] = __float_as_uint(__uint_as_float(v[i]) + __uint_as_float(v1[i]));
@@ -1080,7 +1093,7 @@ static bool encode_x_map(CUtensorMap* xmap, const void* X, int64_t M, int64_t K,
     if (!encode) return false;
     const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)M};
     const cuuint64_t strides[1] = {(cuuint64_t)K * 2};
-    const cuuint32_t box[2] = {64, (cuuint32_t)(M <= PF_SMALL_TOKENS ? M : h)};  // the one-tile kernel: no padding rows
+    const cuuint32_t box[2] = {64, (cuuint32_t)(M < h ? M : h)};  // a single X tile: no padding rows
     const cuuint32_t estr[2] = {1, 1};
     return encode(xmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(X), dims, strides, box, estr,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,

@@ -231,3 +231,23 @@ def test_tiles_cut_by_clusters_of_every_size(B, oracle, bits, dt, K, splits):
         assert ok and tight < 4.0, (M, worst, tight)
         assert np.array_equal(got[0], got[1])
     assert B.pot_debug_errors() == (0, 0, 0)
+
+
+@pytest.mark.parametrize("bits, dt", [(2, "f16"), (3, "bf16"), (4, "f16")])
+@pytest.mark.parametrize("M", [65, 80, 97, 128])
+def test_one_x_tile_shared_by_both_issuers(B, oracle, bits, dt, M):
+    """65 to 128 tokens, 128-column stages: one issuer multiplies the first half of every stage, the other one the second half.  One
+    stage, as many as the ring has, more; unsplit tiles and split ones; both layouts."""
+    for i, (N, K, G) in enumerate([(144, 128, 64), (272, 384, 128), (48, 896, 64), (9600, 256, 128)]):
+        c = PotCase(N, K, bits, G, dist="normal", sigma=0.015, seed=(5, 1000 + 10 * bits + i))
+        X = synth.activations(synth.rng_for(5, 1050 + i), M, K, outliers=True)
+        if dt == "bf16":
+            X = f16_bits_to_bf16_bits(X)
+        rows = np.unique(np.linspace(0, N - 1, 300).astype(np.int64))
+        Y, A = oracle.matmul(c.packed, c.S, K, bits, G, X, rows=rows, dtype=oracle.BF16 if dt == "bf16" else oracle.F16)
+        dX = (bf16_dev if dt == "bf16" else f16_dev)(X)
+        assert B.pot_debug_gemm_plan(M, N, K, bits, G, dt == "bf16")["stage_columns"] == 128
+        for layout, P, S in ((B.TILED, c.tiled(), c.tiled_S()), (B.CANONICAL, c.d_packed, c.d_S)):
+            ok, worst, tight = gate(bits_of(B.pot_gemm(P, S, K, bits, G, dX, layout))[:, rows], Y, A, bf16=dt == "bf16")
+            assert ok and tight < 4.0, (N, K, layout, worst, tight)
+    assert B.pot_debug_errors() == (0, 0, 0)
