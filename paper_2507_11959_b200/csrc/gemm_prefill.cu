@@ -129,6 +129,11 @@ __device__ __forceinline__ uint4 pf_ldg_v4(const uint4* p) {
     asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
     return v;
 }
+__device__ __forceinline__ uint32_t pf_ldg_u32(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
 __device__ __forceinline__ uint32_t pf_ldg_u16(const uint16_t* p) {
     uint16_t v;
     asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(v) : "l"(p));
@@ -398,7 +403,7 @@ __device__ __forceinline__ void pf_add_up(const PfAddUp& a, uint32_t smem, int* 
 // CANON = 1: canonical codes and row-major scales (the 128-column stages only): a producer thread reads its row's 16 BITS
 // contiguous bytes per column block and decodes them with byte look-ups (potl::CanonLut).  There is no workspace on this
 // route: the items of a tile that is cut along K are the CTAs of a thread-block cluster, which add their partial sums through
-// distributed shared memory.  200 tokens x 4099 x 11008, 3 bits: 672 us on the mma.sync kernel that this replaced, 26.5 us
+// distributed shared memory.  200 tokens x 4099 x 11008, 3 bits: 672 us on the mma.sync kernel that this replaced, 25.3 us
 // (clusters of 4, 132 CTAs: the loads of codes, a cache line per row each, and 5 us to add up the sums).
 // CLUSTER = 1: the items of every tile are a cluster (canonical codes: if `clustered`).  An instantiation of its own for tiled codes: with
 // the choice made at run time, launches without clusters took 1 - 3 % longer (301 tokens x 11024 x 4096, BF16: 30.1 -> 31.1 us).
@@ -495,8 +500,12 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
                     const uint4 q = pf_ldg_v4(rowp + t);
                     rec[buf][4 * t + 0] = q.x; rec[buf][4 * t + 1] = q.y; rec[buf][4 * t + 2] = q.z; rec[buf][4 * t + 3] = q.w;
                 }
-                sc2[buf][0] = pf_ldg_u16(scales + (n * ncb + cbx) * spg);
-                sc2[buf][BKS - 1] = pf_ldg_u16(scales + (n * ncb + cbx) * spg + spg - 1);
+                // Every load touches 32 rows, i.e. 32 cache lines, and the load unit takes them one by one: no more loads than needed.
+                // Two groups per column block share an aligned word (two loads, for one group too: 200 tokens x 4096 x 11008, 3 bits
+                // 30.7 us, with one 26.5 us; handing the codes round a warp so that a load touches a third of the lines: 27.3 us).
+                const uint16_t* sp = scales + (n * ncb + cbx) * spg;
+                if (spg == 2) sc2[buf][0] = pf_ldg_u32(reinterpret_cast<const uint32_t*>(sp));
+                else sc2[buf][0] = pf_ldg_u16(sp);
             } else if constexpr (BKS == 2) {
                 const uint4* unit = packed + (rb * ncb + cbx) * (16 * BITS);
 #pragma unroll
@@ -628,7 +637,9 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
                     // (BKS = 1: only) half is decoded before the wait for the stage, so that a stage that has become free is
                     // filled at once
                     auto decode = [&](int hb, uint32_t (&wa)[32]) {
-                        uint32_t sh = sc2[buf][hb];
+                        uint32_t sh;
+                        if constexpr (CANON) sh = spg == 2 ? (sc2[buf][0] >> (16 * hb)) & 0xFFFFu : sc2[buf][0];
+                        else sh = sc2[buf][hb];
                         if (DT == 1) sh = __bfloat16_as_ushort(__float2bfloat16_rn(__half2float(__ushort_as_half((uint16_t)sh))));
                         const uint32_t sh2 = sh * 0x10001u;  // scale pattern in both halves
                         const potl::CanonLut<BITS, DT> lut(sh);
