@@ -96,38 +96,44 @@ __global__ void __launch_bounds__(256) gemv_canonical_kernel(const uint32_t* __r
 // BITS 16-byte loads per row from contiguous memory, and each register is loaded for the next step as soon as it has been
 // decoded.  x is staged in shared memory (272 bytes per column block: the four blocks that the lanes of a fragment read lie
 // in different banks) and sits in every column of B; at 2 bits in the order in which the codes leave the words most cheaply.
-// CTAs of eight warps, two per SM: while one of them finishes, another (of the next launch, too) sets itself up.  The steps of
+// CTAs of eight warps, two per SM, or of four: while one of them finishes, another (of the next launch, too) sets itself up.  The steps of
 // a row block are dealt to 1, 2, 4 or 8 warps of a CTA and, where few row blocks leave SMs idle, to the CTAs of a cluster; the sums are
 // added in warp order, then in CTA order.  (One CTA of 16 warps per SM with a contiguous, equal share of the steps per warp was
 // 5 - 20 % slower: its launches do not overlap.)
 // Bound by instruction issue (16 rows x 128 columns: 70 - 110 instructions to decode, 8 MMAs, 12 loads) and by fixed latencies (launch, x,
 // codes).  HBM-cold, 10007 x 4096: 8.8 us at 2 bits, 11.7 us at 3, 13.0 us at 4 bits in BF16 (one warp per row on CUDA cores: 26.5,
 // 31.9, 26.5 us); 4099 x 11008 at 3 bits: 36.1 -> 11.3 us.
-constexpr int GC_WARPS = 8;
+constexpr int GC_WARPS = 8;                      // (or half as many)
 constexpr int GC_X_STRIDE = 272;                 // bytes per staged column block
 constexpr int64_t GC_MAX_K = 64 * 1024;          // x takes 136 KB at this length
-struct CanonPlan { int wk_shift, cluster; unsigned grid; };  // log2 of the warps per row block, CTAs per row block
+struct CanonPlan { int wk_shift, warps, cluster; unsigned grid; };  // log2 of the warps per row block, warps per CTA, CTAs per row block
 static CanonPlan plan_canonical(int64_t N, int64_t K) {
     const int64_t rbs = (N + 15) / 16, steps = (K / 128 + 3) / 4;
-    CanonPlan p{0, 1, 0};
+    CanonPlan p{0, GC_WARPS, 1, 0};
     while (p.wk_shift < 3 && (rbs << p.wk_shift) < 2 * GC_WARPS * kSmCount && (2 << p.wk_shift) <= steps) ++p.wk_shift;
     while (p.cluster < 4 && p.wk_shift == 3 && rbs * p.cluster * 2 <= kSmCount && 2 * p.cluster * GC_WARPS <= steps) p.cluster *= 2;
-    const int64_t per_cta = GC_WARPS >> p.wk_shift;
+    // Four warps per row block fill a little more than the SMs' 16 warps each: with CTAs of four warps a last wave is one of a few small
+    // CTAs (10007 x 4096, 2 / 3 / 4 bits 9.0 / 11.7 / 13.0 -> 8.2 / 10.0 / 11.3 us, 12000 x 3072 9.0 / 11.7 /
+    // 12.9 -> 8.5 / 10.1 / 10.8), as long as x fits into shared memory four times.
+    if (p.wk_shift == 2 && K <= 24 * 1024) p.warps = GC_WARPS / 2;
+    const int64_t per_cta = p.warps >> p.wk_shift;
     p.grid = (unsigned)((rbs + per_cta - 1) / per_cta * p.cluster);
     return p;
 }
 
-template <int BITS, int DT>
-__global__ void __launch_bounds__(GC_WARPS * 32, 2) gemv_canonical_mma_kernel(const uint4* __restrict__ packed, const uint16_t* __restrict__ scales,
+// (CTAs per SM: as many as 128 registers leave; at 2 bits 102 registers are enough, and a fifth 4-warp CTA is worth 8.5 -> 8.2 us)
+constexpr int gc_ctas_per_sm(int bits, int warps) { return warps == GC_WARPS ? 2 : (bits == 2 ? 5 : 4); }
+template <int BITS, int DT, int W>
+__global__ void __launch_bounds__(W * 32, gc_ctas_per_sm(BITS, W)) gemv_canonical_mma_kernel(const uint4* __restrict__ packed, const uint16_t* __restrict__ scales,
                                                                               int64_t N, int ncb, int spg, const uint4* __restrict__ x,
                                                                               uint16_t* __restrict__ y, int wk_shift, int cluster, int* __restrict__ err) {
     extern __shared__ __align__(16) unsigned char xs[];
-    __shared__ float part[GC_WARPS][16];
+    __shared__ float part[W][16];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int gid = lane >> 2, tig = lane & 3;
     const int WK = 1 << wk_shift;
     const int crank = (int)blockIdx.x % cluster;
-    const int64_t rb = (int64_t)(blockIdx.x / cluster) * (GC_WARPS >> wk_shift) + (warp >> wk_shift);
+    const int64_t rb = (int64_t)(blockIdx.x / cluster) * (W >> wk_shift) + (warp >> wk_shift);
     const int64_t row0 = min(rb * 16 + gid, N - 1), row1 = min(rb * 16 + gid + 8, N - 1);  // (rows past the end repeat the last one and are not stored)
     const int steps = (ncb + 3) / 4, stride = WK * cluster;
     pdl_wait();
@@ -156,7 +162,7 @@ __global__ void __launch_bounds__(GC_WARPS * 32, 2) gemv_canonical_mma_kernel(co
 #pragma unroll
         for (int h = 0; h < 2; ++h) sc[h][hb] = __ldg(ssrc[h] + (spg == 2 ? hb : 0));
     };
-    const bool fits = in_range((uint32_t)(ncb + 1) * GC_X_STRIDE <= dynamic_smem_bytes() && WK <= GC_WARPS && crank < cluster, err, 0x160);
+    const bool fits = in_range((uint32_t)(ncb + 1) * GC_X_STRIDE <= dynamic_smem_bytes() && WK <= W && crank < cluster, err, 0x160);
     int step = fits ? crank * WK + (warp & (WK - 1)) : steps;
     if (step < steps) {
         point(step);
@@ -166,14 +172,14 @@ __global__ void __launch_bounds__(GC_WARPS * 32, 2) gemv_canonical_mma_kernel(co
         load_scales(1);
     }
     if constexpr (BITS == 2) {  // the order of canon_decode32_any
-        for (int i = threadIdx.x; fits && i < ncb * 8; i += GC_WARPS * 32) {
+        for (int i = threadIdx.x; fits && i < ncb * 8; i += W * 32) {
             const uint4 a = ld_dependent16(x + 2 * i), b = ld_dependent16(x + 2 * i + 1);
             uint4* dst = reinterpret_cast<uint4*>(xs + (i >> 3) * GC_X_STRIDE + (i & 7) * 32);
             dst[0] = make_uint4(potl::prmt(a.x, a.y, 0x5410), potl::prmt(a.z, a.w, 0x5410), potl::prmt(b.x, b.y, 0x5410), potl::prmt(b.z, b.w, 0x5410));
             dst[1] = make_uint4(potl::prmt(a.x, a.y, 0x7632), potl::prmt(a.z, a.w, 0x7632), potl::prmt(b.x, b.y, 0x7632), potl::prmt(b.z, b.w, 0x7632));
         }
     } else {
-        for (int i = threadIdx.x; fits && i < ncb * 16; i += GC_WARPS * 32)
+        for (int i = threadIdx.x; fits && i < ncb * 16; i += W * 32)
             *reinterpret_cast<uint4*>(xs + (i >> 4) * GC_X_STRIDE + (i & 15) * 16) = ld_dependent16(x + i);
     }
     if (fits && threadIdx.x < 16) *reinterpret_cast<uint4*>(xs + ncb * GC_X_STRIDE + threadIdx.x * 16) = make_uint4(0, 0, 0, 0);  // x of the block past the end
@@ -277,12 +283,16 @@ static pot_status_t launch_gemv_canonical(const void* packed, const void* scales
         const CanonPlan p = plan_canonical(N, K);
         auto run = [&](auto kernel) -> pot_status_t {
             const size_t smem = (size_t)(K / 128 + 1) * GC_X_STRIDE;
-            return launch_pdl_cluster(kernel, dim3(p.grid), dim3(GC_WARPS * 32), smem, p.cluster, smem > 46 * 1024, s, (const uint4*)packed,
+            return launch_pdl_cluster(kernel, dim3(p.grid), dim3((unsigned)p.warps * 32), smem, p.cluster, smem > 46 * 1024, s, (const uint4*)packed,
                                       (const uint16_t*)scales, N, (int)(K / 128), 128 / group, (const uint4*)x, (uint16_t*)y, p.wk_shift, p.cluster, error_ptr(ERR_GEMV));
         };
-        if (bits == 2) return run(gemv_canonical_mma_kernel<2, DT>);
-        if (bits == 3) return run(gemv_canonical_mma_kernel<3, DT>);
-        return run(gemv_canonical_mma_kernel<4, DT>);
+        auto pick = [&](auto w) -> pot_status_t {
+            constexpr int W = decltype(w)::value;
+            if (bits == 2) return run(gemv_canonical_mma_kernel<2, DT, W>);
+            if (bits == 3) return run(gemv_canonical_mma_kernel<3, DT, W>);
+            return run(gemv_canonical_mma_kernel<4, DT, W>);
+        };
+        return p.warps == GC_WARPS ? pick(std::integral_constant<int, GC_WARPS>()) : pick(std::integral_constant<int, GC_WARPS / 2>());
     }
     const dim3 grid((unsigned)((N + 7) / 8)), block(256);
     auto* P = (const uint32_t*)packed;
