@@ -7,6 +7,7 @@ symbol from it raises.
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 from pathlib import Path
 
 import torch
@@ -31,6 +32,8 @@ EXPORTS = [
 ]
 
 _lib = None
+_fast = None    # the extension module through which a token's calls go, with the addresses of the entry points
+_FASTCALL_PATH = _HERE / "_fastcall.so"
 
 
 class PotError(RuntimeError):
@@ -85,6 +88,23 @@ def lib() -> ctypes.CDLL:
                 fn.restype = i32
         _lib = L
     return _lib
+
+
+def _load_fast():
+    """The calls that a user makes for every token take their way into the library through a C module: ctypes converts twelve
+    arguments in 1.5 us, as long as half of a small kernel."""
+    global _fast
+    if _fast is None:
+        L = lib()
+        if not _FASTCALL_PATH.exists():
+            raise PotError(f"{_FASTCALL_PATH} not built: run `python -m paper_2507_11959_b200.build`")
+        spec = importlib.util.spec_from_file_location("_fastcall", _FASTCALL_PATH)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+        for name in ("pot_gemv", "pot_gemv_bf16", "pot_gemm", "pot_gemm_bf16", "pot_dequant"):
+            setattr(module, name, ctypes.cast(getattr(L, name), ctypes.c_void_p).value)
+        _fast = module
+    return _fast
 
 
 def _check(status: int, what: str) -> None:
@@ -194,7 +214,10 @@ def pot_dequant(packed: torch.Tensor, scales: torch.Tensor, K: int, bits: int, g
     N = packed.shape[0]
     if out is None:
         out = torch.empty((N, K), dtype=torch.float16 if out_dtype == F16 else torch.bfloat16, device=packed.device)
-    _check(lib().pot_dequant(_ptr(packed), _ptr(scales), N, K, bits, group, out_dtype, _ptr(out), _stream(stream)), "pot_dequant")
+    f = _fast or _load_fast()
+    status = f.dequant(f.pot_dequant, _ptr(packed), _ptr(scales), N, K, bits, group, out_dtype, _ptr(out), _stream(stream))
+    if status != POT_OK:
+        _check(status, "pot_dequant")
     return out
 
 
@@ -202,15 +225,18 @@ def pot_gemv(packed, scales, K: int, bits: int, group: int, x: torch.Tensor, lay
              y: torch.Tensor | None = None, workspace: torch.Tensor | None = None, stream=None) -> torch.Tensor:
     """x float16 -> pot_gemv, x bfloat16 -> pot_gemv_bf16 (the output has the activations' dtype)."""
     N = packed.shape[0]
-    assert x.dtype in (torch.float16, torch.bfloat16)
+    dtype = x.dtype
+    assert dtype in (torch.float16, torch.bfloat16)
     if y is None:
-        y = torch.empty(N, dtype=x.dtype, device=x.device)
-    assert y.dtype == x.dtype
+        y = torch.empty(N, dtype=dtype, device=x.device)
+    assert y.dtype == dtype
     if workspace is None and layout == TILED:
         workspace = new_workspace(pot_gemv_workspace_bytes(N, K, bits, group), x.device)
-    fn = lib().pot_gemv if x.dtype == torch.float16 else lib().pot_gemv_bf16
-    _check(fn(_ptr(packed), _ptr(scales), N, K, bits, group, layout, _ptr(x), _ptr(y), _ptr(workspace),
-              0 if workspace is None else workspace.numel(), _stream(stream)), "pot_gemv")
+    f = _fast or _load_fast()
+    status = f.gemv(f.pot_gemv if dtype == torch.float16 else f.pot_gemv_bf16, _ptr(packed), _ptr(scales), N, K, bits, group, layout, _ptr(x),
+                    _ptr(y), _ptr(workspace), 0 if workspace is None else workspace.numel(), _stream(stream))
+    if status != POT_OK:
+        _check(status, "pot_gemv")
     return y
 
 
@@ -227,15 +253,18 @@ def pot_gemv_host(packed, scales, K: int, bits: int, group: int, x_host: torch.T
 def pot_gemm(packed, scales, K: int, bits: int, group: int, X: torch.Tensor, layout: int = CANONICAL,
              Y: torch.Tensor | None = None, workspace: torch.Tensor | None = None, stream=None) -> torch.Tensor:
     N, M = packed.shape[0], X.shape[0]
-    assert X.dtype in (torch.float16, torch.bfloat16)
+    dtype = X.dtype
+    assert dtype in (torch.float16, torch.bfloat16)
     if Y is None:
-        Y = torch.empty((M, N), dtype=X.dtype, device=X.device)
-    assert Y.dtype == X.dtype
+        Y = torch.empty((M, N), dtype=dtype, device=X.device)
+    assert Y.dtype == dtype
     if workspace is None and layout == TILED:
         workspace = new_workspace(pot_gemm_workspace_bytes(M, N, K, bits, group), X.device)
-    fn = lib().pot_gemm if X.dtype == torch.float16 else lib().pot_gemm_bf16
-    _check(fn(_ptr(packed), _ptr(scales), N, K, bits, group, layout, _ptr(X), M, _ptr(Y), _ptr(workspace),
-              0 if workspace is None else workspace.numel(), _stream(stream)), "pot_gemm")
+    f = _fast or _load_fast()
+    status = f.gemm(f.pot_gemm if dtype == torch.float16 else f.pot_gemm_bf16, _ptr(packed), _ptr(scales), N, K, bits, group, layout, _ptr(X), M,
+                    _ptr(Y), _ptr(workspace), 0 if workspace is None else workspace.numel(), _stream(stream))
+    if status != POT_OK:
+        _check(status, "pot_gemm")
     return Y
 
 

@@ -1,4 +1,5 @@
-"""Builds ``libpot_b200.so`` (the C-ABI CUDA library) in-tree with nvcc for sm_100a.
+"""Builds ``libpot_b200.so`` (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and ``_fastcall.so`` (the binding's calls into
+it) with the C compiler.
 
     python -m paper_2507_11959_b200.build [--force] [--verbose]
 """
@@ -7,12 +8,14 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 from pathlib import Path
 
 HERE = Path(__file__).resolve().parent
 CSRC = HERE / "csrc"
 LIB = HERE / "libpot_b200.so"
+FASTCALL = HERE / "_fastcall.so"
 LIB_CHECKED = HERE / "libpot_b200_checked.so"   # the same sources with -DPOT_CHECKED (device-side index checks)
 OBJ_DIR = HERE / "build"
 SOURCES = ["api.cu", "quantize.cu", "dequant.cu", "gemv.cu", "gemm.cu", "gemm_prefill.cu"]
@@ -32,9 +35,24 @@ def _deps_mtime() -> float:
     return max(f.stat().st_mtime for f in files)
 
 
+def build_fastcall(force: bool = False) -> Path:
+    src, header = CSRC / "fastcall.c", HERE.parent / "include" / "pot.h"
+    if not force and FASTCALL.exists() and FASTCALL.stat().st_mtime >= max(f.stat().st_mtime for f in (src, header, Path(__file__))):
+        return FASTCALL
+    tmp = FASTCALL.with_suffix(f".so.tmp{os.getpid()}")
+    cmd = [os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", f"-I{sysconfig.get_paths()['include']}", str(src), "-o", str(tmp)]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        sys.stderr.write(f"$ {' '.join(cmd)}\n{r.stdout}{r.stderr}\n")
+        raise RuntimeError("the C compiler failed on fastcall.c")
+    os.replace(tmp, FASTCALL)
+    return FASTCALL
+
+
 def build(force: bool = False, verbose: bool = False, checked: bool = False) -> Path:
     """Build the library; checked=True builds the variant whose GEMV and GEMM kernels verify their indices before stores,
     atomics and shape-dependent shared-memory accesses and report a violation through the error words instead of accessing."""
+    build_fastcall(force)
     LIB = LIB_CHECKED if checked else globals()["LIB"]
     OBJ_DIR = HERE / ("build_checked" if checked else "build")
     sources = [s for s in SOURCES if (CSRC / s).exists()]

@@ -315,14 +315,10 @@ pot_status_t gemv_stream_launch(const void* packed, const void* scales, int64_t 
     return launch_gemv_stream<SK_POT, 1>(packed, scales, nullptr, N, K, bits, group, x, y, workspace, s);
 }
 
+// (the partial-sum layout depends neither on the kind of codes nor on the occupancy)
 static size_t gemv_stream_workspace(int64_t N, int64_t K, int bits, int group, int tok) {
-    size_t need = 0;
-    for (int occ : {1, 2}) {  // the partial-sum layout does not depend on the occupancy, the check is for safety
-        const StreamPlan p = plan_stream(N, K, 1, bits, group, SK_UINT, tok, 16, occ);
-        if (!p.ok) return 0;
-        if (p.ws_bytes > need) need = p.ws_bytes;
-    }
-    return need;
+    const StreamPlan p = plan_stream(N, K, 1, bits, group, SK_UINT, tok, 16);
+    return p.ok ? p.ws_bytes : 0;
 }
 
 }  // namespace pot
@@ -364,9 +360,9 @@ static pot_status_t check_gemv_args(const void* packed, const void* scales, int6
         return POT_ERR_ALIGN;
     if (layout == POT_LAYOUT_TILED) {
         if (N % 16 != 0) return POT_ERR_SHAPE;
-        if (!plan_stream(N, K, 1, bits, group, SK_POT, 1, 16).ok) return POT_ERR_SHAPE;
-        const size_t need = pot_gemv_workspace_bytes(N, K, bits, group);
-        if (need > 0 && (!workspace || ws_bytes < need)) return POT_ERR_WORKSPACE;
+        const StreamPlan p = plan_stream(N, K, 1, bits, group, SK_POT, 1, 16);
+        if (!p.ok) return POT_ERR_SHAPE;
+        if (p.ws_bytes > 0 && (!workspace || ws_bytes < p.ws_bytes)) return POT_ERR_WORKSPACE;
     }
     return POT_OK;
 }

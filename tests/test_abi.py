@@ -136,3 +136,28 @@ def test_canonical_tiles_are_cut_into_clusters_that_are_resident_at_once(L):
     assert [splits(t, 11008, usual) for t in (1, 15, 16, 22, 23, 26, 27, 33, 34, 45, 46, 74, 75, 5000)] == [8, 8, 6, 6, 5, 5, 4, 4, 3, 3, 2, 2, 1, 1]
     assert [splits(t, 11008, fewer) for t in (12, 13, 32, 33, 73)] == [8, 6, 4, 3, 1]
     assert [splits(1, K, usual) for K in (128, 896, 1024, 1536, 2048, 2560, 3072, 4096)] == [1, 1, 2, 3, 4, 5, 6, 8]  # four column blocks per CTA
+
+
+def test_calls_through_the_extension_module_are_those_through_ctypes(L):
+    """The binding's per-token calls: the same argument errors, in the same order, for pointers that are null, misaligned or plain
+    addresses, for lengths, widths and layouts that are refused; a wrong number or type of arguments raises."""
+    from paper_2507_11959_b200 import binding
+    f = binding._load_fast()
+    ok = dict(packed=4096, scales=4096, N=64, K=256, bits=3, group=128, layout=1, x=4096, y=4096, ws=None, ws_bytes=0, stream=0)
+    bad = [dict(packed=None), dict(x=None), dict(y=0), dict(bits=5), dict(group=32), dict(K=100), dict(N=0), dict(N=-1), dict(layout=7), dict(N=63),
+           dict(packed=4097), dict(x=4098), dict(N=2 ** 40)]  # (nothing that would be launched)
+    for change in bad:
+        a = dict(ok, **change)
+        gemv = (a["packed"], a["scales"], a["N"], a["K"], a["bits"], a["group"], a["layout"], a["x"], a["y"], a["ws"], a["ws_bytes"], a["stream"])
+        gemm = gemv[:8] + (40,) + gemv[8:]
+        for name, args, call in (("pot_gemv", gemv, f.gemv), ("pot_gemv_bf16", gemv, f.gemv), ("pot_gemm", gemm, f.gemm), ("pot_gemm_bf16", gemm, f.gemm)):
+            status = getattr(L, name)(*args)
+            assert status != 0 and call(getattr(f, name), *args) == status, (name, change)
+        if set(change) & {"packed", "y", "bits", "group", "K", "N"} and a["N"] != 63:
+            args = gemv[:6] + (0, a["y"], 0)
+            status = L.pot_dequant(*args)
+            assert status != 0 and f.dequant(f.pot_dequant, *args) == status, change
+    with pytest.raises(TypeError):
+        f.gemv(f.pot_gemv, 1, 2, 3)
+    with pytest.raises(TypeError):
+        f.dequant(f.pot_dequant, 4096, 4096, 1.5, 256, 3, 128, 0, 4096, 0)
