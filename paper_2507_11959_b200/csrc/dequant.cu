@@ -6,6 +6,8 @@
 // pieces in flight.
 #include "common.cuh"
 
+#include <type_traits>
+
 namespace pot {
 
 constexpr int DQ_THREADS = 256;
@@ -33,8 +35,8 @@ __device__ __forceinline__ uint32_t read_piece(const uint32_t* __restrict__ w0, 
     return (8 * BITS == 32) ? v : (v & ((1u << (8 * BITS % 32)) - 1u));
 }
 
-// PoT: FP16 (EBIT = 10) or BF16 (EBIT = 7) output.
-template <int BITS, int EBIT>
+// PoT: FP16 (EBIT = 10) or BF16 (EBIT = 7) output, UNROLL pieces per thread.
+template <int BITS, int EBIT, int UNROLL>
 __global__ void __launch_bounds__(DQ_THREADS) pot_dequant_kernel(const uint32_t* __restrict__ packed,
                                                                  const uint16_t* __restrict__ scales, int64_t n_pieces,
                                                                  int ppg_shift, uint4* __restrict__ out) {
@@ -44,14 +46,14 @@ __global__ void __launch_bounds__(DQ_THREADS) pot_dequant_kernel(const uint32_t*
     pdl_launch_dependents();
     constexpr uint32_t QM2 = (uint32_t)qmax_of(BITS) * 0x10001u;   // exponent mask, both halves
     constexpr uint32_t SM2 = (1u << (BITS - 1)) * 0x10001u;        // sign mask, both halves
-    const int64_t base = ((int64_t)blockIdx.x * DQ_UNROLL) * DQ_THREADS + threadIdx.x;
+    const int64_t base = ((int64_t)blockIdx.x * UNROLL) * DQ_THREADS + threadIdx.x;
     const int64_t bit0 = base * (8 * BITS);
     const uint32_t* w0 = packed + (bit0 >> 5);
     const int sh = (int)(bit0 & 31);
-    uint32_t v[DQ_UNROLL];
-    uint32_t sc[DQ_UNROLL];
+    uint32_t v[UNROLL];
+    uint32_t sc[UNROLL];
 #pragma unroll
-    for (int u = 0; u < DQ_UNROLL; ++u) {
+    for (int u = 0; u < UNROLL; ++u) {
         const int64_t c = base + (int64_t)u * DQ_THREADS;
         if (c < n_pieces) {
             v[u] = read_piece<BITS>(w0 + u * (DQ_THREADS * BITS / 4), sh);
@@ -59,7 +61,7 @@ __global__ void __launch_bounds__(DQ_THREADS) pot_dequant_kernel(const uint32_t*
         }
     }
 #pragma unroll
-    for (int u = 0; u < DQ_UNROLL; ++u) {
+    for (int u = 0; u < UNROLL; ++u) {
         const int64_t c = base + (int64_t)u * DQ_THREADS;
         if (c >= n_pieces) continue;
         uint32_t s16 = sc[u];
@@ -85,21 +87,21 @@ __global__ void __launch_bounds__(DQ_THREADS) pot_dequant_kernel(const uint32_t*
 // PoT, n = 3: the 24-bit pieces of the canonical stream straddle 32-bit words, so the generic kernel needs two
 // loads per piece.  Here a thread takes four consecutive pieces = exactly three words (one coalesced 12-byte
 // read) and the block transposes the decoded pieces through shared memory, so that the stores stay coalesced.
-template <int EBIT>
-__global__ void __launch_bounds__(DQ_THREADS) pot_dequant3_kernel(const uint32_t* __restrict__ packed,
-                                                                  const uint16_t* __restrict__ scales, int64_t n_pieces,
-                                                                  int ppg_shift, uint4* __restrict__ out) {
+template <int EBIT, int THREADS>
+__global__ void __launch_bounds__(THREADS) pot_dequant3_kernel(const uint32_t* __restrict__ packed,
+                                                               const uint16_t* __restrict__ scales, int64_t n_pieces,
+                                                               int ppg_shift, uint4* __restrict__ out) {
     // programmatic dependent launch: this grid may have been scheduled while its predecessor in the stream was still
     // running; nothing is read or written before the predecessor has completed
     pdl_wait();
     pdl_launch_dependents();
     constexpr uint32_t QM2 = (uint32_t)qmax_of(3) * 0x10001u, SM2 = 4u * 0x10001u;
-    __shared__ uint4 tile[4 * DQ_THREADS];
+    __shared__ uint4 tile[4 * THREADS];
     const int t = threadIdx.x;
-    const int64_t base = (int64_t)blockIdx.x * (4 * DQ_THREADS);  // first piece of the block
+    const int64_t base = (int64_t)blockIdx.x * (4 * THREADS);  // first piece of the block
     const int64_t c0 = base + 4 * t;                              // this thread's four pieces (one scale group)
     if (c0 < n_pieces) {
-        const uint32_t* w = packed + (int64_t)blockIdx.x * (3 * DQ_THREADS) + 3 * t;
+        const uint32_t* w = packed + (int64_t)blockIdx.x * (3 * THREADS) + 3 * t;
         const uint32_t w0 = __ldg(w), w1 = __ldg(w + 1), w2 = __ldg(w + 2);
         uint32_t s16 = __ldg(scales + (c0 >> ppg_shift));
         if (EBIT == 7) s16 = __bfloat16_as_ushort(__float2bfloat16_rn(__half2float(__ushort_as_half((uint16_t)s16))));
@@ -115,15 +117,15 @@ __global__ void __launch_bounds__(DQ_THREADS) pot_dequant3_kernel(const uint32_t
                 const uint32_t e = (pr[i] & QM2) * (1u << EBIT) + sc2;
                 o[i] = (pr[i] & SM2) * (1u << 13) + e;
             }
-            tile[j * DQ_THREADS + ((t + 2 * j) & (DQ_THREADS - 1))] = make_uint4(o[0], o[1], o[2], o[3]);
+            tile[j * THREADS + ((t + 2 * j) & (THREADS - 1))] = make_uint4(o[0], o[1], o[2], o[3]);
         }
     }
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        const int o = i * DQ_THREADS + t;  // piece of the block, written by consecutive threads
+        const int o = i * THREADS + t;  // piece of the block, written by consecutive threads
         const int tt = o >> 2, j = o & 3;
-        if (base + o < n_pieces) out[base + o] = tile[j * DQ_THREADS + ((tt + 2 * j) & (DQ_THREADS - 1))];
+        if (base + o < n_pieces) out[base + o] = tile[j * THREADS + ((tt + 2 * j) & (THREADS - 1))];
     }
 }
 
@@ -261,26 +263,34 @@ extern "C" pot_status_t pot_dequant(const void* packed, const void* scales, int6
     if (out_dtype != POT_F16 && out_dtype != POT_BF16) return POT_ERR_UNSUPPORTED;
     if (!aligned16(packed) || !aligned16(scales) || !aligned16(W_out)) return POT_ERR_ALIGN;
     const int64_t n_pieces = N * K / 8;
-    const unsigned grid = (unsigned)((n_pieces + DQ_THREADS * DQ_UNROLL - 1) / (DQ_THREADS * DQ_UNROLL));
     cudaStream_t s = (cudaStream_t)stream;
     auto* P = (const uint32_t*)packed;
     auto* S = (const uint16_t*)scales;
     auto* O = (uint4*)W_out;
     const int ppg = group == 64 ? 3 : 4;  // log2(pieces per group): a 64-bit division per piece would dominate the kernel
-    pot_status_t rc = POT_OK;
-#define POT_DQ(B)                                                                                     \
-    if (out_dtype == POT_F16) rc = launch_pdl(pot_dequant_kernel<B, 10>, dim3(grid), dim3(DQ_THREADS), 0, s, P, S, n_pieces, ppg, O); \
-    else rc = launch_pdl(pot_dequant_kernel<B, 7>, dim3(grid), dim3(DQ_THREADS), 0, s, P, S, n_pieces, ppg, O);
-    if (bits == 2) {
-        POT_DQ(2)
-    } else if (bits == 3) {
-        if (out_dtype == POT_F16) rc = launch_pdl(pot_dequant3_kernel<10>, dim3(grid), dim3(DQ_THREADS), 0, s, P, S, n_pieces, ppg, O);
-        else rc = launch_pdl(pot_dequant3_kernel<7>, dim3(grid), dim3(DQ_THREADS), 0, s, P, S, n_pieces, ppg, O);
-    } else {
-        POT_DQ(4)
-    }
-#undef POT_DQ
-    return rc;
+    auto run = [&](auto kernel, int threads, int per_thread) -> pot_status_t {
+        const int64_t per_block = (int64_t)threads * per_thread;
+        return launch_pdl(kernel, dim3((unsigned)((n_pieces + per_block - 1) / per_block)), dim3((unsigned)threads), 0, s, P, S, n_pieces, ppg, O);
+    };
+    // Blocks of DQ_THREADS threads with DQ_UNROLL pieces each; an SM holds eight.  Where they leave slots empty, less per thread and more
+    // blocks: 2 (4) bits, 2048 x 1024 2.6 (2.8) -> 2.2 us with one piece, 2048 x 2048 3.5 (3.6) -> 2.9 (3.0), 4096 x 2048 4.65 (5.0) -> 4.5
+    // (4.9) with two; 3072 x 3072, 1152 blocks, 4.8 (5.1) either way.  At 3 bits, where a block waits for all its loads, blocks of half
+    // as many threads as soon as there are more than SMs and their slots: 4096 x 3072 6.8 -> 6.5, 4096 x 4096 7.9 -> 7.7 us (2048 x
+    // 2048 3.7 -> 3.8; 28672 x 8192 85.9 either way).
+    const int64_t blocks = (n_pieces + DQ_THREADS * DQ_UNROLL - 1) / (DQ_THREADS * DQ_UNROLL);
+    auto with_type = [&](auto ebit) -> pot_status_t {
+        constexpr int E = decltype(ebit)::value;
+        auto plain = [&](auto b) -> pot_status_t {
+            constexpr int B = decltype(b)::value;
+            if (blocks <= 2 * kSmCount) return run(pot_dequant_kernel<B, E, 1>, DQ_THREADS, 1);
+            if (blocks <= 7 * kSmCount) return run(pot_dequant_kernel<B, E, 2>, DQ_THREADS, 2);
+            return run(pot_dequant_kernel<B, E, DQ_UNROLL>, DQ_THREADS, DQ_UNROLL);
+        };
+        if (bits == 2) return plain(std::integral_constant<int, 2>());
+        if (bits == 4) return plain(std::integral_constant<int, 4>());
+        return blocks > 7 * kSmCount ? run(pot_dequant3_kernel<E, DQ_THREADS / 2>, DQ_THREADS / 2, 4) : run(pot_dequant3_kernel<E, DQ_THREADS>, DQ_THREADS, 4);
+    };
+    return out_dtype == POT_F16 ? with_type(std::integral_constant<int, 10>()) : with_type(std::integral_constant<int, 7>());
 }
 
 extern "C" pot_status_t uint_dequant(const void* packed, const void* scales, const void* zeros, int64_t N, int64_t K,
