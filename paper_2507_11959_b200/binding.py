@@ -1,5 +1,5 @@
-"""Thin ctypes binding of the C-ABI library (``include/pot.h``), same names as the C entry
-points.  It only marshals arguments: every step of the path runs in the library's CUDA
+"""Thin binding of the C-ABI library (``include/pot.h``) by ctypes, and by a small C module for the calls of
+every token, same names as the C entry points.  It only marshals arguments: every step of the path runs in the library's CUDA
 kernels.  Tensors are torch CUDA tensors (PyTorch is used for device memory and streams
 only); there is no CPU fallback -- if the library is missing or fails to load, importing a
 symbol from it raises.
