@@ -80,8 +80,8 @@ const char* pot_status_string(pot_status_t s);
 size_t pot_packed_bytes(int64_t N, int64_t K, int bits);          /* N * K * bits / 8          */
 size_t pot_scales_bytes(int64_t N, int64_t K, int group);         /* N * (K / group) * 2       */
 /* Scratch needed by pot_gemv / uint_gemv with the tiled layout (arrival counters of the row
- * blocks + FP32 partial sums); may be 0.  The workspace must be ZERO before its first use; every
- * call leaves its counters at zero again, so consecutive calls of the SAME entry point with the
+ * blocks + FP32 partial sums, or marked sums on their way from CTA to CTA); may be 0.  The workspace must be ZERO before its
+ * first use; every call leaves its counters and marks at zero again, so consecutive calls of the SAME entry point with the
  * SAME (N, K, bits, group) may reuse one buffer without clearing it.  The position of the
  * counters inside the buffer depends on the shape: a buffer handed to a call with another shape
  * (or to pot_gemm) must be cleared to zero first.  Two calls that may run concurrently
@@ -97,14 +97,18 @@ uint64_t pot_launch_count(void);
  * device, return that word (0 = no wait ever gave up) and clear it.                                   */
 int pot_debug_gemv_error(void);
 /* Host arithmetic only: the launch plan pot_gemv (uniform = 0) / uint_gemv (uniform = 1) would use for a tiled shape:
- * CTAs per SM (1 or 2), whether CTA ranges end on row-block boundaries (1) or the units are split evenly and partial
- * sums cross CTAs through the workspace (0), slots per warp ring, units per slot (2, 4 or 8), and whether x is staged
- * in shared memory.                                                                                                  */
+ * CTAs per SM (1 or 2), whether whole row blocks would give every CTA the same work but for a fifth (1: PoT codes may still be
+ * split evenly, see pot_debug_gemv_split; 0: sums cross CTAs through the workspace), slots per warp ring, units per slot
+ * (2, 4 or 8), and whether x is staged in shared memory.                                                              */
 pot_status_t pot_debug_gemv_plan(int64_t N, int64_t K, int bits, int group, int uniform, int* ctas_per_sm,
                                  int* row_block_split, int* ring_slots, int* units_per_slot, int* x_in_smem);
 /* Host arithmetic only: how pot_gemv (bf16 = 0) / pot_gemv_bf16 (bf16 = 1) would decode a tiled shape: CTAs per SM, and whether
  * the codes are decoded without their scale (BF16: with x as FP16 numbers, where that is exact).                     */
 pot_status_t pot_debug_gemv_decode(int64_t N, int64_t K, int bits, int group, int bf16, int* ctas_per_sm, int* unscaled);
+/* Host arithmetic only: how pot_gemv / pot_gemm with M <= 8 tokens (bf16 = 0), or their BF16 forms, divide a tiled shape among the CTAs: 0 whole
+ * row blocks, 1 the same number of units for every warp (the last one to deliver a row block's sums adds them up), 2 the same number of units for
+ * every CTA (a row block has two CTAs at most, the second of which hands its sums to the first).                       */
+pot_status_t pot_debug_gemv_split(int64_t M, int64_t N, int64_t K, int bits, int group, int bf16, int* split);
 /* Host arithmetic only: how pot_gemv runs canonical codes: warps that share a row block (16 rows) in a CTA, warps per CTA, CTAs of
  * a cluster that share a row block; 0, 8, 0 where x is too long for shared memory (one warp per row).                  */
 pot_status_t pot_debug_canonical_gemv_plan(int64_t N, int64_t K, int bits, int* warps_per_row_block, int* warps_per_cta, int* ctas_per_row_block);

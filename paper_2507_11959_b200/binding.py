@@ -29,7 +29,7 @@ EXPORTS = [
     "pot_status_string", "pot_packed_bytes", "pot_scales_bytes", "pot_gemv_workspace_bytes",
     "pot_gemm_workspace_bytes", "pot_launch_count", "pot_quantize_ref", "pot_validate_scales", "pot_repack", "pot_repack_scales", "pot_layout_scale_index",
     "uint_repack", "pot_dequant", "pot_gemv", "pot_gemv_bf16", "pot_gemv_host", "pot_gemm", "pot_gemm_bf16", "uint_quantize_ref", "uint_dequant",
-    "uint_gemv", "pot_layout_bit", "pot_gemv_noalloc", "pot_gemv_noalloc_max_scratch_bytes", "pot_debug_gemv_error", "pot_debug_gemv_plan", "pot_debug_gemv_decode", "pot_debug_canonical_gemv_plan", "pot_debug_gemm_plan", "pot_debug_gemm_cluster", "pot_debug_canonical_splits", "pot_debug_gemm_error", "pot_debug_prefill_error",
+    "uint_gemv", "pot_layout_bit", "pot_gemv_noalloc", "pot_gemv_noalloc_max_scratch_bytes", "pot_debug_gemv_error", "pot_debug_gemv_plan", "pot_debug_gemv_decode", "pot_debug_gemv_split", "pot_debug_canonical_gemv_plan", "pot_debug_gemm_plan", "pot_debug_gemm_cluster", "pot_debug_canonical_splits", "pot_debug_gemm_error", "pot_debug_prefill_error",
 ]
 
 _lib = None
@@ -68,6 +68,7 @@ def lib() -> ctypes.CDLL:
         L.pot_repack_scales.argtypes = [vp, vp, i64, i64, i32, i32, vp]
         L.pot_debug_gemv_plan.argtypes = [i64, i64, i32, i32, i32, vp, vp, vp, vp, vp]
         L.pot_debug_gemv_decode.argtypes = [i64, i64, i32, i32, i32, vp, vp]
+        L.pot_debug_gemv_split.argtypes = [i64, i64, i64, i32, i32, i32, vp]
         L.pot_debug_canonical_gemv_plan.argtypes = [i64, i64, i32, vp, vp, vp]
         L.pot_debug_gemm_plan.argtypes = [i64, i64, i64, i32, i32, i32] + [vp] * 8
         L.pot_debug_gemm_cluster.argtypes = [i64, i64, i64, i32, i32, i32, vp]
@@ -364,6 +365,13 @@ def pot_debug_gemv_decode(N: int, K: int, bits: int, group: int, bf16: bool = Fa
     v = [ctypes.c_int(-1) for _ in range(2)]
     _check(lib().pot_debug_gemv_decode(N, K, bits, group, 1 if bf16 else 0, *[ctypes.byref(x) for x in v]), "pot_debug_gemv_decode")
     return dict(zip(("ctas_per_sm", "unscaled"), (x.value for x in v)))
+
+
+def pot_debug_gemv_split(M: int, N: int, K: int, bits: int, group: int, bf16: bool = False) -> int:
+    """How M <= 8 tokens on a tiled shape are divided among the CTAs: 0 whole row blocks, 1 units among warps, 2 units among CTAs."""
+    v = ctypes.c_int()
+    _check(lib().pot_debug_gemv_split(M, N, K, bits, group, 1 if bf16 else 0, ctypes.byref(v)), "pot_debug_gemv_split")
+    return v.value
 
 
 def pot_debug_canonical_gemv_plan(N: int, K: int, bits: int) -> tuple[int, int, int]:

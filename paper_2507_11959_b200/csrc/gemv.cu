@@ -354,6 +354,17 @@ extern "C" pot_status_t pot_debug_gemv_plan(int64_t N, int64_t K, int bits, int 
     *x_in_smem = p.x_in_smem ? 1 : 0;
     return POT_OK;
 }
+extern "C" pot_status_t pot_debug_gemv_split(int64_t M, int64_t N, int64_t K, int bits, int group, int bf16, int* split) {
+    if (!split) return POT_ERR_NULL;
+    const pot_status_t st = check_shape(N, K, bits, group);
+    if (st != POT_OK) return st;
+    if (M < 1 || M > 8 || N % 16 != 0) return POT_ERR_SHAPE;
+    const int dt = bf16 ? 1 : 0, tok = M == 1 ? 1 : 8, occ = M == 1 ? gemv_occupancy(N, K, bits, group, SK_POT, dt) : 1;
+    const StreamPlan p = plan_stream(N, K, M, bits, group, SK_POT, tok, 16, occ, dt);
+    if (!p.ok) return POT_ERR_SHAPE;
+    *split = p.even ? 2 : (p.aligned ? 0 : 1);
+    return POT_OK;
+}
 extern "C" pot_status_t pot_debug_canonical_gemv_plan(int64_t N, int64_t K, int bits, int* warps_per_row_block, int* warps_per_cta, int* ctas_per_row_block) {
     if (!warps_per_row_block || !warps_per_cta || !ctas_per_row_block) return POT_ERR_NULL;
     const pot_status_t st = check_shape(N, K, bits, 128);
@@ -511,10 +522,11 @@ extern "C" pot_status_t pot_gemv_noalloc(const void* packed_tiled, const void* s
     st = check_gemv_args(packed_tiled, scales, N, K, bits, group, POT_LAYOUT_TILED, x, y, scratch, kNoAllocScratchBytes);
     if (st != POT_OK) return st;  // nothing has been enqueued yet
     if (need == 0) return pot_gemv(packed_tiled, scales, N, K, bits, group, POT_LAYOUT_TILED, x, y, nullptr, 0, stream);
-    // The array keeps whatever the previous call left in it.  Only the arrival counters have to start
-    // at zero (the partial sums are fully overwritten before they are read), so clear just those.
-    const size_t counters_bytes = plan_stream(N, K, 1, bits, group, SK_POT, 1, 16).ws_counters;
-    if (cudaMemsetAsync(scratch, 0, counters_bytes, (cudaStream_t)stream) != cudaSuccess) return POT_ERR_CUDA;
+    // The array keeps whatever the previous call left in it.  Only the arrival counters, or the places of the sums that go from
+    // CTA to CTA, have to start at zero (partial sums are fully overwritten before they are read), so clear just those.
+    size_t clear = plan_stream(N, K, 1, bits, group, SK_POT, 1, 16).ws_counters;
+    if (clear < sk_box_bytes(1)) clear = sk_box_bytes(1);
+    if (cudaMemsetAsync(scratch, 0, clear, (cudaStream_t)stream) != cudaSuccess) return POT_ERR_CUDA;
     return pot_gemv(packed_tiled, scales, N, K, bits, group, POT_LAYOUT_TILED, x, y, scratch, need, stream);
 }
 

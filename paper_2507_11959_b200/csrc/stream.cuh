@@ -1,9 +1,9 @@
 // Streaming kernel for the decode GEMV (PoT and the uniform twin) and the small-batch GEMM on the tiled layout.
 //
 // Work decomposition.  The matrix is a sequence of units (16 rows x 128 columns, stored contiguously in
-// [row block][column block] order, codes and per-group parameters alike).  The U units are cut into grid * W equal,
-// contiguous ranges, one per consumer warp of the grid (W warps per CTA), so a CTA -- and every warp in it -- streams one
-// contiguous byte range and all SMs move the same number of bytes (+- one unit per warp).
+// [row block][column block] order, codes and per-group parameters alike).  A CTA -- and every warp in it -- streams a contiguous
+// byte range (the even split: a warp two).  Three splits: whole row blocks per CTA; the same number of units for every CTA
+// (even split, where the matrix has a row block for each); the same number for every warp of the grid (unit split).
 //
 // Every warp is its own streaming engine: it owns a private ring of S slots of Q units in shared memory; lane 0 requests
 // a slot's codes and scales with 1-D bulk copies (cp.async.bulk + mbarrier transaction bytes), the warp waits for the
@@ -22,7 +22,8 @@
 //
 // Delivery.  A warp that covered a whole row block writes Y.  Otherwise its sums go to slot (row block, position of the
 // warp among the row block's contributors) of the workspace; a per-row-block arrival counter tells the last contributor,
-// which adds the slots in ascending order -- the result does not depend on timing, and no warp ever waits for another.
+// which adds the slots in ascending order -- the result does not depend on timing, and no warp waits for another (even split: see
+// stream_even.cuh).
 #pragma once
 #include "common.cuh"
 #include "layout.cuh"
@@ -50,6 +51,12 @@ __host__ __device__ constexpr int sk_header_bytes(int warps, int tok) {
     return (warps * 64 + warps * 32 + warps * 4 + warps * 2 * 16 * tok * 4 + 127) / 128 * 128;
 }
 
+// ---- even split (stream_even.cuh)
+// units that are dealt out together (straight-line code; with two of the four in a slot 12288 x 4096 took 8.2 instead of 7.3 us)
+__host__ __device__ constexpr int sk_block(int q) { return q == 2 ? 2 : 4; }
+// the workspace holds a number and a mark, 8 bytes, for each sum that goes from CTA to CTA (16 rows x tok of each CTA)
+constexpr size_t sk_box_bytes(int tok) { return (size_t)kSmCount * 16 * (size_t)tok * 8; }
+
 struct StreamPlan {
     int grid, warps;      // CTAs; consumer warps per CTA
     int ncb;              // column blocks (units per row block)
@@ -65,7 +72,9 @@ struct StreamPlan {
     size_t x_bytes, smem_bytes;
     int max_slots;        // partial-sum slots per row block
     size_t ws_counters, ws_bytes;
-    bool aligned;         // CTA ranges end on row-block boundaries (no partial sums cross CTAs)
+    bool aligned;         // whole row blocks per CTA would differ by a fifth at most
+    bool even;            // even split: see plan_stream
+    uint32_t cta_blocks, cta_more;  // ... of sk_block(q) units: every CTA has cta_blocks of them, the first cta_more CTAs one more
     int nrb;
     bool ok;              // false: the shape cannot run on this kernel (too many units)
 };
@@ -134,6 +143,27 @@ inline StreamPlan plan_stream(int64_t N, int64_t K, int64_t M, int bits, int gro
     if (st > need) st = need;
     if (st > 8) st = 8;
     if (st < 1) st = 1;
+    // Even split (PoT codes): every CTA takes the same number of blocks of units, wherever row blocks end.  A range is at least a row block
+    // long, so that a row block has two CTAs at most.  Instead of the unit split always (us: 2480 x 4096 5.7 -> 3.7, 2400 x 8192 6.9 -> 5.4, 7136 x
+    // 4096 7.6 -> 5.4, 5120 x 13824 12.4 -> 11.4, eight layers of 2048 / 5504 260 -> 227, of 3200 / 8576 270 -> 232); all calls of a shape then keep the
+    // same things in the workspace.  Instead of whole row blocks with one CTA per SM, whose launch nothing hides and which gains by the shorter way
+    // to the first copies: one token always but at 2 bits in BF16 (28672 x 8192 25.0 -> 23.1, 15360 x 8192 17.0 -> 14.7, whole row blocks of
+    // 18944 x 8192 17.1 -> 16.7; BF16, 2 bits 17792 x 7552 15.7 -> 16.4); several tokens, whose sums cost more on their way, where the longest
+    // CTA gets rid of 16 units: 15360 x 5120 (20 units) 12.8 -> 11.3 at 2 tokens, 13.4 -> 12.5 at 4; 4096 x 11008 (23, but of two row
+    // blocks) 10.4 -> 12.0, 8 tokens x 15360 x 5120 13.9 -> 14.3.  Two CTAs per SM: alone 12288 x 4096 7.8 -> 7.3, but 11008 x 4096 6.9 -> 7.25, 4096 x 4096 3.5
+    // -> 4.2, and nothing is left where such launches follow one another (eight layers of 4096 / 11008 274 -> 276, 2 bits 245 -> 250).
+    const int64_t block = sk_block(q), blocks = (U + block - 1) / block, saved = rb_max * ncb - U / p.grid;
+    p.even = kind == SK_POT && p.grid == kSmCount && U / 4 / p.grid * 4 >= ncb && ncb > 1 &&
+             (!p.aligned || (occ == 1 && (tok == 1 ? dt == 0 || bits > 2 : M <= 4 && rb_max >= 3 && saved >= 16)));
+    p.cta_blocks = (uint32_t)(blocks / p.grid);
+    p.cta_more = (uint32_t)(blocks % p.grid);
+    if (p.even) {  // a warp has a part of the CTA's first row block, if that is shared, and a part of the rest
+        const int64_t most = (block * ((p.cta_blocks + 2 + warps) / warps) + q - 1) / q + 1;
+        st = (int64_t)((budget - hdr - p.x_bytes) / ((size_t)warps * slot));
+        if (st > most) st = most;
+        if (st > 8) st = 8;
+        if (st < 1) st = 1;
+    }
     p.stages = (int)st;
     p.smem_bytes = hdr + p.x_bytes + (size_t)warps * (size_t)p.stages * slot;
     const int64_t m = U / GW;  // shortest warp range
@@ -141,6 +171,7 @@ inline StreamPlan plan_stream(int64_t N, int64_t K, int64_t M, int bits, int gro
     if (slots > ncb) slots = ncb;
     p.max_slots = (int)slots;
     p.ws_counters = ((size_t)nrb * 4 + 255) / 256 * 256;
+    // (no smaller than sk_box_bytes(tok) with a row block for every CTA: two slots per row block at least)
     p.ws_bytes = ncb > 1 ? p.ws_counters + (size_t)nrb * (size_t)slots * 16 * (size_t)tok * 4 : 0;
     return p;
 }
@@ -170,6 +201,12 @@ struct StreamArgsUnscaled : StreamArgs {
     uint32_t p2[potl::POT_UNIT_SHIFTS];  // p2[n] = 2^n
     uint32_t zeros_at;                   // shared-memory offset of SK_ZERO_BYTES that are cleared (one group per unit: any that are free)
     uint32_t factors_at;                 // BF16: shared-memory offset of one FP32 factor per unit
+};
+// ... and only the even split
+struct StreamArgsEven : StreamArgsUnscaled {
+    uint32_t cta_blocks, cta_more;  // blocks of sk_block(q) units per CTA; the first cta_more CTAs have one more
+    uint32_t ncb_mul;               // u / ncb = (u * ncb_mul) >> ncb_shift for u < 2^31
+    int ncb_shift;
 };
 template <bool UNSC>
 using StreamKernelArgs = typename std::conditional<UNSC, StreamArgsUnscaled, StreamArgs>::type;
@@ -803,6 +840,10 @@ constexpr auto stream_kernel_of() {
 }
 #endif  // __CUDACC__
 
+}  // namespace pot
+#include "stream_even.cuh"
+namespace pot {
+
 #ifdef SK_TRACE
 inline unsigned long long* g_sk_trace = nullptr;   // next launch's trace block (advanced per launch)
 #endif
@@ -861,6 +902,27 @@ pot_status_t launch_stream(const void* packed, const void* scales, const void* z
     constexpr bool POT = KIND == SK_POT;
     auto pick = [&](auto q) -> pot_status_t {  // q units per slot
         constexpr int Q = decltype(q)::value;
+        if constexpr (POT) {
+            if (p.even) {
+                StreamArgsEven even;
+                static_cast<StreamArgsUnscaled&>(even) = args;
+                if (group == 128) even.zeros_at = (uint32_t)sk_even_slots_at(W);
+                even.cta_blocks = p.cta_blocks;
+                even.cta_more = p.cta_more;
+                even.ncb_shift = 31;  // (Granlund and Montgomery 1994, "Division by invariant integers using multiplication")
+                while ((int64_t(1) << (even.ncb_shift - 31)) < p.ncb) ++even.ncb_shift;
+                even.ncb_mul = (uint32_t)(((uint64_t(1) << even.ncb_shift) + (uint64_t)p.ncb - 1) / (uint64_t)p.ncb);
+                auto run_even = [&](auto kernel) -> pot_status_t {
+                    return launch_pdl_cluster(kernel, dim3((unsigned)p.grid), dim3(W * 32), p.smem_bytes, 1, true, s, even, err);
+                };
+                if constexpr (DT == 0 || TOK == 1)
+                    if (p.unscaled) return run_even(stream_even_kernel<BITS, TOK, true, W, OCC, Q, DT, true>);
+                if constexpr (!(DT == 0 && TOK == 1))
+                    if (p.x_in_smem) return run_even(stream_even_kernel<BITS, TOK, true, W, OCC, Q, DT, false>);
+                if constexpr (OCC == 1 && Q == 2) return run_even(stream_even_kernel<BITS, TOK, false, W, OCC, Q, DT, false>);
+                else return POT_ERR_SHAPE;
+            }
+        }
         if constexpr (POT && (DT == 0 || TOK == 1))
             if (p.unscaled) return run(stream_kernel_of<BITS, KIND, TOK, true, W, OCC, Q, DT, true>());
         if constexpr (!(POT && DT == 0 && TOK == 1))

@@ -1,0 +1,557 @@
+// The streaming kernel of stream.cuh with the units dealt out evenly to the CTAs (PoT codes; plan_stream says where).  As there: warps with rings of
+// their own, decode, MMAs.  Different: which units a warp works on, and the way of the sums.
+//
+// CTA c takes the blocks of units c * cta_blocks + min(c, cta_more) .., as much as every other CTA but for one block.  A range that begins
+// inside a row block begins with a part that the CTA before has the rest of.  All warps work on this part first, and its sums are left in the
+// workspace for that CTA, which adds them to its own when it has come to its end.  Then the warps cut up the other units.  Row blocks that
+// warps share are added up in shared memory by the last one that delivers; the order of additions is fixed.
+// What bounds it: as in stream.cuh.  What the split takes away is the unequal ends: of whole row blocks (28672 x 8192: 16 CTAs have 13 row blocks, 132
+// have 12), of a row block's many contributors (unit split).  Where the kernel has an SM to itself nothing hides its launch: it asks for one
+// chunk per warp, then for the activations, then for the rest of the ring (with all chunks first the activations arrive behind them:
+// 28672 x 8192 24.3 us, so 23.1), and divisions by the number of column blocks are multiplications (the ranges took 1200 cycles).  Before -> after:
+// 28672 x 8192 25.0 -> 23.1 us (3 bits), 28.3 -> 27.7 (4 bits, BF16), 5120 x 13824 12.4 -> 11.4, 2400 x 8192 6.9 -> 5.4, 4 tokens x 15360 x 5120 13.4 -> 12.5.
+#pragma once
+#include "stream.cuh"
+
+#ifdef __CUDACC__
+namespace pot {
+
+__device__ __forceinline__ void st_relaxed64(unsigned long long* p, unsigned long long v) {
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+__device__ __forceinline__ unsigned long long ld_relaxed64(const unsigned long long* p) {
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+// shared-memory header: as sk_header_bytes, with four words between the local arrival counters and the slots of partial sums
+__host__ __device__ constexpr int sk_even_counters_at(int warps) { return warps * 96; }
+__host__ __device__ constexpr int sk_even_slots_at(int warps) { return warps * 100 + 16; }
+
+// Template parameters as of stream_kernel.
+template <int BITS, int TOK, bool XSMEM, int W, int OCC, int SK_Q, int DT, bool UNSC>
+__global__ void __launch_bounds__(W * 32, OCC) stream_even_kernel(const __grid_constant__ StreamArgsEven sa, int* __restrict__ err) {
+    constexpr int UB = sk_unit_bytes(BITS);
+    static_assert(!UNSC || (XSMEM && (DT == 0 || TOK == 1)), "the decode without the scale: x in shared memory, BF16 one token");
+    constexpr bool FACTORS = UNSC && DT == 1;
+    extern __shared__ __align__(128) unsigned char smem[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int gid = lane >> 2, tig = lane & 3;  // MMA fragment coordinates: rows gid and gid + 8, quarter tig
+#ifdef SK_TRACE
+    auto stamp = [&](int i) {
+        if (sa.trace && lane == 0 && (warp == 0 || warp == W - 1)) {
+            unsigned long long t;
+            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+            sa.trace[((size_t)blockIdx.x * 2 + (warp ? 1 : 0)) * 8 + i] = t;
+        }
+    };
+    stamp(0);
+#else
+    auto stamp = [&](int) {};
+#endif
+    const int S = sa.stages;
+    const int spg = 128 / sa.group;
+    const uint32_t PB = 32u * (uint32_t)spg;                 // parameter bytes of one unit
+    const uint32_t slot_bytes = SK_Q * (UB + PB);
+    const uint32_t smem0 = smem_u32(smem);
+    const uint32_t bars = smem0 + (uint32_t)warp * 64u;      // this warp's full barriers (S <= 8)
+    constexpr int HDR = sk_header_bytes(W, TOK);
+    static_assert(sk_even_slots_at(W) + W * 2 * 16 * TOK * 4 <= HDR && sk_even_slots_at(W) % 16 == 0 && SK_ZERO_BYTES <= W * 2 * 16 * TOK * 4, "the header holds it");
+    // What a warp needs only when it requests a chunk or delivers sums: [0] first unit, [1] number of units of its own range; [2], [3] the same of its
+    // part of the CTA's first row block; [4] first, [5] last row block of its range; [6] the warps of the CTA that share the first (lower half)
+    // and the last (upper half) of these; [7] number of chunks
+    uint32_t* wst = reinterpret_cast<uint32_t*>(smem + W * 64) + warp * 8;
+    // local arrival counters; [W] the same of the CTA's part of its first row block, [W + 1] its sums have been added up, [W + 2] the warps that
+    // have a part, [W + 3] the row block that the next CTA has a part of
+    unsigned* lcnt = reinterpret_cast<unsigned*>(smem + sk_even_counters_at(W));
+    float* lslots = reinterpret_cast<float*>(smem + sk_even_slots_at(W));           // [warp][first, last][16 TOK]
+    const unsigned char* xs = smem + HDR;
+    const unsigned char* ringp = xs + sa.x_bytes + (uint32_t)warp * (uint32_t)S * slot_bytes;  // this warp's ring
+    const uint32_t ring = smem0 + (uint32_t)HDR + (uint32_t)sa.x_bytes + (uint32_t)warp * (uint32_t)S * slot_bytes;
+
+    // ---- this warp's ranges ----------------------------------------------------------------------------------
+    const uint32_t ncb = (uint32_t)sa.ncb;
+    constexpr uint32_t BLOCK = sk_block(SK_Q);
+    auto div_ncb = [&](uint32_t u) { return (uint32_t)(((uint64_t)u * sa.ncb_mul) >> sa.ncb_shift); };
+    auto part = [&](uint32_t blocks, uint32_t w) { return w * (blocks / W) + min(w, blocks % W); };
+    const uint32_t base = (blockIdx.x * sa.cta_blocks + min(blockIdx.x, sa.cta_more)) * BLOCK;  // the CTA's units
+    const uint32_t units = min(base + (sa.cta_blocks + (blockIdx.x < sa.cta_more ? 1u : 0u)) * BLOCK, sa.units) - base;
+    const uint32_t first_rb = div_ncb(base), inside = base - first_rb * ncb;
+    const uint32_t lead = inside ? ncb - inside : 0u, rest = units - lead;                      // ... of a row block that the CTA before began; the others
+    const uint32_t lead_blocks = (lead + BLOCK - 1) / BLOCK, all_blocks = lead_blocks + (rest + BLOCK - 1) / BLOCK;
+    const uint32_t l0 = part(lead_blocks, warp), l1 = part(lead_blocks, warp + 1);
+    const uint32_t la = base + min(l0 * BLOCK, lead), ln = base + min(l1 * BLOCK, lead) - la;
+    const uint32_t a = base + lead + min((part(all_blocks, warp) - l0) * BLOCK, rest);
+    const uint32_t n = base + lead + min((part(all_blocks, warp + 1) - l1) * BLOCK, rest) - a;
+    const uint32_t lchunks = (ln + SK_Q - 1) / SK_Q, nchunks = lchunks + (n + SK_Q - 1) / SK_Q;
+
+    // chunk j holds units [a + Q j, a + Q j + Q) (fewer at the end) and lives in slot j % S; the part of the shared row block comes first
+    auto issue = [&](uint32_t a_, uint32_t n_, uint32_t la_, uint32_t ln_, uint32_t j, uint32_t s) {  // one lane: request chunk j into slot s
+        const uint32_t lc = (ln_ + SK_Q - 1) / SK_Q, jj = j < lc ? j : j - lc;
+        const uint32_t u0 = (j < lc ? la_ : a_) + jj * SK_Q, left_j = (j < lc ? ln_ : n_) - jj * SK_Q;
+        const uint32_t cnt = left_j < (uint32_t)SK_Q ? left_j : (uint32_t)SK_Q;
+        const uint32_t bar = bars + s * 8u, dst = ring + s * slot_bytes;
+        if (!in_range(s < (uint32_t)S && (uint64_t)u0 + cnt <= sa.units && cnt >= 1 && cnt <= (uint32_t)SK_Q, err, 0x110)) return;
+        mbar_expect_tx(bar, cnt * (UB + PB));
+        bulk_g2s(dst, sa.packed + (size_t)u0 * UB, cnt * UB, bar);
+        bulk_g2s(dst + SK_Q * UB, sa.scales + (size_t)u0 * PB, cnt * PB, bar);
+    };
+    constexpr bool late = OCC == 1 && XSMEM;   // only the first chunk before the activations
+    if (lane < S) {  // lane s sets up slot s and requests chunk s: the weights do not depend on the predecessor
+        mbar_init(bars + (uint32_t)lane * 8u, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    auto request = [&](uint32_t from, uint32_t to) {
+        if ((uint32_t)lane >= from && (uint32_t)lane < to && lane < S && (uint32_t)lane < nchunks) issue(a, n, la, ln, (uint32_t)lane, (uint32_t)lane);
+    };
+    // Two CTAs per SM: this one's first copies, 100 KB, would be in the way of the activations that the one beside it, of the launch before, is
+    // just waiting for (eight layers of 3200 / 8576 240 us, with this pause 232; of 2048 / 5504 222 and 227; 300 ns: 235, 224).
+    if constexpr (OCC == 2) __nanosleep(1000);
+    request(0, late ? 1u : 8u);
+    __syncwarp();
+    stamp(7);
+    pdl_launch_dependents();
+
+    // ---- row blocks of the range; which of its segments are partial, and their place among the contributors
+    uint32_t rb = 0, cb = 0;
+    auto row_blocks = [&]() {
+        const uint32_t start = base + lead, r1 = first_rb + (lead ? 1u : 0u), m0 = a - start;
+        const uint32_t q0 = div_ncb(m0), qL = n ? div_ncb(m0 + n - 1) : q0, full = div_ncb(rest);
+        rb = r1 + q0;
+        cb = m0 - q0 * ncb;
+        // the warps whose ranges touch the first and the last row block of this one's
+        const uint32_t w = min((uint32_t)lane, (uint32_t)W - 1u);
+        const uint32_t f = min((part(all_blocks, w) - part(lead_blocks, w)) * BLOCK, rest), e = min((part(all_blocks, w + 1) - part(lead_blocks, w + 1)) * BLOCK, rest);
+        const uint32_t m_first = __ballot_sync(0xffffffffu, lane < W && f < e && f < (q0 + 1) * ncb && e > q0 * ncb);
+        const uint32_t m_last = __ballot_sync(0xffffffffu, lane < W && f < e && f < (qL + 1) * ncb && e > qL * ncb);
+        if (lane == 0) {
+            wst[0] = a; wst[1] = n; wst[2] = la; wst[3] = ln; wst[4] = rb; wst[5] = r1 + qL;
+            wst[6] = m_first | (m_last << 16);
+        }
+        if (threadIdx.x == 0) {
+            lcnt[W + 2] = 0xFFFFu >> (16u - min(lead_blocks, (uint32_t)W));
+            lcnt[W + 3] = rest != full * ncb ? r1 + full : 0xffffffffu;
+        }
+        static_assert(W <= 16, "sets of warps in 16 bits");
+        if (lane == 0) wst[7] = nchunks;
+        if (threadIdx.x < W + 2) lcnt[threadIdx.x] = 0u;
+    };
+    // Two CTAs per SM: this one waits anyway.  One: its predecessor on the SM has gone, and so, most of the time, has the previous kernel;
+    // the activations are asked for first.
+    if (!late) row_blocks();
+    [[maybe_unused]] auto behind_loads = [&]() {
+        if (late) {
+            request(1, 8);
+            row_blocks();
+        }
+    };
+
+    stamp(1);
+    pdl_wait();  // x, Y and the workspace may belong to the previous kernel in the stream
+    stamp(2);
+    float* factors = nullptr;  // BF16 without the scale: one per unit
+    if constexpr (FACTORS) factors = reinterpret_cast<float*>(smem + sa.factors_at);
+    bool inexact = false;
+    if constexpr (XSMEM) {
+        uint4* dst = reinterpret_cast<uint4*>(smem + HDR);
+        const uint4* src = reinterpret_cast<const uint4*>(sa.X);
+        const int kc = (int)(sa.K / 8);  // 16-byte chunks per token
+        if constexpr (UNSC && TOK == 1)
+            if (threadIdx.x < SK_ZERO_BYTES / 16) *reinterpret_cast<uint4*>(smem + sa.zeros_at + threadIdx.x * 16) = make_uint4(0, 0, 0, 0);
+        if constexpr (TOK == 1) {
+            // chunk (quarter t, part j) of a unit goes to position j * 4 + t: lanes tig = 0..3 read 64 contiguous bytes
+            // (four loads in flight per thread before the first store: one round trip for K <= 32 * 32 W)
+            // (a bound for whole warps, here and below: 0.5 - 0.8 % of an eight-layer token in the two-CTA build)
+            if (OCC == 1 && (int)(threadIdx.x & ~31u) >= kc) behind_loads();  // (a warp that loads nothing)
+            for (int i0 = threadIdx.x; (i0 & ~31) < kc; i0 += 4 * W * 32) {
+                uint4 v[4];
+#pragma unroll
+                for (int p = 0; p < 4; ++p)
+                    if (i0 + p * W * 32 < kc) v[p] = ld_dependent16(src + i0 + p * W * 32);
+                if (OCC == 1 && i0 == threadIdx.x) behind_loads();
+#pragma unroll
+                for (int p = 0; p < 4; ++p) {
+                    const int i = i0 + p * W * 32;
+                    if constexpr (FACTORS) {  // lanes 0-15 and 16-31 hold one unit each
+                        const float f = sk_normalize(v[p], i < kc);
+                        inexact = inexact || (i < kc && f < 0.f);
+                        if (i < kc && (i & 15) == 0) factors[i >> 4] = f * potl::POT_UNIT_SCALE;
+                    }
+                    if (i < kc) dst[(i & ~15) | ((i & 3) << 2) | ((i >> 2) & 3)] = v[p];
+                }
+            }
+        } else {
+            // T = 2, 4 or 8 token slots (the smallest that holds M).  Chunk (token, unit, quarter t, part j) goes to
+            // 16-byte slot (unit * 4 + j) * 4 T + (token / 2) * 8 + (token % 2) * 4 + t: the eight lanes of a quarter-warp
+            // of the MMA loop (tokens 2q and 2q + 1, quarters 0..3) read one 128-byte line, a warp 4 lines -- no bank
+            // conflict (token-major slots cost four-way conflicts: 11 against 8 us in the loop at 5+ tokens).  With fewer
+            // than 8 slots the MMA columns beyond T repeat the first T tokens; they are never delivered, like the
+            // tokens >= M.  The threads are numbered so that a quarter-warp also STORES one line: t fastest, then the
+            // token's parity, then j -- a warp loads the 256 contiguous bytes of a unit for two tokens.
+            const int ts = sa.token_shift;
+            const int total = kc << ts;
+            if (OCC == 1 && (int)(threadIdx.x & ~31u) >= total) behind_loads();
+            for (int e0 = threadIdx.x; (e0 & ~31) < total; e0 += 8 * W * 32) {  // eight loads in flight per thread
+                uint4 v[8];
+#pragma unroll
+                for (int p = 0; p < 8; ++p) {
+                    const int e = e0 + p * W * 32;
+                    const int t = e & 3, par = (e >> 2) & 1, j = (e >> 3) & 3, hi = (e >> 5) & ((1 << (ts - 1)) - 1), unit_ = e >> (4 + ts);
+                    const int token = (hi << 1) | par;
+                    if (e < total && token < sa.M) v[p] = ld_dependent16(src + (int64_t)token * kc + unit_ * 16 + t * 4 + j);
+                }
+                if (OCC == 1 && e0 == threadIdx.x) behind_loads();
+#pragma unroll
+                for (int p = 0; p < 8; ++p) {
+                    const int e = e0 + p * W * 32;
+                    const int t = e & 3, par = (e >> 2) & 1, j = (e >> 3) & 3, hi = (e >> 5) & ((1 << (ts - 1)) - 1), unit_ = e >> (4 + ts);
+                    const int token = (hi << 1) | par;
+                    if (e < total && token < sa.M) dst[(((unit_ << 2) + j) << (2 + ts)) + (hi << 3) + (par << 2) + t] = v[p];
+                }
+            }
+        }
+    }
+    if constexpr (FACTORS) inexact = __syncthreads_or(inexact);
+    else __syncthreads();
+    stamp(3);
+
+    float acc[2][4];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[i][e] = 0.f;
+
+    // ---- delivery of the sums of rows [16 rb, 16 rb + 16) accumulated so far ---------------------------------
+    auto deliver = [&](uint32_t rbd, bool shared_first) {
+        float v[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            v[e] = acc[0][e] + acc[1][e];
+            acc[0][e] = 0.f;
+            acc[1][e] = 0.f;
+        }
+        if constexpr (UNSC) {
+            if constexpr (TOK == 1) {
+                if (spg == 2) {  // the second group's sums sit in lanes tig = 2, 3
+                    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+                    v[2] += __shfl_xor_sync(0xffffffffu, v[2], 2);
+                }
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if constexpr (!FACTORS) v[e] *= potl::POT_UNIT_SCALE;
+        }
+        const int64_t row0 = (int64_t)rbd * 16;
+        auto store = [&]() {
+            if constexpr (TOK == 1) {
+                if (tig == 0 && in_range(row0 + gid + 8 < sa.N, err, 0x120)) {
+                    sa.Y[row0 + gid] = sk_out<DT>(v[0]);
+                    sa.Y[row0 + gid + 8] = sk_out<DT>(v[2]);
+                }
+            } else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int token = 2 * tig + (e & 1);
+                    if (token < sa.M && in_range(row0 + gid + 8 * (e >> 1) < sa.N, err, 0x121))
+                        sa.Y[(int64_t)token * sa.N + row0 + gid + 8 * (e >> 1)] = sk_out<DT>(v[e]);
+                }
+            }
+        };
+        // the warps of this CTA that have a part of the row block; whether the next CTA has one
+        const uint4 mine4 = *reinterpret_cast<const uint4*>(wst + 4), cta4 = *reinterpret_cast<const uint4*>(lcnt + W);
+        const bool next_cta = !shared_first && rbd == cta4.w;
+        const uint32_t sharers = shared_first ? cta4.z : (rbd == mine4.x ? mine4.z & 0xFFFFu : (rbd == mine4.y ? mine4.z >> 16 : 1u << warp));
+        if (!shared_first && !next_cta && (sharers & (sharers - 1u)) == 0) {
+            store();
+            return;
+        }
+        // slot of warp w: [w][1] if w is the row block's first contributor, else [w][0]; the shared first row block, which is done before a
+        // warp begins with its own range: [w][0]
+        const uint32_t wl = (uint32_t)__ffs(sharers) - 1u, wh = 31u - (uint32_t)__clz(sharers);
+        const bool begins = !shared_first && (uint32_t)warp == wl;
+        if (!in_range(row0 + 16 <= sa.N && ((sharers >> warp) & 1u) && wh < (uint32_t)W && (!(shared_first || next_cta) || sa.counters != nullptr), err, 0x131)) return;
+        if (!shared_first && !begins && wst[3] != 0) {  // [w][0] may still hold sums of the shared row block
+            volatile unsigned* taken = lcnt + W + 1;
+            uint32_t i = 0;
+            while (*taken == 0 && ++i < kSpinLimit) {}
+            __syncwarp();
+            if (__any_sync(0xffffffffu, i >= kSpinLimit)) {
+                if (err && lane == 0) atomicCAS(err, 0, 3 | (warp << 24));
+                return;
+            }
+        }
+        float* mine = lslots + ((size_t)warp * 2 + (begins ? 1 : 0)) * (16 * TOK);
+        if constexpr (TOK == 1) {
+            if (tig == 0) {
+                mine[gid] = v[0];
+                mine[gid + 8] = v[2];
+            }
+        } else {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) mine[(2 * tig + (e & 1)) * 16 + gid + 8 * (e >> 1)] = v[e];
+        }
+        __threadfence_block();
+        __syncwarp();
+        unsigned prev = 0;
+        if (lane == 0) prev = atomicAdd(&lcnt[shared_first ? (uint32_t)W : wl], 1u);
+        prev = __shfl_sync(0xffffffffu, prev, 0);
+        if (prev != (unsigned)__popc(sharers) - 1u) return;
+        __threadfence_block();
+        for (int e = lane; e < 16 * (TOK == 1 ? 1 : sa.M); e += 32) {
+            const float* at = lslots + e;
+            float sum = at[(wl * 2u + (shared_first ? 0u : 1u)) * (16 * TOK)];
+            for (uint32_t w = wl + 1; w <= wh; w += 4) {  // (four loads at a time; a warp between them that has no part of the row block adds nothing)
+                float p[4];
+#pragma unroll
+                for (uint32_t u = 0; u < 4; ++u) p[u] = at[min(w + u, wh) * 2u * (16 * TOK)];
+#pragma unroll
+                for (uint32_t u = 0; u < 4; ++u)
+                    if (w + u <= wh && ((sharers >> (w + u)) & 1u)) sum += p[u];
+            }
+            if (shared_first || next_cta) {
+                // The sums go from CTA to CTA with a mark beside each: no fence, and nothing to wait for where they are left.  The CTA
+                // that takes them, at its end, finds them there but for one that was late to start, and clears them for the next call.
+                unsigned long long* box = reinterpret_cast<unsigned long long*>(sa.counters) + (size_t)(blockIdx.x + (next_cta ? 1u : 0u)) * (16 * TOK) + e;
+                if (shared_first) {
+                    st_relaxed64(box, (1ull << 32) | __float_as_uint(sum));
+                    continue;
+                }
+                unsigned long long got = 0;
+                for (uint32_t i = 0; i < kSpinLimit && got == 0; ++i) got = ld_relaxed64(box);
+                if (got == 0) {  // (the row stays unwritten: the error word says so)
+                    if (err) atomicCAS(err, 0, 4 | (warp << 24));
+                    continue;
+                }
+                st_relaxed64(box, 0ull);
+                sum += __uint_as_float((uint32_t)got);
+            }
+            sa.Y[(int64_t)(e >> 4) * sa.N + row0 + (e & 15)] = sk_out<DT>(sum);
+        }
+        if (shared_first) {
+            __threadfence_block();
+            __syncwarp();
+            if (lane == 0) *(volatile unsigned*)(lcnt + W + 1) = 1u;
+        }
+    };
+
+    // ---- one unit: 2 x 32 codes of this lane -> 32 half2 (decode: needs no activations) -> eight MMAs (multiply) ----
+    auto unit_ok = [&](const unsigned char* code, const unsigned char* param, uint32_t cbu) {
+        return in_range(code >= ringp && code + UB <= ringp + (size_t)S * slot_bytes && param + PB <= ringp + (size_t)S * slot_bytes &&
+                            cbu < ncb && (!XSMEM || ((size_t)(cbu + 1) * 256u << sa.token_shift) <= (size_t)sa.x_bytes),
+                        err, 0x150);
+    };
+    auto decode = [&](const unsigned char* code, const unsigned char* param, uint32_t (&lo)[16], uint32_t (&hi)[16]) {
+        // the scale words {row gid, row gid + 8} of this lane's group
+        const uint32_t poff = ((spg == 2 ? (uint32_t)(tig >> 1) * 8u : 0u) + (uint32_t)gid) * 4u;
+        // plane k of a unit holds word k of every (row, quarter): this lane's word sits at byte 4 * lane
+        uint32_t w[2][BITS];
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int k = 0; k < BITS; ++k) w[h][k] = sk_lds32(code + (uint32_t)(k * 256 + h * 128) + (uint32_t)lane * 4u);
+        if constexpr (UNSC) {
+            potl::pot_units32<BITS>(w[0], sa.p2, sa.bias, lo);
+            potl::pot_units32<BITS>(w[1], sa.p2, sa.bias, hi);
+            return;
+        }
+        const uint32_t scw = sk_lds32(param + poff);  // {row gid, row gid + 8}
+        if constexpr (DT == 0) {
+            potl::pot_decode32<BITS, 1>(w[0], 0, __byte_perm(scw, 0, 0x1010), lo);
+            potl::pot_decode32<BITS, 1>(w[1], 0, __byte_perm(scw, 0, 0x3232), hi);
+        } else {  // the FP16 scale rounded once to BF16
+            const uint32_t s0 = __bfloat16_as_ushort(__float2bfloat16_rn(__half2float(__ushort_as_half((uint16_t)(scw & 0xFFFFu)))));
+            const uint32_t s1 = __bfloat16_as_ushort(__float2bfloat16_rn(__half2float(__ushort_as_half((uint16_t)(scw >> 16)))));
+            potl::pot_decode32_bf16<BITS, 1>(w[0], 0, s0 * 0x10001u, lo);
+            potl::pot_decode32_bf16<BITS, 1>(w[1], 0, s1 * 0x10001u, hi);
+        }
+    };
+    // this lane's column of B (GEMV): x, or zeros if the column belongs to the other group
+    auto zeros = [&]() -> const unsigned char* {
+        if constexpr (UNSC) return smem + sa.zeros_at;
+        else return xs;
+    };
+    const bool zero_column = UNSC && TOK == 1 && spg == 2 && (gid >> 2) != (tig >> 1);
+    const unsigned char* xcol = zero_column ? zeros() + tig * 16 : xs + tig * 16;
+    const uint32_t xstep = zero_column ? 0u : 256u;
+    auto multiply = [&](const uint32_t (&lo)[16], const uint32_t (&hi)[16], const unsigned char* param, uint32_t cbu) {
+        // activations of quarter tig (of token gid): the B fragments of the eight MMAs
+        uint32_t xq[16];
+        if constexpr (XSMEM) {
+            const unsigned char* xa = TOK == 1 ? xcol + cbu * xstep
+                                               : xs + ((((cbu * 16u) << sa.token_shift) + ((((uint32_t)gid & ((1u << sa.token_shift) - 1u)) >> 1) << 3) +
+                                                        (((uint32_t)gid & 1u) << 2) + (uint32_t)tig) << 4);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const uint4 v = sk_lds128(xa + (TOK == 1 ? 64u : (64u << sa.token_shift)) * i);
+                xq[4 * i + 0] = v.x; xq[4 * i + 1] = v.y; xq[4 * i + 2] = v.z; xq[4 * i + 3] = v.w;
+            }
+        } else {
+            const bool live = TOK == 1 || gid < sa.M;
+            const uint4* xp = reinterpret_cast<const uint4*>(sa.X) + (TOK == 1 || !live ? 0 : (int64_t)gid * (sa.K / 8)) +
+                              (int64_t)cbu * 16 + tig * 4;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                uint4 v = make_uint4(0, 0, 0, 0);
+                if (live) v = ld_dependent16(xp + i);
+                xq[4 * i + 0] = v.x; xq[4 * i + 1] = v.y; xq[4 * i + 2] = v.z; xq[4 * i + 3] = v.w;
+            }
+        }
+        if constexpr (UNSC) {
+            float c[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int j = 0; j < 8; ++j) sk_mma(c, lo[2 * j], hi[2 * j], lo[2 * j + 1], hi[2 * j + 1], xq[2 * j], xq[2 * j + 1]);
+            const uint32_t scw = sk_lds32(param + ((spg == 2 ? (uint32_t)(tig >> 1) * 8u : 0u) + (uint32_t)gid) * 4u);  // {row gid, row gid + 8}
+            float2 sc = __half22float2(*reinterpret_cast<const __half2*>(&scw));
+            if constexpr (!FACTORS) {
+                acc[0][0] = fmaf(c[0], sc.x, acc[0][0]);
+                acc[0][2] = fmaf(c[2], sc.y, acc[0][2]);
+                if constexpr (TOK > 1) {
+                    acc[0][1] = fmaf(c[1], sc.x, acc[0][1]);
+                    acc[0][3] = fmaf(c[3], sc.y, acc[0][3]);
+                }
+            } else {  // the FP16 scale rounded once to BF16; times the unit's factor last, so that no product leaves FP32's range early
+                sc = __bfloat1622float2(__float22bfloat162_rn(sc));
+                const float f = factors[cbu];
+                acc[0][0] = fmaf(c[0] * sc.x, f, acc[0][0]);
+                acc[0][2] = fmaf(c[2] * sc.y, f, acc[0][2]);
+            }
+            return;
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j)  // two accumulators: half the length of the dependent chain
+            if constexpr (DT == 0) sk_mma(acc[j & 1], lo[2 * j], hi[2 * j], lo[2 * j + 1], hi[2 * j + 1], xq[2 * j], xq[2 * j + 1]);
+            else sk_mma_bf16(acc[j & 1], lo[2 * j], hi[2 * j], lo[2 * j + 1], hi[2 * j + 1], xq[2 * j], xq[2 * j + 1]);
+    };
+    auto unit = [&](const unsigned char* code, const unsigned char* param, uint32_t cbu) {
+        if (!unit_ok(code, param, cbu)) return;
+        uint32_t lo[16], hi[16];
+        decode(code, param, lo, hi);
+        multiply(lo, hi, param, cbu);
+    };
+    // a unit whose activations are not FP16 numbers times one factor
+    auto unit_bf16 = [&](const unsigned char* code, const unsigned char* param, uint32_t cbu) {
+        if (!unit_ok(code, param, cbu)) return;
+        const unsigned char* sp = param + ((spg == 2 ? (uint32_t)(tig >> 1) * 8u : 0u) + (uint32_t)gid) * 4u;
+        float2 v;
+        if constexpr (OCC == 2) v = sk_unit_bf16_call<BITS>(code + (uint32_t)lane * 4u, sp, xcol + cbu * xstep);
+        else v = sk_unit_bf16<BITS>(code + (uint32_t)lane * 4u, sp, xcol + cbu * xstep);
+        acc[0][0] += v.x;
+        acc[0][2] += v.y;
+    };
+    // ---- main loop over this warp's chunks; MARKS: x has marked units.  False: a copy never arrived -----------------------------
+    // (Two loops: with the marks looked for in the one that most launches run these took 2 - 4 % longer.)
+    auto main_loop = [&](auto marks) -> bool {
+        constexpr bool MARKS = decltype(marks)::value;
+        uint32_t s = 0, phase = 0, left = n;
+        bool shared_first = ln != 0;  // (the part of the row block that the CTA before began)
+        if (shared_first) {
+            left = ln;
+            rb = first_rb;
+            cb = la - first_rb * ncb;
+        }
+        for (uint32_t j = 0; left > 0; ++j) {
+            const unsigned char* code = ringp + s * slot_bytes;
+            const unsigned char* param = code + SK_Q * UB;
+            const uint32_t bar = bars + s * 8u;
+            if (!mbar_test(bar, phase) && !mbar_wait(bar, phase)) {
+                // Record it, request nothing more, deliver nothing more (the rows this warp still owed stay unwritten: the error
+                // word says so), wait -- bounded again -- for the chunks already requested, leave.
+                if (err && lane == 0) atomicCAS(err, 0, 2 | (int)(j << 8) | (warp << 24));
+                uint32_t s2 = s, ph2 = phase;
+                for (uint32_t k = 1; k < (uint32_t)S && j + k < wst[7]; ++k) {
+                    if (++s2 == (uint32_t)S) {
+                        s2 = 0;
+                        ph2 ^= 1u;
+                    }
+                    mbar_wait(bars + s2 * 8u, ph2);
+                }
+                return false;
+            }
+            if (j == 0) stamp(4);
+            const bool full = left >= (uint32_t)SK_Q && cb + (uint32_t)SK_Q <= ncb;
+            bool some = false, all = MARKS;  // some, all units of a full chunk are marked
+            if constexpr (MARKS) {
+                if (full) {
+#pragma unroll
+                    for (int i = 0; i < SK_Q; ++i) {
+                        const bool m = factors[cb + i] < 0.f;
+                        some = some || m;
+                        all = all && m;
+                    }
+                }
+            }
+            if (full && !some) {
+                // the common case: a full chunk inside one row block, straight-line code
+#pragma unroll
+                for (int i = 0; i < SK_Q; ++i) unit(code + i * UB, param + (uint32_t)i * PB, cb + (uint32_t)i);
+                cb += SK_Q;
+                left -= SK_Q;
+                if (cb == ncb || left == 0) {
+                    deliver(rb, shared_first);
+                    cb = 0;
+                    ++rb;
+                }
+            } else if (MARKS && OCC == 1 && full && all) {
+                if constexpr (MARKS) {
+#pragma unroll
+                    for (int i = 0; i < SK_Q; ++i) unit_bf16(code + i * UB, param + (uint32_t)i * PB, cb + (uint32_t)i);
+                }
+                cb += SK_Q;
+                left -= SK_Q;
+                if (cb == ncb || left == 0) {
+                    deliver(rb, shared_first);
+                    cb = 0;
+                    ++rb;
+                }
+            } else {
+                const uint32_t cnt = left < (uint32_t)SK_Q ? left : (uint32_t)SK_Q;
+                left -= cnt;
+                for (uint32_t i = 0; i < cnt;) {
+                    uint32_t step = 1;
+                    if (BLOCK < SK_Q && !MARKS && i + BLOCK <= cnt && cb + BLOCK <= ncb) {
+#pragma unroll
+                        for (uint32_t u = 0; u < BLOCK; ++u) unit(code + u * UB, param + u * PB, cb + u);
+                        step = BLOCK;
+                    } else if constexpr (MARKS) {
+                        if (factors[cb] < 0.f) unit_bf16(code, param, cb);
+                        else unit(code, param, cb);
+                    } else {
+                        unit(code, param, cb);
+                    }
+                    code += step * UB;
+                    param += step * PB;
+                    i += step;
+                    cb += step;
+                    if (cb == ncb || (left == 0 && i == cnt)) {
+                        deliver(rb, shared_first);
+                        cb = 0;
+                        ++rb;
+                    }
+                }
+            }
+            __syncwarp();  // every lane has read the slot: it may be refilled
+            if (lane == 0 && j + (uint32_t)S < wst[7]) issue(wst[0], wst[1], wst[2], wst[3], j + (uint32_t)S, s);
+            if (++s == (uint32_t)S) {
+                s = 0;
+                phase ^= 1u;
+            }
+            if (left == 0 && shared_first) {
+                shared_first = false;
+                left = wst[1];
+                rb = wst[4];
+                cb = wst[0] - rb * ncb;
+            }
+        }
+        return true;
+    };
+    if (FACTORS && inexact) {
+        if constexpr (FACTORS)
+            if (!main_loop(std::true_type())) return;
+    } else {
+        if (!main_loop(std::false_type())) return;
+    }
+    stamp(6);
+}
+
+}  // namespace pot
+#endif

@@ -1,0 +1,77 @@
+"""The streaming kernel with the units dealt out evenly to the CTAs: row blocks that two CTAs share, whose sums go from one to the other."""
+import numpy as np
+import pytest
+
+from tests.gpu_util import GuardedBinding, PotCase, bf16_dev, bits_of, f16_bits_to_bf16_bits, f16_dev, gate
+
+pytestmark = pytest.mark.gpu
+
+# (N, K): row blocks per CTA from just above one to many; K of few and odd numbers of column blocks; shared row blocks of which the second CTA
+# has a single unit or all but one; x that does not fit into shared memory (4 tokens x 14336
+# at 4 bits)
+SHAPES = [(2480, 2048), (2992, 1792), (3088, 4224), (2720, 4224), (13024, 384), (7136, 1152), (5200, 2048), (2400, 8192), (2528, 14336)]
+
+
+@pytest.fixture(scope="module")
+def B():
+    return GuardedBinding()
+
+
+def _acts(M, K, seed):
+    from paper_2507_11959_b200 import synth
+    return synth.activations(synth.rng_for(4, seed), M, K)
+
+
+@pytest.mark.parametrize("N,K", SHAPES)
+@pytest.mark.parametrize("bits,G", [(2, 64), (3, 128), (4, 64)])
+def test_even_split_matches_oracle(B, oracle, N, K, bits, G):
+    from paper_2507_11959_b200 import binding
+    c = PotCase(N, K, bits, G, dist="t5", seed=(4, 900 + bits))
+    tiled, scales = c.tiled(), c.tiled_S()
+    reached = 0
+    for M in (1, 2, 4, 8):
+        X = _acts(M, K, 900 + M)
+        for bf16 in (False, True):
+            Xb = f16_bits_to_bf16_bits(X) if bf16 else X
+            if binding.pot_debug_gemm_plan(M, N, K, bits, G, bf16)["streaming"] == 0:
+                continue
+            reached += binding.pot_debug_gemv_split(M, N, K, bits, G, bf16) == 2
+            Y, A = oracle.matmul(c.packed, c.S, K, bits, G, Xb, dtype=oracle.BF16 if bf16 else oracle.F16)
+            ws = B.new_workspace(binding.pot_gemm_workspace_bytes(M, N, K, bits, G))
+            Xd = bf16_dev(Xb) if bf16 else f16_dev(Xb)
+            first = None
+            for _ in range(3):  # the marks have to be gone after every call; sums in a fixed order
+                y = bits_of(B.pot_gemm(tiled, scales, K, bits, G, Xd, binding.TILED, workspace=ws))
+                first = y if first is None else first
+                assert np.array_equal(y, first), (M, bf16)
+            ok, worst, tight = gate(first, Y, A, bf16)
+            assert ok and tight < 4.0, (M, bf16, worst, tight)
+            assert not ws[:148 * 16 * (1 if M == 1 else 8) * 8].any(), (M, bf16)
+    assert reached >= 2
+
+
+def test_even_split_repeats_itself_in_a_chain(B):
+    """Forty launches behind one another that share a workspace, every one with other numbers: no sum of one call reaches the next."""
+    import torch
+    from paper_2507_11959_b200 import binding
+    N, K, bits, G = 2992, 1792, 3, 128
+    c = PotCase(N, K, bits, G, dist="t5", seed=(4, 950))
+    tiled, scales = c.tiled(), c.tiled_S()
+    assert binding.pot_debug_gemv_split(1, N, K, bits, G) == 2
+    ws = binding.new_workspace(binding.pot_gemv_workspace_bytes(N, K, bits, G))
+    xs = [f16_dev(_acts(1, K, 960 + i)[0]) for i in range(8)]
+    alone = []
+    for x in xs:
+        alone.append(binding.pot_gemv(tiled, scales, K, bits, G, x, binding.TILED, workspace=ws).clone())
+        torch.cuda.synchronize()
+    ys = [torch.empty_like(alone[0]) for _ in range(40)]
+    for i, y in enumerate(ys):
+        binding.pot_gemv(tiled, scales, K, bits, G, xs[i % 8], binding.TILED, y=y, workspace=ws)
+    torch.cuda.synchronize()
+    assert all(torch.equal(y, alone[i % 8]) for i, y in enumerate(ys))
+    # the fixed scratch of pot_gemv_noalloc, after a call that leaves partial sums in it
+    small = PotCase(1024, 4096, bits, G, dist="t5", seed=(4, 951))
+    binding.pot_gemv_noalloc(small.tiled(), small.tiled_S(), 4096, bits, G, f16_dev(_acts(1, 4096, 970)[0]), torch.empty(1024, dtype=torch.float16, device="cuda"))
+    y = binding.pot_gemv_noalloc(tiled, scales, K, bits, G, xs[0], torch.empty_like(alone[0]))
+    assert torch.equal(y, alone[0])
+    assert binding.pot_debug_errors() == (0, 0, 0)
