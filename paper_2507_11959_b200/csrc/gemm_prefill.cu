@@ -67,7 +67,7 @@ __host__ __device__ constexpr int pf_x_bytes(int mt) { return mt == 1 ? PF_SMALL
 // pipe set the pace)
 __host__ __device__ constexpr int pf_bks(int mt, int at, int wide = 0) { return (at && (mt == 1 || wide)) ? 2 : 1; }
 __host__ __device__ constexpr int pf_stage_bytes(int mt, int at = 0, int wide = 0) { return pf_x_bytes(mt) * pf_bks(mt, at, wide) + (at ? 0 : PF_ATOM_BYTES); }
-constexpr size_t pf_smem_bytes_h(int stages, int h, int bks) { return 1024 + (size_t)stages * 2 * h * 128 * bks + 256; }  // tiles of 2 h tokens
+constexpr size_t pf_smem_bytes_h(int stages, int h, int bks, int x_tiles = 2) { return 1024 + (size_t)stages * x_tiles * h * 128 * bks + 256; }  // tiles of 2 h tokens
 constexpr size_t pf_smem_bytes(int stages, int mt, int at = 0, int wide = 0) { return 1024 /*align slack*/ + (size_t)stages * pf_stage_bytes(mt, at, wide) + 256 /*barriers*/; }
 // at = 1, tiles of up to 384 tokens: two X tiles of h tokens (h a multiple of 16, chosen per launch), accumulator columns 0 .. 2h - 1
 // (token t of the tile = column t), then 32 columns per 64-column stage of A: six stages up to h = 128, four up to h = 192
@@ -143,6 +143,12 @@ __device__ __forceinline__ void pf_cluster_sync() {
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
     __syncwarp();
 }
+// the same where nothing that was written has to be seen behind it (a release waits until the stores to Y have reached L2: 200 tokens x
+// 4099 x 11008 25.9 us, without 25.5)
+__device__ __forceinline__ void pf_cluster_sync_relaxed() {
+    asm volatile("barrier.cluster.arrive.relaxed;\n\tbarrier.cluster.wait;" ::: "memory");
+    __syncwarp();
+}
 // address of this CTA's shared-memory location in the CTA with the given rank of the cluster
 __device__ __forceinline__ uint32_t pf_cluster_addr(uint32_t addr, uint32_t rank) {
     uint32_t r;
@@ -205,7 +211,7 @@ __device__ __forceinline__ void pf_issue_at(uint32_t smem0, uint32_t bar0, uint3
 #pragma unroll
     for (int s = 0; s < PF_STAGES; ++s)
 #pragma unroll
-        for (int b = 0; b < BKS; ++b) blo[s][b] = (uint32_t)pf_smem_desc(smem0 + (uint32_t)((s * BKS + b) * PF_MT + (KSPLIT ? 0 : J)) * (h * 128u));
+        for (int b = 0; b < BKS; ++b) blo[s][b] = (uint32_t)pf_smem_desc(smem0 + (uint32_t)(KSPLIT ? s * BKS + b : (s * BKS + b) * PF_MT + J) * (h * 128u));
     constexpr uint32_t desc_hi = (uint32_t)(PF_DESC_CONST >> 32);
     constexpr uint32_t SLOT = 32u * BKS;   // tensor-memory columns of a stage's weights
     const uint32_t d0 = tmem_base + (uint32_t)J * h;
@@ -389,9 +395,11 @@ __device__ __forceinline__ void pf_add_up(const PfAddUp& a, uint32_t smem, int* 
 }
 
 // PF_STAGES stages, NG producer groups (K block kb is decoded by group kb % NG into stage kb % PF_STAGES), NI issuers with
-// their own accumulators, MT token tiles of 128 per CTA.  PF_STAGES is a multiple of NG and of NI: a stage buffer is
-// always filled by the same group, loaded by the same TMA thread and read by the same issuer, so every parity wait is
-// made by a thread that has itself seen the barrier's previous phase (a waiter two phases behind could not tell).
+// their own accumulators, MT token tiles of 128 per CTA.  A parity wait cannot tell a barrier that is two phases behind.  PF_STAGES is a multiple
+// of NG and of NI: a stage buffer is always filled by the same group, loaded by the same TMA thread and read by the same issuer, so every wait is
+// made by a thread that has itself seen the barrier's previous phase.  Or (AT = 1, MT = 2: every issuer reads every stage, in order) NG <= PF_STAGES:
+// a group that comes to stage kb has waited, for stage kb - NG, until stage kb - NG - PF_STAGES had been read, hence every stage up to
+// kb - 2 PF_STAGES, the last but one in the buffer of kb.
 // AT = 0 (diagnostic): the decoded weight tile in shared memory.  <bits, 4, 4, 2, 2> (M > 64: 256-token tiles, four 48 KB
 // stages) and <bits, 8, 4, 2, 1> (M <= 64: one tile of up to 64 tokens, eight 24 KB stages -- a stage buffer's round trip
 // producer -> issuer -> tensor pipe -> producer is ~2000 cycles whatever the tile holds, so more buffers = more stages per
@@ -400,7 +408,7 @@ __device__ __forceinline__ void pf_add_up(const PfAddUp& a, uint32_t smem, int* 
 // shared memory and the MMAs take their A operand from there, which removes a third of the shared-memory traffic of a
 // stage (16 KB written + 16 KB read of 96 KB); see pf_issue_at for the issuers' division of work.  Of the 512 columns
 //   <bits, 6, 3, 2, 1, dt, 1>           (M <= 64)           2 x 64 accumulate, 6 x 64 hold stages of 128 columns of K,
-//   <bits, 3, 3, 2, 2, dt, 1, 3, 1>     (one wave of CTAs)  2 h accumulate (h <= 128), 3 x 64 hold stages of 128 columns,
+//   <bits, 3 or 4, 3, 2, 2, dt, 1, 3, 1> (one wave of CTAs) 2 h accumulate (h <= 128, 112), 3 or 4 x 64 hold stages of 128 columns,
 //   <bits, 6, 2 or 3, 2, 2, dt, 1>      (more waves)        2 h accumulate (h <= 128), 6 x 32 hold stages of 64 columns,
 //   <bits, 4, 2 or 4, 2, 2, dt, 1>      (h > 128)           2 h accumulate (h <= 192), 4 x 32 hold stages of 64 columns;
 // the larger number of producer groups is that of BF16.
@@ -428,7 +436,7 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
     constexpr int BKS = pf_bks(MT, AT, WIDE);   // 64-column sub-blocks per stage
     const int h = AT2 ? tok_h : PF_BM;                      // tokens per X tile
     const int x_tile_bytes = AT2 ? h * 128 : PF_ATOM_BYTES;
-    const int STAGE_BYTES = AT2 ? MT * BKS * x_tile_bytes : pf_stage_bytes(MT, AT, WIDE);
+    const int STAGE_BYTES = AT2 ? (KSPLIT ? 1 : MT) * BKS * x_tile_bytes : pf_stage_bytes(MT, AT, WIDE);
     const int ring_col0 = AT2 ? 2 * h : PF_AT1_RING_COL0;   // AT: first tensor-memory column of the weight ring
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)PF_STAGES * STAGE_BYTES);
     // bars: full[S] (TMA bytes + one arrival per producer warp), empty[S], accum, then the tensor-memory base address
@@ -441,7 +449,7 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
     constexpr int PROD_WARP0 = pf_prod_warp0(NI);
     constexpr int NPT = NG * 128;                       // producer / epilogue threads
     constexpr int TMEM_COLS = AT ? 512 : NI * PF_BN * MT;  // MT accumulators per issuer; AT: 256 accumulator columns + the A ring
-    static_assert(NGP <= NG && (AT2 || PF_STAGES % NI == 0) && PF_STAGES % NGP == 0, "a stage buffer belongs to one issuer and one group");
+    static_assert(NGP <= NG && (AT2 ? NGP <= PF_STAGES : PF_STAGES % NI == 0 && PF_STAGES % NGP == 0), "no parity wait is two phases behind");
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // Work items in launch order: the first n_full are whole output tiles; each of the remaining ("tail") tiles is cut
     // into tail_splits items along K, so that the last, partly filled wave of CTAs is short.  Tiles are numbered
@@ -585,7 +593,7 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
 #pragma unroll
                         for (int mt = 0; mt < MT; ++mt)
                             if (mt < n_mt)
-                                pf_tma_load_2d(a + (sub * MT + mt) * x_tile_bytes, &xmap, ((kb0 + kb) * 2 + sub) * PF_BK, (int)m0 + mt * h, full(s));
+                                pf_tma_load_2d(a + (KSPLIT ? sub : sub * MT + mt) * x_tile_bytes, &xmap, ((kb0 + kb) * 2 + sub) * PF_BK, (int)m0 + mt * h, full(s));
                 } else {
 #pragma unroll
                     for (int mt = 0; mt < MT; ++mt)
@@ -846,7 +854,7 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
     }
     if constexpr (CLUSTER) {  // every thread of the cluster arrives at the barriers: the epilogue warps at the first one above
         if (warp < PROD_WARP0) pf_cluster_sync();
-        if constexpr (CANON) pf_cluster_sync();  // nobody leaves while its partial sums are being read
+        if constexpr (CANON) pf_cluster_sync_relaxed();  // nobody leaves while its partial sums are being read
     }
     // ---------------- teardown: everyone is done with tensor memory, the allocating warp frees it --------
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -970,7 +978,8 @@ static bool prefill_wide_stages_allowed() {
 
 // The instantiation that a launch takes.
 struct PrefillVariant { bool in_tmem; int stages, stage_columns, groups; };
-static PrefillVariant prefill_variant(const PrefillPlan& pl, int64_t M, int dt) {
+static int wide_stages(int64_t M, int64_t K, int h);
+static PrefillVariant prefill_variant(const PrefillPlan& pl, int64_t M, int64_t K, int dt) {
     const bool tmem = prefill_weight_tile_in_tmem();
     // one token tile, three producer groups, six stages of a whole 128-column block with the weight ring in tensor memory
     // (four groups, eight 24 KB stages with the tile in shared memory)
@@ -983,7 +992,8 @@ static PrefillVariant prefill_variant(const PrefillPlan& pl, int64_t M, int dt) 
     // A single wave of CTAs (65 .. 256 tokens on decode-sized matrices) is paced by the stage visits, not by the tensor
     // pipe: three stages of a whole 128-column block (64 KB of X, 64 columns of weights, three producer groups), as in the
     // one-tile kernel (15360 x 5120 at 65 .. 128 tokens: 27.5 - 28.5 -> 22.2 - 23.1 us).
-    if (pl.n_full + (int64_t)pl.n_tail * pl.splits <= kSmCount && prefill_wide_stages_allowed()) return {true, 3, 128, 3};
+    // Four stages where they fit (see wide_stages).
+    if (pl.n_full + (int64_t)pl.n_tail * pl.splits <= kSmCount && prefill_wide_stages_allowed()) return {true, M <= 2 * PF_BM ? wide_stages(M, K, pl.h) : 3, 128, 3};
     return {true, 6, 64, dt == 1 ? 3 : 2};  // 32 KB of X per stage
 }
 // Where the tiles leave SMs idle, a cluster of up to 8 CTAs shares a tile's K range (at least four column
@@ -1027,7 +1037,7 @@ static int tiled_cluster(const PrefillPlan& pl, const PrefillVariant& v, int64_t
 void gemm_prefill_plan_query(int64_t M, int64_t N, int64_t K, int dt, int* tile_tokens, int* ring_stages, int* stage_columns, int* producer_groups,
                              int* tiles, int* split_tiles, int* splits) {
     const PrefillPlan pl = prefill_plan(M, N, K);
-    const PrefillVariant v = prefill_variant(pl, M, dt);
+    const PrefillVariant v = prefill_variant(pl, M, K, dt);
     *tile_tokens = M <= PF_SMALL_TOKENS ? PF_SMALL_TOKENS : 2 * pl.h;
     *ring_stages = v.stages;
     *stage_columns = v.stage_columns;
@@ -1039,7 +1049,7 @@ void gemm_prefill_plan_query(int64_t M, int64_t N, int64_t K, int dt, int* tile_
 
 int gemm_prefill_cluster_query(int64_t M, int64_t N, int64_t K, int dt) {
     const PrefillPlan pl = prefill_plan(M, N, K);
-    return tiled_cluster(pl, prefill_variant(pl, M, dt), K, dt);
+    return tiled_cluster(pl, prefill_variant(pl, M, K, dt), K, dt);
 }
 
 // f(integral_constant<bits>, integral_constant<0: FP16, 1: BF16>)
@@ -1086,6 +1096,12 @@ static bool resident_clusters(const void* kernel, dim3 block, size_t smem, int (
 // Whether the two issuers share the only X tile of a batch: with two stages the epilogue's second accumulator costs more than they save
 // (128 tokens x 2048 x 256, BF16: 4.23 -> 4.44 us), with four it is paid for (100 tokens x 5120 x 512: 2 - 6 % faster).
 static bool one_tile_ksplit(int64_t M, int64_t K) { return M <= PF_BM && K >= 4 * 128; }
+// Stages of 128 columns: four where shared memory (512 h bytes each, 256 h with a single X tile) and tensor memory (2 h + 64 columns each) hold them.
+// Three wait for the tensor pipe's round trip (issuers idle for 250 of 745 cycles per stage at 128 tokens): us, three -> four, 128 tokens x 15360
+// x 5120 20.9 -> 19.9, 70 (4 bits) 19.4 -> 17.4, 100 (2 bits) 18.8 -> 17.2; canonical, 200 x 4099 x 11008 25.7 -> 24.9, 150 x 9000 x 4096 (BF16) 16.7 ->
+// 15.6.  (Two or four producer groups: 1 - 20 % slower, four at 96 registers.)
+constexpr int kWideFourH = 112;
+static int wide_stages(int64_t M, int64_t K, int h) { return one_tile_ksplit(M, K) || h <= kWideFourH ? 4 : 3; }
 pot_status_t gemm_prefill_launch(const void* packed, const void* scales, int64_t N, int64_t K, int bits, int group,
                                  const void* X, int64_t M, void* Y, void* workspace, size_t ws_bytes, cudaStream_t s, int dt) {
     const PrefillPlan pl = prefill_plan(M, N, K);
@@ -1094,7 +1110,7 @@ pot_status_t gemm_prefill_launch(const void* packed, const void* scales, int64_t
     float* partial = pl.ws_bytes > 0 ? (float*)((char*)workspace + pl.counter_bytes) : nullptr;
     CUtensorMap xmap;
     if (!encode_x_map(&xmap, X, M, K, pl.h)) return POT_ERR_CUDA;
-    const PrefillVariant v = prefill_variant(pl, M, dt);
+    const PrefillVariant v = prefill_variant(pl, M, K, dt);
     auto run = [&](auto kernel, int ng, size_t smem, int cluster) -> pot_status_t {
         const int splits = cluster > 1 ? cluster : pl.splits;
         return launch_pdl_cluster(kernel, dim3((unsigned)(pl.n_full + pl.n_tail * splits)), dim3((unsigned)pf_threads(ng, 2)), smem, cluster, true, s,
@@ -1118,10 +1134,12 @@ pot_status_t gemm_prefill_launch(const void* packed, const void* scales, int64_t
         }
         if (!v.in_tmem) return run(pot_gemm_prefill_kernel<B, 4, 4, 2, 2, D>, 4, pf_smem_bytes(4, 2), 1);
         constexpr int NG4 = D == 1 ? 4 : 2, NG6 = D == 1 ? 3 : 2;
-        if (v.stages == 4)
+        if (v.stages == 4 && v.stage_columns == 64)
             return run_split(pot_gemm_prefill_kernel<B, 4, NG4, 2, 2, D, 1>, pot_gemm_prefill_kernel<B, 4, NG4, 2, 2, D, 1, NG4, 0, 0, 1>, NG4, pf_smem_bytes_h(4, pl.h, 1));
-        if (v.stages == 3 && one_tile_ksplit(M, K))
-            return run_split(pot_gemm_prefill_kernel<B, 3, 3, 2, 2, D, 1, 3, 1, 0, 0, 1>, pot_gemm_prefill_kernel<B, 3, 3, 2, 2, D, 1, 3, 1, 0, 1, 1>, 3, pf_smem_bytes_h(3, pl.h, 2));
+        if (v.stage_columns == 128 && one_tile_ksplit(M, K))
+            return run_split(pot_gemm_prefill_kernel<B, 4, 3, 2, 2, D, 1, 3, 1, 0, 0, 1>, pot_gemm_prefill_kernel<B, 4, 3, 2, 2, D, 1, 3, 1, 0, 1, 1>, 3, pf_smem_bytes_h(4, pl.h, 2, 1));
+        if (v.stage_columns == 128 && v.stages == 4)
+            return run_split(pot_gemm_prefill_kernel<B, 4, 3, 2, 2, D, 1, 3, 1>, pot_gemm_prefill_kernel<B, 4, 3, 2, 2, D, 1, 3, 1, 0, 1>, 3, pf_smem_bytes_h(4, pl.h, 2));
         if (v.stages == 3)
             return run_split(pot_gemm_prefill_kernel<B, 3, 3, 2, 2, D, 1, 3, 1>, pot_gemm_prefill_kernel<B, 3, 3, 2, 2, D, 1, 3, 1, 0, 1>, 3, pf_smem_bytes_h(3, pl.h, 2));
         return run(pot_gemm_prefill_kernel<B, 6, NG6, 2, 2, D, 1>, NG6, pf_smem_bytes_h(6, pl.h, 1), 1);
@@ -1165,7 +1183,8 @@ pot_status_t gemm_canonical_launch(const void* packed, const void* scales, int64
         constexpr int B = decltype(b)::value, D = decltype(d)::value;
         if (small) return run(pot_gemm_prefill_kernel<B, 6, 3, 2, 1, D, 1, 3, 0, 1>, pot_gemm_prefill_kernel<B, 6, 3, 2, 1, D, 1, 3, 0, 1, 1>, pf_smem_bytes(6, 1, 1));
         const size_t smem = pf_smem_bytes_h(3, h, 2);
-        if (one_tile_ksplit(M, K)) return run(pot_gemm_prefill_kernel<B, 3, 3, 2, 2, D, 1, 3, 1, 1, 0, 1>, pot_gemm_prefill_kernel<B, 3, 3, 2, 2, D, 1, 3, 1, 1, 1, 1>, smem);
+        if (one_tile_ksplit(M, K)) return run(pot_gemm_prefill_kernel<B, 4, 3, 2, 2, D, 1, 3, 1, 1, 0, 1>, pot_gemm_prefill_kernel<B, 4, 3, 2, 2, D, 1, 3, 1, 1, 1, 1>, pf_smem_bytes_h(4, h, 2, 1));
+        if (h <= kWideFourH) return run(pot_gemm_prefill_kernel<B, 4, 3, 2, 2, D, 1, 3, 1, 1>, pot_gemm_prefill_kernel<B, 4, 3, 2, 2, D, 1, 3, 1, 1, 1>, pf_smem_bytes_h(4, h, 2));
         return run(pot_gemm_prefill_kernel<B, 3, 3, 2, 2, D, 1, 3, 1, 1>, pot_gemm_prefill_kernel<B, 3, 3, 2, 2, D, 1, 3, 1, 1, 1>, smem);
     });
 }
