@@ -9,8 +9,8 @@
 //    codes per lane per step, products accumulated in FP32 with the mixed-precision FMA and reduced with warp shuffles.
 //
 // Programmatic dependent launch: weights and scales do not depend on the previous kernel in the stream, x does.
-// The streaming kernel requests its first weights before it executes griddepcontrol.wait, and touches x, y and the
-// workspace only after it; the canonical kernels wait first.
+// The streaming kernel and the canonical kernel on the tensor cores request their first weights before they execute
+// griddepcontrol.wait, and touch x, y and the workspace only after it; the one with a warp per row waits first.
 #include "common.cuh"
 #include "layout.cuh"
 #include "stream.cuh"
@@ -100,9 +100,9 @@ __global__ void __launch_bounds__(256) gemv_canonical_kernel(const uint32_t* __r
 // a row block are dealt to 1, 2, 4 or 8 warps of a CTA and, where few row blocks leave SMs idle, to the CTAs of a cluster; the sums are
 // added in warp order, then in CTA order.  (One CTA of 16 warps per SM with a contiguous, equal share of the steps per warp was
 // 5 - 20 % slower: its launches do not overlap.)
-// Bound by instruction issue (16 rows x 128 columns: 70 - 110 instructions to decode, 8 MMAs, 12 loads) and by fixed latencies (launch, x,
-// codes).  HBM-cold, 10007 x 4096: 8.2 us at 2 bits, 10.0 us at 3, 11.3 us at 4 bits in BF16 (one warp per row on CUDA cores: 26.5,
-// 31.9, 26.5 us); 4099 x 11008 at 3 bits: 36.1 -> 11.3 us.
+// Bound by instruction issue (16 rows x 128 columns: 70 - 110 instructions to decode, 8 MMAs, 12 loads) and by fixed latencies (launch,
+// x).  HBM-cold, 10007 x 4096: 6.95 us at 2 bits, 9.25 us at 3, 10.5 us at 4 bits in BF16 (one warp per row on CUDA cores: 26.5,
+// 31.9, 26.5 us); 4099 x 11008 at 3 bits: 36.1 -> 9.75 us.
 constexpr int GC_WARPS = 8;                      // (or half as many)
 constexpr int GC_X_STRIDE = 272;                 // bytes per staged column block
 constexpr int64_t GC_MAX_K = 64 * 1024;          // x takes 136 KB at this length
@@ -147,8 +147,6 @@ __global__ void __launch_bounds__(W * 32, gc_ctas_per_sm(BITS, W)) gemv_canonica
     const int64_t rb = (int64_t)(blockIdx.x / cluster) * (W >> wk_shift) + (warp >> wk_shift);
     const int64_t row0 = min(rb * 16 + gid, N - 1), row1 = min(rb * 16 + gid + 8, N - 1);  // (rows past the end repeat the last one and are not stored)
     const int steps = (ncb + 3) / 4, stride = WK * cluster;
-    pdl_wait();
-    pdl_launch_dependents();
 
     uint32_t w[2][4 * BITS], sc[2][2];
     const uint4* src[2];
@@ -182,6 +180,11 @@ __global__ void __launch_bounds__(W * 32, gc_ctas_per_sm(BITS, W)) gemv_canonica
         load_scales(0);
         load_scales(1);
     }
+    // x and y may belong to the previous kernel in the stream; the codes and scales do not, and are on their way (us, before -> behind the wait: 10007 x
+    // 4096 at 2 / 3 / 4 bits 8.05 / 9.7 / 11.1 -> 6.95 / 9.25 / 10.5, 4099 x 11008 11.1 -> 9.75, 1001 x 4096 2.95 -> 2.45).  The next launch is let in
+    // behind the wait: before it, CTAs of several launches share some SMs and leave others empty (4099 x 2944 6.4 us instead of 4.0).
+    pdl_wait();
+    pdl_launch_dependents();
     if constexpr (BITS == 2) {  // the order of canon_decode32_any
         for (int i = threadIdx.x; fits && i < ncb * 8; i += W * 32) {
             const uint4 a = ld_dependent16(x + 2 * i), b = ld_dependent16(x + 2 * i + 1);
