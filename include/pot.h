@@ -107,7 +107,7 @@ pot_status_t pot_debug_gemv_plan(int64_t N, int64_t K, int bits, int group, int 
 pot_status_t pot_debug_gemv_decode(int64_t N, int64_t K, int bits, int group, int bf16, int* ctas_per_sm, int* unscaled);
 /* Host arithmetic only: how pot_gemv / pot_gemm with M <= 8 tokens (bf16 = 0), or their BF16 forms, divide a tiled shape among the CTAs: 0 whole
  * row blocks, 1 the same number of units for every warp (the last one to deliver a row block's sums adds them up), 2 the same number of units for
- * every CTA (a row block has two CTAs at most, the second of which hands its sums to the first).                       */
+ * every CTA (a row block has two CTAs at most, the later of which adds up their sums).                                  */
 pot_status_t pot_debug_gemv_split(int64_t M, int64_t N, int64_t K, int bits, int group, int bf16, int* split);
 /* Host arithmetic only: how pot_gemv runs canonical codes: warps that share a row block (16 rows) in a CTA, warps per CTA, CTAs of
  * a cluster that share a row block; 0, 8, 0 where x is too long for shared memory (one warp per row).                  */

@@ -23,7 +23,7 @@
 // Delivery.  A warp that covered a whole row block writes Y.  Otherwise its sums go to slot (row block, position of the
 // warp among the row block's contributors) of the workspace; a per-row-block arrival counter tells the last contributor,
 // which adds the slots in ascending order -- the result does not depend on timing, and no warp waits for another (even split: see
-// stream_even.cuh).
+// stream_even.cuh; there too no CTA waits for another).
 #pragma once
 #include "common.cuh"
 #include "layout.cuh"

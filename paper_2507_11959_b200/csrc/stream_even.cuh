@@ -3,8 +3,9 @@
 //
 // CTA c takes the blocks of units c * cta_blocks + min(c, cta_more) .., as much as every other CTA but for one block.  A range that begins
 // inside a row block begins with a part that the CTA before has the rest of.  All warps work on this part first, and its sums are left in the
-// workspace for that CTA, which adds them to its own when it has come to its end.  Then the warps cut up the other units.  Row blocks that
-// warps share are added up in shared memory by the last one that delivers; the order of additions is fixed.
+// workspace for that CTA, which adds them to its own when it has come to its end -- or the other way round, where a CTA starts late: the
+// second one adds.  No CTA waits for another.  Then the warps cut up the other units.  Row blocks that warps share are added up in shared
+// memory by the last one that delivers; the order of additions is fixed.
 // What bounds it: as in stream.cuh.  What the split takes away is the unequal ends: of whole row blocks (28672 x 8192: 16 CTAs have 13 row blocks, 132
 // have 12), of a row block's many contributors (unit split).  Where the kernel has an SM to itself nothing hides its launch: it asks for one
 // chunk per warp, then for the activations, then for the rest of the ring (with all chunks first the activations arrive behind them:
@@ -23,6 +24,11 @@ __device__ __forceinline__ unsigned long long ld_relaxed64(const unsigned long l
     unsigned long long v;
     asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
     return v;
+}
+__device__ __forceinline__ unsigned long long exch_relaxed64(unsigned long long* p, unsigned long long v) {
+    unsigned long long old;
+    asm volatile("atom.exch.relaxed.gpu.global.b64 %0, [%1], %2;" : "=l"(old) : "l"(p), "l"(v) : "memory");
+    return old;
 }
 // shared-memory header: as sk_header_bytes, with four words between the local arrival counters and the slots of partial sums
 __host__ __device__ constexpr int sk_even_counters_at(int warps) { return warps * 96; }
@@ -309,19 +315,14 @@ __global__ void __launch_bounds__(W * 32, OCC) stream_even_kernel(const __grid_c
                     if (w + u <= wh && ((sharers >> (w + u)) & 1u)) sum += p[u];
             }
             if (shared_first || next_cta) {
-                // The sums go from CTA to CTA with a mark beside each: no fence, and nothing to wait for where they are left.  The CTA
-                // that takes them, at its end, finds them there but for one that was late to start, and clears them for the next call.
+                // Two CTAs have sums of the row block: the one that finds the other's in the workspace adds the two (in either order the same number),
+                // and clears them for the next call.  Neither waits for the other, which may not have started (another stream's kernel on its SM).
+                // A bounded wait of the first CTA and a plain store in the second were as fast but for 0 - 0.5 us where a launch has an SM to
+                // itself (2400 x 8192 5.45 -> 5.84 us on one GPU, 5.96 -> 5.98 on another; 28672 x 8192 23.0, 5120 x 13824 11.4, both).
                 unsigned long long* box = reinterpret_cast<unsigned long long*>(sa.counters) + (size_t)(blockIdx.x + (next_cta ? 1u : 0u)) * (16 * TOK) + e;
-                if (shared_first) {
-                    st_relaxed64(box, (1ull << 32) | __float_as_uint(sum));
-                    continue;
-                }
-                unsigned long long got = 0;
-                for (uint32_t i = 0; i < kSpinLimit && got == 0; ++i) got = ld_relaxed64(box);
-                if (got == 0) {  // (the row stays unwritten: the error word says so)
-                    if (err) atomicCAS(err, 0, 4 | (warp << 24));
-                    continue;
-                }
+                unsigned long long got = shared_first ? 0ull : ld_relaxed64(box);  // (the CTA after this one is nearly always the first)
+                if (got == 0) got = exch_relaxed64(box, (1ull << 32) | __float_as_uint(sum));
+                if (got == 0) continue;
                 st_relaxed64(box, 0ull);
                 sum += __uint_as_float((uint32_t)got);
             }

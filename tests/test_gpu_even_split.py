@@ -75,3 +75,32 @@ def test_even_split_repeats_itself_in_a_chain(B):
     y = binding.pot_gemv_noalloc(tiled, scales, K, bits, G, xs[0], torch.empty_like(alone[0]))
     assert torch.equal(y, alone[0])
     assert binding.pot_debug_errors() == (0, 0, 0)
+
+
+@pytest.mark.parametrize("M", [1, 4])
+def test_even_split_among_streams(B, M):
+    """Launches of four streams at once, with a product of 2048 tokens beside them: CTAs of a launch start at very different times, and whichever of
+    two that share a row block comes second adds the sums.  The same bits as alone, and nothing left in the workspaces."""
+    import torch
+    from paper_2507_11959_b200 import binding
+    N, K, bits, G = (2400, 8192, 3, 128) if M == 1 else (15360, 5120, 3, 128)
+    c = PotCase(N, K, bits, G, dist="t5", seed=(4, 980 + M))
+    tiled, scales, x = c.tiled(), c.tiled_S(), f16_dev(_acts(M, K, 981))
+    assert binding.pot_debug_gemv_split(M, N, K, bits, G) == 2
+    need = binding.pot_gemm_workspace_bytes(M, N, K, bits, G)
+    alone = binding.pot_gemm(tiled, scales, K, bits, G, x, binding.TILED, workspace=binding.new_workspace(need)).clone()
+    big, wide = f16_dev(_acts(2048, K, 982)), binding.new_workspace(binding.pot_gemm_workspace_bytes(2048, N, K, bits, G))
+    streams = [torch.cuda.Stream() for _ in range(4)]
+    spaces = [binding.new_workspace(need) for _ in streams]
+    ys = [[torch.empty_like(alone) for _ in range(12)] for _ in streams]
+    torch.cuda.synchronize()
+    for i in range(12):
+        for s, ws, y in zip(streams, spaces, ys):
+            with torch.cuda.stream(s):
+                binding.pot_gemm(tiled, scales, K, bits, G, x, binding.TILED, Y=y[i], workspace=ws)
+        if i % 4 == 0:
+            binding.pot_gemm(tiled, scales, K, bits, G, big, binding.TILED, workspace=wide)
+    torch.cuda.synchronize()
+    assert all(torch.equal(v, alone) for y in ys for v in y)
+    assert not any(ws[:148 * 16 * (1 if M == 1 else 8) * 8].any() for ws in spaces)
+    assert binding.pot_debug_errors() == (0, 0, 0)
