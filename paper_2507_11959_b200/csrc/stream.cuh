@@ -54,7 +54,8 @@ __host__ __device__ constexpr int sk_header_bytes(int warps, int tok) {
 // ---- even split (stream_even.cuh)
 // units that are dealt out together (straight-line code; with two of the four in a slot 12288 x 4096 took 8.2 instead of 7.3 us)
 __host__ __device__ constexpr int sk_block(int q) { return q == 2 ? 2 : 4; }
-// the workspace holds a number and a mark, 8 bytes, for each sum that goes from CTA to CTA (16 rows x tok of each CTA)
+// the workspace holds a number and a mark, 8 bytes, for each sum that goes from CTA to CTA (16 rows x tok of each CTA).  These places need not be
+// zero before a call, but they must hold no mark, and none is there after it.
 constexpr size_t sk_box_bytes(int tok) { return (size_t)kSmCount * 16 * (size_t)tok * 8; }
 
 struct StreamPlan {

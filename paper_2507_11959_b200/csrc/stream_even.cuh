@@ -30,6 +30,12 @@ __device__ __forceinline__ unsigned long long exch_relaxed64(unsigned long long*
     asm volatile("atom.exch.relaxed.gpu.global.b64 %0, [%1], %2;" : "=l"(old) : "l"(p), "l"(v) : "memory");
     return old;
 }
+// A sum on its way from CTA to CTA: the number in the lower half, a mark in the upper one.  What else may lie there is zero or the partial sums of a
+// product of more tokens (gemm_prefill.cu), pairs of FP32 numbers as tensor cores and FP32 additions leave them: their NaN is 0x7FFFFFFF and
+// never the mark, which is another one (PF_NO_SUM is a third).
+constexpr uint32_t SK_SUM_MARK = 0x7FD15C0Du;
+__device__ __forceinline__ unsigned long long sk_marked_sum(float v) { return ((unsigned long long)SK_SUM_MARK << 32) | __float_as_uint(v); }
+__device__ __forceinline__ bool sk_is_sum(unsigned long long v) { return (uint32_t)(v >> 32) == SK_SUM_MARK; }
 // shared-memory header: as sk_header_bytes, with four words between the local arrival counters and the slots of partial sums
 __host__ __device__ constexpr int sk_even_counters_at(int warps) { return warps * 96; }
 __host__ __device__ constexpr int sk_even_slots_at(int warps) { return warps * 100 + 16; }
@@ -321,8 +327,8 @@ __global__ void __launch_bounds__(W * 32, OCC) stream_even_kernel(const __grid_c
                 // itself (2400 x 8192 5.45 -> 5.84 us on one GPU, 5.96 -> 5.98 on another; 28672 x 8192 23.0, 5120 x 13824 11.4, both).
                 unsigned long long* box = reinterpret_cast<unsigned long long*>(sa.counters) + (size_t)(blockIdx.x + (next_cta ? 1u : 0u)) * (16 * TOK) + e;
                 unsigned long long got = shared_first ? 0ull : ld_relaxed64(box);  // (the CTA after this one is nearly always the first)
-                if (got == 0) got = exch_relaxed64(box, (1ull << 32) | __float_as_uint(sum));
-                if (got == 0) continue;
+                if (!sk_is_sum(got)) got = exch_relaxed64(box, sk_marked_sum(sum));
+                if (!sk_is_sum(got)) continue;
                 st_relaxed64(box, 0ull);
                 sum += __uint_as_float((uint32_t)got);
             }
