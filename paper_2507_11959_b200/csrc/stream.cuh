@@ -579,17 +579,21 @@ __device__ __forceinline__ void stream_body(const StreamKernelArgs<UNSC>& sa, in
         }
         __threadfence();
         __syncwarp();
+        // Arrivals are counted down: the first one finds zero, or more than the counter can hold, and puts expect - 1 there, the last one finds one and leaves
+        // zero.  So a counter need not be zero before the call: from row block 64 on it lies where a product of more tokens on the same matrix
+        // (gemm_prefill.cu) leaves FP32 partial sums.  As whole numbers these are larger than any count (38 there), but for sums from 2^-149 to 38 x 2^-149,
+        // which no FP16 product has, and a BF16 one only of activations some 2^-100 times the usual ones.
+        // (A sign that no sum can have, raised by a second atomic operation: 2048 x 8192 6.7 -> 7.3 us; bytes in the first 64 words as counters: 7.6.)
         unsigned prev = 0;
-        if (lane == 0) prev = atomicAdd(&sa.counters[rbd], 1u);
+        if (lane == 0) prev = atomicDec(&sa.counters[rbd], expect - 1u);
         prev = __shfl_sync(0xffffffffu, prev, 0);
-        if (prev == expect - 1u) {  // this warp delivered the last slot of the row block: add them in ascending order
+        if (prev == 1u) {  // this warp delivered the last slot of the row block: add them in ascending order
             __threadfence();
             for (int e = lane; e < 16 * (TOK == 1 ? 1 : sa.M); e += 32) {
                 float sum = 0.f;
                 for (uint32_t q = 0; q < expect; ++q) sum += __ldcg(base + (size_t)q * (16 * TOK) + e);
                 sa.Y[(int64_t)(e >> 4) * sa.N + row0 + (e & 15)] = sk_out<DT>(sum);
             }
-            if (lane == 0) sa.counters[rbd] = 0u;  // leave the workspace ready for the next call
         }
     };
 

@@ -38,3 +38,12 @@ def test_even_split_after_partial_sums_of_more_tokens(N, K, bits, G, tokens):
     plans = [(M, B.pot_debug_gemm_plan(M, N, K, bits, G)) for M in tokens]
     assert any(p["split_tiles"] for _, p in plans) and any(p["streaming"] and B.pot_debug_gemv_split(M, N, K, bits, G) == 2 for M, p in plans)
     run_sequence(N, K, bits, G, tokens)
+
+
+@pytest.mark.parametrize("N,K,bits,G,tokens", [
+    (2048, 8192, 3, 128, (32, 4, 1, 300, 2, 512, 8, 1)), (2400, 1152, 2, 64, (64, 4, 1, 16, 8, 2, 1)), (1536, 4608, 4, 128, (16, 4, 1, 300, 2, 1))])
+def test_unit_split_after_partial_sums_of_more_tokens(N, K, bits, G, tokens):
+    """Arrival counters of the row blocks, of which there may be more than 64: partial sums of more tokens lie behind them."""
+    plans = [(M, B.pot_debug_gemm_plan(M, N, K, bits, G)) for M in tokens]
+    assert any(p["split_tiles"] for _, p in plans) and all(B.pot_debug_gemv_split(M, N, K, bits, G) == 1 for M, p in plans if p["streaming"])
+    run_sequence(N, K, bits, G, tokens)
