@@ -84,8 +84,8 @@ size_t pot_scales_bytes(int64_t N, int64_t K, int group);         /* N * (K / gr
  * first use; every call leaves its counters and marks at zero again, so consecutive calls of the SAME entry point with the
  * SAME (N, K, bits, group) may reuse one buffer without clearing it.  The position of the
  * counters inside the buffer depends on the shape: a buffer handed to a call with another shape
- * (or to pot_gemm) must be cleared to zero first.  Two calls that may run concurrently
- * (different streams) need different workspaces.                                              */
+ * (or to pot_gemm) must be cleared to zero first, and so must one of a call after which pot_debug_gemv_error or one of its
+ * siblings reports a wait that gave up.  Two calls that may run concurrently (different streams) need different workspaces.   */
 size_t pot_gemv_workspace_bytes(int64_t N, int64_t K, int bits, int group);
 /* Scratch needed by pot_gemm for the given M; may be 0.                                       */
 size_t pot_gemm_workspace_bytes(int64_t M, int64_t N, int64_t K, int bits, int group);
@@ -292,8 +292,9 @@ pot_status_t pot_gemv_noalloc(const void* packed_tiled, const void* scales_f16, 
  * POT_LAYOUT_CANONICAL (any N, no workspace): M = 1 runs pot_gemv's kernel, larger M the tcgen05 kernel with
  * producers that decode canonical codes; few tiles are split along K over the CTAs of a cluster.  Into how many depends on
  * how many clusters the chip holds at once, so that two GPUs may add in different splits and differ in the last place.
- *   workspace >= pot_gemm_workspace_bytes(M,N,K,bits,group), 16-byte aligned, zero before its
- *   first use (the kernels leave the counters at zero); may be NULL when that size is 0.
+ *   workspace >= pot_gemm_workspace_bytes(M,N,K,bits,group), 16-byte aligned, zero before its first use; may be NULL when that size
+ *   is 0.  Consecutive calls of pot_gemm and pot_gemm_bf16 with the same (N, K, bits, group) and ANY M may share one
+ *   buffer, as large as the largest of them needs, without clearing it: what one call leaves in it is not taken for counters or marks by the next.
  */
 pot_status_t pot_gemm(const void* packed, const void* scales_f16, int64_t N, int64_t K, int bits,
                       int group, pot_layout_t layout, const void* X_f16, int64_t M, void* Y_f16,

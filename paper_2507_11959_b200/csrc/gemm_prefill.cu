@@ -810,13 +810,15 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
         }
         if (!CANON && !CLUSTER && splits > 1 && !gave_up && in_range(tail_index >= 0 && partial != nullptr && counters != nullptr, err, 0x61)) {
             // The CTA that delivers the last split of a tile (an arrival counter tells it) adds the splits in
-            // ascending order -- the result does not depend on timing -- and writes Y.
+            // ascending order -- the result does not depend on timing -- and writes Y.  Counted down from whatever is larger than a count, to
+            // zero, as in stream.cuh: the counters from 64 on lie where a product of another number of tokens on the same matrix, of up to 64 split
+            // tiles, leaves partial sums.  (Halves of the first 64 words: 400 tokens x 2048 x 8192 21.7 -> 21.9 us.)
             __shared__ unsigned s_prev;
             __threadfence();
             asm volatile("bar.sync 2, %0;" ::"n"(NPT) : "memory");
-            if (threadIdx.x == 32 * PROD_WARP0) s_prev = atomicAdd(&counters[tail_index], 1u);
+            if (threadIdx.x == 32 * PROD_WARP0) s_prev = atomicDec(&counters[tail_index], (unsigned)splits - 1u);
             asm volatile("bar.sync 2, %0;" ::"n"(NPT) : "memory");
-            if (s_prev == (unsigned)splits - 1u) {
+            if (s_prev == 1u) {
                 __threadfence();
                 // The epilogue threads walk the tile in 16-byte pieces, consecutive threads on consecutive
                 // pieces (coalesced), four pieces per thread in flight; the splits are added in ascending order.
@@ -848,7 +850,6 @@ pot_gemm_prefill_kernel(const __grid_constant__ CUtensorMap xmap, const uint4* _
                         }
                     }
                 }
-                if (threadIdx.x == 32 * PROD_WARP0) counters[tail_index] = 0u;  // leave the workspace ready for the next call
             }
         }
     }

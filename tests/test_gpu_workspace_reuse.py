@@ -47,3 +47,11 @@ def test_unit_split_after_partial_sums_of_more_tokens(N, K, bits, G, tokens):
     plans = [(M, B.pot_debug_gemm_plan(M, N, K, bits, G)) for M in tokens]
     assert any(p["split_tiles"] for _, p in plans) and all(B.pot_debug_gemv_split(M, N, K, bits, G) == 1 for M, p in plans if p["streaming"])
     run_sequence(N, K, bits, G, tokens)
+
+
+@pytest.mark.parametrize("N,K,bits,G,tokens", [(8192, 28672, 2, 128, (16, 2048, 16)), (1024, 28672, 3, 64, (32, 7680, 32, 7680))])
+def test_more_than_64_split_tiles_after_partial_sums_of_fewer(N, K, bits, G, tokens):
+    """The arrival counters of up to 74 split tiles, the last ten of which lie where products of other token counts leave partial sums."""
+    plans = {M: B.pot_debug_gemm_plan(M, N, K, bits, G) for M in tokens}
+    assert any(p["split_tiles"] > 64 and p["cluster"] == 0 for p in plans.values()) and any(0 < p["split_tiles"] <= 64 for p in plans.values())
+    run_sequence(N, K, bits, G, tokens)
