@@ -920,6 +920,12 @@ pot_status_t launch_stream(const void* packed, const void* scales, const void* z
                 auto run_even = [&](auto kernel) -> pot_status_t {
                     return launch_pdl_cluster(kernel, dim3((unsigned)p.grid), dim3(W * 32), p.smem_bytes, 1, true, s, even, err);
                 };
+                if constexpr (TOK > 1)  // (more than four tokens come here only with their activations in shared memory)
+                    if (M > 4 && p.x_in_smem) {
+                        if constexpr (DT == 0)
+                            if (p.unscaled) return run_even(stream_even_kernel<BITS, TOK, true, W, OCC, Q, DT, true, true>);
+                        return run_even(stream_even_kernel<BITS, TOK, true, W, OCC, Q, DT, false, true>);
+                    }
                 if constexpr (DT == 0 || TOK == 1)
                     if (p.unscaled) return run_even(stream_even_kernel<BITS, TOK, true, W, OCC, Q, DT, true>);
                 if constexpr (!(DT == 0 && TOK == 1))

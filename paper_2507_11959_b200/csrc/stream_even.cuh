@@ -40,8 +40,8 @@ __device__ __forceinline__ bool sk_is_sum(unsigned long long v) { return (uint32
 __host__ __device__ constexpr int sk_even_counters_at(int warps) { return warps * 96; }
 __host__ __device__ constexpr int sk_even_slots_at(int warps) { return warps * 100 + 16; }
 
-// Template parameters as of stream_kernel.
-template <int BITS, int TOK, bool XSMEM, int W, int OCC, int SK_Q, int DT, bool UNSC>
+// Template parameters as of stream_kernel; MANY: more than four tokens.
+template <int BITS, int TOK, bool XSMEM, int W, int OCC, int SK_Q, int DT, bool UNSC, bool MANY = false>
 __global__ void __launch_bounds__(W * 32, OCC) stream_even_kernel(const __grid_constant__ StreamArgsEven sa, int* __restrict__ err) {
     constexpr int UB = sk_unit_bytes(BITS);
     static_assert(!UNSC || (XSMEM && (DT == 0 || TOK == 1)), "the decode without the scale: x in shared memory, BF16 one token");
@@ -309,30 +309,78 @@ __global__ void __launch_bounds__(W * 32, OCC) stream_even_kernel(const __grid_c
         prev = __shfl_sync(0xffffffffu, prev, 0);
         if (prev != (unsigned)__popc(sharers) - 1u) return;
         __threadfence_block();
-        for (int e = lane; e < 16 * (TOK == 1 ? 1 : sa.M); e += 32) {
-            const float* at = lslots + e;
-            float sum = at[(wl * 2u + (shared_first ? 0u : 1u)) * (16 * TOK)];
-            for (uint32_t w = wl + 1; w <= wh; w += 4) {  // (four loads at a time; a warp between them that has no part of the row block adds nothing)
-                float p[4];
+        // Where two CTAs have sums of the row block, the one that finds the other's in the workspace adds the two (in either order the same number),
+        // and clears them for the next call.  Neither waits for the other, which may not have started (another stream's kernel on its SM).
+        // A bounded wait of the first CTA and a plain store in the second were as fast but for 0 - 0.5 us where a launch has an SM to
+        // itself (2400 x 8192 5.45 -> 5.84 us on one GPU, 5.96 -> 5.98 on another; 28672 x 8192 23.0, 5120 x 13824 11.4, both).
+        if constexpr (!MANY) {
+            for (int e = lane; e < 16 * (TOK == 1 ? 1 : sa.M); e += 32) {
+                const float* at = lslots + e;
+                float sum = at[(wl * 2u + (shared_first ? 0u : 1u)) * (16 * TOK)];
+                for (uint32_t w = wl + 1; w <= wh; w += 4) {  // (four loads at a time; a warp between them that has no part of the row block adds nothing)
+                    float p[4];
 #pragma unroll
-                for (uint32_t u = 0; u < 4; ++u) p[u] = at[min(w + u, wh) * 2u * (16 * TOK)];
+                    for (uint32_t u = 0; u < 4; ++u) p[u] = at[min(w + u, wh) * 2u * (16 * TOK)];
 #pragma unroll
-                for (uint32_t u = 0; u < 4; ++u)
-                    if (w + u <= wh && ((sharers >> (w + u)) & 1u)) sum += p[u];
+                    for (uint32_t u = 0; u < 4; ++u)
+                        if (w + u <= wh && ((sharers >> (w + u)) & 1u)) sum += p[u];
+                }
+                if (shared_first || next_cta) {
+                    unsigned long long* box = reinterpret_cast<unsigned long long*>(sa.counters) + (size_t)(blockIdx.x + (next_cta ? 1u : 0u)) * (16 * TOK) + e;
+                    unsigned long long got = shared_first ? 0ull : ld_relaxed64(box);  // (the CTA after this one is nearly always the first)
+                    if (!sk_is_sum(got)) got = exch_relaxed64(box, sk_marked_sum(sum));
+                    if (!sk_is_sum(got)) continue;
+                    st_relaxed64(box, 0ull);
+                    sum += __uint_as_float((uint32_t)got);
+                }
+                sa.Y[(int64_t)(e >> 4) * sa.N + row0 + (e & 15)] = sk_out<DT>(sum);
+            }
+        } else {
+            // Three or four sums per lane: all requests are on their way before the first answer is looked at (in the loop above 5 - 8 tokens take 4 - 10 %
+            // longer, 6 x 3552 x 5888 10.9 us, so 9.95, and on some matrices longer than with the unit split; one or two sums are the loop's: 2
+            // tokens 2 - 5 %, 4 tokens 1 %, and an instantiation of its own because both in one took them 1 - 2 % longer).
+            static_assert(TOK > 1, "several tokens");
+            constexpr int R = TOK / 2;
+            const int last = 16 * sa.M;
+            float sum[R];
+            uint32_t done = 0;  // bit r: sum r is complete
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                if (lane + 32 * r >= last) continue;
+                const float* at = lslots + lane + 32 * r;
+                sum[r] = at[(wl * 2u + (shared_first ? 0u : 1u)) * (16 * TOK)];
+                for (uint32_t w = wl + 1; w <= wh; w += 4) {
+                    float p[4];
+#pragma unroll
+                    for (uint32_t u = 0; u < 4; ++u) p[u] = at[min(w + u, wh) * 2u * (16 * TOK)];
+#pragma unroll
+                    for (uint32_t u = 0; u < 4; ++u)
+                        if (w + u <= wh && ((sharers >> (w + u)) & 1u)) sum[r] += p[u];
+                }
+                done |= 1u << r;
             }
             if (shared_first || next_cta) {
-                // Two CTAs have sums of the row block: the one that finds the other's in the workspace adds the two (in either order the same number),
-                // and clears them for the next call.  Neither waits for the other, which may not have started (another stream's kernel on its SM).
-                // A bounded wait of the first CTA and a plain store in the second were as fast but for 0 - 0.5 us where a launch has an SM to
-                // itself (2400 x 8192 5.45 -> 5.84 us on one GPU, 5.96 -> 5.98 on another; 28672 x 8192 23.0, 5120 x 13824 11.4, both).
-                unsigned long long* box = reinterpret_cast<unsigned long long*>(sa.counters) + (size_t)(blockIdx.x + (next_cta ? 1u : 0u)) * (16 * TOK) + e;
-                unsigned long long got = shared_first ? 0ull : ld_relaxed64(box);  // (the CTA after this one is nearly always the first)
-                if (!sk_is_sum(got)) got = exch_relaxed64(box, sk_marked_sum(sum));
-                if (!sk_is_sum(got)) continue;
-                st_relaxed64(box, 0ull);
-                sum += __uint_as_float((uint32_t)got);
+                unsigned long long* box = reinterpret_cast<unsigned long long*>(sa.counters) + (size_t)(blockIdx.x + (next_cta ? 1u : 0u)) * (16 * TOK) + lane;
+                unsigned long long got[R];
+#pragma unroll
+                for (int r = 0; r < R; ++r) got[r] = !shared_first && ((done >> r) & 1u) ? ld_relaxed64(box + 32 * r) : 0ull;
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+                    if (((done >> r) & 1u) && !sk_is_sum(got[r])) got[r] = exch_relaxed64(box + 32 * r, sk_marked_sum(sum[r]));
+                done = 0;
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+                    if (lane + 32 * r < last && sk_is_sum(got[r])) {
+                        st_relaxed64(box + 32 * r, 0ull);
+                        sum[r] += __uint_as_float((uint32_t)got[r]);
+                        done |= 1u << r;
+                    }
             }
-            sa.Y[(int64_t)(e >> 4) * sa.N + row0 + (e & 15)] = sk_out<DT>(sum);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int e = lane + 32 * r;
+                if ((done >> r) & 1u) sa.Y[(int64_t)(e >> 4) * sa.N + row0 + (e & 15)] = sk_out<DT>(sum[r]);
+            }
         }
         if (shared_first) {
             __threadfence_block();

@@ -104,3 +104,22 @@ def test_even_split_among_streams(B, M):
     assert all(torch.equal(v, alone) for y in ys for v in y)
     assert not any(ws[:148 * 16 * (1 if M == 1 else 8) * 8].any() for ws in spaces)
     assert binding.pot_debug_errors() == (0, 0, 0)
+
+
+@pytest.mark.parametrize("M", [5, 6, 7, 8])
+@pytest.mark.parametrize("bits,G", [(2, 128), (3, 64), (4, 128)])
+def test_even_split_of_five_to_eight_tokens(B, oracle, M, bits, G):
+    """Three or four sums per lane, the last of them with half of its lanes: the same bits from three calls on one workspace, no marks left in it."""
+    from paper_2507_11959_b200 import binding
+    for i, (N, K) in enumerate([(2480, 2048), (3552, 5888)]):
+        c = PotCase(N, K, bits, G, dist="t5", seed=(4, 1100 + 10 * bits + i))
+        X = _acts(M, K, 1110 + M)
+        for bf16 in (False, True):
+            assert binding.pot_debug_gemm_plan(M, N, K, bits, G, bf16)["streaming"] == 1 and binding.pot_debug_gemv_split(M, N, K, bits, G, bf16) == 2
+            Xb = f16_bits_to_bf16_bits(X) if bf16 else X
+            Y, A = oracle.matmul(c.packed, c.S, K, bits, G, Xb, dtype=oracle.BF16 if bf16 else oracle.F16)
+            ws = B.new_workspace(binding.pot_gemm_workspace_bytes(M, N, K, bits, G))
+            y = [bits_of(B.pot_gemm(c.tiled(), c.tiled_S(), K, bits, G, bf16_dev(Xb) if bf16 else f16_dev(Xb), binding.TILED, workspace=ws)) for _ in range(3)]
+            assert np.array_equal(y[0], y[1]) and np.array_equal(y[0], y[2]) and not ws[:148 * 16 * 8 * 8].any()
+            ok, worst, tight = gate(y[0], Y, A, bf16)
+            assert ok and tight < 4.0, (N, bf16, worst, tight)
