@@ -144,18 +144,27 @@ inline StreamPlan plan_stream(int64_t N, int64_t K, int64_t M, int bits, int gro
     if (st > need) st = need;
     if (st > 8) st = 8;
     if (st < 1) st = 1;
-    // Even split (PoT codes): every CTA takes the same number of blocks of units, wherever row blocks end.  A range is at least a row block
-    // long, so that a row block has two CTAs at most.  Instead of the unit split always (us: 2480 x 4096 5.7 -> 3.7, 2400 x 8192 6.9 -> 5.4, 7136 x
-    // 4096 7.6 -> 5.4, 5120 x 13824 12.4 -> 11.4, eight layers of 2048 / 5504 260 -> 227, of 3200 / 8576 270 -> 232); all calls of a shape then keep the
-    // same things in the workspace.  Instead of whole row blocks with one CTA per SM, whose launch nothing hides and which gains by the shorter way
-    // to the first copies: one token always but at 2 bits in BF16 (28672 x 8192 25.0 -> 23.1, 15360 x 8192 17.0 -> 14.7, whole row blocks of
-    // 18944 x 8192 17.1 -> 16.7; BF16, 2 bits 17792 x 7552 15.7 -> 16.4); several tokens, whose sums cost more on their way, where the longest
-    // CTA gets rid of 16 units: 15360 x 5120 (20 units) 12.8 -> 11.3 at 2 tokens, 13.4 -> 12.5 at 4; 4096 x 11008 (23, but of two row
-    // blocks) 10.4 -> 12.0, 8 tokens x 15360 x 5120 13.9 -> 14.3.  Two CTAs per SM: alone 12288 x 4096 7.8 -> 7.3, but 11008 x 4096 6.9 -> 7.25, 4096 x 4096 3.5
-    // -> 4.2, and nothing is left where such launches follow one another (eight layers of 4096 / 11008 274 -> 276, 2 bits 245 -> 250).
+    // Even split (PoT codes): every CTA takes the same number of blocks of units, wherever row blocks end.  A range is no shorter than a row block, or
+    // (the last CTA's, by up to three units) lies inside one, so that a row block has two CTAs at most.  Instead of the unit split always (us: 2480 x 4096
+    // 5.7 -> 3.75, 2400 x 8192 6.9 -> 5.95, 7136 x 4096 7.5 -> 5.8, 5120 x 13824 12.4 -> 11.4, eight layers of 2048 / 5504 259 -> 226, of 3200 / 8576
+    // 269 -> 240).  Instead of whole row blocks with one CTA per SM, whose launch nothing hides and which gains by the shorter way to the first copies:
+    //  * one token always (28672 x 8192 25.0 -> 23.1, 15360 x 8192 17.0 -> 14.7, whole row blocks of 18944 x 8192 17.1 -> 16.7; 4 bits, BF16,
+    //    G = 64, 28672 x 8192 28.3 -> 28.0) but at 2 bits in BF16 (17792 x 7552 15.7 -> 16.4), and on long rows, whose activations come in front of all
+    //    but the first chunk, only where the longest CTA gets rid of 56 units (7104 x 21760, of none, 18.3 -> 19.3; 4352 x 28672, of 37, 16.2 -> 17.1);
+    //  * several tokens, whose sums cost more on their way, where the longest CTA, of three row blocks or more, gets rid of 16 units: two tokens (15360 x
+    //    5120 12.8 -> 11.3; 4096 x 11008, of two row blocks, 10.4 -> 12.0), and BF16, which takes longer per unit.  Three and four FP16 tokens: of 40
+    //    units (13200 x 9088, 38, 17.3 -> 18.3; 6240 x 6528 at 2 bits, 19, 8.7 -> 10.1), 64 at 2 and 3 bits in three or four row blocks (8096 x
+    //    9088, 42, 13.1 -> 14.1); or where x is read through L2 (9200 x 22656 45.2 -> 39.4); or on short rows of 2 or 3 bits in six row blocks and
+    //    more (15360 x 5120, 21, 13.4 -> 12.6; in five 10288 x 4096, 21, 8.9 -> 9.25; 14336 x 3456 at 2 bits 8.55 -> 9.45, at
+    //    4 bits 15440 x 4352 11.7 -> 12.4).
+    // Drawn matrices, of those that the rule takes: one token 0.93 of the time with whole row blocks (250; one above 1.01), two to four 0.94 (400, of
+    // which 4 % take 1 - 6 % longer).
+    // Two CTAs per SM: alone 12288 x 4096 7.8 -> 7.3, but 11008 x 4096 6.9 -> 7.25, 4096 x 4096 3.5 -> 4.2, and nothing is left where such
+    // launches follow one another (eight layers of 4096 / 11008 274 -> 276, 2 bits 245 -> 250).
     const int64_t block = sk_block(q), blocks = (U + block - 1) / block, saved = rb_max * ncb - U / p.grid;
-    p.even = kind == SK_POT && p.grid == kSmCount && U / 4 / p.grid * 4 >= ncb && ncb > 1 &&
-             (!p.aligned || (occ == 1 && (tok == 1 ? dt == 0 || bits > 2 : M <= 4 && rb_max >= 3 && saved >= 16)));
+    const bool pays = tok == 1 ? (dt == 0 || bits > 2) && (ncb <= 110 || saved >= 56)
+                               : M <= 4 && rb_max >= 3 && saved >= 16 && (M == 2 || dt == 1 || saved >= (rb_max > 4 || bits == 4 ? 40 : 64) || !p.x_in_smem || (bits <= 3 && rb_max >= 6 && saved >= 18 && ncb >= (bits == 2 ? 33 : 24) && ncb <= 60));
+    p.even = kind == SK_POT && p.grid == kSmCount && U / 4 / p.grid * 4 >= ncb && ncb > 1 && (!p.aligned || (occ == 1 && pays));
     p.cta_blocks = (uint32_t)(blocks / p.grid);
     p.cta_more = (uint32_t)(blocks % p.grid);
     if (p.even) {  // a warp has a part of the CTA's first row block, if that is shared, and a part of the rest

@@ -260,3 +260,17 @@ def test_four_warp_ctas_of_the_canonical_gemv_where_they_deal_the_row_blocks_out
         assert "".join(str(p[1]) for p in plans) == want and all(p[0] == 4 and p[2] == 1 for p in plans), (N, K, plans)
     assert [B.pot_debug_canonical_gemv_plan(N, K, 3) for N, K in ((38001, 512), (18993, 1152), (1001, 4096), (555, 11008), (96, 28672), (9, 65536), (5, 65664))] == [
         (1, 8, 1), (2, 8, 1), (8, 8, 1), (8, 8, 2), (8, 8, 4), (8, 8, 4), (0, 8, 0)]
+
+
+def test_the_units_are_dealt_out_evenly_where_that_is_faster(L):
+    """Shapes at which whole row blocks per CTA (0), or the even split (2), were measured to be the faster ones; the even split wherever whole row blocks do not
+    divide."""
+    from paper_2507_11959_b200 import binding as B
+    split = lambda M, N, K, bits, G, bf16: B.pot_debug_gemv_split(M, N, K, bits, G, bf16)
+    one = {(28672, 8192, 3, 128, False): 2, (15360, 8192, 3, 128, False): 2, (18944, 8192, 3, 128, False): 2, (28672, 8192, 2, 128, True): 0, (7104, 21760, 3, 64, False): 0,
+           (4352, 28672, 3, 64, False): 0, (9200, 20352, 2, 128, False): 0, (8192, 28672, 3, 128, False): 2, (12288, 4096, 3, 128, False): 0, (5120, 13824, 3, 128, False): 2}
+    assert {k: split(1, *k) for k in one} == one
+    several = {(2, 15360, 5120, 3, 128, False): 2, (2, 4096, 11008, 3, 128, False): 0, (4, 15360, 5120, 3, 128, False): 2, (4, 15360, 5120, 4, 128, False): 0, (4, 6240, 6528, 2, 128, False): 0,
+               (4, 13200, 9088, 3, 128, False): 0, (4, 13200, 9088, 3, 128, True): 2, (3, 8288, 6016, 2, 128, False): 0, (4, 8784, 9472, 3, 128, False): 0, (4, 9200, 22656, 3, 64, False): 2,
+               (4, 10288, 4096, 3, 64, False): 0, (3, 8096, 9088, 3, 128, False): 0, (3, 14336, 3456, 2, 128, False): 0, (4, 15440, 4352, 4, 128, False): 0, (5, 15360, 5120, 3, 128, False): 0, (8, 3552, 5888, 3, 64, False): 2}
+    assert {k: split(*k) for k in several} == several
