@@ -205,8 +205,8 @@ pot_status_t pot_dequant(const void* packed, const void* scales_f16, int64_t N, 
  * accumulation, FP16 output.  Codes are decoded in registers with the integer-add trick (Sec.
  * 4.2).  Tiled layout: every warp streams its own contiguous share of the codes and scales
  * through a private shared-memory ring, the decoded FP16 weights are the A fragments of
- * warp-level tensor-core MMAs whose B columns all hold x, and the matrix is split evenly across
- * all warps of the GPU (partial sums of a row block that spans warps are added in a fixed order --
+ * warp-level tensor-core MMAs whose B columns all hold x, and the matrix is divided by whole row blocks or evenly among the
+ * CTAs, or among all warps of the GPU (pot_debug_gemv_split; partial sums of a row block that spans warps are added in a fixed order --
  * in shared memory inside a CTA, through `workspace` across CTAs -- so results are bit-identical
  * run to run).  Where x fits in shared memory the MMAs take +-2^E and each unit's FP32 sums are multiplied by the scale.
  * Canonical layout: warps of 16 rows on the same MMAs with the codes decoded by byte look-ups, the sums of a row block's

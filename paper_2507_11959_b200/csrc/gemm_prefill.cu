@@ -143,8 +143,9 @@ __device__ __forceinline__ void pf_cluster_sync() {
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
     __syncwarp();
 }
-// the same where nothing that was written has to be seen behind it (a release waits until the stores to Y have reached L2: 200 tokens x
-// 4099 x 11008 25.9 us, without 25.5)
+// The same where nothing that was written has to be seen behind it, and everything that was read from a peer has been used before it: a warp whose
+// stores to Y, which are made of what it read, have been issued has no load from a peer under way any more, so that the peer may go.  (A release
+// waits until the stores have reached L2: 200 tokens x 4099 x 11008 25.9 us, without 25.5.)
 __device__ __forceinline__ void pf_cluster_sync_relaxed() {
     asm volatile("barrier.cluster.arrive.relaxed;\n\tbarrier.cluster.wait;" ::: "memory");
     __syncwarp();

@@ -525,14 +525,11 @@ extern "C" pot_status_t pot_gemv_noalloc(const void* packed_tiled, const void* s
     st = check_gemv_args(packed_tiled, scales, N, K, bits, group, POT_LAYOUT_TILED, x, y, scratch, kNoAllocScratchBytes);
     if (st != POT_OK) return st;  // nothing has been enqueued yet
     if (need == 0) return pot_gemv(packed_tiled, scales, N, K, bits, group, POT_LAYOUT_TILED, x, y, nullptr, 0, stream);
-    // The array keeps whatever the previous call left in it.  Only the arrival counters, or the places of the sums that go from
-    // CTA to CTA, have to start at zero (partial sums are fully overwritten before they are read), so clear just those.
+    // The array keeps whatever the previous call, of any shape, left in it.  Only the arrival counters, or the places of the sums that go
+    // from CTA to CTA, have to start without counts or marks (partial sums are fully overwritten before they are read), so clear just those.
     size_t clear = plan_stream(N, K, 1, bits, group, SK_POT, 1, 16).ws_counters;
     if (clear < sk_box_bytes(1)) clear = sk_box_bytes(1);
     if (cudaMemsetAsync(scratch, 0, clear, (cudaStream_t)stream) != cudaSuccess) return POT_ERR_CUDA;
     return pot_gemv(packed_tiled, scales, N, K, bits, group, POT_LAYOUT_TILED, x, y, scratch, need, stream);
 }
 
-#ifdef SK_TRACE
-extern "C" void pot_debug_set_trace(void* p) { pot::g_sk_trace = (unsigned long long*)p; }
-#endif

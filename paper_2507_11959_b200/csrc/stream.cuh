@@ -200,9 +200,6 @@ struct StreamArgs {
     int token_shift;               // log2 of the token slots of the staged activations
     int fits32;                    // U * gw_total < 2^32: 32-bit range arithmetic
     int aligned, nrb;              // row-block split (see the kernel), number of row blocks
-#ifdef SK_TRACE
-    unsigned long long* trace;     // [launch slot][cta][8] globaltimer stamps
-#endif
 };
 // What only the decode without the scale reads (a type of its own: with twelve more words the parameters of
 // stream_kernel_by_value no longer fit in its registers).
@@ -334,18 +331,6 @@ __device__ __forceinline__ void stream_body(const StreamKernelArgs<UNSC>& sa, in
     extern __shared__ __align__(128) unsigned char smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int gid = lane >> 2, tig = lane & 3;  // MMA fragment coordinates: rows gid and gid + 8, quarter tig
-#ifdef SK_TRACE
-    auto stamp = [&](int i) {
-        if (sa.trace && lane == 0 && (warp == 0 || warp == W - 1)) {
-            unsigned long long t;
-            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-            sa.trace[((size_t)blockIdx.x * 2 + (warp ? 1 : 0)) * 8 + i] = t;
-        }
-    };
-    stamp(0);
-#else
-    auto stamp = [&](int) {};
-#endif
     const int S = sa.stages;
     const int spg = 128 / sa.group;
     const uint32_t PB = 32u * (uint32_t)spg;                 // parameter bytes of one unit
@@ -399,7 +384,6 @@ __device__ __forceinline__ void stream_body(const StreamKernelArgs<UNSC>& sa, in
         if ((uint32_t)lane < nchunks) issue(a, n, (uint32_t)lane, (uint32_t)lane);
     }
     __syncwarp();
-    stamp(7);
     pdl_launch_dependents();
 
     // ---- row blocks of the range; which of its segments are partial, and their place among the contributors
@@ -429,9 +413,7 @@ __device__ __forceinline__ void stream_body(const StreamKernelArgs<UNSC>& sa, in
     }
     if (threadIdx.x < W) lcnt[threadIdx.x] = 0u;
 
-    stamp(1);
     pdl_wait();  // x, Y and the workspace may belong to the previous kernel in the stream
-    stamp(2);
     float* factors = nullptr;  // BF16 without the scale: one per unit
     if constexpr (FACTORS) factors = reinterpret_cast<float*>(smem + sa.factors_at);
     bool inexact = false;
@@ -492,7 +474,6 @@ __device__ __forceinline__ void stream_body(const StreamKernelArgs<UNSC>& sa, in
     }
     if constexpr (FACTORS) inexact = __syncthreads_or(inexact);
     else __syncthreads();
-    stamp(3);
 
     float acc[2][4];
 #pragma unroll
@@ -761,7 +742,6 @@ __device__ __forceinline__ void stream_body(const StreamKernelArgs<UNSC>& sa, in
                 }
                 return false;
             }
-            if (j == 0) stamp(4);
             const bool full = left >= (uint32_t)SK_Q && cb + (uint32_t)SK_Q <= ncb;
             bool some = false, all = MARKS;  // some, all units of a full chunk are marked
             if constexpr (MARKS) {
@@ -831,9 +811,7 @@ __device__ __forceinline__ void stream_body(const StreamKernelArgs<UNSC>& sa, in
     } else {
         if (!main_loop(std::false_type())) return;
     }
-    stamp(5);
     if (n && cb != 0) deliver(rb);
-    stamp(6);
 }
 
 template <int BITS, int KIND, int TOK, bool XSMEM, int W, int OCC, int SK_Q, int DT, bool UNSC>
@@ -858,9 +836,6 @@ constexpr auto stream_kernel_of() {
 #include "stream_even.cuh"
 namespace pot {
 
-#ifdef SK_TRACE
-inline unsigned long long* g_sk_trace = nullptr;   // next launch's trace block (advanced per launch)
-#endif
 // ---- host side --------------------------------------------------------------------------------------------
 inline StreamArgs stream_args(const StreamPlan& p, const void* packed, const void* scales, const void* zeros, int64_t N,
                               int64_t K, int group, const void* X, int M, void* Y, void* workspace) {
@@ -885,10 +860,6 @@ inline StreamArgs stream_args(const StreamPlan& p, const void* packed, const voi
     sa.max_slots = p.max_slots;
     sa.M = M;
     sa.token_shift = p.token_shift;
-#ifdef SK_TRACE
-    sa.trace = g_sk_trace;
-    if (g_sk_trace) g_sk_trace += 148 * 2 * 8;
-#endif
     sa.fits32 = ((uint64_t)p.units + 1) * ((uint64_t)sa.gw_total + 1) < (uint64_t(1) << 32) ? 1 : 0;
     return sa;
 }

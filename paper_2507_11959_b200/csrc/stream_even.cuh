@@ -10,7 +10,7 @@
 // have 12), of a row block's many contributors (unit split).  Where the kernel has an SM to itself nothing hides its launch: it asks for one
 // chunk per warp, then for the activations, then for the rest of the ring (with all chunks first the activations arrive behind them:
 // 28672 x 8192 24.3 us, so 23.1), and divisions by the number of column blocks are multiplications (the ranges took 1200 cycles).  Before -> after:
-// 28672 x 8192 25.0 -> 23.1 us (3 bits), 28.3 -> 27.7 (4 bits, BF16), 5120 x 13824 12.4 -> 11.4, 2400 x 8192 6.9 -> 5.4, 4 tokens x 15360 x 5120 13.4 -> 12.5.
+// 28672 x 8192 25.0 -> 23.1 us (3 bits), 28.2 -> 28.0 (4 bits, BF16, G = 64), 5120 x 13824 12.4 -> 11.4, 2400 x 8192 6.9 -> 5.95, 4 tokens x 15360 x 5120 13.4 -> 12.6.
 #pragma once
 #include "stream.cuh"
 
@@ -49,18 +49,6 @@ __global__ void __launch_bounds__(W * 32, OCC) stream_even_kernel(const __grid_c
     extern __shared__ __align__(128) unsigned char smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int gid = lane >> 2, tig = lane & 3;  // MMA fragment coordinates: rows gid and gid + 8, quarter tig
-#ifdef SK_TRACE
-    auto stamp = [&](int i) {
-        if (sa.trace && lane == 0 && (warp == 0 || warp == W - 1)) {
-            unsigned long long t;
-            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-            sa.trace[((size_t)blockIdx.x * 2 + (warp ? 1 : 0)) * 8 + i] = t;
-        }
-    };
-    stamp(0);
-#else
-    auto stamp = [&](int) {};
-#endif
     const int S = sa.stages;
     const int spg = 128 / sa.group;
     const uint32_t PB = 32u * (uint32_t)spg;                 // parameter bytes of one unit
@@ -117,11 +105,14 @@ __global__ void __launch_bounds__(W * 32, OCC) stream_even_kernel(const __grid_c
         if ((uint32_t)lane >= from && (uint32_t)lane < to && lane < S && (uint32_t)lane < nchunks) issue(a, n, la, ln, (uint32_t)lane, (uint32_t)lane);
     };
     // Two CTAs per SM: this one's first copies, 100 KB, would be in the way of the activations that the one beside it, of the launch before, is
-    // just waiting for (eight layers of 3200 / 8576 240 us, with this pause 232; of 2048 / 5504 222 and 227; 300 ns: 235, 224).
+    // just waiting for.  us with this pause / without it / without it and with all but the first chunk behind the activations: eight layers of
+    // 3200 / 8576 240.1 / 247.3 / 243.7, of 2048 / 5504 226.3 / 222.2 / 226.2, of 2816 / 7040 202.2 / 203.8 / 204.3, of 2560 / 6912 at 2 bits 171.5 /
+    // 174.1 / 176.6.  Behind another kernel, which does not let this one in early, it is lost time: 2480 x 4096 6.7 / 6.2 / 6.3 (unit split 8.0),
+    // 7136 x 4096 10.2 / 9.7 / 9.3 (11.4), 5120 x 13824 16.0 / 15.5 / 14.6 (16.4).  A pause that ends with the previous kernel: 240 -> 238 and 226
+    // -> 228, but 2480 x 2048 at 2 bits 2.8 -> 3.1; with both orders in one launch the chains took 1 - 4 % longer.
     if constexpr (OCC == 2) __nanosleep(1000);
     request(0, late ? 1u : 8u);
     __syncwarp();
-    stamp(7);
     pdl_launch_dependents();
 
     // ---- row blocks of the range; which of its segments are partial, and their place among the contributors
@@ -158,9 +149,7 @@ __global__ void __launch_bounds__(W * 32, OCC) stream_even_kernel(const __grid_c
         }
     };
 
-    stamp(1);
     pdl_wait();  // x, Y and the workspace may belong to the previous kernel in the stream
-    stamp(2);
     float* factors = nullptr;  // BF16 without the scale: one per unit
     if constexpr (FACTORS) factors = reinterpret_cast<float*>(smem + sa.factors_at);
     bool inexact = false;
@@ -225,7 +214,6 @@ __global__ void __launch_bounds__(W * 32, OCC) stream_even_kernel(const __grid_c
     }
     if constexpr (FACTORS) inexact = __syncthreads_or(inexact);
     else __syncthreads();
-    stamp(3);
 
     float acc[2][4];
 #pragma unroll
@@ -522,7 +510,6 @@ __global__ void __launch_bounds__(W * 32, OCC) stream_even_kernel(const __grid_c
                 }
                 return false;
             }
-            if (j == 0) stamp(4);
             const bool full = left >= (uint32_t)SK_Q && cb + (uint32_t)SK_Q <= ncb;
             bool some = false, all = MARKS;  // some, all units of a full chunk are marked
             if constexpr (MARKS) {
@@ -605,7 +592,6 @@ __global__ void __launch_bounds__(W * 32, OCC) stream_even_kernel(const __grid_c
     } else {
         if (!main_loop(std::false_type())) return;
     }
-    stamp(6);
 }
 
 }  // namespace pot

@@ -2,14 +2,14 @@
 import numpy as np
 import pytest
 
-from tests.gpu_util import GuardedBinding, PotCase, bf16_dev, bits_of, f16_bits_to_bf16_bits, f16_dev, gate
+from tests.gpu_util import GuardedBinding, PotCase, bf16_dev, bits_of, f16_bits_to_bf16_bits, f16_dev, gate, to_dev
 
 pytestmark = pytest.mark.gpu
 
 # (N, K): row blocks per CTA from just above one to many; K of few and odd numbers of column blocks; shared row blocks of which the second CTA
 # has a single unit or all but one; x that does not fit into shared memory (4 tokens x 14336
-# at 4 bits)
-SHAPES = [(2480, 2048), (2992, 1792), (3088, 4224), (2720, 4224), (13024, 384), (7136, 1152), (5200, 2048), (2400, 8192), (2528, 14336)]
+# at 4 bits); a last CTA whose units all lie in a row block that the one before it began (2528 x 2432: 18 units of 19, 2480 x 4992: 37 of 39)
+SHAPES = [(2480, 2048), (2992, 1792), (3088, 4224), (2720, 4224), (13024, 384), (7136, 1152), (5200, 2048), (2400, 8192), (2528, 14336), (2528, 2432), (2480, 4992)]
 
 
 @pytest.fixture(scope="module")
@@ -28,14 +28,13 @@ def test_even_split_matches_oracle(B, oracle, N, K, bits, G):
     from paper_2507_11959_b200 import binding
     c = PotCase(N, K, bits, G, dist="t5", seed=(4, 900 + bits))
     tiled, scales = c.tiled(), c.tiled_S()
-    reached = 0
     for M in (1, 2, 4, 8):
         X = _acts(M, K, 900 + M)
         for bf16 in (False, True):
             Xb = f16_bits_to_bf16_bits(X) if bf16 else X
             if binding.pot_debug_gemm_plan(M, N, K, bits, G, bf16)["streaming"] == 0:
                 continue
-            reached += binding.pot_debug_gemv_split(M, N, K, bits, G, bf16) == 2
+            assert binding.pot_debug_gemv_split(M, N, K, bits, G, bf16) == 2
             Y, A = oracle.matmul(c.packed, c.S, K, bits, G, Xb, dtype=oracle.BF16 if bf16 else oracle.F16)
             ws = B.new_workspace(binding.pot_gemm_workspace_bytes(M, N, K, bits, G))
             Xd = bf16_dev(Xb) if bf16 else f16_dev(Xb)
@@ -47,7 +46,31 @@ def test_even_split_matches_oracle(B, oracle, N, K, bits, G):
             ok, worst, tight = gate(first, Y, A, bf16)
             assert ok and tight < 4.0, (M, bf16, worst, tight)
             assert not ws[:148 * 16 * (1 if M == 1 else 8) * 8].any(), (M, bf16)
-    assert reached >= 2
+
+
+# One CTA per SM, whose ring is filled behind the activations: slots of 8 units (2 and 3 bits) and of 4; row blocks shared by two CTAs and not;
+# BF16 with and without the scale (2 bits keep whole row blocks)
+@pytest.mark.parametrize("N,K", [(28672, 8192), (18944, 8192), (15376, 9088)])
+@pytest.mark.parametrize("bits,G", [(2, 64), (2, 128), (3, 64), (3, 128), (4, 64), (4, 128)])
+def test_one_token_with_one_cta_per_sm_matches_oracle(B, oracle, N, K, bits, G):
+    from paper_2507_11959_b200 import binding
+    small = PotCase(1009, K, bits, G, dist="t5", seed=(4, 1200 + bits))
+    row = np.arange(N) % small.N     # the matrix repeats the rows of a small one
+    tiled, scales = binding.pot_repack(to_dev(small.packed[row]), K, bits, 0), binding.pot_repack_scales(f16_dev(small.S[row]), K, G, 0)
+    X = _acts(1, K, 1210)
+    for bf16 in (False, True):
+        plan = binding.pot_debug_gemv_decode(N, K, bits, G, bf16)
+        if plan["ctas_per_sm"] != 1:
+            assert N * K < 28672 * 8192
+            continue
+        assert binding.pot_debug_gemv_split(1, N, K, bits, G, bf16) == (0 if bf16 and bits == 2 else 2)
+        Xb = f16_bits_to_bf16_bits(X) if bf16 else X
+        Y, A = oracle.matmul(small.packed, small.S, K, bits, G, Xb, dtype=oracle.BF16 if bf16 else oracle.F16)
+        ws = B.new_workspace(binding.pot_gemv_workspace_bytes(N, K, bits, G))
+        y = [bits_of(B.pot_gemv(tiled, scales, K, bits, G, bf16_dev(Xb[0]) if bf16 else f16_dev(Xb[0]), binding.TILED, workspace=ws)) for _ in range(3)]
+        assert np.array_equal(y[0], y[1]) and np.array_equal(y[0], y[2]) and not ws[:148 * 16 * 8].any()
+        ok, worst, tight = gate(y[0], Y[0][row], A[0][row], bf16)
+        assert ok and tight < 4.0, (bf16, worst, tight)
 
 
 def test_even_split_repeats_itself_in_a_chain(B):

@@ -47,12 +47,13 @@ def test_config1_gemv_4096x4096_3bit(B, oracle):
 @pytest.mark.parametrize("bits", [2, 3])
 def test_config2_llama7b_projections(B, oracle, bits):
     """The five 7B projections as bench.py runs them: every one takes the two-CTAs-per-SM variant (a chain must not mix
-    the variants); the one-CTA variant is reached by the 28672 x 8192 and 13B tests below."""
+    the variants) with whole row blocks per CTA; the one-CTA variant is reached by the 28672 x 8192 test below and in test_gpu_even_split."""
     seen = set()
     for i, pr in enumerate(synth.LLAMA2_7B):
         if pr.name == "up":
             continue  # same shape as gate
         plan = check_gemv(B, oracle, pr.N, pr.K, bits, "t5", (2, 2 * i))
+        assert B.pot_debug_gemv_split(1, pr.N, pr.K, bits, 128) == 0
         seen.add(plan["ctas_per_sm"])
         assert plan["units_per_slot"] == (2 if pr.K == 11008 and bits == 3 else 4), (pr.name, plan)
     assert seen == {2}, seen
@@ -71,10 +72,13 @@ def test_config2_uniform_twin_gate_and_down(B, oracle, bits):
         assert ok and tight < 4.0, (N, K, worst, tight)
 
 
-def test_unit_split_with_sums_crossing_ctas_at_full_width(B, oracle):
-    """13B down (5120 x 13824) keeps the even unit split: 320 row blocks of 108 units on 148 CTAs, so most row blocks are
-    shared between CTAs and go through the workspace."""
+def test_sums_crossing_ctas_at_full_width(B, oracle):
+    """13B down (5120 x 13824): 320 row blocks of 108 units on 148 CTAs, the even split, so most row blocks are shared by two CTAs.  2048 x 28672 has a row
+    block for fewer CTAs than there are: the unit split, whose row blocks several warps of two or three CTAs share."""
     check_gemv(B, oracle, 5120, 13824, 3, "t5", (4, 30), {"row_block_split": 0})
+    assert B.pot_debug_gemv_split(1, 5120, 13824, 3, 128) == 2
+    check_gemv(B, oracle, 2048, 28672, 3, "t5", (4, 32), {"row_block_split": 0})
+    assert B.pot_debug_gemv_split(1, 2048, 28672, 3, 128) == 1
 
 
 @pytest.mark.parametrize("M", list(synth.SMALL_BATCH_M))
@@ -126,6 +130,7 @@ def test_config3_dequant_largest_matrix_sampled_rows(B, oracle, bits):
     # the same matrix through the fused GEMV (a share per CTA large enough for the one-CTA-per-SM variant)
     plan = B.pot_debug_gemv_plan(N, K, bits, G)
     assert plan["ctas_per_sm"] == 1 and plan["units_per_slot"] == (4 if bits == 4 else 8), plan
+    assert B.pot_debug_gemv_split(1, N, K, bits, G) == 2
     X = synth.activations(synth.rng_for(3, 650 + bits), 1, K)
     Y, A = oracle.matmul(c.packed, c.S, K, bits, G, X, rows=rows)
     y = bits_of(B.pot_gemv(c.tiled(), c.tiled_S(), K, bits, G, f16_dev(X[0]), B.TILED))
