@@ -154,63 +154,7 @@ __global__ void __launch_bounds__(W * 32, OCC) stream_even_kernel(const __grid_c
     if constexpr (FACTORS) factors = reinterpret_cast<float*>(smem + sa.factors_at);
     bool inexact = false;
     if constexpr (XSMEM) {
-        uint4* dst = reinterpret_cast<uint4*>(smem + HDR);
-        const uint4* src = reinterpret_cast<const uint4*>(sa.X);
-        const int kc = (int)(sa.K / 8);  // 16-byte chunks per token
-        if constexpr (UNSC && TOK == 1)
-            if (threadIdx.x < SK_ZERO_BYTES / 16) *reinterpret_cast<uint4*>(smem + sa.zeros_at + threadIdx.x * 16) = make_uint4(0, 0, 0, 0);
-        if constexpr (TOK == 1) {
-            // chunk (quarter t, part j) of a unit goes to position j * 4 + t: lanes tig = 0..3 read 64 contiguous bytes
-            // (four loads in flight per thread before the first store: one round trip for K <= 32 * 32 W)
-            // (a bound for whole warps, here and below: 0.5 - 0.8 % of an eight-layer token in the two-CTA build)
-            if (OCC == 1 && (int)(threadIdx.x & ~31u) >= kc) behind_loads();  // (a warp that loads nothing)
-            for (int i0 = threadIdx.x; (i0 & ~31) < kc; i0 += 4 * W * 32) {
-                uint4 v[4];
-#pragma unroll
-                for (int p = 0; p < 4; ++p)
-                    if (i0 + p * W * 32 < kc) v[p] = ld_dependent16(src + i0 + p * W * 32);
-                if (OCC == 1 && i0 == threadIdx.x) behind_loads();
-#pragma unroll
-                for (int p = 0; p < 4; ++p) {
-                    const int i = i0 + p * W * 32;
-                    if constexpr (FACTORS) {  // lanes 0-15 and 16-31 hold one unit each
-                        const float f = sk_normalize(v[p], i < kc);
-                        inexact = inexact || (i < kc && f < 0.f);
-                        if (i < kc && (i & 15) == 0) factors[i >> 4] = f * potl::POT_UNIT_SCALE;
-                    }
-                    if (i < kc) dst[(i & ~15) | ((i & 3) << 2) | ((i >> 2) & 3)] = v[p];
-                }
-            }
-        } else {
-            // T = 2, 4 or 8 token slots (the smallest that holds M).  Chunk (token, unit, quarter t, part j) goes to
-            // 16-byte slot (unit * 4 + j) * 4 T + (token / 2) * 8 + (token % 2) * 4 + t: the eight lanes of a quarter-warp
-            // of the MMA loop (tokens 2q and 2q + 1, quarters 0..3) read one 128-byte line, a warp 4 lines -- no bank
-            // conflict (token-major slots cost four-way conflicts: 11 against 8 us in the loop at 5+ tokens).  With fewer
-            // than 8 slots the MMA columns beyond T repeat the first T tokens; they are never delivered, like the
-            // tokens >= M.  The threads are numbered so that a quarter-warp also STORES one line: t fastest, then the
-            // token's parity, then j -- a warp loads the 256 contiguous bytes of a unit for two tokens.
-            const int ts = sa.token_shift;
-            const int total = kc << ts;
-            if (OCC == 1 && (int)(threadIdx.x & ~31u) >= total) behind_loads();
-            for (int e0 = threadIdx.x; (e0 & ~31) < total; e0 += 8 * W * 32) {  // eight loads in flight per thread
-                uint4 v[8];
-#pragma unroll
-                for (int p = 0; p < 8; ++p) {
-                    const int e = e0 + p * W * 32;
-                    const int t = e & 3, par = (e >> 2) & 1, j = (e >> 3) & 3, hi = (e >> 5) & ((1 << (ts - 1)) - 1), unit_ = e >> (4 + ts);
-                    const int token = (hi << 1) | par;
-                    if (e < total && token < sa.M) v[p] = ld_dependent16(src + (int64_t)token * kc + unit_ * 16 + t * 4 + j);
-                }
-                if (OCC == 1 && e0 == threadIdx.x) behind_loads();
-#pragma unroll
-                for (int p = 0; p < 8; ++p) {
-                    const int e = e0 + p * W * 32;
-                    const int t = e & 3, par = (e >> 2) & 1, j = (e >> 3) & 3, hi = (e >> 5) & ((1 << (ts - 1)) - 1), unit_ = e >> (4 + ts);
-                    const int token = (hi << 1) | par;
-                    if (e < total && token < sa.M) dst[(((unit_ << 2) + j) << (2 + ts)) + (hi << 3) + (par << 2) + t] = v[p];
-                }
-            }
-        }
+        inexact = sk_stage_x<TOK, W, UNSC, FACTORS>(sa, smem, smem + HDR, factors, behind_loads);
     }
     if constexpr (FACTORS) inexact = __syncthreads_or(inexact);
     else __syncthreads();
@@ -384,29 +328,7 @@ __global__ void __launch_bounds__(W * 32, OCC) stream_even_kernel(const __grid_c
                         err, 0x150);
     };
     auto decode = [&](const unsigned char* code, const unsigned char* param, uint32_t (&lo)[16], uint32_t (&hi)[16]) {
-        // the scale words {row gid, row gid + 8} of this lane's group
-        const uint32_t poff = ((spg == 2 ? (uint32_t)(tig >> 1) * 8u : 0u) + (uint32_t)gid) * 4u;
-        // plane k of a unit holds word k of every (row, quarter): this lane's word sits at byte 4 * lane
-        uint32_t w[2][BITS];
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int k = 0; k < BITS; ++k) w[h][k] = sk_lds32(code + (uint32_t)(k * 256 + h * 128) + (uint32_t)lane * 4u);
-        if constexpr (UNSC) {
-            potl::pot_units32<BITS>(w[0], sa.p2, sa.bias, lo);
-            potl::pot_units32<BITS>(w[1], sa.p2, sa.bias, hi);
-            return;
-        }
-        const uint32_t scw = sk_lds32(param + poff);  // {row gid, row gid + 8}
-        if constexpr (DT == 0) {
-            potl::pot_decode32<BITS, 1>(w[0], 0, __byte_perm(scw, 0, 0x1010), lo);
-            potl::pot_decode32<BITS, 1>(w[1], 0, __byte_perm(scw, 0, 0x3232), hi);
-        } else {  // the FP16 scale rounded once to BF16
-            const uint32_t s0 = __bfloat16_as_ushort(__float2bfloat16_rn(__half2float(__ushort_as_half((uint16_t)(scw & 0xFFFFu)))));
-            const uint32_t s1 = __bfloat16_as_ushort(__float2bfloat16_rn(__half2float(__ushort_as_half((uint16_t)(scw >> 16)))));
-            potl::pot_decode32_bf16<BITS, 1>(w[0], 0, s0 * 0x10001u, lo);
-            potl::pot_decode32_bf16<BITS, 1>(w[1], 0, s1 * 0x10001u, hi);
-        }
+        sk_decode_pot<BITS, DT, UNSC>(sa, code, param, spg, lane, gid, tig, lo, hi);
     };
     // this lane's column of B (GEMV): x, or zeros if the column belongs to the other group
     auto zeros = [&]() -> const unsigned char* {
@@ -417,53 +339,7 @@ __global__ void __launch_bounds__(W * 32, OCC) stream_even_kernel(const __grid_c
     const unsigned char* xcol = zero_column ? zeros() + tig * 16 : xs + tig * 16;
     const uint32_t xstep = zero_column ? 0u : 256u;
     auto multiply = [&](const uint32_t (&lo)[16], const uint32_t (&hi)[16], const unsigned char* param, uint32_t cbu) {
-        // activations of quarter tig (of token gid): the B fragments of the eight MMAs
-        uint32_t xq[16];
-        if constexpr (XSMEM) {
-            const unsigned char* xa = TOK == 1 ? xcol + cbu * xstep
-                                               : xs + ((((cbu * 16u) << sa.token_shift) + ((((uint32_t)gid & ((1u << sa.token_shift) - 1u)) >> 1) << 3) +
-                                                        (((uint32_t)gid & 1u) << 2) + (uint32_t)tig) << 4);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const uint4 v = sk_lds128(xa + (TOK == 1 ? 64u : (64u << sa.token_shift)) * i);
-                xq[4 * i + 0] = v.x; xq[4 * i + 1] = v.y; xq[4 * i + 2] = v.z; xq[4 * i + 3] = v.w;
-            }
-        } else {
-            const bool live = TOK == 1 || gid < sa.M;
-            const uint4* xp = reinterpret_cast<const uint4*>(sa.X) + (TOK == 1 || !live ? 0 : (int64_t)gid * (sa.K / 8)) +
-                              (int64_t)cbu * 16 + tig * 4;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                uint4 v = make_uint4(0, 0, 0, 0);
-                if (live) v = ld_dependent16(xp + i);
-                xq[4 * i + 0] = v.x; xq[4 * i + 1] = v.y; xq[4 * i + 2] = v.z; xq[4 * i + 3] = v.w;
-            }
-        }
-        if constexpr (UNSC) {
-            float c[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-            for (int j = 0; j < 8; ++j) sk_mma(c, lo[2 * j], hi[2 * j], lo[2 * j + 1], hi[2 * j + 1], xq[2 * j], xq[2 * j + 1]);
-            const uint32_t scw = sk_lds32(param + ((spg == 2 ? (uint32_t)(tig >> 1) * 8u : 0u) + (uint32_t)gid) * 4u);  // {row gid, row gid + 8}
-            float2 sc = __half22float2(*reinterpret_cast<const __half2*>(&scw));
-            if constexpr (!FACTORS) {
-                acc[0][0] = fmaf(c[0], sc.x, acc[0][0]);
-                acc[0][2] = fmaf(c[2], sc.y, acc[0][2]);
-                if constexpr (TOK > 1) {
-                    acc[0][1] = fmaf(c[1], sc.x, acc[0][1]);
-                    acc[0][3] = fmaf(c[3], sc.y, acc[0][3]);
-                }
-            } else {  // the FP16 scale rounded once to BF16; times the unit's factor last, so that no product leaves FP32's range early
-                sc = __bfloat1622float2(__float22bfloat162_rn(sc));
-                const float f = factors[cbu];
-                acc[0][0] = fmaf(c[0] * sc.x, f, acc[0][0]);
-                acc[0][2] = fmaf(c[2] * sc.y, f, acc[0][2]);
-            }
-            return;
-        }
-#pragma unroll
-        for (int j = 0; j < 8; ++j)  // two accumulators: half the length of the dependent chain
-            if constexpr (DT == 0) sk_mma(acc[j & 1], lo[2 * j], hi[2 * j], lo[2 * j + 1], hi[2 * j + 1], xq[2 * j], xq[2 * j + 1]);
-            else sk_mma_bf16(acc[j & 1], lo[2 * j], hi[2 * j], lo[2 * j + 1], hi[2 * j + 1], xq[2 * j], xq[2 * j + 1]);
+        sk_multiply<TOK, XSMEM, DT, UNSC, FACTORS>(sa, lo, hi, param, cbu, spg, gid, tig, xs, xcol, xstep, factors, acc);
     };
     auto unit = [&](const unsigned char* code, const unsigned char* param, uint32_t cbu) {
         if (!unit_ok(code, param, cbu)) return;
