@@ -31,9 +31,8 @@ __device__ __forceinline__ unsigned long long exch_relaxed64(unsigned long long*
     return old;
 }
 // A sum on its way from CTA to CTA: the number in the lower half, a mark in the upper one.  What else may lie there is zero or the partial sums of a
-// product of more tokens (gemm_prefill.cu), pairs of FP32 numbers as tensor cores and FP32 additions leave them: their NaN is 0x7FFFFFFF and
-// never the mark, which is another one (PF_NO_SUM is a third).
-constexpr uint32_t SK_SUM_MARK = 0x7FD15C0Du;
+// product of more tokens (gemm_prefill.cu), pairs of FP32 numbers.  The mark is a signaling NaN, which no operation returns, and not PF_NO_SUM.
+constexpr uint32_t SK_SUM_MARK = 0x7F95C0DEu;
 __device__ __forceinline__ unsigned long long sk_marked_sum(float v) { return ((unsigned long long)SK_SUM_MARK << 32) | __float_as_uint(v); }
 __device__ __forceinline__ bool sk_is_sum(unsigned long long v) { return (uint32_t)(v >> 32) == SK_SUM_MARK; }
 // shared-memory header: as sk_header_bytes, with four words between the local arrival counters and the slots of partial sums
