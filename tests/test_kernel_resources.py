@@ -35,6 +35,8 @@ def test_sums_of_a_cluster_that_may_be_incomplete_are_not_stored():
     assert add_up.index("p[u][z].x != PF_NO_SUM") < add_up.index("if (!complete) continue;") < add_up.index("uint16_t* dst = a.Y")
     pattern = int(re.search(r"PF_NO_SUM = (0x[0-9A-F]+)u", text).group(1), 16)
     assert 0x7F800000 < pattern < 0x7FC00000   # a signaling NaN: sums of products, and NaN that additions pass on, are none
+    mark = int(re.search(r"SK_SUM_MARK = (0x[0-9A-F]+)u", (build.CSRC / "stream_even.cuh").read_text()).group(1), 16)
+    assert 0x7F800000 < mark < 0x7FC00000 and mark != pattern   # (looked for where such sums may lie)
 
 
 def test_the_scale_search_does_not_spill(tmp_path):
